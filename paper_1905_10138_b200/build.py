@@ -1,14 +1,18 @@
-"""Builds ``libsqnn.so`` (C-ABI library: host encoder + sm_100a kernels) in-tree with nvcc."""
+"""Builds ``libsqnn.so`` (C-ABI library: host encoder + sm_100a kernels) in-tree with nvcc, and
+``_sqnn_python.so`` (marshalling of torch tensors for its device entry points) with the host compiler."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIB = os.path.join(HERE, "libsqnn.so")
+PY_MODULE = os.path.join(HERE, "_sqnn_python.so")
+PY_SOURCE = "sqnn_python.cpp"
 SOURCES = ["sqnn_host.cpp", "sqnn_api.cu", "sqnn_mma.cu", "sqnn_search.cu"]
 SHAPE_SOURCE = "sqnn_shape.cu"
 # (n_out, n_in) with compile-time kernels -- the list in csrc/sqnn_shapes.h -- plus the run-time shape (0, 0)
@@ -23,16 +27,35 @@ def _nvcc() -> str:
     return "nvcc"
 
 
-def _stale() -> bool:
-    if not os.path.exists(LIB):
+def _stale(target: str, sources) -> bool:
+    if not os.path.exists(target):
         return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, s) for s in SOURCES + HEADERS] + [os.path.join(INCLUDE, "sqnn.h")]
+    t = os.path.getmtime(target)
+    deps = [os.path.join(CSRC, s) for s in sources] + [os.path.join(INCLUDE, "sqnn.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _build_python_module(force: bool) -> None:
+    """The module uses torch's C++ tensor type, so it is compiled against the headers of the installed torch."""
+    if not force and not _stale(PY_MODULE, [PY_SOURCE]):
+        return
+    from torch.utils import cpp_extension
+    import torch
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(_nvcc()))), "include")
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I", INCLUDE, "-I", sysconfig.get_paths()["include"], "-I", cuda]
+    for d in cpp_extension.include_paths():
+        cmd += ["-isystem", d]
+    for d in cpp_extension.library_paths():
+        cmd += ["-L", d]
+    cmd += [os.path.join(CSRC, PY_SOURCE), "-o", PY_MODULE, "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+    subprocess.run(cmd, check=True)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    if not force and not _stale():
+    _build_python_module(force)
+    if not force and not _stale(LIB, SOURCES + HEADERS):
         return LIB
     objdir = os.path.join(HERE, "_build")
     os.makedirs(objdir, exist_ok=True)

@@ -1,4 +1,6 @@
-"""Thin ctypes binding over ``libsqnn.so`` -- same names as ``include/sqnn.h``.
+"""Thin binding over ``libsqnn.so`` -- same names as ``include/sqnn.h``.  Host functions go through ctypes,
+the device entry points through a small C++ module (``csrc/sqnn_python.cpp``), because what a call costs
+on the host is what a small layer costs.
 
 Argument marshalling only: every step of the decode / product path runs in the library's
 kernels.  Device buffers are torch CUDA tensors (torch is used for device memory and
@@ -308,11 +310,27 @@ def _stream_ptr(stream):
     return ctypes.c_void_p(s.cuda_stream)
 
 
+_native_module = None
+
+
+def _native():
+    """The marshalling module of the device entry points (csrc/sqnn_python.cpp), bound to the loaded library."""
+    global _native_module
+    if _native_module is None:
+        import torch  # noqa: F401 -- its libraries must be loaded before the module that links against them
+        from . import _sqnn_python as mod
+        L = lib()
+        mod.bind(*(ctypes.cast(getattr(L, f), ctypes.c_void_p).value
+                   for f in ("sqnn_decode", "sqnn_decode_matmul", "sqnn_decode_matmul_static")))
+        _native_module = mod
+    return _native_module
+
+
 def sqnn_decode(desc: Desc, d_blob, d_mask, d_alpha, mode: int, d_out, d_status=None, stream=None):
     """Queues the decode kernel on ``stream`` (default: torch's current stream).  Tensors are CUDA."""
-    _check(lib().sqnn_decode(ctypes.byref(desc), _dev_ptr(d_blob), _dev_ptr(d_mask), _dev_ptr(d_alpha),
-                             int(mode), _dev_ptr(d_out), d_out.numel() * d_out.element_size(),
-                             _dev_ptr(d_status), _stream_ptr(stream)), "sqnn_decode")
+    status = (_native_module or _native()).decode(desc, d_blob, d_mask, d_alpha, mode, d_out, d_status, stream)
+    if status:
+        raise SqnnError(status, "sqnn_decode")
 
 
 def sqnn_store_probe(d_out, chunk_bytes: int = 3200, stream=None):
@@ -336,23 +354,9 @@ def sqnn_decode_matmul(desc: Desc, d_blob, d_mask, d_alpha, d_x, d_y, d_workspac
     """Y[b, r] = sum_c W[r, c] X[b, c].  d_x: [batch, n] float32 or bfloat16 (row stride free);
     d_y: [batch, m] float32.  batch >= 16 needs ``d_workspace`` of ``sqnn_workspace_bytes`` bytes.
     Queues on ``stream``; does not synchronise."""
-    import torch
-    if d_x.dim() != 2 or d_y.dim() != 2 or d_x.stride(1) != 1 or d_y.stride(1) != 1:
-        raise ValueError("X and Y must be 2-D with unit inner stride")
-    if d_x.dtype == torch.float32:
-        xdt = X_F32
-    elif d_x.dtype == torch.bfloat16:
-        xdt = X_BF16
-    else:
-        raise ValueError("X must be float32 or bfloat16")
-    if d_y.dtype != torch.float32:
-        raise ValueError("Y must be float32")
-    batch = d_x.shape[0]
-    ws_bytes = d_workspace.numel() * d_workspace.element_size() if d_workspace is not None else 0
-    _check(lib().sqnn_decode_matmul(ctypes.byref(desc), _dev_ptr(d_blob), _dev_ptr(d_mask), _dev_ptr(d_alpha),
-                                    _dev_ptr(d_x), xdt, batch, d_x.stride(0), _dev_ptr(d_y), d_y.stride(0),
-                                    _dev_ptr(d_workspace), ws_bytes, _dev_ptr(d_status), _stream_ptr(stream)),
-           "sqnn_decode_matmul")
+    status = (_native_module or _native()).matmul(desc, d_blob, d_mask, d_alpha, d_x, d_y, d_workspace, d_status, stream)
+    if status:
+        raise SqnnError(status, "sqnn_decode_matmul")
 
 
 def sqnn_decode_matmul_static(desc: Desc, d_blob, d_mask, d_alpha, d_x, d_y, d_status=None, stream=None):
@@ -361,12 +365,6 @@ def sqnn_decode_matmul_static(desc: Desc, d_blob, d_mask, d_alpha, d_x, d_y, d_s
     cannot allocate device memory (stream capture, a framework-owned heap, a frozen memory plan).
     Layers whose ``sqnn_workspace_bytes`` exceeds ``STATIC_SCRATCH_BYTES`` are refused.  Calls share
     that one array, so calls that may overlap on the GPU must be serialised by the caller."""
-    import torch
-    if d_x.dim() != 2 or d_y.dim() != 2 or d_x.stride(1) != 1 or d_y.stride(1) != 1:
-        raise ValueError("X and Y must be 2-D with unit inner stride")
-    if d_x.dtype != torch.bfloat16 or d_y.dtype != torch.float32:
-        raise ValueError("X must be bfloat16 and Y float32")
-    _check(lib().sqnn_decode_matmul_static(ctypes.byref(desc), _dev_ptr(d_blob), _dev_ptr(d_mask),
-                                           _dev_ptr(d_alpha), _dev_ptr(d_x), X_BF16, d_x.shape[0],
-                                           d_x.stride(0), _dev_ptr(d_y), d_y.stride(0), _dev_ptr(d_status),
-                                           _stream_ptr(stream)), "sqnn_decode_matmul_static")
+    status = (_native_module or _native()).matmul_static(desc, d_blob, d_mask, d_alpha, d_x, d_y, d_status, stream)
+    if status:
+        raise SqnnError(status, "sqnn_decode_matmul_static")
