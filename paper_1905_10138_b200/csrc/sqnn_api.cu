@@ -16,13 +16,13 @@ namespace sqnn {
 
 template <int N_OUT, int N_IN>
 int decode_shape(const DecodeArgs &A, sqnn_out_mode mode, const uint64_t *d_mask, const float *d_alpha,
-                 uint64_t n, void *d_out, cudaStream_t st);
+                 uint64_t n, void *d_out, const ClearArgs &clear, cudaStream_t st);
 template <int N_OUT, int N_IN>
 int gemv_shape(const DecodeArgs &A, const uint64_t *d_mask, const float *d_alpha, const void *d_x, int x_dtype,
                int64_t ldx, uint32_t batch, float *d_y, int64_t ldy, uint64_t m, uint64_t n, cudaStream_t st);
 #define SQNN_DECLARE(NO, NI)                                                                                  \
     template <> int decode_shape<NO, NI>(const DecodeArgs &, sqnn_out_mode, const uint64_t *, const float *,  \
-                                         uint64_t, void *, cudaStream_t);                                     \
+                                         uint64_t, void *, const ClearArgs &, cudaStream_t);                                   \
     template <> int gemv_shape<NO, NI>(const DecodeArgs &, const uint64_t *, const float *, const void *, int, \
                                        int64_t, uint32_t, float *, int64_t, uint64_t, uint64_t, cudaStream_t);
 SQNN_FOR_SHAPES(SQNN_DECLARE)
@@ -109,13 +109,13 @@ static int gemv_dispatch(const DecodeArgs &A, const uint64_t *d_mask, const floa
     return gemv_shape<0, 0>(A, d_mask, d_alpha, d_x, x_dtype, ldx, batch, d_y, ldy, m, n, st);
 }
 
-int decode_bits_dispatch(const DecodeArgs &A, void *d_out, cudaStream_t st)
+int decode_bits_dispatch(const DecodeArgs &A, void *d_out, const ClearArgs &clear, cudaStream_t st)
 {
 #define SQNN_BITS_CASE(NO, NI) \
-    if (A.n_out == NO && A.n_in == NI) return decode_shape<NO, NI>(A, SQNN_OUT_BITS, nullptr, nullptr, 0, d_out, st);
+    if (A.n_out == NO && A.n_in == NI) return decode_shape<NO, NI>(A, SQNN_OUT_BITS, nullptr, nullptr, 0, d_out, clear, st);
     SQNN_FOR_SHAPES(SQNN_BITS_CASE)
 #undef SQNN_BITS_CASE
-    return decode_shape<0, 0>(A, SQNN_OUT_BITS, nullptr, nullptr, 0, d_out, st);
+    return decode_shape<0, 0>(A, SQNN_OUT_BITS, nullptr, nullptr, 0, d_out, clear, st);
 }
 
 namespace {
@@ -182,10 +182,10 @@ static int decode_queue(const sqnn_desc *desc, const void *d_blob, const uint64_
     if (mode == SQNN_OUT_BF16 && (!d_mask || !d_alpha)) return SQNN_E_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)cuda_stream;
 #define SQNN_DECODE_CASE(NO, NI) \
-    if (A.n_out == NO && A.n_in == NI) return decode_shape<NO, NI>(A, mode, d_mask, d_alpha, desc->n, d_out, st);
+    if (A.n_out == NO && A.n_in == NI) return decode_shape<NO, NI>(A, mode, d_mask, d_alpha, desc->n, d_out, ClearArgs{}, st);
     SQNN_FOR_SHAPES(SQNN_DECODE_CASE)
 #undef SQNN_DECODE_CASE
-    return decode_shape<0, 0>(A, mode, d_mask, d_alpha, desc->n, d_out, st);
+    return decode_shape<0, 0>(A, mode, d_mask, d_alpha, desc->n, d_out, ClearArgs{}, st);
 }
 
 extern "C" int sqnn_decode(const sqnn_desc *desc, const void *d_blob, const uint64_t *d_mask,

@@ -45,6 +45,21 @@ struct DecodeArgs {
     PlanePtrs pl[8];
 };
 
+// Rows of Y the decode kernel clears for the product kernel that follows it (batch 0: nothing).
+struct ClearArgs {
+    float *y;
+    uint64_t m;
+    int64_t ldy;
+    uint32_t batch;
+};
+
+// Programmatic dependent launch.  A kernel of this library may be scheduled before the kernel queued ahead of
+// it has finished; wait_prior_grid() returns once that one is complete and its results are visible, and nothing
+// in global memory is read or written before it.  launch_dependents() lets the next kernel in (it waits in
+// turn for all of this one), and is called once this kernel has nothing left to wait for.
+SQNN_DEV void wait_prior_grid() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+SQNN_DEV void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+
 SQNN_DEV uint32_t extract_bits(const uint32_t *__restrict__ base, uint64_t bitpos, uint32_t width)
 {
     const uint64_t w = bitpos >> 5;

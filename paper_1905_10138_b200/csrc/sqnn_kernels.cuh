@@ -58,9 +58,11 @@ inline uint32_t decode_bits_table_words(const DecodeArgs &A, bool rep)
 // being looked up by a plane index in every step).
 template <int N_OUT, int N_IN, bool SINK, bool ONE_PLANE, bool REP>
 __global__ void __launch_bounds__(DECODE_BITS_THREADS, 1)
-k_decode_bits(DecodeArgs A, uint64_t *__restrict__ out)
+k_decode_bits(DecodeArgs A, uint64_t *__restrict__ out, const ClearArgs clear)
 {
     extern __shared__ __align__(16) uint32_t smem[];
+    wait_prior_grid();
+    launch_dependents();
     uint32_t tab_words_s;
     if constexpr (N_OUT != 0 && REP) {
         tab_words_s = table_words_replicated(N_OUT, N_IN);       // filled below, after the first fetches are out
@@ -100,6 +102,19 @@ k_decode_bits(DecodeArgs A, uint64_t *__restrict__ out)
         }
     };
 
+    if (clear.batch) {
+        // every block clears a run of Y's elements (counted without the gaps between rows)
+        const uint64_t total = clear.m * clear.batch, per = (total + gridDim.x - 1) / gridDim.x;
+        const uint64_t lo = blockIdx.x * per, hi = lo + per < total ? lo + per : total;
+        if (clear.ldy == (int64_t)clear.m) {
+            for (uint64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) clear.y[i] = 0.0f;
+        } else {
+            for (uint64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+                const uint64_t b = i / clear.m;
+                clear.y[(int64_t)b * clear.ldy + (int64_t)(i - b * clear.m)] = 0.0f;
+            }
+        }
+    }
     auto plane_of = [&](const TilePos &p) -> const PlanePtrs & { return ONE_PLANE ? A.pl[0] : A.pl[p.plane]; };
     if constexpr (N_OUT != 0) {
         using S = Shape<N_OUT, N_IN>;
@@ -344,7 +359,8 @@ inline uint32_t grid_for(uint64_t warp_tiles, uint32_t warps, uint32_t blocks_pe
 
 template <int N_OUT, int N_IN>
 inline int launch_decode(const DecodeArgs &A, sqnn_out_mode mode, const uint64_t *d_mask,
-                         const float *d_alpha, uint64_t n, void *d_out, cudaStream_t st)
+                         const float *d_alpha, uint64_t n, void *d_out, const ClearArgs &clear,
+                         cudaStream_t st)
 {
     size_t smem = 0;
     if (mode == SQNN_OUT_BITS || mode == SQNN_OUT_SINK) {
@@ -358,13 +374,16 @@ inline int launch_decode(const DecodeArgs &A, sqnn_out_mode mode, const uint64_t
         if (tab + per_warp > limit) return SQNN_E_UNSUPPORTED;
         uint32_t warps = (uint32_t)((limit - tab) / per_warp);
         if (warps > DECODE_BITS_THREADS / 32) warps = DECODE_BITS_THREADS / 32;
+        // a layer with fewer tiles than all SMs have warps: as many blocks as SMs with as few warps as that takes
+        const uint64_t share = (live * A.n_q + sm_count() - 1) / sm_count();
+        const uint32_t want = share > 4 ? (share < 32 ? (uint32_t)share : 32u) : 4u;
+        if (warps > want) warps = want;
         smem = tab + warps * per_warp;
         const uint32_t grid = grid_for(live * A.n_q, warps, 1);
 #define SQNN_BITS_LAUNCH2(SINKV, ONEV, REPV)                                                             \
     do {                                                                                                 \
         auto k = k_decode_bits<N_OUT, N_IN, SINKV, ONEV, REPV>;                                          \
-        if (prepare(k, smem)) return SQNN_E_CUDA;                                                        \
-        k<<<grid, warps * 32, smem, st>>>(A, (uint64_t *)d_out);                                         \
+        return launch_kernel(k, grid, warps * 32, smem, st, A, (uint64_t *)d_out, clear);                \
     } while (0)
 #define SQNN_BITS_LAUNCH(SINKV, ONEV)                                                                    \
     do {                                                                                                 \
@@ -403,7 +422,7 @@ inline int launch_decode(const DecodeArgs &A, sqnn_out_mode mode, const uint64_t
 // One network shape = one translation unit (sqnn_shape.cu compiled with -DSQNN_NO / -DSQNN_NI).
 template <int N_OUT, int N_IN>
 int decode_shape(const DecodeArgs &A, sqnn_out_mode mode, const uint64_t *d_mask, const float *d_alpha,
-                 uint64_t n, void *d_out, cudaStream_t st);
+                 uint64_t n, void *d_out, const ClearArgs &clear, cudaStream_t st);
 template <int N_OUT, int N_IN>
 int gemv_shape(const DecodeArgs &A, const uint64_t *d_mask, const float *d_alpha, const void *d_x, int x_dtype,
                int64_t ldx, uint32_t batch, float *d_y, int64_t ldy, uint64_t m, uint64_t n, cudaStream_t st);

@@ -9,8 +9,29 @@ int sm_count();
 // Raises a kernel's dynamic shared-memory limit when `smem` needs it; remembered per kernel and
 // device so that repeated launches cost nothing on the host.
 int ensure_dynamic_smem(const void *kernel, size_t smem);
-// Queues the packed-bits decode of every plane into `d_out` (n_q * ceil(mn/64) uint64).
-int decode_bits_dispatch(const DecodeArgs &A, void *d_out, cudaStream_t st);
+// Queues the packed-bits decode of every plane into `d_out` (n_q * ceil(mn/64) uint64); the same kernel clears
+// what `clear` describes.
+int decode_bits_dispatch(const DecodeArgs &A, void *d_out, const ClearArgs &clear, cudaStream_t st);
+
+// Launches a kernel that begins with wait_prior_grid() (sqnn_decode.cuh): it may be scheduled while the
+// kernel queued before it on the stream is finishing, so that consecutive launches do not each pay the launch
+// latency.
+template <typename... P, typename... Q>
+inline int launch_kernel(void (*kernel)(P...), uint32_t grid, uint32_t threads, size_t smem, cudaStream_t st, const Q &...args)
+{
+    if (ensure_dynamic_smem(reinterpret_cast<const void *>(kernel), smem) != SQNN_OK) return SQNN_E_CUDA;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...) == cudaSuccess ? SQNN_OK : SQNN_E_CUDA;
+}
 size_t mma_workspace_bytes(const sqnn_desc *desc, uint32_t batch);
 int mma_dispatch(const sqnn_desc *desc, const DecodeArgs &A, const uint64_t *d_mask, const float *d_alpha,
                  const void *d_x, int64_t ldx, uint32_t batch, float *d_y, int64_t ldy, void *d_workspace,

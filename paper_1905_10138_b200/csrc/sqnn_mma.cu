@@ -2,27 +2,33 @@
 //
 //   Y[b][r] = sum_i alpha[r][i] * sum_c s_i[r][c] X[b][c],      s_i = mask * (2 b_i - 1) in {-1, 0, +1}
 //
-//   D (TMEM, fp32) [128 batch rows x 256 weight rows] += A (shared, bf16, K-major) [128 x 64] . B (shared) [256 x 64]^T
+//   D_u (TMEM, fp32) [128 weight rows x N batch rows] += A (TMEM, bf16) [128 x 64] . B (shared, bf16, K-major) [N x 64]^T
 //
-// One CTA owns 256 rows of W of ONE plane and a range of columns.  Per 64-column step
-//   - one thread fetches the activations X[bc .. bc+128) x [64 columns] with TMA into the A stage (every CTA
-//     fetches its own tile; rows past the batch are filled with zeros by the copy engine);
-//   - the decode warps expand the plane's sign tile -1 / 0 / +1 (mask and sign only, four weights per table
-//     read) into the B stage (bf16, 128-byte rows, 128-byte swizzle) -- the expanded weights exist only in
-//     shared memory;
-//   - one thread issues tcgen05.mma (M = 128, N = 256, K = 16 each) that accumulate in tensor memory, never
-//     twice in a row into the same accumulator.
-// A tcgen05.mma of M = 128 takes about as long whatever its N, so the weight rows sit on the N side at the
-// full N = 256.  The scale alpha[r][i] is applied to the accumulator in the epilogue, so the weights stay
-// exact (one tile of rescaled weights rounded to bf16 would not meet the tolerance: a row has only 2^n_q
-// distinct values and their rounding errors add up coherently).  Planes and column ranges of different CTAs
-// are summed with fp32 vector reductions on Y (cleared beforehand).  Batches beyond 128 are taken 128 rows
-// at a time, two accumulators (256 batch rows) per pass over the columns.
+// The planes have been decoded to packed bits in the workspace by the tiled decode kernel (queued just before
+// this one) and sit in L2.  A tile of work is a group of rows (one or two times 128), a group of planes and a
+// chunk of N batch rows; its units u = (128 rows, plane) have an accumulator each and share the activation
+// tile.  Per 64-column step and unit
+//   - one thread fetches the activations with TMA (once for all units; rows past the batch and columns past n
+//     are filled with zeros by the copy engine);
+//   - the four warps of an expander group turn 64 bits of mask and plane per row into bf16 in registers and
+//     store them to a slot of tensor memory (lane = weight row), so the expanded weights never touch shared
+//     memory: its bandwidth is left to the activation operand;
+//   - the unit's own MMA warp issues four tcgen05.mma (M = 128, K = 16, A from tensor memory) and commits the
+//     slot.  (One warp for all units could not keep up: with its instruction stream evicted by the expanders'
+//     between steps, a step of 256 tensor-core cycles took it 340.)
+// The scale alpha[r][i] is applied to the accumulator in the epilogue, so the weights stay exact (one tile of
+// rescaled weights rounded to bf16 would not meet the tolerance: a row has only 2^n_q distinct values and
+// their rounding errors add up coherently).
 //
-// Where the bits come from.  The planes have been decoded to packed bits in the workspace by the tiled
-// decode kernel (queued just before this one) and sit in L2.  A decode thread owns (row, half of a 64-column
-// step); when rows start on 16-byte boundaries it takes the bits of 256 columns with one 16-byte load per
-// vector (plane, mask) and trades words with its neighbour by shuffle, otherwise it reads word by word.
+// Expansion.  A weight is 0, +2 or -2 in bf16 (0x0000, 0x4000, 0xc000; the factor 2 is taken out of alpha):
+// only the two top bits of a half word carry information, so once mask and sign bits are interleaved (mask bit
+// 2f, sign bit 2f + 1 of a half word, even columns in the low, odd ones in the high half) two weights cost one
+// shift and one AND.
+//
+// Split of the work.  All tiles x 256-column macros form one line that is cut into equal runs, one per CTA and
+// at most one CTA per SM, whatever the shape; a CTA's run covers one or more tiles in part, and each part is
+// added to Y (cleared by the decode kernel) with coalesced fp32 reductions.  Within a part the expander groups
+// take units and column ranges in turn, so that consecutive slots come from different groups.
 //
 // Every wait on an mbarrier is bounded; a wait that gives up sets SQNN_E_TIMEOUT in the status word and
 // makes all roles leave their loops, so the kernel always frees its tensor memory and returns.
@@ -39,18 +45,15 @@ namespace sqnn {
 
 namespace {
 
-constexpr uint32_t NROWS = 256;           // rows of W per CTA = MMA N
-constexpr uint32_t MB = 128;              // batch rows per accumulator = MMA M
-constexpr uint32_t KC = 64;               // columns per pipeline step
-constexpr uint32_t MACRO = 256;           // columns whose bits a decode thread takes at a time
-constexpr uint32_t STEPS_PER_MACRO = MACRO / KC;
-constexpr uint32_t LUT_COPIES = 16;       // copies of the 256-entry sign table: lane l of a half-warp reads copy l
-constexpr uint32_t DEC_WARPS = 16;
-constexpr uint32_t DEC_THREADS = DEC_WARPS * 32;
-constexpr uint32_t THREADS = DEC_THREADS + 64;  // + TMA warp + MMA warp
-constexpr uint32_t B_STAGE_BYTES = NROWS * KC * 2;
-constexpr uint32_t A_TILE_BYTES = MB * KC * 2;
-constexpr uint32_t MAX_STAGES = 4;
+constexpr uint32_t MROWS = 128;           // weight rows per unit = MMA M = TMEM lanes
+constexpr uint32_t KC = 64;               // columns per step (one A slot, one X stage)
+constexpr uint32_t STEPS = 4;             // steps per macro
+constexpr uint32_t MACRO = KC * STEPS;    // columns whose bits an expander thread takes at a time
+constexpr uint32_t MAX_SLOTS = 8;         // A slots per unit
+constexpr uint32_t MAX_XSTAGES = 12;
+constexpr uint32_t MAX_UNITS = 4;
+constexpr uint32_t MAX_ACC_COLS = 384;    // TMEM columns of all accumulators; the other 128 and more are A slots
+constexpr uint32_t XSTAGE_BUDGET = 192 * 1024;
 constexpr uint64_t WAIT_LIMIT_CYCLES = 4000000000ull;   // about 2 s at 2 GHz
 
 // Set by sqnn_set_debug_flags (for the library's own tests).
@@ -61,19 +64,22 @@ struct MmaArgs {
     const uint32_t *bits32;       // decoded planes in the workspace
     uint64_t plane_words32;       // 32-bit words per plane in the workspace
     const uint32_t *mask32;
-    uint64_t mask_words32;        // number of valid 32-bit mask words
     const float *alpha;
     float *y;
     int64_t ldy;
     uint64_t m, n;
     uint32_t n_q;
     uint32_t batch;
-    uint32_t nchunks;             // accumulators (128 batch rows each) per pass: 1 or 2
-    uint32_t stages;
-    uint32_t splits;              // CTAs per (row tile, plane)
-    uint32_t macros_per_split;
-    uint32_t aligned;             // 1: rows of the packed vectors start on 16-byte boundaries
-    uint32_t vec_y;               // 1: Y rows allow 16-byte vector reductions
+    uint32_t N;                   // batch rows per tile = MMA N (multiple of 16)
+    uint32_t chunks;              // batch chunks
+    uint32_t mt;                  // 128-row groups per tile
+    uint32_t planes;              // planes per tile
+    uint32_t plane_groups;
+    uint32_t phases;              // column ranges the expander groups of one unit take side by side
+    uint32_t macros;              // 256-column macros per row
+    uint64_t total;               // tiles x macros
+    uint32_t slots, xstages;      // A slots per unit (a power of two), X stages
+    uint32_t acc_cols;            // first TMEM column of the A slots
     uint32_t skip_loads;          // test only: the TMA role issues no loads
     uint64_t wait_limit;          // cycles a bounded wait may take
     uint32_t *status;
@@ -82,31 +88,28 @@ struct MmaArgs {
 // ---------------------------------------------------------------------------------------
 // PTX wrappers
 // ---------------------------------------------------------------------------------------
-SQNN_DEV void mbar_init(uint64_t *bar, uint32_t count)
+SQNN_DEV void mbar_init(uint32_t bar, uint32_t count)
 {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" :: "r"(smem_addr(bar)), "r"(count) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" :: "r"(bar), "r"(count) : "memory");
 }
-SQNN_DEV void mbar_arrive(uint64_t *bar)
+SQNN_DEV void mbar_arrive(uint32_t bar)
 {
-    asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" :: "r"(smem_addr(bar)) : "memory");
+    asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" :: "r"(bar) : "memory");
 }
-SQNN_DEV void mbar_expect_tx(uint64_t *bar, uint32_t bytes)
+SQNN_DEV void mbar_expect_tx(uint32_t bar, uint32_t bytes)
 {
     asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n}\n"
-                 :: "r"(smem_addr(bar)), "r"(bytes) : "memory");
+                 :: "r"(bar), "r"(bytes) : "memory");
 }
-SQNN_DEV bool mbar_try(uint64_t *bar, uint32_t parity)
+SQNN_DEV bool mbar_try(uint32_t bar, uint32_t parity)
 {
-    // The last operand lets the hardware park the thread for up to ~1 ms while the phase is
-    // pending (it wakes as soon as the phase completes), so that waiting threads do not take
-    // issue slots from working ones; the caller's loop still bounds the total wait.
     uint32_t ok;
-    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}\n"
-                 : "=r"(ok) : "r"(smem_addr(bar)), "r"(parity), "r"(1000000u) : "memory");
+    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
 // Bounded wait.  Returns false if the wait was abandoned (limit reached or another role gave up).
-SQNN_DEV bool mbar_wait(uint64_t *bar, uint32_t parity, volatile uint32_t *abort_flag, uint32_t *status, uint64_t limit)
+SQNN_DEV bool mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag, uint32_t *status, uint64_t limit)
 {
     if (mbar_try(bar, parity)) return true;
     const long long t0 = clock64();
@@ -120,10 +123,23 @@ SQNN_DEV bool mbar_wait(uint64_t *bar, uint32_t parity, volatile uint32_t *abort
         }
     }
 }
-SQNN_DEV void tma_load_2d(void *sdst, const CUtensorMap *map, uint64_t *bar, int32_t x, int32_t y)
+// The same for a converged warp: true in all lanes or in none.  (One instruction of a converged warp gives all
+// its lanes the same answer, so only the slow way needs a vote.)
+SQNN_DEV bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag, uint32_t *status, uint64_t limit)
+{
+    if (mbar_try(bar, parity)) return true;
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status, limit));
+}
+// The same without a report, for copies that must land before the kernel may leave.
+SQNN_DEV void mbar_drain(uint32_t bar, uint32_t parity, uint64_t limit)
+{
+    const long long t0 = clock64();
+    while (!mbar_try(bar, parity) && (uint64_t)(clock64() - t0) <= limit) {}
+}
+SQNN_DEV void tma_load_2d(uint32_t sdst, const CUtensorMap *map, uint32_t bar, int32_t x, int32_t y)
 {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];\n"
-                 :: "r"(smem_addr(sdst)), "l"(map), "r"(smem_addr(bar)), "r"(x), "r"(y) : "memory");
+                 :: "r"(sdst), "l"(map), "r"(bar), "r"(x), "r"(y) : "memory");
 }
 SQNN_DEV void tmem_alloc(uint32_t *slot, uint32_t cols)
 {
@@ -137,35 +153,62 @@ SQNN_DEV void tmem_dealloc(uint32_t taddr, uint32_t cols)
 }
 SQNN_DEV void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
 SQNN_DEV void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
-SQNN_DEV void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
+// The tcgen05.mma of one A slot (SLICES of K = 16) and the commit that frees it, by one elected lane of a
+// converged warp: A from tensor memory (128 lanes x 16 bf16 each, two per column), B from shared memory.
+// Issued from converged code the operands are uniform registers; issued under a lane test they were moved
+// there one by one and a step took over 800 cycles instead of the 256 the tensor cores need at N = 128.
+template <uint32_t SLICES>
+SQNN_DEV void mma_slot(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate, uint32_t free_a)
 {
-    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                 " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-                 :: "r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
+    static_assert(SLICES == 2 || SLICES == 4, "slots of 32 or 64 columns");
+    if constexpr (SLICES == 4) {
+        asm volatile("{\n .reg .pred e, p, t;\n .reg .b32 a1, a2, a3;\n .reg .b64 b1, b2, b3;\n"
+                     " elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %4, 0;\n setp.eq.b32 t, %4, %4;\n"
+                     " add.u32 a1, %1, 8;\n add.u32 a2, %1, 16;\n add.u32 a3, %1, 24;\n"
+                     " add.u64 b1, %2, 2;\n add.u64 b2, %2, 4;\n add.u64 b3, %2, 6;\n"
+                     " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n"
+                     " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a1], b1, %3, t;\n"
+                     " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a2], b2, %3, t;\n"
+                     " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a3], b3, %3, t;\n"
+                     " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n}\n"
+                     :: "r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(free_a) : "memory");
+    } else {
+        asm volatile("{\n .reg .pred e, p, t;\n .reg .b32 a1;\n .reg .b64 b1;\n"
+                     " elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %4, 0;\n setp.eq.b32 t, %4, %4;\n"
+                     " add.u32 a1, %1, 8;\n add.u64 b1, %2, 2;\n"
+                     " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n"
+                     " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a1], b1, %3, t;\n"
+                     " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n}\n"
+                     :: "r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(free_a) : "memory");
+    }
 }
-// Makes the mbarrier track completion of all MMAs this thread issued so far.
-SQNN_DEV void mma_commit(uint64_t *bar)
+// Makes the mbarrier track completion of all MMAs the elected lane issued so far (converged warp).
+SQNN_DEV void mma_commit(uint32_t bar)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
-                 :: "r"(smem_addr(bar)) : "memory");
+    asm volatile("{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
+                 " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n"
+                 :: "r"(bar) : "memory");
 }
-// 32 consecutive accumulator columns of this thread's lane (one wait for the whole load).
-SQNN_DEV void tmem_ld32(uint32_t taddr, uint32_t (&v)[32])
+// 16 consecutive accumulator columns of this thread's lane (one wait for the whole load).
+SQNN_DEV void tmem_ld16(uint32_t taddr, uint32_t (&v)[16])
 {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-                 "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n"
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n"
                  : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                   "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-                   "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
-                   "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+                   "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
                  : "r"(taddr) : "memory");
     asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 }
-SQNN_DEV void red_add_v4(float *gdst, float a, float b, float c, float d)
+// 16 consecutive columns of this thread's lane; tmem_st_wait() completes all stores of the warp.
+SQNN_DEV void tmem_st16(uint32_t taddr, const uint32_t *v)
 {
-    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};\n" :: "l"(gdst), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], "
+                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15};\n"
+                 :: "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
+                    "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]),
+                    "r"(taddr) : "memory");
 }
+SQNN_DEV void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
 
 // Shared-memory matrix descriptor of a K-major bf16 tile with 128-byte rows and 128-byte
 // swizzle: rows 128 B apart, groups of 8 rows 1024 B apart (stride byte offset), descriptor
@@ -184,301 +227,296 @@ SQNN_DEV uint64_t smem_desc_sw128(uint32_t addr)
 // Instruction descriptor: D fp32, A and B bf16, both K-major, M = 128, N = n.
 SQNN_DEV uint32_t instr_desc_bf16(uint32_t n)
 {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | ((MB >> 4) << 24);
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | ((MROWS >> 4) << 24);
 }
 
-// Barrier over the decode threads that also ORs a flag, so that all of them take the same exit.
-SQNN_DEV bool decode_barrier_any(uint32_t flagged)
+// Expands 32 columns (mask word m, plane word b, bit j = column j) into 16 registers of two bf16 each.
+SQNN_DEV void expand32(uint32_t m, uint32_t b, uint32_t *v)
 {
-    uint32_t any;
-    asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 q, %1, 0;\n bar.red.or.pred p, 1, %2, q;\n selp.u32 %0, 1, 0, p;\n}\n"
-                 : "=r"(any) : "r"(flagged), "n"(DEC_THREADS) : "memory");
-    return any != 0;
+    const uint32_t s = ~b;                                                    // bit set: minus
+    const uint32_t even = (m & 0x55555555u) | ((s << 1) & 0xaaaaaaaau);       // fields of columns 0, 2, .. 30
+    const uint32_t odd = ((m >> 1) & 0x55555555u) | (s & 0xaaaaaaaau);        // fields of columns 1, 3, .. 31
+    const uint32_t z0 = __byte_perm(even, odd, 0x5410), z1 = __byte_perm(even, odd, 0x7632);
+#pragma unroll
+    for (uint32_t j = 0; j < 8; ++j) {
+        v[j] = (z0 << (14 - 2 * j)) & 0xc000c000u;
+        v[8 + j] = (z1 << (14 - 2 * j)) & 0xc000c000u;
+    }
 }
 
-// 32 bits of a packed vector starting at bit position p (words past `valid` read as zero).
-SQNN_DEV uint32_t bits_at(const uint32_t *__restrict__ src, uint64_t valid, uint64_t p)
-{
-    const uint64_t w = p >> 5;
-    const uint32_t sh = (uint32_t)(p & 31);
-    const uint32_t lo = w < valid ? __ldg(src + w) : 0u;
-    const uint32_t hi = (sh != 0 && w + 1 < valid) ? __ldg(src + w + 1) : 0u;
-    return __funnelshift_r(lo, hi, sh);
-}
+// Bits of 256 columns of one row as eight words.  ALIGNED: rows start on 16-byte boundaries; otherwise the
+// three 16-byte vectors that cover them are fetched and shifted into place when the bits are used.
+template <bool ALIGNED>
+struct MacroBits {
+    static constexpr uint32_t RAW = ALIGNED ? 8 : 12;
+    uint32_t t[RAW];
+    // first, last: valid words of the vector counted from `base` (16-byte aligned); pos: bit position from `base`
+    SQNN_DEV void fetch(const uint32_t *__restrict__ base, uint64_t first, uint64_t last, uint64_t pos)
+    {
+        const uint64_t w = (pos >> 7) << 2;
+        if (w >= first && w + RAW <= last) {
+#pragma unroll
+            for (uint32_t k = 0; k < RAW; k += 4)
+                asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                             : "=r"(t[k]), "=r"(t[k + 1]), "=r"(t[k + 2]), "=r"(t[k + 3]) : "l"(base + w + k));
+        } else {
+#pragma unroll
+            for (uint32_t k = 0; k < RAW; ++k) {
+                t[k] = 0u;
+                if (w + k >= first && w + k < last) t[k] = base[w + k];
+            }
+        }
+    }
+    SQNN_DEV void take(uint32_t shift, uint32_t (&out)[8])
+    {
+        uint32_t q[RAW];
+#pragma unroll
+        for (uint32_t k = 0; k < RAW; ++k) q[k] = settle(t[k]);
+        if constexpr (!ALIGNED) {
+            const bool two = (shift & 64u) != 0, one = (shift & 32u) != 0;
+#pragma unroll
+            for (uint32_t k = 0; k < 10; ++k) q[k] = two ? q[k + 2] : q[k];
+#pragma unroll
+            for (uint32_t k = 0; k < 9; ++k) q[k] = one ? q[k + 1] : q[k];
+#pragma unroll
+            for (uint32_t k = 0; k < 8; ++k) out[k] = __funnelshift_r(q[k], q[k + 1], shift & 31u);
+        } else {
+#pragma unroll
+            for (uint32_t k = 0; k < 8; ++k) out[k] = q[k];
+        }
+    }
+};
 
-__global__ void __launch_bounds__(THREADS, 1)
+// One part of the work of a CTA: macros [m0, m0 + len) of a tile, and how the phases share them.
+struct Part {
+    uint32_t chunk, pg, group;    // batch chunk, plane group, row group
+    uint32_t m0, len, base, rem;  // phase p takes base + (p < rem) macros from first(p) on
+    SQNN_DEV Part(const MmaArgs &M, uint64_t pos, uint64_t end)
+    {
+        const uint64_t tile = pos / M.macros;
+        m0 = (uint32_t)(pos - tile * M.macros);
+        const uint64_t left = end - pos;
+        len = M.macros - m0 < left ? M.macros - m0 : (uint32_t)left;
+        chunk = (uint32_t)(tile % M.chunks);
+        const uint64_t rest = tile / M.chunks;
+        pg = (uint32_t)(rest % M.plane_groups);
+        group = (uint32_t)(rest / M.plane_groups);
+        base = len / M.phases;
+        rem = len - base * M.phases;
+    }
+    SQNN_DEV uint32_t first(uint32_t p) const { return m0 + p * base + (p < rem ? p : rem); }
+    SQNN_DEV uint32_t count(uint32_t p) const { return base + (p < rem ? 1u : 0u); }
+    SQNN_DEV uint32_t rounds() const { return base + (rem ? 1u : 0u); }
+    SQNN_DEV uint32_t active(uint32_t i, uint32_t phases) const { return i < base ? phases : rem; }
+};
+
+// Order of the X stages inside a part, the same for all roles: round i (one macro of every active phase), step h
+// of the macro, phase p.  Every unit has its own ring of A slots, filled in that order; a slot holds SLOT_COLS
+// TMEM columns (two bf16 each): the 64 columns of a step, or half of them where the accumulators leave less.
+template <bool ALIGNED, uint32_t SLOT_COLS>
+__global__ void __launch_bounds__(4 * MAX_UNITS * 32 + 32 + MAX_UNITS * 32, 1)
 k_decode_mma(const __grid_constant__ CUtensorMap xmap, const MmaArgs M)
 {
     extern __shared__ __align__(16) uint8_t smem_raw[];
-    // carve shared memory (A / B stages need 1024-byte alignment for the 128-byte swizzle)
-    uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint8_t *b_stages = base;                                               // [stage][256 rows][128 B]
-    const uint32_t a_stage_bytes = M.nchunks * A_TILE_BYTES;
-    uint8_t *a_stages = b_stages + M.stages * B_STAGE_BYTES;                 // [stage][chunk][128 rows][128 B]
-    uint2 *lut256 = reinterpret_cast<uint2 *>(a_stages + M.stages * a_stage_bytes);   // [256][LUT_COPIES]
-    float *alpha_s = reinterpret_cast<float *>(lut256 + 256 * LUT_COPIES);  // [256]
-    uint64_t *bars = reinterpret_cast<uint64_t *>(alpha_s + NROWS);
-    uint64_t *full_a = bars, *full_b = bars + MAX_STAGES, *empty = bars + 2 * MAX_STAGES;
-    uint64_t *accum = bars + 3 * MAX_STAGES;
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(accum + 1);
-    volatile uint32_t *abort_flag = tmem_slot + 1;
-
+    __shared__ uint64_t bars[2 * MAX_UNITS * MAX_SLOTS + 2 * MAX_XSTAGES + 2];
+    __shared__ uint32_t tmem_slot, abort_word;
+    const uint32_t x_sa = (smem_addr(smem_raw) + 1023u) & ~1023u;
+    volatile uint32_t *abort_flag = &abort_word;
+    // barriers by shared address: barrier i of a kind is 8 i bytes further on
+    const uint32_t full_a = smem_addr(bars), empty_a = full_a + 8 * MAX_UNITS * MAX_SLOTS, full_x = empty_a + 8 * MAX_UNITS * MAX_SLOTS;
+    const uint32_t empty_x = full_x + 8 * MAX_XSTAGES, accum = empty_x + 8 * MAX_XSTAGES, acc_free = accum + 8;
     const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // work item: (row tile, plane, column range)
-    const uint32_t split = blockIdx.x % M.splits;
-    const uint32_t plane = (blockIdx.x / M.splits) % M.n_q;
-    const uint32_t row_tile = blockIdx.x / (M.splits * M.n_q);
-    const uint64_t r0 = (uint64_t)row_tile * NROWS;
-    const uint32_t total_macros = (uint32_t)((M.n + MACRO - 1) / MACRO);
-    const uint32_t macro_begin = split * M.macros_per_split;
-    const uint32_t macro_end = macro_begin + M.macros_per_split < total_macros ? macro_begin + M.macros_per_split : total_macros;
-    const uint32_t total_steps = (uint32_t)((M.n + KC - 1) / KC);
-    const uint32_t step_begin = macro_begin * STEPS_PER_MACRO;
-    const uint32_t step_end = macro_end * STEPS_PER_MACRO < total_steps ? macro_end * STEPS_PER_MACRO : total_steps;
-    const uint32_t nsteps = step_end > step_begin ? step_end - step_begin : 0;
-    // Two accumulators always: with two batch chunks one per chunk; with one chunk the K = 16 slices
-    // alternate between them and the epilogue adds them up.  (Measured: a tcgen05.mma that accumulates
-    // into the accumulator of the one before it is issued about 300 cycles after it at N = 256; when
-    // consecutive ones go to different accumulators the spacing is about 160 cycles.)
-    const uint32_t tmem_cols = 2 * NROWS;
+    const uint32_t units = M.mt * M.planes, groups = units * M.phases;       // expander groups of four warps
+    const uint32_t x_bytes = M.N * KC * 2;
+    const uint64_t begin = M.total * blockIdx.x / gridDim.x, end = M.total * (blockIdx.x + 1) / gridDim.x;
+    constexpr uint32_t PER_STEP = KC / 2 / SLOT_COLS;                        // slots per step
+    const uint32_t slot_mask = M.slots - 1, slot_shift = 31 - __clz((int)M.slots);
 
     if (tid == 0) {
-        for (uint32_t s = 0; s < MAX_STAGES; ++s) {
-            mbar_init(full_b + s, DEC_WARPS);        // one arrival per decode warp
-            mbar_init(full_a + s, 1);
-            mbar_init(empty + s, 1);
-        }
-        mbar_init(accum, 1);
-        *abort_flag = 0;
+        for (uint32_t s = 0; s < M.slots * units; ++s) { mbar_init(full_a + 8 * s, 4); mbar_init(empty_a + 8 * s, 1); }
+        for (uint32_t s = 0; s < M.xstages; ++s) { mbar_init(full_x + 8 * s, 1); mbar_init(empty_x + 8 * s, units); }
+        mbar_init(accum, units);
+        mbar_init(acc_free, 4 * groups);
+        abort_word = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
-    if (warp == DEC_WARPS + 1) tmem_alloc(tmem_slot, tmem_cols);
-    if (tid < 256) {
-        // 4 weights at a time: index = mask nibble << 4 | bit nibble -> 4 bf16 of -1, 0, +1
-        uint32_t h[4];
+    if (warp == 4 * groups + 1) tmem_alloc(&tmem_slot, 512);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = tmem_slot;
+    launch_dependents();
+
+    if (warp < 4 * groups) {
+        // ------------------------------ expander groups ------------------------------
+        const uint32_t g = warp >> 2, quad = warp & 3;
+        const uint32_t u = g % units, p = g / units;
+        const uint32_t lane_sel = (quad * 32) << 16;
+        const uint32_t *mask_base = reinterpret_cast<const uint32_t *>(reinterpret_cast<uintptr_t>(M.mask32) & ~(uintptr_t)15);
+        const uint64_t mask_first = (uint64_t)(M.mask32 - mask_base), mask_last = mask_first + M.plane_words32;
+        uint32_t seq0 = 0, part_no = 0;
+        wait_prior_grid();                                   // workspace and cleared Y are in place
+        for (uint64_t pos = begin; pos < end;) {
+            const Part P(M, pos, end);
+            const uint64_t row_in = (uint64_t)P.group * M.mt * MROWS + (u / M.planes) * MROWS + quad * 32 + lane;
+            const uint64_t row = row_in < M.m ? row_in : M.m - 1;           // rows past the end repeat the last one
+            uint32_t plane = P.pg * M.planes + u % M.planes;
+            if (plane >= M.n_q) plane = M.n_q - 1;                          // weighted with zero in the epilogue
+            const uint64_t plane_at = (uint64_t)plane * M.plane_words32;    // the workspace is 256-byte aligned
+            const uint64_t c0 = row * M.n + (uint64_t)P.first(p) * MACRO;
+            uint64_t pos_m = mask_first * 32 + c0, pos_b = plane_at * 32 + c0;
+            const uint32_t shift_m = (uint32_t)pos_m & 127u, shift_b = (uint32_t)pos_b & 127u;
+            const uint32_t count = P.count(p);
+            MacroBits<ALIGNED> fm, fb;
+            if (count) {
+                fm.fetch(mask_base, mask_first, mask_last, pos_m);
+                fb.fetch(M.bits32, plane_at, plane_at + M.plane_words32, pos_b);
+            }
+            uint32_t seq = seq0;
+            bool stop = false;
+            for (uint32_t i = 0; i < count && !stop; ++i) {
+                uint32_t mw[8], bw[8];
+                fm.take(shift_m, mw);
+                fb.take(shift_b, bw);
+                if (i + 1 < count) {
+                    pos_m += MACRO;
+                    pos_b += MACRO;
+                    fm.fetch(mask_base, mask_first, mask_last, pos_m);
+                    fb.fetch(M.bits32, plane_at, plane_at + M.plane_words32, pos_b);
+                }
+                const uint32_t act = P.active(i, M.phases);
 #pragma unroll
-        for (uint32_t k = 0; k < 4; ++k)
-            h[k] = ((tid >> (4 + k)) & 1u) ? (((tid >> k) & 1u) ? 0x3f80u : 0xbf80u) : 0u;
+                for (uint32_t h = 0; h < STEPS; ++h) {
+                    if (stop) continue;
+                    uint32_t v[32];
+                    expand32(mw[2 * h], bw[2 * h], v);
+                    expand32(mw[2 * h + 1], bw[2 * h + 1], v + 16);
 #pragma unroll
-        for (uint32_t c = 0; c < LUT_COPIES; ++c)
-            lut256[tid * LUT_COPIES + c] = make_uint2(h[0] | (h[1] << 16), h[2] | (h[3] << 16));
-    } else if (tid < 256 + NROWS) {
-        const uint64_t r = r0 + (tid - 256);
-        alpha_s[tid - 256] = r < M.m ? __ldg(M.alpha + r * M.n_q + plane) : 0.0f;
+                    for (uint32_t part = 0; part < PER_STEP; ++part) {
+                        const uint32_t s = seq + (h * act + p) * PER_STEP + part, use = s >> slot_shift;
+                        const uint32_t slot = u * M.slots + (s & slot_mask);
+                        if (stop) continue;
+                        if (use > 0) {
+                            if (!mbar_wait_warp(empty_a + 8 * slot, (use - 1) & 1u, abort_flag, M.status, M.wait_limit)) { stop = true; continue; }
+                            tc_fence_after();
+                        }
+                        const uint32_t at = tmem_base + lane_sel + M.acc_cols + slot * SLOT_COLS;
+#pragma unroll
+                        for (uint32_t k = 0; k < SLOT_COLS; k += 16) tmem_st16(at + k, v + part * SLOT_COLS + k);
+                        tmem_st_wait();
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(full_a + 8 * slot);
+                    }
+                }
+                seq += STEPS * act * PER_STEP;
+            }
+            seq0 += STEPS * P.len * PER_STEP;
+            // ------------------------------ epilogue of the part ------------------------------
+            if (stop || !mbar_wait_warp(accum, part_no & 1u, abort_flag, M.status, M.wait_limit)) break;
+            tc_fence_after();
+            const uint32_t b0 = P.chunk * M.N;
+            for (uint32_t t = 0; t < M.mt; ++t) {
+                const uint64_t r = ((uint64_t)P.group * M.mt + t) * MROWS + quad * 32 + lane;
+                float al[MAX_UNITS];
+#pragma unroll
+                for (uint32_t k = 0; k < MAX_UNITS; ++k) {
+                    const uint32_t pl = P.pg * M.planes + k;
+                    al[k] = k < M.planes && pl < M.n_q && r < M.m ? 0.5f * __ldg(M.alpha + r * M.n_q + pl) : 0.0f;
+                }
+                for (uint32_t j = g; j < M.N / 16; j += groups) {
+                    if (b0 + j * 16 >= M.batch) break;
+                    float sum[16];
+#pragma unroll
+                    for (uint32_t e = 0; e < 16; ++e) sum[e] = 0.0f;
+#pragma unroll
+                    for (uint32_t k = 0; k < MAX_UNITS; ++k) {
+                        if (k >= M.planes) break;
+                        uint32_t d[16];
+                        tmem_ld16(tmem_base + lane_sel + (t * M.planes + k) * M.N + j * 16, d);
+#pragma unroll
+                        for (uint32_t e = 0; e < 16; ++e) sum[e] = fmaf(al[k], __uint_as_float(d[e]), sum[e]);
+                    }
+                    if (r < M.m) {
+                        float *dst = M.y + (int64_t)(b0 + j * 16) * M.ldy + (int64_t)r;
+#pragma unroll
+                        for (uint32_t e = 0; e < 16; ++e)
+                            if (b0 + j * 16 + e < M.batch) atomicAdd(dst + (int64_t)e * M.ldy, sum[e]);
+                    }
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acc_free);
+            ++part_no;
+            pos += P.len;
+        }
+    } else if (warp == 4 * groups) {
+        // ------------------------------ activations by TMA ------------------------------
+        if (lane == 0 && !M.skip_loads) {
+            uint32_t stage = 0, use = 0;
+            bool ok = true;
+            for (uint64_t pos = begin; pos < end && ok;) {
+                const Part P(M, pos, end);
+                for (uint32_t i = 0; i < P.rounds() && ok; ++i) {
+                    const uint32_t act = P.active(i, M.phases);
+                    for (uint32_t h = 0; h < STEPS && ok; ++h)
+                        for (uint32_t p = 0; p < act && ok; ++p) {
+                            if (use > 0) ok = mbar_wait(empty_x + 8 * stage, (use - 1) & 1u, abort_flag, M.status, M.wait_limit);
+                            if (!ok) break;
+                            mbar_expect_tx(full_x + 8 * stage, x_bytes);
+                            tma_load_2d(x_sa + stage * x_bytes, &xmap, full_x + 8 * stage,
+                                        (int32_t)((P.first(p) + i) * MACRO + h * KC), (int32_t)(P.chunk * M.N));
+                            if (++stage == M.xstages) { stage = 0; ++use; }
+                        }
+                }
+                pos += P.len;
+            }
+            // after a wait that gave up: copies in flight must land before the block's shared memory goes away
+            if (!ok)
+                for (uint32_t s = 0; s < M.xstages; ++s) {
+                    const uint32_t issued = use + (s < stage ? 1u : 0u);
+                    if (issued) mbar_drain(full_x + 8 * s, (issued - 1) & 1u, M.wait_limit);
+                }
+        }
+    } else {
+        // ------------------------------ MMA issuers (one converged warp per unit) ------------------------------
+        const uint32_t u = warp - (4 * groups + 1);
+        const uint32_t idesc = instr_desc_bf16(M.N), d_tmem = tmem_base + u * M.N, a_tmem = tmem_base + M.acc_cols;
+        // descriptors differ only in the start-address field (units of 16 bytes)
+        const uint64_t x_desc0 = smem_desc_sw128(x_sa);
+        const uint32_t x_step = x_bytes >> 4;
+        uint32_t stage = 0, x_parity = 0, seq = 0, part_no = 0;
+        bool ok = true;
+        for (uint64_t pos = begin; pos < end && ok;) {
+            const Part P(M, pos, end);
+            if (part_no) ok = mbar_wait_warp(acc_free, (part_no - 1) & 1u, abort_flag, M.status, M.wait_limit);
+            const uint32_t steps = STEPS * P.len;
+            for (uint32_t k = 0; k < steps && ok; ++k) {
+                ok = mbar_wait_warp(full_x + 8 * stage, x_parity, abort_flag, M.status, M.wait_limit);
+#pragma unroll
+                for (uint32_t part = 0; part < PER_STEP; ++part, ++seq) {
+                    const uint32_t slot = u * M.slots + (seq & slot_mask);
+                    ok = ok && mbar_wait_warp(full_a + 8 * slot, (seq >> slot_shift) & 1u, abort_flag, M.status, M.wait_limit);
+                    if (!ok) break;
+                    tc_fence_after();
+                    // the first step of a part overwrites the accumulator
+                    mma_slot<SLOT_COLS / 8>(d_tmem, a_tmem + slot * SLOT_COLS, x_desc0 + stage * x_step + part * (SLOT_COLS / 4),
+                                            idesc, k + part, empty_a + 8 * slot);
+                }
+                if (!ok) break;
+                mma_commit(empty_x + 8 * stage);
+                if (++stage == M.xstages) { stage = 0; x_parity ^= 1u; }
+            }
+            if (ok) mma_commit(accum);
+            ++part_no;
+            pos += P.len;
+        }
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
-
-    uint32_t step_count = 0;                    // pipeline steps issued so far (all roles count alike)
-    uint32_t accum_parity = 0;
-    for (uint32_t bc = 0; bc < M.batch; bc += MB * M.nchunks) {
-        if (warp < DEC_WARPS) {
-            // ------------------------------ decode warps ------------------------------
-            // thread = (row, half): 32 columns of a 64-column step; two threads of a row are neighbours
-            const uint32_t row = tid >> 1, half = tid & 1, sw = row & 7;
-            const uint64_t r = r0 + row;
-            const bool live = r < M.m;
-            const uint32_t *src_b = M.bits32 + (uint64_t)plane * M.plane_words32;
-            const uint2 *lut_mine = lut256 + (lane & (LUT_COPIES - 1));
-            // shared addresses: this row inside stage 0, its four 16-byte chunks (swizzled), this lane's table copy
-            const uint32_t brow0 = smem_addr(b_stages) + (row >> 3) * 1024 + sw * 128;
-            uint32_t chunk_off[4];
-#pragma unroll
-            for (uint32_t j = 0; j < 4; ++j) chunk_off[j] = ((half * 4 + j) ^ sw) << 4;
-            const uint32_t lut_sa = smem_addr(lut_mine);
-            uint32_t stage = step_count % M.stages, use = step_count / M.stages;       // advanced step by step below
-            bool stop = false;
-            // bits of the current macro: aligned rows -> 4 words of this thread's 128 columns per vector
-            uint4 cur_m = make_uint4(0, 0, 0, 0), cur_b = make_uint4(0, 0, 0, 0);
-            auto fetch_macro = [&](uint32_t mc, uint4 &vm, uint4 &vb) {
-                vm = vb = make_uint4(0, 0, 0, 0);
-                const uint64_t c = (uint64_t)mc * MACRO + 128 * half;       // first column of this thread's 128
-                if (live && c < M.n) {
-                    const uint64_t w = (r * M.n + c) >> 5;                  // a multiple of 4
-                    if (w + 4 <= M.mask_words32) vm = ldg_ahead(reinterpret_cast<const uint4 *>(M.mask32 + w));
-                    else {
-                        vm.x = w < M.mask_words32 ? __ldg(M.mask32 + w) : 0u;
-                        vm.y = w + 1 < M.mask_words32 ? __ldg(M.mask32 + w + 1) : 0u;
-                        vm.z = w + 2 < M.mask_words32 ? __ldg(M.mask32 + w + 2) : 0u;
-                    }
-                    if (w + 4 <= M.plane_words32) vb = ldg_ahead(reinterpret_cast<const uint4 *>(src_b + w));
-                    else {
-                        vb.x = w < M.plane_words32 ? __ldg(src_b + w) : 0u;
-                        vb.y = w + 1 < M.plane_words32 ? __ldg(src_b + w + 1) : 0u;
-                        vb.z = w + 2 < M.plane_words32 ? __ldg(src_b + w + 2) : 0u;
-                    }
-                }
-            };
-            if (M.aligned && macro_begin < macro_end) fetch_macro(macro_begin, cur_m, cur_b);
-            for (uint32_t mc = macro_begin; mc < macro_end && !stop; ++mc) {
-                // take delivery of this macro's bits before the next macro's are requested (a warp's few
-                // scoreboards are shared between loads: a first use after the new request would wait for it)
-                cur_m.x = settle(cur_m.x); cur_m.y = settle(cur_m.y); cur_m.z = settle(cur_m.z); cur_m.w = settle(cur_m.w);
-                cur_b.x = settle(cur_b.x); cur_b.y = settle(cur_b.y); cur_b.z = settle(cur_b.z); cur_b.w = settle(cur_b.w);
-                uint4 nxt_m = make_uint4(0, 0, 0, 0), nxt_b = make_uint4(0, 0, 0, 0);
-                if (M.aligned && mc + 1 < macro_end) fetch_macro(mc + 1, nxt_m, nxt_b);
-                const uint32_t st_lo = mc * STEPS_PER_MACRO;
-#pragma unroll
-                for (uint32_t ks = 0; ks < STEPS_PER_MACRO; ++ks) {
-                    if (st_lo + ks >= step_end || stop) continue;           // the same in every thread
-                    // mask and sign word of this thread's 32 columns
-                    uint32_t mw, bw;
-                    if (M.aligned) {
-                        // words 2 ks and 2 ks + 1 of the macro: the lower four live in the half-0 thread,
-                        // the upper four in the half-1 thread; the neighbour hands over the one this thread lacks
-                        const uint32_t am[4] = {cur_m.x, cur_m.y, cur_m.z, cur_m.w};
-                        const uint32_t ab[4] = {cur_b.x, cur_b.y, cur_b.z, cur_b.w};
-                        const uint32_t m0 = am[(2 * ks) & 3u], m1 = am[(2 * ks + 1) & 3u];      // compile-time picks
-                        const uint32_t b0 = ab[(2 * ks) & 3u], b1 = ab[(2 * ks + 1) & 3u];
-                        const uint32_t gm = __shfl_xor_sync(0xffffffffu, half ? m0 : m1, 1);
-                        const uint32_t gb = __shfl_xor_sync(0xffffffffu, half ? b0 : b1, 1);
-                        const bool mine = half == (ks >> 1);                // the owner of words 2 ks, 2 ks + 1
-                        mw = mine ? (half ? m1 : m0) : gm;
-                        bw = mine ? (half ? b1 : b0) : gb;
-                    } else {
-                        const uint64_t c = (uint64_t)(st_lo + ks) * KC + 32 * half;
-                        mw = bw = 0;
-                        if (live && c < M.n) {
-                            mw = bits_at(M.mask32, M.mask_words32, r * M.n + c);
-                            bw = bits_at(src_b, M.plane_words32, r * M.n + c);
-                        }
-                    }
-                    // table indices (mask nibble << 4 | sign nibble) of the eight groups of four weights, one per
-                    // byte: byte j of `lo` for weights 8j .. 8j+3, byte j of `hi` for weights 8j+4 .. 8j+7
-                    const uint32_t lo = ((mw & 0x0f0f0f0fu) << 4) | (bw & 0x0f0f0f0fu);
-                    const uint32_t hi = (mw & 0xf0f0f0f0u) | ((bw >> 4) & 0x0f0f0f0fu);
-                    uint2 e[8];
-#pragma unroll
-                    for (uint32_t j = 0; j < 4; ++j) {
-                        const uint32_t a0 = lut_sa + ((lo >> (8 * j)) & 0xffu) * (LUT_COPIES * 8);
-                        const uint32_t a1 = lut_sa + ((hi >> (8 * j)) & 0xffu) * (LUT_COPIES * 8);
-                        asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(e[2 * j].x), "=r"(e[2 * j].y) : "r"(a0));
-                        asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(e[2 * j + 1].x), "=r"(e[2 * j + 1].y) : "r"(a1));
-                    }
-                    // one lane per warp watches the barrier that frees the stage; the warp follows it
-                    if (use > 0) {
-                        uint32_t freed = 1;
-                        if (lane == 0) freed = mbar_wait(empty + stage, (use - 1) & 1u, abort_flag, M.status, M.wait_limit) ? 1u : 0u;
-                        if (!__shfl_sync(0xffffffffu, freed, 0)) { stop = true; continue; }
-                    }
-                    const uint32_t brow = brow0 + stage * B_STAGE_BYTES;
-#pragma unroll
-                    for (uint32_t j = 0; j < 4; ++j)                        // 8 weights = one 16-byte chunk
-                        asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};"
-                                     :: "r"(brow + chunk_off[j]), "r"(e[2 * j].x), "r"(e[2 * j].y), "r"(e[2 * j + 1].x), "r"(e[2 * j + 1].y) : "memory");
-                    fence_async_smem();                 // generic-proxy writes -> visible to the tensor core
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(full_b + stage);     // the warp's 16 rows are in place
-                    if (++stage == M.stages) { stage = 0; ++use; }
-                }
-                cur_m = nxt_m;
-                cur_b = nxt_b;
-                // a warp that gave up makes every decode thread leave at the same macro
-                if (decode_barrier_any(stop || *abort_flag)) stop = true;
-            }
-        } else if (warp == DEC_WARPS) {
-            // ------------------------------ TMA producer ------------------------------
-            if (lane == 0 && !M.skip_loads) {
-                uint32_t it = step_count;
-                for (uint32_t st = step_begin; st < step_end; ++st, ++it) {
-                    const uint32_t stage = it % M.stages, use = it / M.stages;
-                    if (use > 0 && !mbar_wait(empty + stage, (use - 1) & 1u, abort_flag, M.status, M.wait_limit)) break;
-                    uint8_t *a_stage = a_stages + (size_t)stage * a_stage_bytes;
-                    mbar_expect_tx(full_a + stage, a_stage_bytes);
-                    for (uint32_t c = 0; c < M.nchunks; ++c)
-                        tma_load_2d(a_stage + c * A_TILE_BYTES, &xmap, full_a + stage, (int32_t)(st * KC), (int32_t)(bc + c * MB));
-                }
-            }
-        } else {
-            // ------------------------------ MMA issuer ------------------------------
-            if (lane == 0) {
-                uint32_t it = step_count;
-                const uint32_t idesc = instr_desc_bf16(NROWS);
-                // descriptors differ only in the start-address field (units of 16 bytes): keep the
-                // constant part and add offsets, so that issuing an MMA costs a few instructions
-                const uint64_t a_desc0 = smem_desc_sw128(smem_addr(a_stages));
-                const uint64_t b_desc0 = smem_desc_sw128(smem_addr(b_stages));
-                bool ok = true;
-                uint32_t acc = 0;                       // 0 for the very first MMA of every accumulator
-                for (uint32_t st = step_begin; st < step_end && ok; ++st, ++it) {
-                    const uint32_t stage = it % M.stages, use = it / M.stages;
-                    ok = mbar_wait(full_b + stage, use & 1u, abort_flag, M.status, M.wait_limit) &&
-                         mbar_wait(full_a + stage, use & 1u, abort_flag, M.status, M.wait_limit);
-                    if (!ok) break;
-                    tc_fence_after();
-                    const uint64_t a_desc = a_desc0 + (uint64_t)(stage * (a_stage_bytes >> 4));
-                    const uint64_t b_desc = b_desc0 + (uint64_t)(stage * (B_STAGE_BYTES >> 4));
-                    if (M.nchunks == 2) {
-#pragma unroll
-                        for (uint32_t k16 = 0; k16 < KC / 16; ++k16)
-#pragma unroll
-                            for (uint32_t c = 0; c < 2; ++c)
-                                mma_bf16(tmem_base + c * NROWS, a_desc + (uint64_t)(c * (A_TILE_BYTES >> 4)) + 2 * k16,
-                                         b_desc + 2 * k16, idesc, (acc | k16) ? 1u : 0u);
-                    } else {
-#pragma unroll
-                        for (uint32_t k16 = 0; k16 < KC / 16; ++k16)
-                            mma_bf16(tmem_base + (k16 & 1u) * NROWS, a_desc + 2 * k16, b_desc + 2 * k16, idesc,
-                                     (acc | (k16 >> 1)) ? 1u : 0u);
-                    }
-                    acc = 1;
-                    mma_commit(empty + stage);          // frees the stage when these MMAs are done
-                }
-                if (ok && nsteps) mma_commit(accum);
-            }
-        }
-        step_count += nsteps;
-
-        // ------------------------------ epilogue ------------------------------
-        if (warp < DEC_WARPS && nsteps) {
-            const bool ready = mbar_wait(accum, accum_parity, abort_flag, M.status, M.wait_limit);
-            if (__all_sync(0xffffffffu, ready)) {                  // tcgen05.ld needs the whole warp
-                tc_fence_after();
-                const uint32_t quad = warp & 3, part = warp >> 2;       // TMEM lane quarter (batch rows), column quarter
-                for (uint32_t c = 0; c < M.nchunks; ++c) {
-                    const uint32_t b = bc + c * MB + quad * 32 + lane;  // batch row of this thread
-                    if (bc + c * MB + quad * 32 >= M.batch) continue;   // the same in the whole warp
-#pragma unroll 1
-                    for (uint32_t q = 0; q < 2; ++q) {
-                        const uint32_t col = part * 64 + q * 32;        // first of 32 weight rows
-                        uint32_t v[32];
-                        tmem_ld32(tmem_base + ((quad * 32) << 16) + c * NROWS + col, v);
-                        if (M.nchunks == 1) {                           // the second accumulator of the only chunk
-                            uint32_t u[32];
-                            tmem_ld32(tmem_base + ((quad * 32) << 16) + NROWS + col, u);
-#pragma unroll
-                            for (uint32_t e = 0; e < 32; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) + __uint_as_float(u[e]));
-                        }
-                        if (b < M.batch) {
-                            float *dst = M.y + (int64_t)b * M.ldy + (int64_t)(r0 + col);
-#pragma unroll
-                            for (uint32_t e = 0; e < 32; e += 4) {
-                                const float o0 = alpha_s[col + e] * __uint_as_float(v[e]);
-                                const float o1 = alpha_s[col + e + 1] * __uint_as_float(v[e + 1]);
-                                const float o2 = alpha_s[col + e + 2] * __uint_as_float(v[e + 2]);
-                                const float o3 = alpha_s[col + e + 3] * __uint_as_float(v[e + 3]);
-                                if (M.vec_y && r0 + col + e + 4 <= M.m) {
-                                    red_add_v4(dst + e, o0, o1, o2, o3);
-                                } else {
-                                    if (r0 + col + e < M.m) atomicAdd(dst + e, o0);
-                                    if (r0 + col + e + 1 < M.m) atomicAdd(dst + e + 1, o1);
-                                    if (r0 + col + e + 2 < M.m) atomicAdd(dst + e + 2, o2);
-                                    if (r0 + col + e + 3 < M.m) atomicAdd(dst + e + 3, o3);
-                                }
-                            }
-                        }
-                    }
-                }
-            }
-        }
-        if (nsteps) accum_parity ^= 1;
-        tc_fence_before();
-        __syncthreads();                       // accumulators are read before the next pass overwrites them
-        tc_fence_after();
-    }
-    if (warp == DEC_WARPS + 1) tmem_dealloc(tmem_base, tmem_cols);
+    if (warp == 4 * groups + 1) tmem_dealloc(tmem_base, 512);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -520,7 +558,6 @@ int mma_dispatch(const sqnn_desc *desc, const DecodeArgs &A0, const uint64_t *d_
     M.bits32 = (const uint32_t *)d_workspace;
     M.plane_words32 = A0.words64 * 2;
     M.mask32 = (const uint32_t *)d_mask;
-    M.mask_words32 = A0.words64 * 2;
     M.alpha = d_alpha;
     M.y = d_y;
     M.ldy = ldy;
@@ -528,54 +565,53 @@ int mma_dispatch(const sqnn_desc *desc, const DecodeArgs &A0, const uint64_t *d_
     M.n = desc->n;
     M.n_q = desc->n_q;
     M.batch = batch;
-    M.nchunks = batch > MB ? 2u : 1u;
     M.status = A0.status;
-    // rows of the packed vectors start on 16-byte boundaries when n is a multiple of 128 (the workspace is
-    // 256-byte aligned and every plane in it starts on a multiple of 8 bytes: check that too)
-    M.aligned = (desc->n % 128 == 0 && ((uintptr_t)d_mask & 15) == 0 && (M.plane_words32 % 4 == 0 || desc->n_q == 1)) ? 1u : 0u;
-    M.vec_y = (((uintptr_t)d_y & 15) == 0 && ldy % 4 == 0) ? 1u : 0u;
     const uint32_t dbg = g_debug_flags.load();
     M.skip_loads = (dbg & 1u) ? 1u : 0u;
     M.wait_limit = g_debug_wait_cycles.load() ? g_debug_wait_cycles.load() : WAIT_LIMIT_CYCLES;
 
-    const size_t budget = 225 * 1024;        // + 1 KB of static shared memory stays within the 227 KB a block may have
-    const size_t fixed = 256 * 8 * LUT_COPIES + NROWS * 4 + (3 * MAX_STAGES + 1) * 8 + 16 + 1024;
-    const size_t per_stage = B_STAGE_BYTES + (size_t)M.nchunks * A_TILE_BYTES;
-    M.stages = MAX_STAGES;
-    while (M.stages > 1 && fixed + (size_t)M.stages * per_stage > budget) --M.stages;
-    const size_t smem = fixed + (size_t)M.stages * per_stage;
-    if (smem > budget) return SQNN_E_UNSUPPORTED;
-
-    const uint64_t row_tiles = (desc->m + NROWS - 1) / NROWS;
-    const uint32_t total_macros = (uint32_t)((desc->n + MACRO - 1) / MACRO);
-    const uint64_t items = row_tiles * desc->n_q;
-    uint32_t splits = items >= (uint64_t)sm_count() ? 1u : (uint32_t)((uint64_t)sm_count() / items);
-    if (splits < 1) splits = 1;
-    if (splits > total_macros) splits = total_macros;
-    M.macros_per_split = (total_macros + splits - 1) / splits;
-    M.splits = (total_macros + M.macros_per_split - 1) / M.macros_per_split;
-    if (items * M.splits > 0x7fffffffull) return SQNN_E_UNSUPPORTED;
+    // Units of a tile.  All planes of 128 rows share the activation tile (up to four; more planes are taken in
+    // equal groups); one plane alone takes 256 rows, so that an activation tile is used twice there as well.
+    M.planes = M.n_q <= 4 ? M.n_q : M.n_q <= 6 ? 3u : 4u;
+    M.plane_groups = (M.n_q + M.planes - 1) / M.planes;
+    M.mt = M.planes == 1 && M.m > MROWS ? 2u : 1u;
+    const uint32_t units = M.mt * M.planes;
+    // Batch rows per tile: what the accumulators leave room for, in equal chunks.
+    const uint32_t n_max = units == 1 ? 256u : MAX_ACC_COLS / units / 16 * 16;
+    M.chunks = (batch + n_max - 1) / n_max;
+    M.N = ((batch + M.chunks - 1) / M.chunks + 15) / 16 * 16;
+    M.acc_cols = (units * M.N + 31) / 32 * 32;
+    // A slots of a whole step (32 TMEM columns) if every unit gets at least two, else of half a step
+    const uint32_t per_unit = (512 - M.acc_cols) / units, slot_cols = per_unit >= 64 ? 32u : 16u;
+    M.slots = per_unit / slot_cols >= 8 ? 8u : per_unit / slot_cols >= 4 ? 4u : 2u;
+    // Groups of four warps: four, or three for three planes, so that every group always serves the same unit.
+    M.phases = units == 1 ? 4u : units == 2 ? 2u : 1u;
+    const uint32_t threads = units * M.phases * 128 + 32 + units * 32;
+    const size_t x_bytes = (size_t)M.N * KC * 2;
+    M.xstages = (uint32_t)(XSTAGE_BUDGET / x_bytes < MAX_XSTAGES ? XSTAGE_BUDGET / x_bytes : MAX_XSTAGES);
+    const size_t smem = M.xstages * x_bytes + 1024;
+    M.macros = (uint32_t)((desc->n + MACRO - 1) / MACRO);
+    M.total = (M.m + M.mt * MROWS - 1) / (M.mt * MROWS) * M.plane_groups * M.chunks * M.macros;
+    const uint32_t grid = M.total < (uint64_t)sm_count() ? (uint32_t)M.total : (uint32_t)sm_count();
+    // rows of mask and planes start on 16-byte boundaries
+    const bool aligned = desc->n % 128 == 0 && ((uintptr_t)d_mask & 15) == 0 && (M.plane_words32 % 4 == 0 || M.n_q == 1);
 
     CUtensorMap xmap;
     const cuuint64_t gdim[2] = {(cuuint64_t)desc->n, (cuuint64_t)batch};
     const cuuint64_t gstride[1] = {(cuuint64_t)ldx * 2};
-    const cuuint32_t box[2] = {KC, MB};
+    const cuuint32_t box[2] = {KC, M.N};
     const cuuint32_t estride[2] = {1, 1};
     if (encode(&xmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(d_x), gdim, gstride, box, estride,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return SQNN_E_CUDA;
 
-    cudaError_t e = (ldy == (int64_t)desc->m)
-        ? cudaMemsetAsync(d_y, 0, (size_t)batch * desc->m * sizeof(float), st)
-        : cudaMemset2DAsync(d_y, (size_t)ldy * sizeof(float), 0, (size_t)desc->m * sizeof(float), batch, st);
-    if (e != cudaSuccess) return SQNN_E_CUDA;
-    if (ensure_dynamic_smem(reinterpret_cast<const void *>(k_decode_mma), smem) != SQNN_OK) return SQNN_E_CUDA;
-    // stage 1: the decode kernel writes the planes as packed bits into the workspace
-    const int rc = decode_bits_dispatch(A0, d_workspace, st);
+    // stage 1: the decode kernel writes the planes as packed bits into the workspace and clears Y
+    const int rc = decode_bits_dispatch(A0, d_workspace, ClearArgs{d_y, desc->m, ldy, batch}, st);
     if (rc != SQNN_OK) return rc;
-    k_decode_mma<<<(uint32_t)(items * M.splits), THREADS, smem, st>>>(xmap, M);
-    return cudaGetLastError() == cudaSuccess ? SQNN_OK : SQNN_E_CUDA;
+    auto k = slot_cols == 32 ? (aligned ? k_decode_mma<true, 32> : k_decode_mma<false, 32>)
+                             : (aligned ? k_decode_mma<true, 16> : k_decode_mma<false, 16>);
+    return launch_kernel(k, grid, threads, smem, st, xmap, M);
 }
 
 }  // namespace sqnn

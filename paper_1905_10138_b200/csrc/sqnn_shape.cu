@@ -10,9 +10,10 @@ namespace sqnn {
 
 template <>
 int decode_shape<SQNN_NO, SQNN_NI>(const DecodeArgs &A, sqnn_out_mode mode, const uint64_t *d_mask,
-                                   const float *d_alpha, uint64_t n, void *d_out, cudaStream_t st)
+                                   const float *d_alpha, uint64_t n, void *d_out, const ClearArgs &clear,
+                                   cudaStream_t st)
 {
-    return launch_decode<SQNN_NO, SQNN_NI>(A, mode, d_mask, d_alpha, n, d_out, st);
+    return launch_decode<SQNN_NO, SQNN_NI>(A, mode, d_mask, d_alpha, n, d_out, clear, st);
 }
 
 template <>
