@@ -46,11 +46,10 @@ namespace sqnn {
 namespace {
 
 constexpr uint32_t MROWS = 128;           // weight rows per unit = MMA M = TMEM lanes
-constexpr uint32_t KC = 64;               // columns per step (one A slot, one X stage)
-constexpr uint32_t STEPS = 4;             // steps per macro
-constexpr uint32_t MACRO = KC * STEPS;    // columns whose bits an expander thread takes at a time
+constexpr uint32_t KX = 128;              // columns per X stage (two TMA boxes of 64)
+constexpr uint32_t MACRO = 2 * KX;        // columns whose bits an expander thread takes at a time
 constexpr uint32_t MAX_SLOTS = 8;         // A slots per unit
-constexpr uint32_t MAX_XSTAGES = 12;
+constexpr uint32_t MAX_XSTAGES = 8;
 constexpr uint32_t MAX_UNITS = 4;
 constexpr uint32_t MAX_ACC_COLS = 384;    // TMEM columns of all accumulators; the other 128 and more are A slots
 constexpr uint32_t XSTAGE_BUDGET = 192 * 1024;
@@ -75,9 +74,8 @@ struct MmaArgs {
     uint32_t mt;                  // 128-row groups per tile
     uint32_t planes;              // planes per tile
     uint32_t plane_groups;
-    uint32_t phases;              // column ranges the expander groups of one unit take side by side
     uint32_t macros;              // 256-column macros per row
-    uint64_t total;               // tiles x macros
+    uint32_t total;               // tiles x macros
     uint32_t slots, xstages;      // A slots per unit (a power of two), X stages
     uint32_t acc_cols;            // first TMEM column of the A slots
     uint32_t skip_loads;          // test only: the TMA role issues no loads
@@ -109,12 +107,12 @@ SQNN_DEV bool mbar_try(uint32_t bar, uint32_t parity)
     return ok != 0;
 }
 // Bounded wait.  Returns false if the wait was abandoned (limit reached or another role gave up).
-SQNN_DEV bool mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag, uint32_t *status, uint64_t limit)
+__device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag, uint32_t *status, uint64_t limit)
 {
-    if (mbar_try(bar, parity)) return true;
     const long long t0 = clock64();
     while (true) {
-        if (mbar_try(bar, parity)) return true;
+        for (uint32_t k = 0; k < 16; ++k)
+            if (mbar_try(bar, parity)) return true;
         if (*abort_flag) return false;
         if ((uint64_t)(clock64() - t0) > limit) {
             *abort_flag = 1u;
@@ -123,12 +121,19 @@ SQNN_DEV bool mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t *abort_
         }
     }
 }
+SQNN_DEV bool mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag, uint32_t *status, uint64_t limit)
+{
+    for (uint32_t k = 0; k < 4; ++k)
+        if (mbar_try(bar, parity)) return true;
+    return mbar_wait_slow(bar, parity, abort_flag, status, limit);
+}
 // The same for a converged warp: true in all lanes or in none.  (One instruction of a converged warp gives all
 // its lanes the same answer, so only the slow way needs a vote.)
 SQNN_DEV bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag, uint32_t *status, uint64_t limit)
 {
-    if (mbar_try(bar, parity)) return true;
-    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status, limit));
+    for (uint32_t k = 0; k < 4; ++k)
+        if (mbar_try(bar, parity)) return true;
+    return __all_sync(0xffffffffu, mbar_wait_slow(bar, parity, abort_flag, status, limit));
 }
 // The same without a report, for copies that must land before the kernel may leave.
 SQNN_DEV void mbar_drain(uint32_t bar, uint32_t parity, uint64_t limit)
@@ -153,35 +158,41 @@ SQNN_DEV void tmem_dealloc(uint32_t taddr, uint32_t cols)
 }
 SQNN_DEV void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
 SQNN_DEV void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
-// The tcgen05.mma of one A slot (SLICES of K = 16) and the commit that frees it, by one elected lane of a
-// converged warp: A from tensor memory (128 lanes x 16 bf16 each, two per column), B from shared memory.
+// The tcgen05.mma of one A slot (4 or 8 slices of K = 16) and the commit that frees it, by one elected lane of
+// a converged warp: A from tensor memory (128 lanes x 16 bf16 each, two per column), B from shared memory.
 // Issued from converged code the operands are uniform registers; issued under a lane test they were moved
-// there one by one and a step took over 800 cycles instead of the 256 the tensor cores need at N = 128.
+// there one by one and a step of 64 columns took over 800 cycles instead of the 256 the tensor cores need at
+// N = 128.  `bdesc_hi`: descriptor step from the first four slices (one box of 64 columns) to the next four.
+#define SQNN_MMA(D, A, B, P) " @e tcgen05.mma.cta_group::1.kind::f16 [" D "], [" A "], " B ", %3, " P ";\n"
 template <uint32_t SLICES>
-SQNN_DEV void mma_slot(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate, uint32_t free_a)
+SQNN_DEV void mma_slot(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate, uint32_t free_a,
+                       uint64_t bdesc_hi)
 {
-    static_assert(SLICES == 2 || SLICES == 4, "slots of 32 or 64 columns");
-    if constexpr (SLICES == 4) {
+    static_assert(SLICES == 4 || SLICES == 8, "slots of 64 or 128 columns");
+    if constexpr (SLICES == 8) {
+        asm volatile("{\n .reg .pred e, p, t;\n .reg .b32 a1, a2, a3, a4, a5, a6, a7;\n .reg .b64 b1, b2, b3, b4, b5, b6, b7;\n"
+                     " elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %4, 0;\n setp.eq.b32 t, %4, %4;\n"
+                     " add.u32 a1, %1, 8;\n add.u32 a2, %1, 16;\n add.u32 a3, %1, 24;\n add.u32 a4, %1, 32;\n"
+                     " add.u32 a5, %1, 40;\n add.u32 a6, %1, 48;\n add.u32 a7, %1, 56;\n"
+                     " add.u64 b1, %2, 2;\n add.u64 b2, %2, 4;\n add.u64 b3, %2, 6;\n add.u64 b4, %2, %6;\n"
+                     " add.u64 b5, b4, 2;\n add.u64 b6, b4, 4;\n add.u64 b7, b4, 6;\n"
+                     SQNN_MMA("%0", "%1", "%2", "p") SQNN_MMA("%0", "a1", "b1", "t") SQNN_MMA("%0", "a2", "b2", "t")
+                     SQNN_MMA("%0", "a3", "b3", "t") SQNN_MMA("%0", "a4", "b4", "t") SQNN_MMA("%0", "a5", "b5", "t")
+                     SQNN_MMA("%0", "a6", "b6", "t") SQNN_MMA("%0", "a7", "b7", "t")
+                     " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n}\n"
+                     :: "r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(free_a), "l"(bdesc_hi) : "memory");
+    } else {
         asm volatile("{\n .reg .pred e, p, t;\n .reg .b32 a1, a2, a3;\n .reg .b64 b1, b2, b3;\n"
                      " elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %4, 0;\n setp.eq.b32 t, %4, %4;\n"
                      " add.u32 a1, %1, 8;\n add.u32 a2, %1, 16;\n add.u32 a3, %1, 24;\n"
                      " add.u64 b1, %2, 2;\n add.u64 b2, %2, 4;\n add.u64 b3, %2, 6;\n"
-                     " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n"
-                     " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a1], b1, %3, t;\n"
-                     " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a2], b2, %3, t;\n"
-                     " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a3], b3, %3, t;\n"
-                     " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n}\n"
-                     :: "r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(free_a) : "memory");
-    } else {
-        asm volatile("{\n .reg .pred e, p, t;\n .reg .b32 a1;\n .reg .b64 b1;\n"
-                     " elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %4, 0;\n setp.eq.b32 t, %4, %4;\n"
-                     " add.u32 a1, %1, 8;\n add.u64 b1, %2, 2;\n"
-                     " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n"
-                     " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a1], b1, %3, t;\n"
+                     SQNN_MMA("%0", "%1", "%2", "p") SQNN_MMA("%0", "a1", "b1", "t") SQNN_MMA("%0", "a2", "b2", "t")
+                     SQNN_MMA("%0", "a3", "b3", "t")
                      " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n}\n"
                      :: "r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(free_a) : "memory");
     }
 }
+#undef SQNN_MMA
 // Makes the mbarrier track completion of all MMAs the elected lane issued so far (converged warp).
 SQNN_DEV void mma_commit(uint32_t bar)
 {
@@ -244,30 +255,44 @@ SQNN_DEV void expand32(uint32_t m, uint32_t b, uint32_t *v)
     }
 }
 
-// Bits of 256 columns of one row as eight words.  ALIGNED: rows start on 16-byte boundaries; otherwise the
-// three 16-byte vectors that cover them are fetched and shifted into place when the bits are used.
+// A row's packed bits as a stream of 256-column macros, eight words each.  ALIGNED: rows start on 16-byte
+// boundaries; otherwise the three 16-byte vectors that cover a macro are fetched and shifted into place when
+// the bits are used.
 template <bool ALIGNED>
-struct MacroBits {
+struct BitStream {
     static constexpr uint32_t RAW = ALIGNED ? 8 : 12;
     uint32_t t[RAW];
-    // first, last: valid words of the vector counted from `base` (16-byte aligned); pos: bit position from `base`
-    SQNN_DEV void fetch(const uint32_t *__restrict__ base, uint64_t first, uint64_t last, uint64_t pos)
+    const uint32_t *at, *first, *last;   // next macro; the vector's first word and the end of its last one
+    uint32_t shift;
+    bool inside;                         // all macros of this stream lie inside the vector with their slack
+    // vec: 8-byte aligned, `words` long; from bit `pos` of it, `count` macros
+    SQNN_DEV void open(const uint32_t *__restrict__ vec, uint64_t words, uint64_t pos, uint32_t count)
     {
-        const uint64_t w = (pos >> 7) << 2;
-        if (w >= first && w + RAW <= last) {
+        const uint32_t lead = (uint32_t)(reinterpret_cast<uintptr_t>(vec) >> 2) & 3u;     // words past a 16-byte boundary
+        const uint64_t p = pos + 32 * lead;
+        first = vec;
+        last = vec + words;
+        at = vec - lead + ((p >> 7) << 2);
+        shift = (uint32_t)p & 127u;
+        inside = at >= first && at + (uint64_t)count * 8 + (RAW - 8) <= last;
+    }
+    SQNN_DEV void fetch()
+    {
+        if (inside) {
 #pragma unroll
             for (uint32_t k = 0; k < RAW; k += 4)
                 asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];"
-                             : "=r"(t[k]), "=r"(t[k + 1]), "=r"(t[k + 2]), "=r"(t[k + 3]) : "l"(base + w + k));
+                             : "=r"(t[k]), "=r"(t[k + 1]), "=r"(t[k + 2]), "=r"(t[k + 3]) : "l"(at + k));
         } else {
 #pragma unroll
             for (uint32_t k = 0; k < RAW; ++k) {
                 t[k] = 0u;
-                if (w + k >= first && w + k < last) t[k] = base[w + k];
+                if (at + k >= first && at + k < last) t[k] = at[k];
             }
         }
+        at += 8;
     }
-    SQNN_DEV void take(uint32_t shift, uint32_t (&out)[8])
+    SQNN_DEV void take(uint32_t (&out)[8])
     {
         uint32_t q[RAW];
 #pragma unroll
@@ -288,59 +313,67 @@ struct MacroBits {
 };
 
 // One part of the work of a CTA: macros [m0, m0 + len) of a tile, and how the phases share them.
+template <uint32_t PHASES>
 struct Part {
     uint32_t chunk, pg, group;    // batch chunk, plane group, row group
     uint32_t m0, len, base, rem;  // phase p takes base + (p < rem) macros from first(p) on
-    SQNN_DEV Part(const MmaArgs &M, uint64_t pos, uint64_t end)
+    SQNN_DEV Part(const MmaArgs &M, uint32_t pos, uint32_t end)
     {
-        const uint64_t tile = pos / M.macros;
-        m0 = (uint32_t)(pos - tile * M.macros);
-        const uint64_t left = end - pos;
-        len = M.macros - m0 < left ? M.macros - m0 : (uint32_t)left;
-        chunk = (uint32_t)(tile % M.chunks);
-        const uint64_t rest = tile / M.chunks;
-        pg = (uint32_t)(rest % M.plane_groups);
-        group = (uint32_t)(rest / M.plane_groups);
-        base = len / M.phases;
-        rem = len - base * M.phases;
+        const uint32_t tile = pos / M.macros;
+        m0 = pos - tile * M.macros;
+        len = min(M.macros - m0, end - pos);
+        const uint32_t rest = tile / M.chunks;
+        chunk = tile - rest * M.chunks;
+        group = rest / M.plane_groups;
+        pg = rest - group * M.plane_groups;
+        base = len / PHASES;
+        rem = len - base * PHASES;
     }
-    SQNN_DEV uint32_t first(uint32_t p) const { return m0 + p * base + (p < rem ? p : rem); }
+    SQNN_DEV uint32_t first(uint32_t p) const { return m0 + p * base + min(p, rem); }
     SQNN_DEV uint32_t count(uint32_t p) const { return base + (p < rem ? 1u : 0u); }
     SQNN_DEV uint32_t rounds() const { return base + (rem ? 1u : 0u); }
-    SQNN_DEV uint32_t active(uint32_t i, uint32_t phases) const { return i < base ? phases : rem; }
+    SQNN_DEV uint32_t active(uint32_t i) const { return i < base ? PHASES : rem; }
 };
 
-// Order of the X stages inside a part, the same for all roles: round i (one macro of every active phase), step h
-// of the macro, phase p.  Every unit has its own ring of A slots, filled in that order; a slot holds SLOT_COLS
-// TMEM columns (two bf16 each): the 64 columns of a step, or half of them where the accumulators leave less.
-template <bool ALIGNED, uint32_t SLOT_COLS>
-__global__ void __launch_bounds__(4 * MAX_UNITS * 32 + 32 + MAX_UNITS * 32, 1)
+// Expander groups (four warps each) of the unit counts: every unit has as many (its phases), four in all where
+// that divides.
+SQNN_HD constexpr uint32_t phases_of(uint32_t units) { return units == 1 ? 4 : units == 2 ? 2 : 1; }
+SQNN_HD constexpr uint32_t threads_of(uint32_t units) { return units * phases_of(units) * 128 + 32 + units * 32; }
+
+// Order of the X stages inside a part, the same for all roles: round i (one macro of every active phase), half
+// c of the macro, phase p.  Every unit has its own ring of A slots; within (i, c) the slots of the phases
+// alternate.  A slot holds SLOT_COLS TMEM columns (two bf16 each): the 128 columns of an X stage or half of them.
+template <uint32_t UNITS, bool ALIGNED, uint32_t SLOT_COLS>
+__global__ void __launch_bounds__(threads_of(UNITS), 1)
 k_decode_mma(const __grid_constant__ CUtensorMap xmap, const MmaArgs M)
 {
     extern __shared__ __align__(16) uint8_t smem_raw[];
     __shared__ uint64_t bars[2 * MAX_UNITS * MAX_SLOTS + 2 * MAX_XSTAGES + 2];
     __shared__ uint32_t tmem_slot, abort_word;
-    const uint32_t x_sa = (smem_addr(smem_raw) + 1023u) & ~1023u;
     volatile uint32_t *abort_flag = &abort_word;
     // barriers by shared address: barrier i of a kind is 8 i bytes further on
     const uint32_t full_a = smem_addr(bars), empty_a = full_a + 8 * MAX_UNITS * MAX_SLOTS, full_x = empty_a + 8 * MAX_UNITS * MAX_SLOTS;
     const uint32_t empty_x = full_x + 8 * MAX_XSTAGES, accum = empty_x + 8 * MAX_XSTAGES, acc_free = accum + 8;
+    const uint32_t x_sa = (smem_addr(smem_raw) + 1023u) & ~1023u;
     const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint32_t units = M.mt * M.planes, groups = units * M.phases;       // expander groups of four warps
-    const uint32_t x_bytes = M.N * KC * 2;
-    const uint64_t begin = M.total * blockIdx.x / gridDim.x, end = M.total * (blockIdx.x + 1) / gridDim.x;
-    constexpr uint32_t PER_STEP = KC / 2 / SLOT_COLS;                        // slots per step
+    constexpr uint32_t units = UNITS, PHASES = phases_of(UNITS), groups = units * PHASES;
+    const uint32_t box_bytes = M.N * 128, x_bytes = 2 * box_bytes;
+    const uint32_t begin = (uint32_t)((uint64_t)M.total * blockIdx.x / gridDim.x);
+    const uint32_t end = (uint32_t)((uint64_t)M.total * (blockIdx.x + 1) / gridDim.x);
+    constexpr uint32_t PER_X = KX / 2 / SLOT_COLS;                           // slots per X stage and unit
     const uint32_t slot_mask = M.slots - 1, slot_shift = 31 - __clz((int)M.slots);
 
-    if (tid == 0) {
-        for (uint32_t s = 0; s < M.slots * units; ++s) { mbar_init(full_a + 8 * s, 4); mbar_init(empty_a + 8 * s, 1); }
-        for (uint32_t s = 0; s < M.xstages; ++s) { mbar_init(full_x + 8 * s, 1); mbar_init(empty_x + 8 * s, units); }
-        mbar_init(accum, units);
-        mbar_init(acc_free, 4 * groups);
-        abort_word = 0;
+    if (warp == 4 * groups + 1) tmem_alloc(&tmem_slot, 512);
+    if (warp == 4 * groups) {
+        for (uint32_t s = lane; s < M.slots * units; s += 32) { mbar_init(full_a + 8 * s, 4); mbar_init(empty_a + 8 * s, 1); }
+        if (lane < M.xstages) { mbar_init(full_x + 8 * lane, 1); mbar_init(empty_x + 8 * lane, units); }
+        if (lane == 31) {
+            mbar_init(accum, units);
+            mbar_init(acc_free, 4 * groups);
+            abort_word = 0;
+        }
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
-    if (warp == 4 * groups + 1) tmem_alloc(&tmem_slot, 512);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -350,81 +383,74 @@ k_decode_mma(const __grid_constant__ CUtensorMap xmap, const MmaArgs M)
     if (warp < 4 * groups) {
         // ------------------------------ expander groups ------------------------------
         const uint32_t g = warp >> 2, quad = warp & 3;
-        const uint32_t u = g % units, p = g / units;
+        const uint32_t p = g / units, u = g - p * units, mt_u = u / M.planes, plane_u = u - mt_u * M.planes;
         const uint32_t lane_sel = (quad * 32) << 16;
-        const uint32_t *mask_base = reinterpret_cast<const uint32_t *>(reinterpret_cast<uintptr_t>(M.mask32) & ~(uintptr_t)15);
-        const uint64_t mask_first = (uint64_t)(M.mask32 - mask_base), mask_last = mask_first + M.plane_words32;
         uint32_t seq0 = 0, part_no = 0;
-        wait_prior_grid();                                   // workspace and cleared Y are in place
-        for (uint64_t pos = begin; pos < end;) {
-            const Part P(M, pos, end);
-            const uint64_t row_in = (uint64_t)P.group * M.mt * MROWS + (u / M.planes) * MROWS + quad * 32 + lane;
+        for (uint32_t pos = begin; pos < end;) {
+            const Part<PHASES> P(M, pos, end);
+            const uint32_t row_in = (P.group * M.mt + mt_u) * MROWS + quad * 32 + lane;
             const uint64_t row = row_in < M.m ? row_in : M.m - 1;           // rows past the end repeat the last one
-            uint32_t plane = P.pg * M.planes + u % M.planes;
+            uint32_t plane = P.pg * M.planes + plane_u;
             if (plane >= M.n_q) plane = M.n_q - 1;                          // weighted with zero in the epilogue
-            const uint64_t plane_at = (uint64_t)plane * M.plane_words32;    // the workspace is 256-byte aligned
             const uint64_t c0 = row * M.n + (uint64_t)P.first(p) * MACRO;
-            uint64_t pos_m = mask_first * 32 + c0, pos_b = plane_at * 32 + c0;
-            const uint32_t shift_m = (uint32_t)pos_m & 127u, shift_b = (uint32_t)pos_b & 127u;
             const uint32_t count = P.count(p);
-            MacroBits<ALIGNED> fm, fb;
-            if (count) {
-                fm.fetch(mask_base, mask_first, mask_last, pos_m);
-                fb.fetch(M.bits32, plane_at, plane_at + M.plane_words32, pos_b);
-            }
+            BitStream<ALIGNED> sm, sb;
+            sm.open(M.mask32, M.plane_words32, c0, count);
+            sb.open(M.bits32 + plane * M.plane_words32, M.plane_words32, c0, count);
+            if (count) sm.fetch();
+            if (part_no == 0) wait_prior_grid();             // decoded planes and cleared Y are in place
+            if (count) sb.fetch();
             uint32_t seq = seq0;
-            bool stop = false;
-            for (uint32_t i = 0; i < count && !stop; ++i) {
+            for (uint32_t i = 0; i < count; ++i) {
                 uint32_t mw[8], bw[8];
-                fm.take(shift_m, mw);
-                fb.take(shift_b, bw);
-                if (i + 1 < count) {
-                    pos_m += MACRO;
-                    pos_b += MACRO;
-                    fm.fetch(mask_base, mask_first, mask_last, pos_m);
-                    fb.fetch(M.bits32, plane_at, plane_at + M.plane_words32, pos_b);
-                }
-                const uint32_t act = P.active(i, M.phases);
+                sm.take(mw);
+                sb.take(bw);
+                if (i + 1 < count) { sm.fetch(); sb.fetch(); }
+                const uint32_t act = P.active(i);
+                constexpr uint32_t WORDS = SLOT_COLS / 16;                  // 2 or 4: 32 columns each
 #pragma unroll
-                for (uint32_t h = 0; h < STEPS; ++h) {
-                    if (stop) continue;
+                for (uint32_t k = 0; k < 2 * PER_X; ++k) {                  // slots of the macro
+                    const uint32_t s = seq + k * act + p, use = s >> slot_shift, slot = u * M.slots + (s & slot_mask);
+                    const uint32_t at = tmem_base + lane_sel + M.acc_cols + slot * SLOT_COLS;
                     uint32_t v[32];
-                    expand32(mw[2 * h], bw[2 * h], v);
-                    expand32(mw[2 * h + 1], bw[2 * h + 1], v + 16);
-#pragma unroll
-                    for (uint32_t part = 0; part < PER_STEP; ++part) {
-                        const uint32_t s = seq + (h * act + p) * PER_STEP + part, use = s >> slot_shift;
-                        const uint32_t slot = u * M.slots + (s & slot_mask);
-                        if (stop) continue;
-                        if (use > 0) {
-                            if (!mbar_wait_warp(empty_a + 8 * slot, (use - 1) & 1u, abort_flag, M.status, M.wait_limit)) { stop = true; continue; }
-                            tc_fence_after();
-                        }
-                        const uint32_t at = tmem_base + lane_sel + M.acc_cols + slot * SLOT_COLS;
-#pragma unroll
-                        for (uint32_t k = 0; k < SLOT_COLS; k += 16) tmem_st16(at + k, v + part * SLOT_COLS + k);
-                        tmem_st_wait();
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(full_a + 8 * slot);
+                    expand32(mw[k * WORDS], bw[k * WORDS], v);
+                    expand32(mw[k * WORDS + 1], bw[k * WORDS + 1], v + 16);
+                    if (use > 0) {
+                        if (!mbar_wait_warp(empty_a + 8 * slot, (use - 1) & 1u, abort_flag, M.status, M.wait_limit)) goto leave;
+                        tc_fence_after();
                     }
+                    tmem_st16(at, v);
+                    tmem_st16(at + 16, v + 16);
+                    if constexpr (WORDS == 4) {
+                        expand32(mw[k * WORDS + 2], bw[k * WORDS + 2], v);
+                        expand32(mw[k * WORDS + 3], bw[k * WORDS + 3], v + 16);
+                        tmem_st16(at + 32, v);
+                        tmem_st16(at + 48, v + 16);
+                    }
+                    tmem_st_wait();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(full_a + 8 * slot);
                 }
-                seq += STEPS * act * PER_STEP;
+                seq += 2 * PER_X * act;
             }
-            seq0 += STEPS * P.len * PER_STEP;
+            seq0 += 2 * PER_X * P.len;
             // ------------------------------ epilogue of the part ------------------------------
-            if (stop || !mbar_wait_warp(accum, part_no & 1u, abort_flag, M.status, M.wait_limit)) break;
-            tc_fence_after();
             const uint32_t b0 = P.chunk * M.N;
             for (uint32_t t = 0; t < M.mt; ++t) {
-                const uint64_t r = ((uint64_t)P.group * M.mt + t) * MROWS + quad * 32 + lane;
+                const uint32_t r = (P.group * M.mt + t) * MROWS + quad * 32 + lane;
                 float al[MAX_UNITS];
 #pragma unroll
                 for (uint32_t k = 0; k < MAX_UNITS; ++k) {
                     const uint32_t pl = P.pg * M.planes + k;
-                    al[k] = k < M.planes && pl < M.n_q && r < M.m ? 0.5f * __ldg(M.alpha + r * M.n_q + pl) : 0.0f;
+                    al[k] = k < M.planes && pl < M.n_q && r < M.m ? 0.5f * __ldg(M.alpha + (uint64_t)r * M.n_q + pl) : 0.0f;
                 }
-                for (uint32_t j = g; j < M.N / 16; j += groups) {
+                if (t == 0) {
+                    if (!mbar_wait_warp(accum, part_no & 1u, abort_flag, M.status, M.wait_limit)) goto leave;
+                    tc_fence_after();
+                }
+                float *dst = M.y + (int64_t)(b0 + g * 16) * M.ldy + (int64_t)r;
+                for (uint32_t j = g; j < M.N / 16; j += groups, dst += (int64_t)groups * 16 * M.ldy) {
                     if (b0 + j * 16 >= M.batch) break;
                     float sum[16];
 #pragma unroll
@@ -438,10 +464,10 @@ k_decode_mma(const __grid_constant__ CUtensorMap xmap, const MmaArgs M)
                         for (uint32_t e = 0; e < 16; ++e) sum[e] = fmaf(al[k], __uint_as_float(d[e]), sum[e]);
                     }
                     if (r < M.m) {
-                        float *dst = M.y + (int64_t)(b0 + j * 16) * M.ldy + (int64_t)r;
+                        float *q = dst;
 #pragma unroll
-                        for (uint32_t e = 0; e < 16; ++e)
-                            if (b0 + j * 16 + e < M.batch) atomicAdd(dst + (int64_t)e * M.ldy, sum[e]);
+                        for (uint32_t e = 0; e < 16; ++e, q += M.ldy)
+                            if (b0 + j * 16 + e < M.batch) atomicAdd(q, sum[e]);
                     }
                 }
             }
@@ -456,19 +482,21 @@ k_decode_mma(const __grid_constant__ CUtensorMap xmap, const MmaArgs M)
         if (lane == 0 && !M.skip_loads) {
             uint32_t stage = 0, use = 0;
             bool ok = true;
-            for (uint64_t pos = begin; pos < end && ok;) {
-                const Part P(M, pos, end);
+            for (uint32_t pos = begin; pos < end && ok;) {
+                const Part<PHASES> P(M, pos, end);
+                const int32_t b0 = (int32_t)(P.chunk * M.N);
                 for (uint32_t i = 0; i < P.rounds() && ok; ++i) {
-                    const uint32_t act = P.active(i, M.phases);
-                    for (uint32_t h = 0; h < STEPS && ok; ++h)
-                        for (uint32_t p = 0; p < act && ok; ++p) {
-                            if (use > 0) ok = mbar_wait(empty_x + 8 * stage, (use - 1) & 1u, abort_flag, M.status, M.wait_limit);
-                            if (!ok) break;
-                            mbar_expect_tx(full_x + 8 * stage, x_bytes);
-                            tma_load_2d(x_sa + stage * x_bytes, &xmap, full_x + 8 * stage,
-                                        (int32_t)((P.first(p) + i) * MACRO + h * KC), (int32_t)(P.chunk * M.N));
-                            if (++stage == M.xstages) { stage = 0; ++use; }
-                        }
+                    const uint32_t act = P.active(i);
+                    for (uint32_t cp = 0; cp < 2 * act && ok; ++cp) {
+                        const uint32_t c = cp >= act ? 1u : 0u, p = cp - c * act;
+                        if (use > 0) ok = mbar_wait(empty_x + 8 * stage, (use - 1) & 1u, abort_flag, M.status, M.wait_limit);
+                        if (!ok) break;
+                        const int32_t col = (int32_t)((P.first(p) + i) * MACRO + c * KX);
+                        mbar_expect_tx(full_x + 8 * stage, x_bytes);
+                        tma_load_2d(x_sa + stage * x_bytes, &xmap, full_x + 8 * stage, col, b0);
+                        tma_load_2d(x_sa + stage * x_bytes + box_bytes, &xmap, full_x + 8 * stage, col + 64, b0);
+                        if (++stage == M.xstages) { stage = 0; ++use; }
+                    }
                 }
                 pos += P.len;
             }
@@ -482,37 +510,41 @@ k_decode_mma(const __grid_constant__ CUtensorMap xmap, const MmaArgs M)
     } else {
         // ------------------------------ MMA issuers (one converged warp per unit) ------------------------------
         const uint32_t u = warp - (4 * groups + 1);
-        const uint32_t idesc = instr_desc_bf16(M.N), d_tmem = tmem_base + u * M.N, a_tmem = tmem_base + M.acc_cols;
+        const uint32_t idesc = instr_desc_bf16(M.N), d_tmem = tmem_base + u * M.N, a_tmem = tmem_base + M.acc_cols + u * M.slots * SLOT_COLS;
         // descriptors differ only in the start-address field (units of 16 bytes)
         const uint64_t x_desc0 = smem_desc_sw128(x_sa);
-        const uint32_t x_step = x_bytes >> 4;
-        uint32_t stage = 0, x_parity = 0, seq = 0, part_no = 0;
-        bool ok = true;
-        for (uint64_t pos = begin; pos < end && ok;) {
-            const Part P(M, pos, end);
-            if (part_no) ok = mbar_wait_warp(acc_free, (part_no - 1) & 1u, abort_flag, M.status, M.wait_limit);
-            const uint32_t steps = STEPS * P.len;
-            for (uint32_t k = 0; k < steps && ok; ++k) {
-                ok = mbar_wait_warp(full_x + 8 * stage, x_parity, abort_flag, M.status, M.wait_limit);
+        const uint32_t x_step = x_bytes >> 4, box_step = box_bytes >> 4;
+        const uint32_t my_full = full_a + 8 * u * M.slots, my_empty = empty_a + 8 * u * M.slots;
+        uint32_t xs = 0, x_parity = 0, seq = 0, part_no = 0;      // first X stage of the round and its parity
+        for (uint32_t pos = begin; pos < end;) {
+            const Part<PHASES> P(M, pos, end);
+            if (part_no && !mbar_wait_warp(acc_free, (part_no - 1) & 1u, abort_flag, M.status, M.wait_limit)) goto leave;
+            uint32_t accumulate = 0;                              // the first slot of a part overwrites the accumulator
+            for (uint32_t i2 = 0; i2 < 2 * P.rounds(); ++i2) {
+                const uint32_t act = P.active(i2 >> 1);
 #pragma unroll
-                for (uint32_t part = 0; part < PER_STEP; ++part, ++seq) {
-                    const uint32_t slot = u * M.slots + (seq & slot_mask);
-                    ok = ok && mbar_wait_warp(full_a + 8 * slot, (seq >> slot_shift) & 1u, abort_flag, M.status, M.wait_limit);
-                    if (!ok) break;
-                    tc_fence_after();
-                    // the first step of a part overwrites the accumulator
-                    mma_slot<SLOT_COLS / 8>(d_tmem, a_tmem + slot * SLOT_COLS, x_desc0 + stage * x_step + part * (SLOT_COLS / 4),
-                                            idesc, k + part, empty_a + 8 * slot);
+                for (uint32_t j = 0; j < PER_X; ++j) {
+                    uint32_t stage = xs, parity = x_parity;
+                    for (uint32_t p = 0; p < act; ++p, ++seq) {
+                        const uint32_t slot = seq & slot_mask;
+                        if (j == 0 && !mbar_wait_warp(full_x + 8 * stage, parity, abort_flag, M.status, M.wait_limit)) goto leave;
+                        if (!mbar_wait_warp(my_full + 8 * slot, (seq >> slot_shift) & 1u, abort_flag, M.status, M.wait_limit)) goto leave;
+                        tc_fence_after();
+                        mma_slot<SLOT_COLS / 8>(d_tmem, a_tmem + slot * SLOT_COLS, x_desc0 + stage * x_step + j * box_step, idesc,
+                                                accumulate, my_empty + 8 * slot, box_step);
+                        accumulate = 1;
+                        if (j == PER_X - 1) mma_commit(empty_x + 8 * stage);
+                        if (++stage == M.xstages) { stage = 0; parity ^= 1u; }
+                    }
+                    if (j == PER_X - 1) { xs = stage; x_parity = parity; }
                 }
-                if (!ok) break;
-                mma_commit(empty_x + 8 * stage);
-                if (++stage == M.xstages) { stage = 0; x_parity ^= 1u; }
             }
-            if (ok) mma_commit(accum);
+            mma_commit(accum);
             ++part_no;
             pos += P.len;
         }
     }
+leave:
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -581,25 +613,25 @@ int mma_dispatch(const sqnn_desc *desc, const DecodeArgs &A0, const uint64_t *d_
     M.chunks = (batch + n_max - 1) / n_max;
     M.N = ((batch + M.chunks - 1) / M.chunks + 15) / 16 * 16;
     M.acc_cols = (units * M.N + 31) / 32 * 32;
-    // A slots of a whole step (32 TMEM columns) if every unit gets at least two, else of half a step
-    const uint32_t per_unit = (512 - M.acc_cols) / units, slot_cols = per_unit >= 64 ? 32u : 16u;
-    M.slots = per_unit / slot_cols >= 8 ? 8u : per_unit / slot_cols >= 4 ? 4u : 2u;
-    // Groups of four warps: four, or three for three planes, so that every group always serves the same unit.
-    M.phases = units == 1 ? 4u : units == 2 ? 2u : 1u;
-    const uint32_t threads = units * M.phases * 128 + 32 + units * 32;
-    const size_t x_bytes = (size_t)M.N * KC * 2;
+    // A slots of 64 TMEM columns if every unit gets two of them, else of 32; one slot of 32 per unit is enough
+    // where three or four units take turns on the tensor cores
+    const uint32_t per_unit = (512 - M.acc_cols) / units, slot_cols = per_unit >= 128 ? 64u : 32u;
+    M.slots = per_unit / slot_cols >= 8 ? 8u : per_unit / slot_cols >= 4 ? 4u : per_unit / slot_cols >= 2 ? 2u : 1u;
+    const size_t x_bytes = (size_t)M.N * KX * 2;
     M.xstages = (uint32_t)(XSTAGE_BUDGET / x_bytes < MAX_XSTAGES ? XSTAGE_BUDGET / x_bytes : MAX_XSTAGES);
     const size_t smem = M.xstages * x_bytes + 1024;
     M.macros = (uint32_t)((desc->n + MACRO - 1) / MACRO);
-    M.total = (M.m + M.mt * MROWS - 1) / (M.mt * MROWS) * M.plane_groups * M.chunks * M.macros;
-    const uint32_t grid = M.total < (uint64_t)sm_count() ? (uint32_t)M.total : (uint32_t)sm_count();
+    const uint64_t total = (M.m + M.mt * MROWS - 1) / (M.mt * MROWS) * M.plane_groups * M.chunks * M.macros;
+    if (total > 0x7fffffffull || M.m > 0x7fffff00ull) return SQNN_E_UNSUPPORTED;
+    M.total = (uint32_t)total;
+    const uint32_t grid = M.total < (uint32_t)sm_count() ? M.total : (uint32_t)sm_count();
     // rows of mask and planes start on 16-byte boundaries
     const bool aligned = desc->n % 128 == 0 && ((uintptr_t)d_mask & 15) == 0 && (M.plane_words32 % 4 == 0 || M.n_q == 1);
 
     CUtensorMap xmap;
     const cuuint64_t gdim[2] = {(cuuint64_t)desc->n, (cuuint64_t)batch};
     const cuuint64_t gstride[1] = {(cuuint64_t)ldx * 2};
-    const cuuint32_t box[2] = {KC, M.N};
+    const cuuint32_t box[2] = {KX / 2, M.N};
     const cuuint32_t estride[2] = {1, 1};
     if (encode(&xmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(d_x), gdim, gstride, box, estride,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -609,9 +641,13 @@ int mma_dispatch(const sqnn_desc *desc, const DecodeArgs &A0, const uint64_t *d_
     // stage 1: the decode kernel writes the planes as packed bits into the workspace and clears Y
     const int rc = decode_bits_dispatch(A0, d_workspace, ClearArgs{d_y, desc->m, ldy, batch}, st);
     if (rc != SQNN_OK) return rc;
-    auto k = slot_cols == 32 ? (aligned ? k_decode_mma<true, 32> : k_decode_mma<false, 32>)
-                             : (aligned ? k_decode_mma<true, 16> : k_decode_mma<false, 16>);
-    return launch_kernel(k, grid, threads, smem, st, xmap, M);
+#define SQNN_MMA_PICK(U, COLS) (aligned ? k_decode_mma<U, true, COLS> : k_decode_mma<U, false, COLS>)
+    auto k = units == 1   ? SQNN_MMA_PICK(1, 64)
+             : units == 2 ? (slot_cols == 64 ? SQNN_MMA_PICK(2, 64) : SQNN_MMA_PICK(2, 32))
+             : units == 3 ? (slot_cols == 64 ? SQNN_MMA_PICK(3, 64) : SQNN_MMA_PICK(3, 32))
+                          : SQNN_MMA_PICK(4, 32);
+#undef SQNN_MMA_PICK
+    return launch_kernel(k, grid, threads_of(units), smem, st, xmap, M);
 }
 
 }  // namespace sqnn
