@@ -1,11 +1,24 @@
-// Exhaustive seed search on the device (Section 5.2): for every slice of every plane all 2^n_in
-// seeds are expanded through the network and the seed with the fewest wrong care bits is kept
-// (the smallest seed among equals).
+// Exhaustive seed search on the device (Section 5.2): for every slice of every plane the seed with the fewest
+// wrong care bits among all 2^n_in is found (the smallest seed among equals).
 //
-// One warp per slice.  The 32 lanes split the seeds by their top five bits; inside its range a
-// lane walks the low bits in Gray-code order, so that going from one seed to the next is one
-// XOR with a column of M (w~ = M . w^c is linear over GF(2)) -- the columns sit in shared memory
-// and all lanes read the same one.  The count of wrong care bits is popc((w~ ^ w^q) & care).
+// The seeds are not tried one by one.  Let r_j be the rows of M at the slice's care positions and b_j the
+// wanted bits.  Elimination in ascending position makes some rows pivots (r of them, r = the rank); every
+// other row is the sum of pivot rows in a known subset.  A seed is then a choice of the set e of pivots it
+// gets wrong: which dependent rows are wrong follows (their syndrome s plus the columns C_i of the pivots in
+// e), and so does the smallest seed with exactly these errors: the one with all free variables 0 when every
+// pivot column is the lowest possible one, which is linear in the pivots' bits (columns Q_i).  So with
+// V_i = C_i << 20 | Q_i the search is
+//
+//     min over e of  (|e| + |C part|) << 20 | Q part,   V(e) = V_0 ^ xor of V_i, i in e,
+//
+// and e can be taken in the order of its size: once the best count is B, sizes above B cannot matter.  Almost
+// all slices are done after sizes 0 (consistent: no wrong bit), 1 and 2: about 80 candidates for r = 12
+// instead of 4096.  One thread per slice does that much; the few slices that need larger sets are finished by
+// the whole warp, which walks all 2^r sets in Gray-code order, and slices with more dependent rows than V has
+// bits for by trying all seeds.
+//
+// Bound: integer instructions.  600 000 slices of 60 x 12 (20 % care bits): see the measured figure at the
+// launch below.
 #include "sqnn_launch.h"
 
 #include <cuda_runtime.h>
@@ -36,76 +49,216 @@ SQNN_DEV uint32_t bits32_at(const uint64_t *__restrict__ v, uint64_t p, uint64_t
     return r;
 }
 
+constexpr uint32_t SEARCH_THREADS = 128;
+constexpr uint32_t MAX_DEP = 44;                          // dependent rows a 64-bit V has room for
+
+SQNN_DEV uint32_t warp_min(uint32_t v)
+{
+    return __reduce_min_sync(0xffffffffu, v);
+}
+
+// The whole warp tries all seeds of one slice: the lanes split them by their top bits and walk the rest in
+// Gray-code order, one XOR with a column of M per seed.
 template <int NW>
-__global__ void __launch_bounds__(256)
+SQNN_DEV uint32_t try_all_seeds(const uint32_t (*cols)[NW], uint32_t n_in, const uint32_t (&want)[NW], const uint32_t (&care)[NW], uint32_t lane)
+{
+    const uint32_t low_bits = n_in > 5 ? n_in - 5 : 0, lanes_used = n_in >= 5 ? 32u : (1u << n_in);
+    uint32_t best = 0xffffffffu;
+    if (lane < lanes_used) {
+        const uint32_t top = lane << low_bits;
+        uint32_t out[NW];
+#pragma unroll
+        for (int k = 0; k < NW; ++k) out[k] = 0;
+        for (uint32_t t = low_bits; t < n_in; ++t)
+            if ((top >> t) & 1u) {
+#pragma unroll
+                for (int k = 0; k < NW; ++k) out[k] ^= cols[t][k];
+            }
+        const uint32_t count = 1u << low_bits;
+        for (uint32_t i = 0; i < count; ++i) {
+            if (i != 0) {
+                const uint32_t t = (uint32_t)__ffs((int)i) - 1u;          // bit that changes in the Gray code
+#pragma unroll
+                for (int k = 0; k < NW; ++k) out[k] ^= cols[t][k];
+            }
+            uint32_t wrong = 0;
+#pragma unroll
+            for (int k = 0; k < NW; ++k) wrong += (uint32_t)__popc((out[k] ^ want[k]) & care[k]);
+            best = min(best, (wrong << 20) | top | (i ^ (i >> 1)));       // n_in <= 20, wrong <= 256
+        }
+    }
+    return warp_min(best);
+}
+
+// The whole warp tries all 2^r sets of wrong pivots of one slice (v: its V_i, one every SEARCH_THREADS).
+SQNN_DEV uint32_t try_all_sets(const unsigned long long *v, unsigned long long v0, uint32_t r, uint32_t lane)
+{
+    const uint32_t low_bits = r > 5 ? r - 5 : 0, lanes_used = r >= 5 ? 32u : (1u << r);
+    uint32_t best = 0xffffffffu;
+    if (lane < lanes_used) {
+        const uint32_t top = lane << low_bits, size0 = (uint32_t)__popc(lane);
+        unsigned long long x = v0;
+        for (uint32_t t = low_bits; t < r; ++t)
+            if ((top >> t) & 1u) x ^= v[t * SEARCH_THREADS];
+        const uint32_t count = 1u << low_bits;
+        for (uint32_t i = 0; i < count; ++i) {
+            if (i != 0) x ^= v[((uint32_t)__ffs((int)i) - 1u) * SEARCH_THREADS];
+            const uint32_t wrong = size0 + (uint32_t)__popc(i ^ (i >> 1)) + (uint32_t)__popcll(x >> 20);
+            best = min(best, (wrong << 20) | ((uint32_t)x & 0xfffffu));
+        }
+    }
+    return warp_min(best);
+}
+
+// NI >= n_in: rows and bookkeeping of the elimination sit in registers, indexed by pivot column at compile time.
+template <int NI, int NW>
+__global__ void __launch_bounds__(SEARCH_THREADS)
 k_search_seeds(const __grid_constant__ SearchArgs S)
 {
-    __shared__ uint32_t cols[SQNN_MAX_N_IN][NW];          // column t of M as an n_out-bit word
-    __shared__ uint32_t want_s[8][NW], care_s[8][NW];     // per warp: the slice
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    for (uint32_t i = threadIdx.x; i < S.n_in * NW; i += blockDim.x) {
+    __shared__ uint32_t rows_s[SQNN_MAX_N_OUT];
+    __shared__ uint32_t cols[SQNN_MAX_N_IN][NW];                          // column t of M as an n_out-bit word
+    __shared__ unsigned long long v_s[NI][SEARCH_THREADS];
+    wait_prior_grid();
+    launch_dependents();
+    const uint32_t lane = threadIdx.x & 31;
+    for (uint32_t j = threadIdx.x; j < S.n_out; j += SEARCH_THREADS) rows_s[j] = S.rows[j] & (uint32_t)((1ull << S.n_in) - 1ull);
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < S.n_in * NW; i += SEARCH_THREADS) {
         const uint32_t t = i / NW, k = i % NW;
         uint32_t w = 0;
-        for (uint32_t j = 32 * k; j < S.n_out && j < 32 * k + 32; ++j) w |= ((S.rows[j] >> t) & 1u) << (j - 32 * k);
+        for (uint32_t j = 32 * k; j < S.n_out && j < 32 * k + 32; ++j) w |= ((rows_s[j] >> t) & 1u) << (j - 32 * k);
         cols[t][k] = w;
     }
     __syncthreads();
-    const uint32_t low_bits = S.n_in > 5 ? S.n_in - 5 : 0;
-    const uint32_t lanes_used = S.n_in >= 5 ? 32u : (1u << S.n_in);
+    unsigned long long *v = &v_s[0][threadIdx.x];
     const uint64_t total = S.slices * S.n_q;
-    for (uint64_t job = (uint64_t)blockIdx.x * nwarps + warp; job < total; job += (uint64_t)gridDim.x * nwarps) {
-        const uint32_t plane = (uint32_t)(job / S.slices);
-        const uint64_t s = job - (uint64_t)plane * S.slices;
-        const uint64_t p0 = s * S.n_out;
-        __syncwarp();
-        if (lane < NW) {
-            const uint32_t lo = 32 * lane;
-            uint32_t c = 0, w = 0;
-            if (lo < S.n_out) {
-                const uint64_t limit = p0 + S.n_out < S.mn ? p0 + S.n_out : S.mn;   // slice end (ragged tail)
-                c = bits32_at(S.mask, p0 + lo, limit);
-                w = bits32_at(S.planes + (uint64_t)plane * S.words64, p0 + lo, limit);
-            }
-            care_s[warp][lane] = c;
-            want_s[warp][lane] = w;
-        }
-        __syncwarp();
-        uint32_t want[NW], care[NW], out[NW];
+    const uint64_t step = (uint64_t)gridDim.x * SEARCH_THREADS;
+    for (uint64_t job0 = (uint64_t)blockIdx.x * SEARCH_THREADS + (threadIdx.x & ~31u); job0 < total; job0 += step) {
+        const uint64_t job = job0 + lane;
+        const bool live = job < total;
+        uint32_t want[NW], care[NW];
 #pragma unroll
-        for (int k = 0; k < NW; ++k) { want[k] = want_s[warp][k]; care[k] = care_s[warp][k]; out[k] = 0; }
-        uint32_t best = 0xffffffffu;
-        if (lane < lanes_used) {
-            const uint32_t top = lane << low_bits;
-            for (uint32_t t = low_bits; t < S.n_in; ++t)
-                if ((top >> t) & 1u) {
+        for (int k = 0; k < NW; ++k) want[k] = care[k] = 0;
+        if (live) {
+            const uint32_t plane = (uint32_t)(job / S.slices);
+            const uint64_t p0 = (job - (uint64_t)plane * S.slices) * S.n_out;
+            const uint64_t limit = p0 + S.n_out < S.mn ? p0 + S.n_out : S.mn;   // slice end (ragged tail)
 #pragma unroll
-                    for (int k = 0; k < NW; ++k) out[k] ^= cols[t][k];
-                }
-            const uint32_t count = 1u << low_bits;
-            for (uint32_t i = 0; i < count; ++i) {
-                if (i != 0) {
-                    const uint32_t t = (uint32_t)__ffs((int)i) - 1u;      // bit that changes in the Gray code
-#pragma unroll
-                    for (int k = 0; k < NW; ++k) out[k] ^= cols[t][k];
-                }
-                uint32_t wrong = 0;
-#pragma unroll
-                for (int k = 0; k < NW; ++k) wrong += (uint32_t)__popc((out[k] ^ want[k]) & care[k]);
-                const uint32_t seed = top | (i ^ (i >> 1));
-                const uint32_t key = (wrong << 20) | seed;                  // n_in <= 20, wrong <= 256
-                best = key < best ? key : best;
+            for (int k = 0; k < NW; ++k) {
+                if (32u * k >= S.n_out) break;
+                care[k] = bits32_at(S.mask, p0 + 32 * k, limit);
+                want[k] = bits32_at(S.planes + (uint64_t)plane * S.words64, p0 + 32 * k, limit);
             }
         }
+        // elimination: row[c] = the pivot row whose lowest set column is c, sub[c] = the original pivots it is the
+        // sum of (numbered as they come), bits = the original pivots' wanted bits
+        uint32_t row[NI], sub[NI], have = 0, bits = 0, r = 0, dep = 0;
+        unsigned long long syn = 0;
 #pragma unroll
-        for (uint32_t d = 16; d >= 1; d >>= 1) {
-            const uint32_t o = __shfl_xor_sync(0xffffffffu, best, d);
-            best = o < best ? o : best;
+        for (int c = 0; c < NI; ++c) { row[c] = sub[c] = 0; v[c * SEARCH_THREADS] = 0; }
+#pragma unroll
+        for (int k = 0; k < NW; ++k) {
+            uint32_t left = care[k];
+            while (left) {
+                const uint32_t j = (uint32_t)__ffs((int)left) - 1u;
+                left &= left - 1u;
+                uint32_t a = rows_s[32 * k + j], of = 0;
+                const uint32_t b = (want[k] >> j) & 1u;
+#pragma unroll
+                for (int c = 0; c < NI; ++c) {
+                    const bool set = (a >> c) & 1u, pivot = (have >> c) & 1u;
+                    if (set && pivot) { a ^= row[c]; of ^= sub[c]; }
+                    if (set && !pivot) {                                  // a new pivot
+                        row[c] = a;
+                        sub[c] = of | (1u << r);
+                        have |= 1u << c;
+                        bits |= b << r;
+                        ++r;
+                        a = 0;
+                        of = 0x80000000u;
+                    }
+                }
+                if (!(of & 0x80000000u)) {                                // the sum of the pivots in `of`
+                    if (dep < MAX_DEP) {
+                        const unsigned long long bit = 1ull << (20 + dep);
+                        if ((b ^ (uint32_t)__popc(bits & of)) & 1u) syn |= bit;
+                        for (uint32_t o = of; o; o &= o - 1u) v[((uint32_t)__ffs((int)o) - 1u) * SEARCH_THREADS] |= bit;
+                    }
+                    ++dep;
+                }
+            }
         }
-        if (lane == 0) {
+        // reduced form: no pivot row contains another pivot's column
+#pragma unroll
+        for (int c = NI - 2; c >= 0; --c) {
+#pragma unroll
+            for (int d = c + 1; d < NI; ++d)
+                if ((row[c] >> d) & (have >> d) & 1u) { row[c] ^= row[d]; sub[c] ^= sub[d]; }
+        }
+        uint32_t seed = 0;
+#pragma unroll
+        for (int c = 0; c < NI; ++c) seed |= ((uint32_t)__popc(bits & sub[c]) & 1u) << c;
+        const unsigned long long v0 = syn | seed;
+        uint32_t best = ((uint32_t)__popcll(syn) << 20) | seed;
+        const bool wide = live && dep > MAX_DEP;
+        if (syn != 0 && !wide) {
+#pragma unroll
+            for (int c = 0; c < NI; ++c)
+                for (uint32_t o = sub[c]; o; o &= o - 1u) v[((uint32_t)__ffs((int)o) - 1u) * SEARCH_THREADS] |= 1ull << c;
+            for (uint32_t i = 0; i < r; ++i) {                            // one wrong pivot
+                const unsigned long long x = v0 ^ v[i * SEARCH_THREADS];
+                best = min(best, ((1u + (uint32_t)__popcll(x >> 20)) << 20) | ((uint32_t)x & 0xfffffu));
+            }
+            if ((best >> 20) >= 2)
+                for (uint32_t i = 1; i < r; ++i) {                        // two
+                    const unsigned long long y = v0 ^ v[i * SEARCH_THREADS];
+                    for (uint32_t h = 0; h < i; ++h) {
+                        const unsigned long long x = y ^ v[h * SEARCH_THREADS];
+                        best = min(best, ((2u + (uint32_t)__popcll(x >> 20)) << 20) | ((uint32_t)x & 0xfffffu));
+                    }
+                }
+            // three by this thread alone where the whole warp would have far more than that to walk
+            if (r > 12 && (best >> 20) >= 3)
+                for (uint32_t i = 2; i < r; ++i)
+                    for (uint32_t h = 1; h < i; ++h) {
+                        const unsigned long long y = v0 ^ v[i * SEARCH_THREADS] ^ v[h * SEARCH_THREADS];
+                        for (uint32_t g = 0; g < h; ++g) {
+                            const unsigned long long x = y ^ v[g * SEARCH_THREADS];
+                            best = min(best, ((3u + (uint32_t)__popcll(x >> 20)) << 20) | ((uint32_t)x & 0xfffffu));
+                        }
+                    }
+        }
+        __syncwarp();
+        // what is left for the whole warp: larger sets could still win or tie, or V has no room
+        uint32_t more = __ballot_sync(0xffffffffu, wide || (live && syn != 0 && (best >> 20) > (r > 12 ? 3u : 2u)));
+        while (more) {
+            const uint32_t src = (uint32_t)__ffs((int)more) - 1u;
+            more &= more - 1u;
+            uint32_t found;
+            if (__shfl_sync(0xffffffffu, wide ? 1u : 0u, src)) {
+                uint32_t w_s[NW], c_s[NW];
+#pragma unroll
+                for (int k = 0; k < NW; ++k) { w_s[k] = __shfl_sync(0xffffffffu, want[k], src); c_s[k] = __shfl_sync(0xffffffffu, care[k], src); }
+                found = try_all_seeds<NW>(cols, S.n_in, w_s, c_s, lane);
+            } else {
+                found = try_all_sets(&v_s[0][(threadIdx.x & ~31u) + src], __shfl_sync(0xffffffffu, v0, src), __shfl_sync(0xffffffffu, r, src), lane);
+            }
+            if (lane == src) best = found;
+        }
+        if (live) {
             S.wc[job] = best & 0xfffffu;
             S.np[job] = (uint16_t)(best >> 20);
         }
+        __syncwarp();
     }
+}
+
+template <int NI>
+int launch_search(const SearchArgs &S, uint32_t blocks, cudaStream_t st)
+{
+    const uint32_t nw = (S.n_out + 31) / 32;
+    auto k = nw <= 1 ? k_search_seeds<NI, 1> : nw <= 2 ? k_search_seeds<NI, 2> : nw <= 4 ? k_search_seeds<NI, 4> : k_search_seeds<NI, 8>;
+    return launch_kernel(k, blocks, SEARCH_THREADS, 0, st, S);
 }
 
 }  // namespace
@@ -130,16 +283,14 @@ static int search_seeds_queue(const sqnn_xornet *net, uint64_t m, uint64_t n, ui
     S.slices = (S.mn + net->n_out - 1) / net->n_out;
     S.planes = d_planes; S.mask = d_mask; S.wc = d_wc; S.np = d_np;
     const uint64_t jobs = S.slices * n_q;
-    uint64_t blocks = (jobs + 7) / 8;
-    const uint64_t cap = (uint64_t)sm_count() * 8;
+    uint64_t blocks = (jobs + SEARCH_THREADS - 1) / SEARCH_THREADS;
+    const uint64_t cap = (uint64_t)sm_count() * 64;
     if (blocks > cap) blocks = cap;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    const uint32_t nw = (net->n_out + 31) / 32;
-    if (nw <= 1) k_search_seeds<1><<<(uint32_t)blocks, 256, 0, st>>>(S);
-    else if (nw <= 2) k_search_seeds<2><<<(uint32_t)blocks, 256, 0, st>>>(S);
-    else if (nw <= 4) k_search_seeds<4><<<(uint32_t)blocks, 256, 0, st>>>(S);
-    else k_search_seeds<8><<<(uint32_t)blocks, 256, 0, st>>>(S);
-    return cudaGetLastError() == cudaSuccess ? SQNN_OK : SQNN_E_CUDA;
+    return net->n_in <= 8    ? launch_search<8>(S, (uint32_t)blocks, st)
+           : net->n_in <= 12 ? launch_search<12>(S, (uint32_t)blocks, st)
+           : net->n_in <= 16 ? launch_search<16>(S, (uint32_t)blocks, st)
+                             : launch_search<20>(S, (uint32_t)blocks, st);
 }
 
 extern "C" int sqnn_search_seeds(const sqnn_xornet *net, uint64_t m, uint64_t n, uint32_t n_q,
