@@ -7,6 +7,7 @@
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <vector>
 
@@ -53,54 +54,92 @@ inline void load_slice(const uint64_t *plane, const uint64_t *mask, uint64_t mn,
     }
 }
 
-// w~ = M . w^c over GF(2): bit j = parity(rows[j] AND seed)
-inline void expand(const uint32_t *rows, uint32_t n_out, uint32_t seed, uint64_t out[4])
-{
-    out[0] = out[1] = out[2] = out[3] = 0;
-    for (uint32_t j = 0; j < n_out; ++j)
-        out[j >> 6] |= (uint64_t)(__builtin_popcount(rows[j] & seed) & 1) << (j & 63);
-}
+// w~ = M . w^c over GF(2) by table: the seed is cut into bytes, an entry is the XOR of the columns of M its byte
+// selects.  (Taking the parity of every row with the seed was four fifths of the encoder's time.)
+struct Expander {
+    uint32_t words, bytes;
+    std::vector<uint64_t> tab;                            // [byte][value][words]
+    Expander(const uint32_t *rows, uint32_t n_out, uint32_t n_in)
+        : words((n_out + 63) / 64), bytes((n_in + 7) / 8), tab((size_t)bytes * 256 * words, 0)
+    {
+        for (uint32_t t = 0; t < n_in; ++t) {             // the columns first: entries with one bit
+            uint64_t *e = &tab[((size_t)(t >> 3) * 256 + (1u << (t & 7))) * words];
+            for (uint32_t j = 0; j < n_out; ++j) e[j >> 6] |= (uint64_t)((rows[j] >> t) & 1) << (j & 63);
+        }
+        for (uint32_t b = 0; b < bytes; ++b)
+            for (uint32_t v = 1; v < 256; ++v)
+                if (v & (v - 1)) {
+                    uint64_t *e = &tab[((size_t)b * 256 + v) * words];
+                    const uint64_t *x = &tab[((size_t)b * 256 + (v & (v - 1))) * words], *y = &tab[((size_t)b * 256 + (v & (0u - v))) * words];
+                    for (uint32_t k = 0; k < words; ++k) e[k] = x[k] ^ y[k];
+                }
+    }
+    void operator()(uint32_t seed, uint64_t out[4]) const
+    {
+        out[0] = out[1] = out[2] = out[3] = 0;
+        for (uint32_t b = 0; b < bytes; ++b, seed >>= 8) {
+            const uint64_t *e = &tab[((size_t)b * 256 + (seed & 255u)) * words];
+            for (uint32_t k = 0; k < words; ++k) out[k] ^= e[k];
+        }
+    }
+};
 
-// Algorithm 1 on one slice.  The augmented matrix is kept in reduced row-echelon form while
-// care rows are appended in ascending position: a new row is first reduced against the pivots;
-// if it reduces to 0 = 1 it is the unsolvable case and is dropped (it will show up as a patch),
-// if it reduces to 0 = 0 it is redundant, otherwise its lowest set column becomes a new pivot
-// and is eliminated from the older rows.  Free variables are 0, so a pivot variable equals the
-// right-hand side of its row.
-inline uint32_t encode_alg1(const uint32_t *rows, uint32_t n_out, const SliceBits &sb)
+// Algorithm 1 on one slice.  Care rows are appended in ascending position to a system kept in echelon form
+// (a row's pivot is its lowest set column, its right-hand side rides in bit 32): a new row is reduced until its
+// lowest column has no pivot yet and is kept there; one that reduces to 0 = 1 is the unsolvable case and is
+// dropped (it will show up as a patch), one that reduces to 0 = 0 is redundant.  With `full` pivots (the rank
+// of M) no further row can be kept.  Free variables are 0, so the pivot variables follow from the highest
+// column down.
+inline uint32_t encode_alg1(const uint32_t *rows, uint32_t n_out, uint32_t full, const SliceBits &sb)
 {
-    uint32_t prow[SQNN_MAX_N_IN], pcol[SQNN_MAX_N_IN];
-    uint8_t prhs[SQNN_MAX_N_IN];
-    uint32_t npiv = 0;
-    for (uint32_t k = 0; k * 64 < n_out; ++k) {
+    uint64_t piv[SQNN_MAX_N_IN];
+    uint32_t have = 0, count = 0;
+    for (uint32_t k = 0; k * 64 < n_out && count < full; ++k) {
         uint64_t c = sb.care[k];
         while (c) {
             const uint32_t j = k * 64 + (uint32_t)__builtin_ctzll(c);
             c &= c - 1;
-            uint32_t a = rows[j];
-            uint8_t b = (uint8_t)((sb.want[k] >> (j & 63)) & 1);
-            for (uint32_t q = 0; q < npiv; ++q)
-                if ((a >> pcol[q]) & 1) { a ^= prow[q]; b ^= prhs[q]; }
-            if (a == 0) continue;                 // redundant or contradictory: nothing to keep
-            const uint32_t col = (uint32_t)ctz32(a);
-            for (uint32_t q = 0; q < npiv; ++q)
-                if ((prow[q] >> col) & 1) { prow[q] ^= a; prhs[q] ^= b; }
-            prow[npiv] = a; prhs[npiv] = b; pcol[npiv] = col;
-            ++npiv;
+            uint64_t a = (uint64_t)rows[j] | ((sb.want[k] >> (j & 63)) & 1) << 32;
+            while ((uint32_t)a) {
+                const uint32_t col = (uint32_t)ctz32((uint32_t)a);
+                if ((have >> col) & 1) { a ^= piv[col]; continue; }
+                piv[col] = a;
+                have |= 1u << col;
+                ++count;
+                break;
+            }
+            if (count == full) break;
         }
     }
     uint32_t seed = 0;
-    for (uint32_t q = 0; q < npiv; ++q)
-        if (prhs[q]) seed |= 1u << pcol[q];
+    for (uint32_t left = have; left;) {
+        const uint32_t col = 31u - (uint32_t)__builtin_clz(left);
+        left &= ~(1u << col);
+        const uint64_t a = piv[col];
+        seed |= (((uint32_t)(a >> 32) ^ (uint32_t)__builtin_popcount((uint32_t)a & seed)) & 1u) << col;
+    }
     return seed;
+}
+
+// Rank of the rows over GF(2).
+uint32_t rank_of(const uint32_t *rows, uint32_t n_out)
+{
+    uint32_t piv[SQNN_MAX_N_IN] = {0}, rank = 0;
+    for (uint32_t j = 0; j < n_out; ++j) {
+        uint32_t a = rows[j];
+        while (a && piv[ctz32(a)]) a ^= piv[ctz32(a)];
+        if (a) { piv[ctz32(a)] = a; ++rank; }
+    }
+    return rank;
 }
 
 // All 2^n_in outputs of the network, 4 words each.
 void build_outputs(const uint32_t *rows, uint32_t n_out, uint32_t n_in, std::vector<uint64_t> &tab)
 {
     const uint64_t cnt = (uint64_t)1 << n_in;
+    const Expander expand(rows, n_out, n_in);
     tab.assign(cnt * 4, 0);
-    for (uint64_t v = 0; v < cnt; ++v) expand(rows, n_out, (uint32_t)v, &tab[v * 4]);
+    for (uint64_t v = 0; v < cnt; ++v) expand((uint32_t)v, &tab[v * 4]);
 }
 
 inline uint32_t encode_exhaustive(const std::vector<uint64_t> &tab, uint32_t n_in, const SliceBits &sb)
@@ -120,7 +159,6 @@ inline uint32_t encode_exhaustive(const std::vector<uint64_t> &tab, uint32_t n_i
 struct PlaneArrays {
     std::vector<uint32_t> wc;
     std::vector<uint16_t> np;
-    std::vector<uint8_t> dp;
 };
 
 uint64_t round_up(uint64_t v, uint64_t a) { return (v + a - 1) / a * a; }
@@ -132,7 +170,7 @@ void pack_fields(const T *vals, uint64_t count, uint32_t width, uint32_t *dst)
 {
     if (width == 0) return;
     const int64_t groups = (int64_t)((count + 31) / 32);
-#pragma omp parallel for schedule(static)
+#pragma omp parallel for schedule(static) if (count >= 8192)
     for (int64_t g = 0; g < groups; ++g) {
         uint32_t *w = dst + (uint64_t)g * width;
         uint64_t acc = 0;
@@ -164,19 +202,18 @@ void build_tables(const uint32_t *rows, uint32_t n_out, uint32_t n_in, uint32_t 
     const uint32_t nch = sqnn::table_chunks(n_in, nwp), cb = sqnn::chunk_bits(n_in, nwp);
     std::memset(tab, 0, (size_t)sqnn::table_words(n_out, n_in) * 4);
     for (uint32_t ch = 0; ch < nch; ++ch)
-        for (uint32_t v = 0; v < (1u << cb); ++v) {
-            // chunk bits that lie past n_in select no column
-            const uint64_t sel64 = (uint64_t)v << (ch * cb);
-            const uint32_t sel = (uint32_t)(sel64 & (n_in >= 32 ? 0xffffffffull : ((1ull << n_in) - 1ull)));
+        for (uint32_t v = 1; v < (1u << cb); ++v) {
             uint32_t *e = tab + (size_t)(((ch << cb) | v)) * nwp;
-            for (uint32_t j = 0; j < n_out; ++j)
-                e[j >> 5] |= (uint32_t)(__builtin_popcount(rows[j] & sel) & 1) << (j & 31);
+            if (v & (v - 1)) {                            // the sum of two entries made before it
+                const uint32_t *x = tab + (size_t)((ch << cb) | (v & (v - 1))) * nwp, *y = tab + (size_t)((ch << cb) | (v & (0u - v))) * nwp;
+                for (uint32_t k = 0; k < nwp; ++k) e[k] = x[k] ^ y[k];
+                continue;
+            }
+            const uint32_t t = ch * cb + (uint32_t)ctz32(v);           // one column of M; bits past n_in select none
+            if (t < n_in)
+                for (uint32_t j = 0; j < n_out; ++j) e[j >> 5] |= ((rows[j] >> t) & 1u) << (j & 31);
         }
 }
-
-struct BlobPlan {
-    sqnn_desc d;
-};
 
 // Section offsets of a device blob for the given patch totals.
 void plan_blob(uint64_t m, uint64_t n, uint32_t n_q, uint32_t n_out, uint32_t n_in, const uint64_t *n_pp, sqnn_desc *out)
@@ -207,60 +244,78 @@ void plan_blob(uint64_t m, uint64_t n, uint32_t n_q, uint32_t n_out, uint32_t n_
     *out = d;
 }
 
-int build_blob(const sqnn_xornet *net, uint64_t m, uint64_t n, uint32_t n_q,
-               const uint32_t *const *wc, const uint16_t *const *np, const uint8_t *const *dp8,
-               const uint16_t *const *dp16, void **blob, size_t *blob_bytes)
+// Host loops over slices or tiles run in parallel from this many slices on (below it a thread team costs more
+// than it saves).
+constexpr uint64_t PARALLEL_FROM = 8192;
+
+// Allocates a blob for the given patch totals: header, rows of M and tables in place, streams zero.
+uint8_t *start_blob(const sqnn_xornet *net, uint64_t m, uint64_t n, uint32_t n_q, const uint64_t *n_pp, sqnn_desc *d)
 {
-    const uint64_t mn = m * n;
-    const uint32_t n_out = net->n_out, n_in = net->n_in;
-    const uint64_t l = (mn + n_out - 1) / n_out;
-    uint64_t n_pp[SQNN_MAX_PLANES] = {0};
-    for (uint32_t i = 0; i < n_q; ++i) {
-        uint64_t sum = 0;
-        for (uint64_t s = 0; s < l; ++s) {
-            if (np[i][s] > n_out) return SQNN_E_INVALID_ARG;
-            sum += np[i][s];
-        }
-        if (sum > 0xffffffffull) return SQNN_E_INVALID_ARG;
-        n_pp[i] = sum;
-    }
-    sqnn_desc d;
-    plan_blob(m, n, n_q, n_out, n_in, n_pp, &d);
-    const uint64_t lp = d.slices_padded;
-    uint8_t *b = (uint8_t *)std::calloc(d.total_bytes, 1);
-    if (!b) return SQNN_E_NOMEM;
+    plan_blob(m, n, n_q, net->n_out, net->n_in, n_pp, d);
+    uint8_t *b = (uint8_t *)std::calloc(d->total_bytes, 1);
+    if (!b) return nullptr;
     sqnn_blob_header *h = (sqnn_blob_header *)b;
     std::memcpy(h->magic, SQNN_BLOB_MAGIC, 8);
     h->version = SQNN_BLOB_VERSION;
     h->header_bytes = SQNN_BLOB_HEADER_BYTES;
-    h->desc = d;
-    std::memcpy(b + d.off_xornet, net->rows, (size_t)n_out * 4);
-    build_tables(net->rows, n_out, n_in, (uint32_t *)(b + d.off_tables));
+    h->desc = *d;
+    std::memcpy(b + d->off_xornet, net->rows, (size_t)net->n_out * 4);
+    build_tables(net->rows, net->n_out, net->n_in, (uint32_t *)(b + d->off_tables));
+    return b;
+}
+
+int build_blob(const sqnn_xornet *net, uint64_t m, uint64_t n, uint32_t n_q,
+               const uint32_t *const *wc, const uint16_t *const *np, const uint16_t *const *dp, void **blob, size_t *blob_bytes)
+{
+    const uint64_t mn = m * n;
+    const uint32_t n_out = net->n_out, n_in = net->n_in;
+    const uint64_t l = (mn + n_out - 1) / n_out;
+    const int64_t tiles = (int64_t)((l + SQNN_TILE_SLICES - 1) / SQNN_TILE_SLICES);
+    const bool par = l >= PARALLEL_FROM;
+    uint64_t n_pp[SQNN_MAX_PLANES] = {0};
+    std::vector<std::vector<uint64_t>> first(n_q, std::vector<uint64_t>((size_t)tiles + 1));   // entries before each tile
+    int bad = 0;
     for (uint32_t i = 0; i < n_q; ++i) {
-        if (n_in < 32)
-            for (uint64_t s = 0; s < l; ++s)
-                if (wc[i][s] >> n_in) { std::free(b); return SQNN_E_INVALID_ARG; }
+#pragma omp parallel for schedule(static) if (par) reduction(| : bad)
+        for (int64_t t = 0; t < tiles; ++t) {
+            const uint64_t lo = (uint64_t)t * SQNN_TILE_SLICES, hi = std::min<uint64_t>(l, lo + SQNN_TILE_SLICES);
+            uint64_t sum = 0;
+            for (uint64_t s = lo; s < hi; ++s) {
+                bad |= np[i][s] > n_out;
+                bad |= n_in < 32 && (wc[i][s] >> n_in) != 0;
+                sum += np[i][s];
+            }
+            first[i][(size_t)t + 1] = sum;
+        }
+        if (bad) return SQNN_E_INVALID_ARG;
+        for (int64_t t = 0; t < tiles; ++t) first[i][(size_t)t + 1] += first[i][(size_t)t];
+        n_pp[i] = first[i][(size_t)tiles];
+        if (n_pp[i] > 0xffffffffull) return SQNN_E_INVALID_ARG;
+    }
+    sqnn_desc d;
+    uint8_t *b = start_blob(net, m, n, n_q, n_pp, &d);
+    if (!b) return SQNN_E_NOMEM;
+    for (uint32_t i = 0; i < n_q; ++i) {
         pack_fields(wc[i], l, n_in, (uint32_t *)(b + d.off_wc[i]));
         uint32_t *idx = (uint32_t *)(b + d.off_idx[i]);
         uint16_t *dst = (uint16_t *)(b + d.off_pp[i]);
-        uint64_t run = 0;
-        const uint64_t tiles = lp / SQNN_TILE_SLICES;
-        for (uint64_t t = 0; t <= tiles; ++t) {
-            idx[t] = (uint32_t)run;
-            if (t == tiles) break;
-            const uint64_t lo = t * SQNN_TILE_SLICES, hi = std::min<uint64_t>(l, lo + SQNN_TILE_SLICES);
+        for (uint64_t t = 0; t <= d.slices_padded / SQNN_TILE_SLICES; ++t) idx[t] = (uint32_t)first[i][std::min<uint64_t>(t, (uint64_t)tiles)];
+#pragma omp parallel for schedule(static) if (par) reduction(| : bad)
+        for (int64_t t = 0; t < tiles; ++t) {
+            const uint64_t lo = (uint64_t)t * SQNN_TILE_SLICES, hi = std::min<uint64_t>(l, lo + SQNN_TILE_SLICES);
+            uint64_t run = first[i][(size_t)t];
             for (uint64_t s = lo; s < hi; ++s) {
                 int64_t prev = -1;
                 for (uint32_t k = 0; k < np[i][s]; ++k, ++run) {
-                    const uint32_t pos = dp8 ? dp8[i][run] : dp16[i][run];
+                    const uint32_t pos = dp[i][run];
                     // positions inside a slice ascend strictly; the last slice holds real positions only
-                    if (pos >= n_out || (int64_t)pos <= prev || s * n_out + pos >= mn) { std::free(b); return SQNN_E_INVALID_ARG; }
+                    bad |= pos >= n_out || (int64_t)pos <= prev || s * n_out + pos >= mn;
                     prev = pos;
                     dst[run] = (uint16_t)((s - lo) * n_out + pos);
                 }
             }
         }
-        if (run != n_pp[i]) { std::free(b); return SQNN_E_INVALID_ARG; }
+        if (bad) { std::free(b); return SQNN_E_INVALID_ARG; }
     }
     *blob = b;
     *blob_bytes = d.total_bytes;
@@ -294,9 +349,35 @@ const char *sqnn_status_string(int status)
     }
 }
 
+// Size accounting from the totals of a layer: hist over all planes, sum and max of n_patch per plane.
+static void fill_stats(const sqnn_desc &d, const uint64_t *sum, const uint32_t *maxp, const uint64_t *hist, sqnn_stats *stats)
+{
+    std::memset(stats, 0, sizeof *stats);
+    const uint64_t mn = d.m * d.n, l = d.slices, lp = d.slices_padded;
+    stats->slices = l;
+    std::memcpy(stats->patch_hist, hist, sizeof stats->patch_hist);
+    double eq1_bits = 0.0;
+    for (uint32_t i = 0; i < d.n_q; ++i) {
+        stats->patches[i] = sum[i];
+        stats->max_patch[i] = maxp[i];
+        // Eq. 1, literally: n_in/n_out * mn + l * ceil(lg max p) + sum p * ceil(lg n_out)
+        eq1_bits += (double)d.n_in / (double)d.n_out * (double)mn +
+                    (double)l * ceil_lg_u64(maxp[i]) + (double)sum[i] * ceil_lg_u64(d.n_out);
+        stats->bits_wc += (round_up(lp * d.n_in / 8, 16) + 16) * 8;
+        stats->bits_index += (round_up((lp / SQNN_TILE_SLICES + 1) * 4, 16) + 16) * 8;
+        stats->bits_dpatch += (round_up(sum[i] * 2, 16) + 16) * 8;
+    }
+    stats->bits_tables = (round_up(d.tables_bytes, 16) + 16) * 8;
+    stats->bits_index += stats->bits_tables;
+    stats->bpw_eq1 = eq1_bits / (double)mn;
+    stats->bpw_actual = (double)(stats->bits_wc + stats->bits_npatch + stats->bits_index + stats->bits_dpatch) / (double)mn;
+}
+
 // Shared by sqnn_encode_host and sqnn_encode_seeds_host: seeds come from Algorithm 1, from the
 // exhaustive search, or from the caller (given != NULL); patch counts and positions follow by
-// expanding each seed and comparing on the care bits.
+// expanding each seed and comparing on the care bits.  One parallel pass over the format tiles makes seeds,
+// patch entries (kept in a buffer of the thread) and statistics; a second one, once the totals are known,
+// packs the streams straight into the blob.
 static int encode_impl(const sqnn_xornet *net, const sqnn_planes *layer, bool exhaustive,
                        const uint32_t *const *given, void **blob, size_t *blob_bytes, sqnn_stats *stats)
 {
@@ -305,69 +386,110 @@ static int encode_impl(const sqnn_xornet *net, const sqnn_planes *layer, bool ex
         const uint32_t n_out = net->n_out, n_in = net->n_in, n_q = layer->n_q;
         const uint64_t l = (mn + n_out - 1) / n_out;
         const uint64_t words = (mn + 63) / 64;
+        const int64_t tiles = (int64_t)((l + SQNN_TILE_SLICES - 1) / SQNN_TILE_SLICES), items = tiles * n_q;
+        const Expander expand(net->rows, n_out, n_in);
+        const uint32_t full = rank_of(net->rows, n_out);
         std::vector<uint64_t> tab;
         if (exhaustive && !given) build_outputs(net->rows, n_out, n_in, tab);
-        std::vector<PlaneArrays> pa(n_q);
+        struct TileOut { const uint16_t *pp; uint32_t count; };
+        std::vector<TileOut> made((size_t)items);
+        std::unique_ptr<uint32_t[]> seeds(new uint32_t[(size_t)(l * n_q)]);
+        // entries of a thread's tiles in blocks that never move (a tile has at most 256 * n_out entries)
+        std::vector<std::unique_ptr<uint16_t[]>> blocks;
+        uint64_t sum[SQNN_MAX_PLANES] = {0}, hist[SQNN_PATCH_HIST_BINS] = {0};
+        uint32_t maxp[SQNN_MAX_PLANES] = {0};
+        int bad_seed = 0, no_memory = 0;
+        const uint32_t tile_bits = SQNN_TILE_SLICES * n_out;
+#pragma omp parallel if (l * n_q >= PARALLEL_FROM)
+        {
+            uint64_t t_sum[SQNN_MAX_PLANES] = {0}, t_hist[SQNN_PATCH_HIST_BINS] = {0};
+            uint32_t t_max[SQNN_MAX_PLANES] = {0};
+            std::vector<std::unique_ptr<uint16_t[]>> t_blocks;
+            uint32_t room = 0;
+            uint16_t *at = nullptr;
+            int t_bad = 0, t_nomem = 0;
+#pragma omp for schedule(dynamic, 4)
+            for (int64_t it = 0; it < items; ++it) {
+                if (t_nomem) continue;
+                const uint32_t i = (uint32_t)(it / tiles);
+                const uint64_t lo = (uint64_t)(it - (int64_t)i * tiles) * SQNN_TILE_SLICES, hi = std::min<uint64_t>(l, lo + SQNN_TILE_SLICES);
+                const uint64_t *plane = layer->planes + (uint64_t)i * words;
+                if (room < tile_bits) {
+                    room = std::max<uint32_t>(tile_bits, 1u << 17);
+                    uint16_t *fresh = new (std::nothrow) uint16_t[room];
+                    if (!fresh) { t_nomem = 1; continue; }
+                    try { t_blocks.emplace_back(fresh); } catch (const std::bad_alloc &) { delete[] fresh; t_nomem = 1; continue; }
+                    at = fresh;
+                }
+                uint16_t *const begin = at;
+                for (uint64_t s = lo; s < hi; ++s) {
+                    SliceBits sb;
+                    load_slice(plane, layer->mask, mn, n_out, s, sb);
+                    uint32_t seed;
+                    if (given) {
+                        seed = given[i][s];
+                        if (n_in < 32 && (seed >> n_in)) { t_bad = 1; seed = 0; }
+                    } else {
+                        seed = exhaustive ? encode_exhaustive(tab, n_in, sb) : encode_alg1(net->rows, n_out, full, sb);
+                        if (n_in < 32 && (seed >> n_in)) { t_bad = 1; seed = 0; }      // rows of M wider than n_in
+                    }
+                    seeds[(size_t)(i * l + s)] = seed;
+                    uint64_t out[4];
+                    expand(seed, out);
+                    const uint16_t *const before = at;
+                    const uint32_t base = (uint32_t)(s - lo) * n_out;
+                    for (uint32_t k = 0; k * 64 < n_out; ++k) {
+                        uint64_t bad = (out[k] ^ sb.want[k]) & sb.care[k];
+                        while (bad) {
+                            *at++ = (uint16_t)(base + k * 64 + (uint32_t)__builtin_ctzll(bad));
+                            bad &= bad - 1;
+                        }
+                    }
+                    const uint32_t p = (uint32_t)(at - before);
+                    t_max[i] = std::max(t_max[i], p);
+                    ++t_hist[p < SQNN_PATCH_HIST_BINS - 1 ? p : SQNN_PATCH_HIST_BINS - 1];
+                }
+                const uint32_t count = (uint32_t)(at - begin);
+                made[(size_t)it] = TileOut{begin, count};
+                t_sum[i] += count;
+                room -= count;
+            }
+#pragma omp critical
+            {
+                for (uint32_t i = 0; i < n_q; ++i) { sum[i] += t_sum[i]; maxp[i] = std::max(maxp[i], t_max[i]); }
+                for (uint32_t k = 0; k < SQNN_PATCH_HIST_BINS; ++k) hist[k] += t_hist[k];
+                bad_seed |= t_bad;
+                no_memory |= t_nomem;
+                try {
+                    for (auto &b : t_blocks) blocks.push_back(std::move(b));
+                } catch (const std::bad_alloc &) { no_memory = 1; }
+            }
+        }
+        if (no_memory) return SQNN_E_NOMEM;
+        if (bad_seed) return SQNN_E_INVALID_ARG;
+        for (uint32_t i = 0; i < n_q; ++i)
+            if (sum[i] > 0xffffffffull) return SQNN_E_INVALID_ARG;
+        sqnn_desc d;
+        uint8_t *b = start_blob(net, layer->m, layer->n, n_q, sum, &d);
+        if (!b) return SQNN_E_NOMEM;
         for (uint32_t i = 0; i < n_q; ++i) {
-            const uint64_t *plane = layer->planes + (uint64_t)i * words;
-            pa[i].wc.assign(l, 0);
-            pa[i].np.assign(l, 0);
-            int bad_seed = 0;
-            // pass 1: seed and patch count of every slice (slices are independent)
-#pragma omp parallel for schedule(dynamic, 4096)
-            for (int64_t s = 0; s < (int64_t)l; ++s) {
-                SliceBits sb;
-                load_slice(plane, layer->mask, mn, n_out, (uint64_t)s, sb);
-                uint32_t seed;
-                if (given) {
-                    seed = given[i][s];
-                    if (n_in < 32 && (seed >> n_in)) {
-#pragma omp atomic write
-                        bad_seed = 1;
-                        seed = 0;
-                    }
-                } else {
-                    seed = exhaustive ? encode_exhaustive(tab, n_in, sb) : encode_alg1(net->rows, n_out, sb);
-                }
-                uint64_t out[4];
-                expand(net->rows, n_out, seed, out);
-                int wrong = 0;
-                for (int k = 0; k < 4; ++k) wrong += popc64((out[k] ^ sb.want[k]) & sb.care[k]);
-                pa[i].wc[s] = seed;
-                pa[i].np[s] = (uint16_t)wrong;
+            uint32_t *idx = (uint32_t *)(b + d.off_idx[i]);
+            uint32_t run = 0;
+            for (uint64_t t = 0; t <= d.slices_padded / SQNN_TILE_SLICES; ++t) {
+                idx[t] = run;
+                if ((int64_t)t < tiles) run += made[(size_t)(i * tiles + (int64_t)t)].count;
             }
-            if (bad_seed) return SQNN_E_INVALID_ARG;
-            // pass 2: positions of the wrong care bits, written at the running offset
-            std::vector<uint64_t> start(l + 1, 0);
-            for (uint64_t s = 0; s < l; ++s) start[s + 1] = start[s] + pa[i].np[s];
-            pa[i].dp.assign(start[l] + 1, 0);
-#pragma omp parallel for schedule(dynamic, 4096)
-            for (int64_t s = 0; s < (int64_t)l; ++s) {
-                if (!pa[i].np[s]) continue;
-                SliceBits sb;
-                load_slice(plane, layer->mask, mn, n_out, (uint64_t)s, sb);
-                uint64_t out[4];
-                expand(net->rows, n_out, pa[i].wc[s], out);
-                uint64_t at = start[s];
-                for (uint32_t k = 0; k * 64 < n_out; ++k) {
-                    uint64_t bad = (out[k] ^ sb.want[k]) & sb.care[k];
-                    while (bad) {
-                        pa[i].dp[at++] = (uint8_t)(k * 64 + (uint32_t)__builtin_ctzll(bad));
-                        bad &= bad - 1;
-                    }
-                }
-            }
+            pack_fields(&seeds[(size_t)(i * l)], l, n_in, (uint32_t *)(b + d.off_wc[i]));
         }
-        std::vector<const uint32_t *> wcp(n_q);
-        std::vector<const uint16_t *> npp(n_q);
-        std::vector<const uint8_t *> dpp(n_q);
-        for (uint32_t i = 0; i < n_q; ++i) { wcp[i] = pa[i].wc.data(); npp[i] = pa[i].np.data(); dpp[i] = pa[i].dp.data(); }
-        int rc = build_blob(net, layer->m, layer->n, n_q, wcp.data(), npp.data(), dpp.data(), nullptr, blob, blob_bytes);
-        if (rc != SQNN_OK) return rc;
-        if (stats) {
-            rc = sqnn_stats_host(*blob, *blob_bytes, stats);
-            if (rc != SQNN_OK) { std::free(*blob); *blob = nullptr; return rc; }
+#pragma omp parallel for schedule(static) if (l * n_q >= PARALLEL_FROM)
+        for (int64_t it = 0; it < items; ++it) {
+            const uint32_t i = (uint32_t)(it / tiles);
+            const uint32_t *idx = (const uint32_t *)(b + d.off_idx[i]);
+            std::memcpy(b + d.off_pp[i] + (size_t)idx[it - (int64_t)i * tiles] * 2, made[(size_t)it].pp, (size_t)made[(size_t)it].count * 2);
         }
+        if (stats) fill_stats(d, sum, maxp, hist, stats);
+        *blob = b;
+        *blob_bytes = d.total_bytes;
         return SQNN_OK;
     } catch (const std::bad_alloc &) {
         return SQNN_E_NOMEM;
@@ -408,7 +530,7 @@ int sqnn_pack_host(const sqnn_xornet *net, uint64_t m, uint64_t n, uint32_t n_q,
     for (uint32_t i = 0; i < n_q; ++i)
         if (!wc[i] || !np[i] || !dp[i]) return SQNN_E_INVALID_ARG;
     try {
-        return build_blob(net, m, n, n_q, wc, np, nullptr, dp, blob, blob_bytes);
+        return build_blob(net, m, n, n_q, wc, np, dp, blob, blob_bytes);
     } catch (const std::bad_alloc &) {
         return SQNN_E_NOMEM;
     }
@@ -512,39 +634,24 @@ int sqnn_stats_host(const void *blob, size_t blob_bytes, sqnn_stats *stats)
     sqnn_desc d;
     int rc = sqnn_describe_host(blob, blob_bytes, &d);
     if (rc != SQNN_OK) return rc;
-    std::memset(stats, 0, sizeof *stats);
     const uint8_t *b = (const uint8_t *)blob;
-    const uint64_t mn = d.m * d.n, l = d.slices, lp = d.slices_padded;
-    stats->slices = l;
-    double eq1_bits = 0.0;
+    uint64_t sum[SQNN_MAX_PLANES] = {0}, hist[SQNN_PATCH_HIST_BINS] = {0};
+    uint32_t maxp[SQNN_MAX_PLANES] = {0};
     try {
-        std::vector<uint16_t> np(l ? l : 1);
+        std::vector<uint16_t> np(d.slices ? d.slices : 1);
         for (uint32_t i = 0; i < d.n_q; ++i) {
             count_patches(b, d, i, np.data());
-            uint32_t maxp = 0;
-            uint64_t sum = 0;
-            for (uint64_t s = 0; s < l; ++s) {
+            for (uint64_t s = 0; s < d.slices; ++s) {
                 const uint32_t p = np[s];
-                maxp = std::max(maxp, p);
-                sum += p;
-                ++stats->patch_hist[p < SQNN_PATCH_HIST_BINS - 1 ? p : SQNN_PATCH_HIST_BINS - 1];
+                maxp[i] = std::max(maxp[i], p);
+                sum[i] += p;
+                ++hist[p < SQNN_PATCH_HIST_BINS - 1 ? p : SQNN_PATCH_HIST_BINS - 1];
             }
-            stats->patches[i] = sum;
-            stats->max_patch[i] = maxp;
-            // Eq. 1, literally: n_in/n_out * mn + l * ceil(lg max p) + sum p * ceil(lg n_out)
-            eq1_bits += (double)d.n_in / (double)d.n_out * (double)mn +
-                        (double)l * ceil_lg_u64(maxp) + (double)sum * ceil_lg_u64(d.n_out);
-            stats->bits_wc += (round_up(lp * d.n_in / 8, 16) + 16) * 8;
-            stats->bits_index += (round_up((lp / SQNN_TILE_SLICES + 1) * 4, 16) + 16) * 8;
-            stats->bits_dpatch += (round_up(sum * 2, 16) + 16) * 8;
         }
     } catch (const std::bad_alloc &) {
         return SQNN_E_NOMEM;
     }
-    stats->bits_tables = (round_up(d.tables_bytes, 16) + 16) * 8;
-    stats->bits_index += stats->bits_tables;
-    stats->bpw_eq1 = eq1_bits / (double)mn;
-    stats->bpw_actual = (double)(stats->bits_wc + stats->bits_npatch + stats->bits_index + stats->bits_dpatch) / (double)mn;
+    fill_stats(d, sum, maxp, hist, stats);
     return SQNN_OK;
 }
 
@@ -847,7 +954,7 @@ int sqnn_load_host(const void *stored, size_t stored_bytes, void **blob, size_t 
         std::vector<const uint32_t *> wcp(h.n_q);
         std::vector<const uint16_t *> npp(h.n_q), dpp(h.n_q);
         for (uint32_t i = 0; i < h.n_q; ++i) { wcp[i] = pa[i].wc.data(); npp[i] = pa[i].np.data(); dpp[i] = dp16[i].data(); }
-        const int rc = build_blob(&net, h.m, h.n, h.n_q, wcp.data(), npp.data(), nullptr, dpp.data(), blob, blob_bytes);
+        const int rc = build_blob(&net, h.m, h.n, h.n_q, wcp.data(), npp.data(), dpp.data(), blob, blob_bytes);
         return rc == SQNN_E_INVALID_ARG ? SQNN_E_BAD_BLOB : rc;     // bad contents, not a bad call
     } catch (const std::bad_alloc &) {
         return SQNN_E_NOMEM;
