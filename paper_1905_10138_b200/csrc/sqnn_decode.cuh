@@ -60,15 +60,6 @@ struct ClearArgs {
 SQNN_DEV void wait_prior_grid() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 SQNN_DEV void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 
-SQNN_DEV uint32_t extract_bits(const uint32_t *__restrict__ base, uint64_t bitpos, uint32_t width)
-{
-    const uint64_t w = bitpos >> 5;
-    const uint32_t sh = (uint32_t)(bitpos & 31);
-    const uint32_t lo = __ldg(base + w), hi = __ldg(base + w + 1);   // sections end with slack
-    const uint32_t v = __funnelshift_r(lo, hi, sh);
-    return width >= 32 ? v : (v & ((1u << width) - 1u));
-}
-
 SQNN_DEV void flag(uint32_t *status, uint32_t code)
 {
     if (status) atomicMax(status, code);
@@ -426,45 +417,141 @@ SQNN_DEV void tile_expand(const TileSeeds<N_OUT, N_IN> &in, uint32_t *region, co
     }
 }
 
-// Run-time shape: plain loops, every read through extract_bits.  Ends with the warp synchronised.
-SQNN_DEV void decode_ktile_generic(const DecodeArgs &A, uint32_t plane, uint64_t ktile,
-                                   uint32_t *region, const uint32_t *tab, uint32_t lane)
+// Table entry e of NWP words (run-time shapes).
+template <int NWP>
+SQNN_DEV void xor_entry(const uint32_t *tab, uint32_t e, uint32_t (&x)[NWP])
+{
+    uint32_t y[NWP];
+    load_entry<NWP, false>(tab, e, 0, y);
+#pragma unroll
+    for (int k = 0; k < NWP; ++k) x[k] ^= y[k];
+}
+template <int NWP>
+SQNN_DEV void lookup(const DecodeArgs &A, const uint32_t *tab, uint32_t seed, uint32_t (&x)[NWP])
+{
+    const uint32_t cb = A.cb, cmask = (1u << cb) - 1u;
+    load_entry<NWP, false>(tab, seed & cmask, 0, x);
+    for (uint32_t ch = 1; ch < A.nchunks; ++ch) {
+        seed >>= cb;
+        xor_entry<NWP>(tab, (ch << cb) | (seed & cmask), x);
+    }
+}
+
+// Run-time shape with n_out a multiple of 32: every slice is NW whole output words, so the lanes take slices in
+// turn (lane l: slices l, l + 32, ...) and nothing has to be shifted into place; the stores of a warp are
+// consecutive.  (With eight consecutive slices per lane all lanes would store to the same bank.)
+template <int NW>
+SQNN_DEV void expand_whole_words(const DecodeArgs &A, const PlanePtrs &P, uint64_t tile, uint32_t *region, const uint32_t *tab, uint32_t lane)
+{
+    constexpr int NWP = (int)(NW <= 2 ? NW : NW <= 4 ? 4 : 8);
+    const uint32_t n_in = A.n_in, smask = n_in >= 32 ? 0xffffffffu : (1u << n_in) - 1u;
+    uint32_t seed[8];
+#pragma unroll
+    for (uint32_t i = 0; i < 8; ++i) {
+        const uint64_t bit = (tile * SQNN_TILE_SLICES + 32 * i + lane) * n_in;
+        const uint32_t *w = P.wc + (bit >> 5);
+        seed[i] = __funnelshift_r(__ldg(w), __ldg(w + 1), (uint32_t)bit & 31u) & smask;     // sections end with slack
+    }
+#pragma unroll
+    for (uint32_t i = 0; i < 8; ++i) {
+        uint32_t x[NWP];
+        lookup<NWP>(A, tab, seed[i], x);
+        uint32_t *out = region + (32 * i + lane) * NW;
+        if constexpr (NW % 4 == 0) {
+#pragma unroll
+            for (int k = 0; k < NW; k += 4) *reinterpret_cast<uint4 *>(out + k) = make_uint4(x[k], x[k + 1], x[k + 2], x[k + 3]);
+        } else if constexpr (NW % 2 == 0) {
+#pragma unroll
+            for (int k = 0; k < NW; k += 2) *reinterpret_cast<uint2 *>(out + k) = make_uint2(x[k], x[k + 1]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < NW; ++k) out[k] = x[k];
+        }
+    }
+}
+
+// Any other run-time shape: a lane owns 8 * KT consecutive slices and shifts their entries together.  The seeds of
+// eight slices (n_in bytes) are fetched at once and move through registers.
+template <int NWP>
+SQNN_DEV void expand_shifted(const DecodeArgs &A, const PlanePtrs &P, uint64_t ktile, uint32_t *region, const uint32_t *tab, uint32_t lane)
+{
+    const uint32_t n_in = A.n_in, nw = A.nw, smask = n_in >= 32 ? 0xffffffffu : (1u << n_in) - 1u;
+    const uint32_t last = A.n_out - 32 * (nw - 1);              // bits of an entry's last word, 1 .. 32
+    uint32_t *out = region + lane * A.W;
+    uint32_t have = 0, top = 0;                                  // pending bits: the upper `have` bits of `top`
+    for (uint32_t f = 0; f < A.KT; ++f) {
+        const uint64_t byte = ((ktile * 32 + lane) * A.KT + f) * n_in;
+        const uint32_t *w = P.wc + (byte >> 2);
+        const uint32_t sh = ((uint32_t)byte & 3u) * 8, bits = 8 * n_in + sh;
+        uint32_t al[9];
+#pragma unroll
+        for (uint32_t k = 0; k < 9; ++k) al[k] = 32 * k < bits ? __ldg(w + k) : 0u;
+#pragma unroll
+        for (uint32_t k = 0; k < 8; ++k) al[k] = __funnelshift_r(al[k], al[k + 1], sh);
+#pragma unroll
+        for (uint32_t i = 0; i < 8; ++i) {
+            uint32_t x[NWP];
+            lookup<NWP>(A, tab, al[0] & smask, x);
+#pragma unroll
+            for (uint32_t k = 0; k < 7; ++k) al[k] = __funnelshift_rc(al[k], al[k + 1], n_in);
+            al[7] = n_in >= 32 ? 0u : al[7] >> n_in;
+            uint32_t prev = top, end = x[0];
+#pragma unroll
+            for (uint32_t k = 0; k < NWP; ++k) {
+                if (k + 1 < nw) {                                // whole words
+                    *out++ = __funnelshift_l(prev, x[k], have);
+                    prev = x[k];
+                    if (k + 1 < NWP) end = x[k + 1];
+                }
+            }
+            const uint32_t word = __funnelshift_l(prev, end, have);          // bits past the pending ones are 0
+            if (have + last >= 32) {
+                *out++ = word;
+                have = have + last - 32;
+                top = last >= 32 ? end : end << (32 - last);
+            } else {
+                have += last;
+                top = word << (32 - have);
+            }
+        }
+    }
+}
+
+// Run-time shape: one kernel tile.  Ends with the warp synchronised.
+SQNN_DEV void decode_ktile_generic(const DecodeArgs &A, uint32_t plane, uint64_t ktile, uint32_t *region, const uint32_t *tab, uint32_t lane)
 {
     const PlanePtrs &P = A.pl[plane];
-    const uint32_t n_out = A.n_out, n_in = A.n_in, G = A.G, W = A.W;
-    const uint32_t nw = A.nw, nwp = A.nwp, nch = A.nchunks, cb = A.cb;
-    const uint32_t cmask = (1u << cb) - 1u;
-    const uint64_t s0 = (ktile * 32 + lane) * G;
-    uint32_t *mine = region + lane * W;
-    uint64_t acc = 0;
-    uint32_t have = 0, wp = 0;
-    for (uint32_t i = 0; i < G; ++i) {
-        const uint32_t seed = extract_bits(P.wc, (s0 + i) * n_in, n_in);
-        for (uint32_t k = 0; k < nw; ++k) {
-            uint32_t x = 0;
-            for (uint32_t ch = 0; ch < nch; ++ch)
-                x ^= tab[((ch << cb) | ((seed >> (ch * cb)) & cmask)) * nwp + k];
-            const uint32_t bits = (k == nw - 1) ? n_out - 32 * k : 32;
-            acc |= (uint64_t)x << have;
-            have += bits;
-            if (have >= 32) { mine[wp++] = (uint32_t)acc; acc >>= 32; have -= 32; }
+    const uint32_t tile_bits = SQNN_TILE_SLICES * A.n_out;
+    uint32_t pw[PATCH_AHEAD];
+    TileRun run = fetch_run(P, ktile * A.KT);
+    if (A.n_out % 32 == 0) {
+        switch (A.nw) {
+            case 1: expand_whole_words<1>(A, P, ktile, region, tab, lane); break;
+            case 2: expand_whole_words<2>(A, P, ktile, region, tab, lane); break;
+            case 3: expand_whole_words<3>(A, P, ktile, region, tab, lane); break;
+            case 4: expand_whole_words<4>(A, P, ktile, region, tab, lane); break;
+            case 5: expand_whole_words<5>(A, P, ktile, region, tab, lane); break;
+            case 6: expand_whole_words<6>(A, P, ktile, region, tab, lane); break;
+            case 7: expand_whole_words<7>(A, P, ktile, region, tab, lane); break;
+            default: expand_whole_words<8>(A, P, ktile, region, tab, lane); break;
+        }
+    } else {
+        switch (A.nwp) {
+            case 1: expand_shifted<1>(A, P, ktile, region, tab, lane); break;
+            case 2: expand_shifted<2>(A, P, ktile, region, tab, lane); break;
+            case 4: expand_shifted<4>(A, P, ktile, region, tab, lane); break;
+            default: expand_shifted<8>(A, P, ktile, region, tab, lane); break;
         }
     }
+    fetch_patches(A, P, run, lane, pw);
     __syncwarp();
-    // patches (Section 3.2), one format tile after the other
-    const uint32_t tile_bits = SQNN_TILE_SLICES * n_out;
-    const uint32_t region_sa = smem_addr(region);
-    uint32_t bad = 0;
-    for (uint32_t f = 0; f < A.KT; ++f) {
-        const uint64_t ft = ktile * A.KT + f;
-        uint32_t base = __ldg(P.idx + ft), end = __ldg(P.idx + ft + 1);
-        if (end < base || end > P.n_pp) { flag(A.status, 2u); continue; }
-        for (uint32_t e = base + lane; e < end; e += 32) {
-            const uint32_t pos = P.pp[e];
-            if (pos < tile_bits) smem_flip(region_sa, f * tile_bits + pos); else bad = 1;
+    for (uint32_t f = 0; f < A.KT; ++f) {                        // one format tile after the other
+        tile_patch(A, P, run, pw, region, f * tile_bits, tile_bits, lane);
+        if (f + 1 < A.KT) {
+            run = fetch_run(P, ktile * A.KT + f + 1);
+            fetch_patches(A, P, run, lane, pw);
         }
     }
-    if (bad) flag(A.status, 1u);
     __syncwarp();
 }
 
