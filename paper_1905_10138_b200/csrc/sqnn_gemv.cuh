@@ -118,6 +118,8 @@ __global__ void __launch_bounds__(1024, 1)
 k_decode_gemv(const GemvArgs g)
 {
     extern __shared__ __align__(16) uint32_t smem[];
+    wait_prior_grid();
+    launch_dependents();
     const DecodeArgs &A = g.A;
     const uint32_t W = words_per_lane<N_OUT>(A);
     const uint32_t TW = 32 * W;                                  // words per kernel tile
@@ -422,9 +424,7 @@ inline int launch_gemv_bt(const DecodeArgs &A, const uint64_t *d_mask, const flo
                     (size_t)g.region_words * 4 < (1u << 20)) ? 1u : 0u;
 #define SQNN_GEMV_LAUNCH(XSV, NQV)                                                                       \
     do {                                                                                                 \
-        auto k = k_decode_gemv<N_OUT, N_IN, BT, XT, XSV, NQV>;                                           \
-        if (prepare(k, smem)) return SQNN_E_CUDA;                                                        \
-        k<<<(uint32_t)grid, nwarps * 32, smem, st>>>(g);                                                 \
+        return launch_kernel(k_decode_gemv<N_OUT, N_IN, BT, XT, XSV, NQV>, (uint32_t)grid, nwarps * 32, smem, st, g); \
     } while (0)
     if (xs) {
         if (A.n_q == 1) SQNN_GEMV_LAUNCH(true, 1);
@@ -436,7 +436,6 @@ inline int launch_gemv_bt(const DecodeArgs &A, const uint64_t *d_mask, const flo
         else SQNN_GEMV_LAUNCH(false, 0);
     }
 #undef SQNN_GEMV_LAUNCH
-    return cudaGetLastError() == cudaSuccess ? SQNN_OK : SQNN_E_CUDA;
 }
 
 template <int N_OUT, int N_IN, typename XT>

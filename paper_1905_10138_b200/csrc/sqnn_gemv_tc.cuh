@@ -1,0 +1,422 @@
+// K3: decryption fused with Y[b][r] = sum_c W[r][c] X[b][c] for small batch (<= 15) on the tensor cores, as a
+// template over the network shape, with its launcher.
+//
+// Work split.  As in sqnn_gemv.cuh a block owns a run of whole rows of W and decodes the kernel tiles that cover
+// them into shared memory, next to the same range of the pruning mask.  The product then runs on tcgen05.mma
+// with the expanded weights as the A operand in tensor memory:
+//
+//   - a tile is 16 rows; its columns are cut into 8 equal ranges (kq) of Kq columns, and TMEM lane
+//     32 w + 8 i + kq holds row 4 w + i, range kq: the M = 128 lanes are all in use whatever the number of rows;
+//   - B row 8 q + kq holds the activations of range kq, vector q (Kq columns, K-major), so lane (row, kq) of the
+//     accumulator finds its own product in columns 8 q + kq (one column in eight; the others are the price of
+//     sharing B, and cost nothing at these N);
+//   - four expander groups of four warps each take an equal run of the list (tile, plane, 128 columns), with
+//     an accumulator and A slots of their own, each fed to the tensor cores by a warp of its own; the scale of
+//     a row and plane is applied to the accumulator, so weights are exact.  fp32 activations enter as three bf16
+//     pieces that add up to them exactly (8 + 8 + 8 bits).
+//
+// Kq is an odd multiple of 128 columns: the 8 lanes of a row then read 16-byte vectors of mask and plane bits
+// from different banks, whatever the row length.  Sums over the 8 ranges (shuffles) and the four groups (shared
+// memory) have a fixed order: results are bit-identical from run to run.
+//
+// Bound: integer instructions of the expansion (1.4 per weight and plane, against 42 per unpruned weight of the
+// walk over care bits in sqnn_gemv.cuh, 3.8 per weight at 9 % density) and the latency of the block's phases
+// (launch, staging, decode, product, reduction).
+#pragma once
+#include "sqnn_gemv.cuh"
+#include "sqnn_tc.cuh"
+
+namespace sqnn {
+
+constexpr uint32_t TC_GROUPS = 4;                         // expander groups
+constexpr uint32_t TC_THREADS = TC_GROUPS * 128 + TC_GROUPS * 32;
+constexpr uint32_t TC_TILE_ROWS = 16, TC_RANGES = 8;
+constexpr uint32_t TC_MAX_Q = 12;                         // activation columns (vectors x pieces) per pass: N <= 96
+constexpr uint64_t TC_WAIT_LIMIT = 2000000000ull;         // about a second
+
+struct TcArgs {
+    DecodeArgs A;
+    const uint32_t *mask32;
+    uint64_t mask_words;
+    const float *alpha;
+    const void *x;
+    int64_t ldx;
+    float *y;
+    int64_t ldy;
+    uint64_t m;
+    uint32_t n, batch;
+    uint32_t rows_per_block, rows_per_chunk;
+    uint32_t region_words;        // words of one bit vector of a chunk in shared memory (with slack for the last row's ranges)
+    uint32_t kq, units;           // columns per range, kq / 128
+    uint32_t bt;                  // activation vectors per pass
+    uint32_t N;                   // MMA N: 8 x bt x pieces, rounded up to 16
+    uint32_t slots;               // A slots (64 columns) per group: 1 or 2
+    uint32_t alpha_words, part_words;
+    uint32_t x_vec;               // rows of X start on 16-byte boundaries
+};
+
+SQNN_DEV void named_arrive(uint32_t id) { asm volatile("bar.arrive %0, 160;\n" :: "r"(id) : "memory"); }
+SQNN_DEV void named_sync(uint32_t id) { asm volatile("bar.sync %0, 160;\n" :: "r"(id) : "memory"); }
+
+// 128 columns of one row from bit `o` of a packed vector in shared memory (address sa, 16-byte aligned).
+template <bool ALIGNED>
+SQNN_DEV void lds_bits128(uint32_t sa, uint32_t o, uint32_t (&out)[4])
+{
+    const uint32_t at = sa + ((o >> 7) << 4);
+    uint32_t q[8];
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(q[0]), "=r"(q[1]), "=r"(q[2]), "=r"(q[3]) : "r"(at));
+    if constexpr (ALIGNED) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) out[k] = q[k];
+    } else {
+        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(q[4]), "=r"(q[5]), "=r"(q[6]), "=r"(q[7]) : "r"(at + 16));
+        const bool two = (o & 64u) != 0, one = (o & 32u) != 0;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) q[k] = two ? q[k + 2] : q[k];
+#pragma unroll
+        for (int k = 0; k < 5; ++k) q[k] = one ? q[k + 1] : q[k];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) out[k] = __funnelshift_r(q[k], q[k + 1], o & 31u);
+    }
+}
+
+// Two bf16 values (round toward zero, exact when they have at most 8 significant bits) in one word.
+SQNN_DEV uint32_t high_halves(float lo, float hi) { return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632); }
+
+// Stages activation vectors [bc, bc + bt) as B rows: vector q, range kq, piece p -> row 8 (q * PIECES + p) + kq of
+// every 64-column step's box ([N rows][128 bytes], 128-byte swizzle).  Columns past n and vectors past the batch
+// are zero.  Values that are not finite are staged as zero and reported: a pruned weight must not meet them.
+template <typename XT>
+SQNN_DEV void tc_stage_x(const TcArgs &g, uint32_t x_sa, uint32_t bc, uint32_t *not_finite)
+{
+    constexpr uint32_t PIECES = sizeof(XT) == 4 ? 3 : 1;
+    const XT *x = reinterpret_cast<const XT *>(g.x);
+    const uint32_t chunks = g.kq / 8, per_q = TC_RANGES * chunks, total = per_q * g.bt;       // of 8 columns
+    bool odd = false;
+    for (uint32_t i = threadIdx.x; i < total; i += TC_THREADS) {
+        const uint32_t q = i / per_q, rest = i - q * per_q, kq = rest / chunks, ch = rest - kq * chunks;
+        const uint32_t c = kq * g.kq + ch * 8;
+        float v[8];
+        const XT *src = x + (int64_t)(bc + q) * g.ldx + c;
+        if (bc + q < g.batch && c + 8 <= g.n && g.x_vec) {
+            if constexpr (PIECES == 1) {
+                const uint4 t = __ldg(reinterpret_cast<const uint4 *>(src));
+                const uint32_t w[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) { v[2 * e] = __uint_as_float(w[e] << 16); v[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u); }
+            } else {
+                const float4 t = __ldg(reinterpret_cast<const float4 *>(src)), u = __ldg(reinterpret_cast<const float4 *>(src) + 1);
+                v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w; v[4] = u.x; v[5] = u.y; v[6] = u.z; v[7] = u.w;
+            }
+        } else {
+#pragma unroll
+            for (uint32_t e = 0; e < 8; ++e) v[e] = bc + q < g.batch && c + e < g.n ? to_float(src[e]) : 0.0f;
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            if ((__float_as_uint(v[e]) & 0x7f800000u) == 0x7f800000u) { odd = true; v[e] = 0.0f; }
+        const uint32_t box = x_sa + (ch >> 3) * g.N * 128;
+#pragma unroll
+        for (uint32_t p = 0; p < PIECES; ++p) {
+            const uint32_t row = 8 * (q * PIECES + p) + kq;
+            const uint32_t at = box + row * 128 + (((ch & 7u) ^ (row & 7u)) << 4);
+            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" :: "r"(at), "r"(high_halves(v[0], v[1])), "r"(high_halves(v[2], v[3])),
+                         "r"(high_halves(v[4], v[5])), "r"(high_halves(v[6], v[7])) : "memory");
+            if (p + 1 < PIECES) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[e] -= __uint_as_float(__float_as_uint(v[e]) & 0xffff0000u);
+            }
+        }
+    }
+    if (odd) atomicOr(not_finite, 1u);
+}
+
+template <int N_OUT, int N_IN, typename XT, bool ALIGNED>
+__global__ void __launch_bounds__(TC_THREADS, 1)
+k_gemv_tc(const TcArgs g)
+{
+    extern __shared__ __align__(16) uint32_t smem[];
+    __shared__ uint64_t bars[3 * TC_GROUPS];              // per group: two A slots free, accumulator complete
+    __shared__ uint32_t tmem_slot, abort_word, not_finite;
+    constexpr uint32_t PIECES = sizeof(XT) == 4 ? 3 : 1;
+    const DecodeArgs &A = g.A;
+    volatile uint32_t *abort_flag = &abort_word;
+    const uint32_t W = words_per_lane<N_OUT>(A);
+    const uint32_t TW = 32 * W;                                  // words per kernel tile
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr uint32_t nwarps = TC_THREADS / 32;
+    const uint32_t n = g.n, n_q = A.n_q;
+    uint32_t *tab_s = smem;
+    uint32_t *bits_s = tab_s + A.tab_words;                      // [plane][region_words]
+    uint32_t *mask_s = bits_s + n_q * g.region_words;
+    float *alpha_s = reinterpret_cast<float *>(mask_s + g.region_words);
+    float *part_s = alpha_s + g.alpha_words;                     // [group][row][bt]
+    const uint32_t x_sa = (smem_addr(part_s + g.part_words) + 1023u) & ~1023u;
+    const uint32_t bars_sa = smem_addr(bars);
+    const bool mask_vec = (reinterpret_cast<uintptr_t>(g.mask32) & 15) == 0;
+    const uint64_t row0 = (uint64_t)blockIdx.x * g.rows_per_block;
+    const uint64_t row_end = row0 + g.rows_per_block < g.m ? row0 + g.rows_per_block : g.m;
+
+    if (warp == nwarps - 1) tmem_alloc(&tmem_slot, 512);
+    if (threadIdx.x == 0) {
+        for (uint32_t i = 0; i < 3 * TC_GROUPS; ++i) mbar_init(bars_sa + 8 * i, 1);
+        abort_word = not_finite = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    __syncthreads();
+    wait_prior_grid();
+    launch_dependents();
+    tables_request(A, tab_s);                                    // commit group: tables
+    uint32_t slot_seq = 0, parts_done = 0;                       // per group: A slots filled, accumulators read
+    bool first = true;
+
+    for (uint64_t ra = row0; ra < row_end; ra += g.rows_per_chunk) {
+        const uint64_t rb = ra + g.rows_per_chunk < row_end ? ra + g.rows_per_chunk : row_end;
+        const uint32_t nrows = (uint32_t)(rb - ra);
+        // kernel tiles that cover the bits [ra * n, rb * n)
+        const uint64_t tile_bits = 32ull * TW;
+        const uint64_t kt0 = (ra * n) / tile_bits, kt1 = (rb * n + tile_bits - 1) / tile_bits;
+        const uint32_t nt = (uint32_t)(kt1 - kt0);
+        const uint64_t gw0 = kt0 * TW;                           // first word of the chunk's regions
+        if (!first) __syncthreads();                             // the product of the previous chunk is over
+        stage_mask(mask_s, g.mask32, gw0, g.mask_words, nt * TW, threadIdx.x, TC_THREADS, mask_vec);
+        for (uint32_t i = threadIdx.x; i < nrows * n_q; i += TC_THREADS) cp_async4(alpha_s + i, g.alpha + ra * n_q + i);
+        cp_async_commit();                                       // commit group: mask and scales
+        for (uint32_t i = threadIdx.x; i < TC_GROUPS * nrows * g.bt; i += TC_THREADS) part_s[i] = 0.0f;
+
+        // decode: item = (tile, plane), dealt out over the warps; a warp's first item is fetched before anybody
+        // waits for the tables, and the activations are staged while it is under way
+        const uint32_t items = nt * n_q;
+        uint32_t item = warp;
+        if constexpr (N_OUT != 0) {
+            using S = Shape<N_OUT, N_IN>;
+            TileSeeds<N_OUT, N_IN> s;
+            TileRun run{0u, 0u};
+            uint32_t pw[PATCH_AHEAD];
+            auto fetch = [&](uint32_t it) {
+                const uint32_t t = it / n_q, pl = it - t * n_q;
+                fetch_seeds<N_OUT, N_IN>(A.pl[pl], kt0 + t, lane, s);
+                run = fetch_run(A.pl[pl], kt0 + t);
+                fetch_patches(A, A.pl[pl], run, lane, pw);
+            };
+            if (item < items) fetch(item);
+            if (first) {
+                tc_stage_x<XT>(g, x_sa, 0, &not_finite);
+                cp_async_wait_group<1>();                        // tables (mask and scales may be pending)
+                __syncthreads();
+            }
+            while (item < items) {
+                const uint32_t t = item / n_q, pl = item - t * n_q;
+                uint32_t *region = bits_s + pl * g.region_words + t * TW;
+                tile_expand<N_OUT, N_IN>(s, region, tab_s, lane);
+                __syncwarp();
+                tile_patch(A, A.pl[pl], run, pw, region, 0u, S::TILE_BITS, lane);
+                item += nwarps;
+                if (item < items) fetch(item);
+            }
+        } else {
+            if (first) {
+                tc_stage_x<XT>(g, x_sa, 0, &not_finite);
+                cp_async_wait_group<1>();
+                __syncthreads();
+            }
+            for (; item < items; item += nwarps) {
+                const uint32_t t = item / n_q, pl = item - t * n_q;
+                decode_ktile_generic(A, pl, kt0 + t, bits_s + pl * g.region_words + t * TW, tab_s, lane);
+            }
+        }
+        first = false;
+        cp_async_wait_all();
+        fence_async_smem();                                      // staged activations -> visible to the tensor cores
+        tc_fence_before();
+        __syncthreads();                                         // bits, mask, scales, activations in place
+        tc_fence_after();
+
+        // a group's run of the list (tile, plane, 128 columns)
+        const uint32_t tiles = (nrows + TC_TILE_ROWS - 1) / TC_TILE_ROWS, list = tiles * n_q * g.units;
+        const uint32_t grp = warp < 4 * TC_GROUPS ? warp >> 2 : warp - 4 * TC_GROUPS;
+        const uint32_t u_begin = list * grp / TC_GROUPS, u_end = list * (grp + 1) / TC_GROUPS;
+        const uint32_t d_tmem = tmem_slot + grp * g.N, a_tmem = tmem_slot + TC_GROUPS * g.N + grp * g.slots * 32;
+        const uint32_t free_a = bars_sa + 24 * grp, done = free_a + 16;
+        const uint32_t slot_mask = g.slots - 1, slot_shift = g.slots - 1;      // 1 slot: 0, 2 slots: 1
+        for (uint32_t bc = 0; bc < g.batch; bc += g.bt) {
+            if (bc != 0 || (ra != row0 && g.bt < g.batch)) {     // another pass: its activations replace the last one's
+                __syncthreads();
+                tc_stage_x<XT>(g, x_sa, bc, &not_finite);
+                for (uint32_t i = threadIdx.x; i < TC_GROUPS * nrows * g.bt; i += TC_THREADS) part_s[i] = 0.0f;
+                fence_async_smem();
+                __syncthreads();
+            }
+            if (warp < 4 * TC_GROUPS) {
+                const uint32_t quad = warp & 3, kq = lane & 7, lane_sel = (quad * 32) << 16;
+                const uint32_t mask_sa = smem_addr(mask_s), bits_sa = smem_addr(bits_s);
+                float acc[TC_MAX_Q];
+#pragma unroll
+                for (uint32_t q = 0; q < TC_MAX_Q; ++q) acc[q] = 0.0f;
+                for (uint32_t u = u_begin; u < u_end;) {
+                    const uint32_t it = u / g.units, t0 = u - it * g.units, tile = it / n_q, pl = it - tile * n_q;
+                    const uint32_t len = min(g.units - t0, u_end - u);
+                    const uint32_t rl = min(tile * TC_TILE_ROWS + quad * 4 + (lane >> 3), nrows - 1);
+                    uint32_t o = (uint32_t)((ra + rl) * n - gw0 * 32) + kq * g.kq + t0 * 128;
+                    const uint32_t plane_sa = bits_sa + pl * g.region_words * 4;
+                    for (uint32_t k = 0; k < len; ++k, o += 128) {
+                        uint32_t mw[4], bw[4];
+                        lds_bits128<ALIGNED>(mask_sa, o, mw);
+                        lds_bits128<ALIGNED>(plane_sa, o, bw);
+#pragma unroll
+                        for (uint32_t h = 0; h < 2; ++h, ++slot_seq) {
+                            uint32_t v[32];
+                            expand32(mw[2 * h], bw[2 * h], v);
+                            expand32(mw[2 * h + 1], bw[2 * h + 1], v + 16);
+                            const uint32_t slot = slot_seq & slot_mask, use = slot_seq >> slot_shift;
+                            if (use > 0) {
+                                mbar_wait_warp(free_a + 8 * slot, (use - 1) & 1u, abort_flag, A.status, TC_WAIT_LIMIT);
+                                tc_fence_after();
+                            }
+                            tmem_st16(a_tmem + lane_sel + slot * 32, v);
+                            tmem_st16(a_tmem + lane_sel + slot * 32 + 16, v + 16);
+                            tmem_st_wait();
+                            tc_fence_before();
+                            named_arrive(1 + 2 * grp + slot);
+                        }
+                    }
+                    u += len;
+                    // the part's accumulator: this lane's range, scaled
+                    const float al = 0.5f * alpha_s[rl * n_q + pl];
+                    mbar_wait_warp(done, parts_done & 1u, abort_flag, A.status, TC_WAIT_LIMIT);
+                    ++parts_done;
+                    tc_fence_after();
+#pragma unroll
+                    for (uint32_t q2 = 0; q2 < TC_MAX_Q / 2; ++q2) {
+                        if (16 * q2 >= g.N) break;
+                        uint32_t d[16];
+                        tmem_ld16(d_tmem + lane_sel + 16 * q2, d);
+#pragma unroll
+                        for (uint32_t e = 0; e < 2; ++e) {
+                            uint32_t a4[4], a2[2];
+#pragma unroll
+                            for (uint32_t k = 0; k < 4; ++k) a4[k] = (kq & 4u) ? d[8 * e + k + 4] : d[8 * e + k];
+#pragma unroll
+                            for (uint32_t k = 0; k < 2; ++k) a2[k] = (kq & 2u) ? a4[k + 2] : a4[k];
+                            const float mine = __uint_as_float((kq & 1u) ? a2[1] : a2[0]);
+                            const uint32_t q = 2 * q2 + e;
+                            acc[q / PIECES] = fmaf(al, mine, acc[q / PIECES]);
+                        }
+                    }
+                    tc_fence_before();
+                    // the tile is complete for this group: sum over the ranges, hand over
+                    if (u == u_end || u / g.units / n_q != tile) {
+#pragma unroll
+                        for (uint32_t q = 0; q < TC_MAX_Q / PIECES; ++q) {
+                            if (q >= g.bt) break;
+                            float sum = acc[q];
+                            sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+                            sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+                            sum += __shfl_xor_sync(0xffffffffu, sum, 4);
+                            if (kq == 0 && tile * TC_TILE_ROWS + quad * 4 + (lane >> 3) < nrows) part_s[(grp * nrows + rl) * g.bt + q] = sum;
+                            acc[q] = 0.0f;
+                        }
+                    }
+                }
+            } else {
+                // the group's MMA warp: one slot at a time, in the order they are filled
+                const uint32_t idesc = instr_desc_bf16(g.N);
+                const uint64_t x_desc0 = smem_desc_sw128(x_sa);
+                const uint32_t box_step = g.N * 128 >> 4;
+                for (uint32_t u = u_begin; u < u_end;) {
+                    const uint32_t it = u / g.units, t0 = u - it * g.units;
+                    const uint32_t len = min(g.units - t0, u_end - u);
+                    for (uint32_t k = 0; k < 2 * len; ++k, ++slot_seq) {
+                        const uint32_t slot = slot_seq & slot_mask;
+                        named_sync(1 + 2 * grp + slot);
+                        tc_fence_after();
+                        mma_slot<4>(d_tmem, a_tmem + slot * 32, x_desc0 + (2 * t0 + k) * box_step, idesc, k, free_a + 8 * slot, 0);
+                    }
+                    mma_commit(done);
+                    u += len;
+                }
+            }
+            __syncthreads();
+            for (uint32_t i = threadIdx.x; i < nrows * g.bt; i += TC_THREADS) {
+                const uint32_t rl = i / g.bt, q = i - rl * g.bt;
+                if (bc + q >= g.batch) continue;
+                float sum = 0.0f;
+#pragma unroll
+                for (uint32_t p = 0; p < TC_GROUPS; ++p) sum += part_s[(p * nrows + rl) * g.bt + q];
+                if (not_finite) {                                // add what was left out of the staged activations
+                    const XT *x = reinterpret_cast<const XT *>(g.x) + (int64_t)(bc + q) * g.ldx;
+                    const uint32_t o = (uint32_t)((ra + rl) * n - gw0 * 32);
+                    for (uint32_t c = 0; c < n; ++c) {
+                        const float xv = to_float(x[c]);
+                        if ((__float_as_uint(xv) & 0x7f800000u) != 0x7f800000u || !((mask_s[(o + c) >> 5] >> ((o + c) & 31u)) & 1u)) continue;
+                        float w = 0.0f;
+                        for (uint32_t pl = 0; pl < n_q; ++pl) {
+                            const float a = alpha_s[rl * n_q + pl];
+                            w += ((bits_s[pl * g.region_words + ((o + c) >> 5)] >> ((o + c) & 31u)) & 1u) ? a : -a;
+                        }
+                        sum = fmaf(w, xv, sum);
+                    }
+                }
+                g.y[(int64_t)(bc + q) * g.ldy + (int64_t)(ra + rl)] = sum;
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == nwarps - 1) tmem_dealloc(tmem_slot, 512);
+}
+
+// ------------------------------------------------------------------------------------------
+// launcher
+// ------------------------------------------------------------------------------------------
+// Returns SQNN_E_UNSUPPORTED when this kernel is not the one to take (the caller falls back to the walk).
+template <int N_OUT, int N_IN, typename XT>
+inline int launch_gemv_tc(const DecodeArgs &A, const uint64_t *d_mask, const float *d_alpha, const void *d_x,
+                          int64_t ldx, uint32_t batch, float *d_y, int64_t ldy, uint64_t m, uint64_t n, cudaStream_t st)
+{
+    constexpr uint32_t PIECES = sizeof(XT) == 4 ? 3 : 1;
+    const size_t limit = 220 * 1024;
+    const uint32_t sms = (uint32_t)sm_count();
+    TcArgs g;
+    g.A = A;
+    g.mask32 = (const uint32_t *)d_mask;
+    g.mask_words = A.words64 * 2;
+    g.alpha = d_alpha;
+    g.x = d_x; g.ldx = ldx; g.y = d_y; g.ldy = ldy;
+    g.m = m; g.n = (uint32_t)n; g.batch = batch;
+    const uint64_t R = (m + sms - 1) / sms, grid = (m + R - 1) / R;
+    if (R > 0xffffffffull || n > (1u << 24)) return SQNN_E_UNSUPPORTED;
+    g.rows_per_block = (uint32_t)R;
+    g.units = (uint32_t)((n + 128 * TC_RANGES - 1) / (128 * TC_RANGES)) | 1u;      // odd: see above
+    g.kq = g.units * 128;
+    const uint32_t bt_max = TC_MAX_Q / PIECES, passes = (batch + bt_max - 1) / bt_max;
+    g.bt = (batch + passes - 1) / passes;
+    g.N = (8 * g.bt * PIECES + 15) / 16 * 16;
+    g.slots = g.N <= 64 ? 2u : 1u;
+    const size_t tab = (size_t)A.tab_words * 4, x_bytes = (size_t)(g.kq / 64) * g.N * 128 + 1024;
+    const uint64_t TW = 32ull * A.W, tile_bits = 32 * TW;
+    // bits a lane may read past the end of the last row: its range's padding and the second vector
+    const uint64_t slack = (TC_RANGES * (uint64_t)g.kq - n) / 32 + 12;
+    uint64_t RC = R;
+    size_t smem = 0;
+    for (;; RC = (RC + 1) / 2) {
+        const uint64_t tiles = (RC * n + tile_bits - 1) / tile_bits + 1;
+        const uint64_t region_words = (tiles * TW + slack + 3) & ~3ull;
+        g.alpha_words = (uint32_t)((RC * A.n_q + 3) & ~3ull);
+        g.part_words = (uint32_t)((TC_GROUPS * RC * g.bt + 3) & ~3ull);
+        const uint64_t need = tab + (uint64_t)(A.n_q + 1) * region_words * 4 + 4ull * (g.alpha_words + g.part_words) + x_bytes;
+        if (need <= limit) {
+            g.region_words = (uint32_t)region_words;
+            g.rows_per_chunk = (uint32_t)RC;
+            smem = (size_t)need;
+            break;
+        }
+        if (RC <= 8) return SQNN_E_UNSUPPORTED;                  // rows too long for chunks that fill a tile half
+    }
+    g.x_vec = (((uintptr_t)d_x & 15) == 0 && (ldx * (int64_t)sizeof(XT)) % 16 == 0) ? 1u : 0u;
+    return n % 128 == 0 ? launch_kernel(k_gemv_tc<N_OUT, N_IN, XT, true>, (uint32_t)grid, TC_THREADS, smem, st, g)
+                        : launch_kernel(k_gemv_tc<N_OUT, N_IN, XT, false>, (uint32_t)grid, TC_THREADS, smem, st, g);
+}
+
+}  // namespace sqnn
