@@ -80,55 +80,82 @@ SQNN_DEV void lds_bits128(uint32_t sa, uint32_t o, uint32_t (&out)[4])
     }
 }
 
-// Two bf16 values (round toward zero, exact when they have at most 8 significant bits) in one word.
-SQNN_DEV uint32_t high_halves(float lo, float hi) { return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632); }
+SQNN_DEV void sts128(uint32_t at, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" :: "r"(at), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
 
 // Stages activation vectors [bc, bc + bt) as B rows: vector q, range kq, piece p -> row 8 (q * PIECES + p) + kq of
 // every 64-column step's box ([N rows][128 bytes], 128-byte swizzle).  Columns past n and vectors past the batch
-// are zero.  Values that are not finite are staged as zero and reported: a pruned weight must not meet them.
+// are zero.  A warp takes 32 chunks (of 8 columns) of one B row at a time.  bf16 rows on 16-byte boundaries go
+// straight to shared memory (cp.async, the caller commits and waits); everything else passes through registers.
 template <typename XT>
-SQNN_DEV void tc_stage_x(const TcArgs &g, uint32_t x_sa, uint32_t bc, uint32_t *not_finite)
+SQNN_DEV void tc_stage_x(const TcArgs &g, uint32_t x_sa, uint32_t bc)
 {
     constexpr uint32_t PIECES = sizeof(XT) == 4 ? 3 : 1;
     const XT *x = reinterpret_cast<const XT *>(g.x);
-    const uint32_t chunks = g.kq / 8, per_q = TC_RANGES * chunks, total = per_q * g.bt;       // of 8 columns
-    bool odd = false;
-    for (uint32_t i = threadIdx.x; i < total; i += TC_THREADS) {
-        const uint32_t q = i / per_q, rest = i - q * per_q, kq = rest / chunks, ch = rest - kq * chunks;
-        const uint32_t c = kq * g.kq + ch * 8;
-        float v[8];
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t chunks = g.kq / 8, blocks = (chunks + 31) / 32, items = TC_RANGES * g.bt * blocks;
+    for (uint32_t it = warp; it < items; it += TC_THREADS / 32) {
+        const uint32_t row = it / blocks, ch = (it - row * blocks) * 32 + lane;                // row = 8 q + kq
+        if (ch >= chunks) continue;
+        const uint32_t q = row >> 3, kq = row & 7u, c = kq * g.kq + ch * 8;
+        const uint32_t valid = bc + q < g.batch && c < g.n ? min(g.n - c, 8u) : 0u;
         const XT *src = x + (int64_t)(bc + q) * g.ldx + c;
-        if (bc + q < g.batch && c + 8 <= g.n && g.x_vec) {
-            if constexpr (PIECES == 1) {
-                const uint4 t = __ldg(reinterpret_cast<const uint4 *>(src));
-                const uint32_t w[4] = {t.x, t.y, t.z, t.w};
-#pragma unroll
-                for (int e = 0; e < 4; ++e) { v[2 * e] = __uint_as_float(w[e] << 16); v[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u); }
+        const uint32_t box = x_sa + (ch >> 3) * g.N * 128;
+        if constexpr (PIECES == 1) {
+            const uint32_t at = box + row * 128 + (((ch & 7u) ^ kq) << 4);
+            if (g.x_vec) {
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" :: "r"(at), "l"(valid ? src : x), "r"(2 * valid) : "memory");
             } else {
-                const float4 t = __ldg(reinterpret_cast<const float4 *>(src)), u = __ldg(reinterpret_cast<const float4 *>(src) + 1);
-                v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w; v[4] = u.x; v[5] = u.y; v[6] = u.z; v[7] = u.w;
+                const unsigned short *h = reinterpret_cast<const unsigned short *>(src);
+                uint32_t w[4];
+#pragma unroll
+                for (uint32_t k = 0; k < 4; ++k)
+                    w[k] = (2 * k < valid ? (uint32_t)__ldg(h + 2 * k) : 0u) | (2 * k + 1 < valid ? (uint32_t)__ldg(h + 2 * k + 1) << 16 : 0u);
+                sts128(at, w[0], w[1], w[2], w[3]);
             }
         } else {
+            float v[8];
+            if (g.x_vec && valid == 8) {
+                const float4 t = __ldg(reinterpret_cast<const float4 *>(src)), u = __ldg(reinterpret_cast<const float4 *>(src) + 1);
+                v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w; v[4] = u.x; v[5] = u.y; v[6] = u.z; v[7] = u.w;
+            } else {
 #pragma unroll
-            for (uint32_t e = 0; e < 8; ++e) v[e] = bc + q < g.batch && c + e < g.n ? to_float(src[e]) : 0.0f;
-        }
+                for (uint32_t k = 0; k < 8; ++k) v[k] = k < valid ? __ldg(reinterpret_cast<const float *>(src) + k) : 0.0f;
+            }
+            // the upper half of an fp32 word is a bf16 with its first 8 significant bits; what is left after
+            // subtracting it has 16, and so on: three pieces, exactly
 #pragma unroll
-        for (int e = 0; e < 8; ++e)
-            if ((__float_as_uint(v[e]) & 0x7f800000u) == 0x7f800000u) { odd = true; v[e] = 0.0f; }
-        const uint32_t box = x_sa + (ch >> 3) * g.N * 128;
+            for (uint32_t p = 0; p < PIECES; ++p) {
+                const uint32_t r = 8 * (q * PIECES + p) + kq;
+                uint32_t w[4];
 #pragma unroll
-        for (uint32_t p = 0; p < PIECES; ++p) {
-            const uint32_t row = 8 * (q * PIECES + p) + kq;
-            const uint32_t at = box + row * 128 + (((ch & 7u) ^ (row & 7u)) << 4);
-            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" :: "r"(at), "r"(high_halves(v[0], v[1])), "r"(high_halves(v[2], v[3])),
-                         "r"(high_halves(v[4], v[5])), "r"(high_halves(v[6], v[7])) : "memory");
-            if (p + 1 < PIECES) {
+                for (uint32_t k = 0; k < 4; ++k) w[k] = __byte_perm(__float_as_uint(v[2 * k]), __float_as_uint(v[2 * k + 1]), 0x7632);
+                sts128(box + r * 128 + (((ch & 7u) ^ kq) << 4), w[0], w[1], w[2], w[3]);
 #pragma unroll
-                for (int e = 0; e < 8; ++e) v[e] -= __uint_as_float(__float_as_uint(v[e]) & 0xffff0000u);
+                for (uint32_t k = 0; k < 8; ++k) v[k] -= __uint_as_float(__float_as_uint(v[k]) & 0xffff0000u);
             }
         }
     }
-    if (odd) atomicOr(not_finite, 1u);
+}
+
+// One output by a plain walk over the care bits: for sums that came out as no finite number.  A pruned weight must
+// not meet an activation that is infinite or not a number, and in the matrix product it does (as zero).
+template <typename XT>
+SQNN_DEV float tc_walk(const TcArgs &g, const XT *x, const uint32_t *mask_s, const uint32_t *bits_s, const float *al, uint32_t o)
+{
+    float sum = 0.0f;
+#pragma unroll 1
+    for (uint32_t c = 0; c < g.n; ++c) {
+        if (!((mask_s[(o + c) >> 5] >> ((o + c) & 31u)) & 1u)) continue;
+        float w = 0.0f;
+#pragma unroll 1
+        for (uint32_t pl = 0; pl < g.A.n_q; ++pl)
+            w += ((bits_s[pl * g.region_words + ((o + c) >> 5)] >> ((o + c) & 31u)) & 1u) ? al[pl] : -al[pl];
+        sum = fmaf(w, to_float(x[c]), sum);
+    }
+    return sum;
 }
 
 template <int N_OUT, int N_IN, typename XT, bool ALIGNED>
@@ -137,7 +164,7 @@ k_gemv_tc(const TcArgs g)
 {
     extern __shared__ __align__(16) uint32_t smem[];
     __shared__ uint64_t bars[3 * TC_GROUPS];              // per group: two A slots free, accumulator complete
-    __shared__ uint32_t tmem_slot, abort_word, not_finite;
+    __shared__ uint32_t tmem_slot, abort_word;
     constexpr uint32_t PIECES = sizeof(XT) == 4 ? 3 : 1;
     const DecodeArgs &A = g.A;
     volatile uint32_t *abort_flag = &abort_word;
@@ -160,13 +187,11 @@ k_gemv_tc(const TcArgs g)
     if (warp == nwarps - 1) tmem_alloc(&tmem_slot, 512);
     if (threadIdx.x == 0) {
         for (uint32_t i = 0; i < 3 * TC_GROUPS; ++i) mbar_init(bars_sa + 8 * i, 1);
-        abort_word = not_finite = 0;
+        abort_word = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
-    __syncthreads();
     wait_prior_grid();
     launch_dependents();
-    tables_request(A, tab_s);                                    // commit group: tables
     uint32_t slot_seq = 0, parts_done = 0;                       // per group: A slots filled, accumulators read
     bool first = true;
 
@@ -179,15 +204,27 @@ k_gemv_tc(const TcArgs g)
         const uint32_t nt = (uint32_t)(kt1 - kt0);
         const uint64_t gw0 = kt0 * TW;                           // first word of the chunk's regions
         if (!first) __syncthreads();                             // the product of the previous chunk is over
-        stage_mask(mask_s, g.mask32, gw0, g.mask_words, nt * TW, threadIdx.x, TC_THREADS, mask_vec);
-        for (uint32_t i = threadIdx.x; i < nrows * n_q; i += TC_THREADS) cp_async4(alpha_s + i, g.alpha + ra * n_q + i);
-        cp_async_commit();                                       // commit group: mask and scales
-        for (uint32_t i = threadIdx.x; i < TC_GROUPS * nrows * g.bt; i += TC_THREADS) part_s[i] = 0.0f;
-
-        // decode: item = (tile, plane), dealt out over the warps; a warp's first item is fetched before anybody
-        // waits for the tables, and the activations are staged while it is under way
+        // decode: item = (tile, plane), dealt out over the warps.  A warp's first item is requested before
+        // everything else, its patch entries (whose place the first answer tells) after the requests for tables,
+        // activations, mask and scales.
         const uint32_t items = nt * n_q;
         uint32_t item = warp;
+        auto stage_all = [&] {
+            if (first) {
+                tables_request(A, tab_s);                        // commit group: tables
+                tc_stage_x<XT>(g, x_sa, 0);
+            }
+            stage_mask(mask_s, g.mask32, gw0, g.mask_words, nt * TW, threadIdx.x, TC_THREADS, mask_vec);
+            for (uint32_t i = threadIdx.x; i < nrows * n_q; i += TC_THREADS) cp_async4(alpha_s + i, g.alpha + ra * n_q + i);
+            cp_async_commit();                                   // commit group: activations, mask and scales
+            for (uint32_t i = threadIdx.x; i < TC_GROUPS * nrows * g.bt; i += TC_THREADS) part_s[i] = 0.0f;
+        };
+        auto tables_ready = [&] {
+            if (first) {
+                cp_async_wait_group<1>();                        // (the younger group may be pending)
+                __syncthreads();
+            }
+        };
         if constexpr (N_OUT != 0) {
             using S = Shape<N_OUT, N_IN>;
             TileSeeds<N_OUT, N_IN> s;
@@ -195,16 +232,13 @@ k_gemv_tc(const TcArgs g)
             uint32_t pw[PATCH_AHEAD];
             auto fetch = [&](uint32_t it) {
                 const uint32_t t = it / n_q, pl = it - t * n_q;
-                fetch_seeds<N_OUT, N_IN>(A.pl[pl], kt0 + t, lane, s);
                 run = fetch_run(A.pl[pl], kt0 + t);
-                fetch_patches(A, A.pl[pl], run, lane, pw);
+                fetch_seeds<N_OUT, N_IN>(A.pl[pl], kt0 + t, lane, s);
             };
             if (item < items) fetch(item);
-            if (first) {
-                tc_stage_x<XT>(g, x_sa, 0, &not_finite);
-                cp_async_wait_group<1>();                        // tables (mask and scales may be pending)
-                __syncthreads();
-            }
+            stage_all();
+            if (item < items) fetch_patches(A, A.pl[item % n_q], run, lane, pw);
+            tables_ready();
             while (item < items) {
                 const uint32_t t = item / n_q, pl = item - t * n_q;
                 uint32_t *region = bits_s + pl * g.region_words + t * TW;
@@ -212,14 +246,11 @@ k_gemv_tc(const TcArgs g)
                 __syncwarp();
                 tile_patch(A, A.pl[pl], run, pw, region, 0u, S::TILE_BITS, lane);
                 item += nwarps;
-                if (item < items) fetch(item);
+                if (item < items) { fetch(item); fetch_patches(A, A.pl[item % n_q], run, lane, pw); }
             }
         } else {
-            if (first) {
-                tc_stage_x<XT>(g, x_sa, 0, &not_finite);
-                cp_async_wait_group<1>();
-                __syncthreads();
-            }
+            stage_all();
+            tables_ready();
             for (; item < items; item += nwarps) {
                 const uint32_t t = item / n_q, pl = item - t * n_q;
                 decode_ktile_generic(A, pl, kt0 + t, bits_s + pl * g.region_words + t * TW, tab_s, lane);
@@ -242,7 +273,9 @@ k_gemv_tc(const TcArgs g)
         for (uint32_t bc = 0; bc < g.batch; bc += g.bt) {
             if (bc != 0 || (ra != row0 && g.bt < g.batch)) {     // another pass: its activations replace the last one's
                 __syncthreads();
-                tc_stage_x<XT>(g, x_sa, bc, &not_finite);
+                tc_stage_x<XT>(g, x_sa, bc);
+                cp_async_commit();
+                cp_async_wait_all();
                 for (uint32_t i = threadIdx.x; i < TC_GROUPS * nrows * g.bt; i += TC_THREADS) part_s[i] = 0.0f;
                 fence_async_smem();
                 __syncthreads();
@@ -287,19 +320,19 @@ k_gemv_tc(const TcArgs g)
                     ++parts_done;
                     tc_fence_after();
 #pragma unroll
-                    for (uint32_t q2 = 0; q2 < TC_MAX_Q / 2; ++q2) {
-                        if (16 * q2 >= g.N) break;
-                        uint32_t d[16];
-                        tmem_ld16(d_tmem + lane_sel + 16 * q2, d);
+                    for (uint32_t q4 = 0; q4 < TC_MAX_Q / 4; ++q4) {
+                        if (32 * q4 >= g.N) break;
+                        uint32_t d[32];
+                        tmem_ld32(d_tmem + lane_sel + 32 * q4, d);           // (N = 16, 48, ..: the second half is not used)
 #pragma unroll
-                        for (uint32_t e = 0; e < 2; ++e) {
+                        for (uint32_t e = 0; e < 4; ++e) {
                             uint32_t a4[4], a2[2];
 #pragma unroll
                             for (uint32_t k = 0; k < 4; ++k) a4[k] = (kq & 4u) ? d[8 * e + k + 4] : d[8 * e + k];
 #pragma unroll
                             for (uint32_t k = 0; k < 2; ++k) a2[k] = (kq & 2u) ? a4[k + 2] : a4[k];
                             const float mine = __uint_as_float((kq & 1u) ? a2[1] : a2[0]);
-                            const uint32_t q = 2 * q2 + e;
+                            const uint32_t q = 4 * q4 + e;
                             acc[q / PIECES] = fmaf(al, mine, acc[q / PIECES]);
                         }
                     }
@@ -337,28 +370,16 @@ k_gemv_tc(const TcArgs g)
                 }
             }
             __syncthreads();
-            for (uint32_t i = threadIdx.x; i < nrows * g.bt; i += TC_THREADS) {
-                const uint32_t rl = i / g.bt, q = i - rl * g.bt;
-                if (bc + q >= g.batch) continue;
-                float sum = 0.0f;
+            for (uint32_t q = warp; q < g.bt && bc + q < g.batch; q += nwarps)
+                for (uint32_t rl = lane; rl < nrows; rl += 32) {
+                    float sum = 0.0f;
 #pragma unroll
-                for (uint32_t p = 0; p < TC_GROUPS; ++p) sum += part_s[(p * nrows + rl) * g.bt + q];
-                if (not_finite) {                                // add what was left out of the staged activations
-                    const XT *x = reinterpret_cast<const XT *>(g.x) + (int64_t)(bc + q) * g.ldx;
-                    const uint32_t o = (uint32_t)((ra + rl) * n - gw0 * 32);
-                    for (uint32_t c = 0; c < n; ++c) {
-                        const float xv = to_float(x[c]);
-                        if ((__float_as_uint(xv) & 0x7f800000u) != 0x7f800000u || !((mask_s[(o + c) >> 5] >> ((o + c) & 31u)) & 1u)) continue;
-                        float w = 0.0f;
-                        for (uint32_t pl = 0; pl < n_q; ++pl) {
-                            const float a = alpha_s[rl * n_q + pl];
-                            w += ((bits_s[pl * g.region_words + ((o + c) >> 5)] >> ((o + c) & 31u)) & 1u) ? a : -a;
-                        }
-                        sum = fmaf(w, xv, sum);
-                    }
+                    for (uint32_t p = 0; p < TC_GROUPS; ++p) sum += part_s[(p * nrows + rl) * g.bt + q];
+                    if ((__float_as_uint(sum) & 0x7f800000u) == 0x7f800000u)
+                        sum = tc_walk<XT>(g, reinterpret_cast<const XT *>(g.x) + (int64_t)(bc + q) * g.ldx, mask_s, bits_s,
+                                          alpha_s + rl * n_q, (uint32_t)((ra + rl) * n - gw0 * 32));
+                    g.y[(int64_t)(bc + q) * g.ldy + (int64_t)(ra + rl)] = sum;
                 }
-                g.y[(int64_t)(bc + q) * g.ldy + (int64_t)(ra + rl)] = sum;
-            }
         }
     }
     tc_fence_before();
