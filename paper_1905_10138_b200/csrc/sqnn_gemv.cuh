@@ -1,5 +1,6 @@
-// K3: decryption fused with Y[b][r] = sum_c W[r][c] X[b][c] for small batch (<= 15), fp32
-// accumulation on the plain ALUs, as a template over the network shape, with its launcher.
+// K3 for rows too long for the tensor-core form (sqnn_gemv_tc.cuh): decryption fused with
+// Y[b][r] = sum_c W[r][c] X[b][c] for small batch (<= 15), fp32 accumulation on the plain ALUs, as a template over
+// the network shape, with its launcher.
 //
 // Work split.  A block owns a run of whole rows of W.  The bits of those rows are one contiguous
 // range of every flattened plane, so the block decodes the kernel tiles that cover that range
@@ -381,7 +382,7 @@ inline int launch_gemv_bt(const DecodeArgs &A, const uint64_t *d_mask, const flo
     const uint64_t TW = 32ull * A.W, tile_bits = 32 * TW;
     const size_t tab = (size_t)A.tab_words * 4;
     const size_t xbytes = ((size_t)n * BT * sizeof(XT) + 15) & ~(size_t)15;
-    bool xs = xbytes <= 128 * 1024;
+    bool xs = BT == 1 && xbytes <= 128 * 1024;      // several long vectors never fit
     // Warps sharing a row.  A warp walks its run of a row's words 32 at a time, and every item (a row, or one
     // of `parts` runs of it) costs about one such step more for its set-up and reduction, so the walk of a chunk
     // takes (rounds of items over the warps) x (steps per item + 1); the cheapest split wins, the smaller one on
@@ -426,15 +427,14 @@ inline int launch_gemv_bt(const DecodeArgs &A, const uint64_t *d_mask, const flo
     do {                                                                                                 \
         return launch_kernel(k_decode_gemv<N_OUT, N_IN, BT, XT, XSV, NQV>, (uint32_t)grid, nwarps * 32, smem, st, g); \
     } while (0)
-    if (xs) {
-        if (A.n_q == 1) SQNN_GEMV_LAUNCH(true, 1);
-        else if (A.n_q == 2) SQNN_GEMV_LAUNCH(true, 2);
-        else if (A.n_q == 3) SQNN_GEMV_LAUNCH(true, 3);
-        else SQNN_GEMV_LAUNCH(true, 0);
-    } else {
-        if (A.n_q == 1) SQNN_GEMV_LAUNCH(false, 1);
-        else SQNN_GEMV_LAUNCH(false, 0);
+    if constexpr (BT == 1) {
+        if (xs) {
+            if (A.n_q == 1) SQNN_GEMV_LAUNCH(true, 1);
+            else SQNN_GEMV_LAUNCH(true, 0);
+        }
     }
+    if (A.n_q == 1) SQNN_GEMV_LAUNCH(false, 1);
+    else SQNN_GEMV_LAUNCH(false, 0);
 #undef SQNN_GEMV_LAUNCH
 }
 

@@ -411,29 +411,35 @@ inline int launch_gemv_tc(const DecodeArgs &A, const uint64_t *d_mask, const flo
     g.rows_per_block = (uint32_t)R;
     g.units = (uint32_t)((n + 128 * TC_RANGES - 1) / (128 * TC_RANGES)) | 1u;      // odd: see above
     g.kq = g.units * 128;
-    const uint32_t bt_max = TC_MAX_Q / PIECES, passes = (batch + bt_max - 1) / bt_max;
-    g.bt = (batch + passes - 1) / passes;
-    g.N = (8 * g.bt * PIECES + 15) / 16 * 16;
-    g.slots = g.N <= 64 ? 2u : 1u;
-    const size_t tab = (size_t)A.tab_words * 4, x_bytes = (size_t)(g.kq / 64) * g.N * 128 + 1024;
+    const size_t tab = (size_t)A.tab_words * 4;
     const uint64_t TW = 32ull * A.W, tile_bits = 32 * TW;
     // bits a lane may read past the end of the last row: its range's padding and the second vector
     const uint64_t slack = (TC_RANGES * (uint64_t)g.kq - n) / 32 + 12;
-    uint64_t RC = R;
+    // Activation vectors per pass: as many as the accumulators allow, fewer where they would leave too little
+    // shared memory for a chunk of rows (every pass expands the weights again, every chunk decodes its boundary
+    // tiles again and may leave a tile of 16 rows half empty).
+    const uint32_t bt_max = TC_MAX_Q / PIECES;
     size_t smem = 0;
-    for (;; RC = (RC + 1) / 2) {
-        const uint64_t tiles = (RC * n + tile_bits - 1) / tile_bits + 1;
-        const uint64_t region_words = (tiles * TW + slack + 3) & ~3ull;
-        g.alpha_words = (uint32_t)((RC * A.n_q + 3) & ~3ull);
-        g.part_words = (uint32_t)((TC_GROUPS * RC * g.bt + 3) & ~3ull);
-        const uint64_t need = tab + (uint64_t)(A.n_q + 1) * region_words * 4 + 4ull * (g.alpha_words + g.part_words) + x_bytes;
-        if (need <= limit) {
-            g.region_words = (uint32_t)region_words;
-            g.rows_per_chunk = (uint32_t)RC;
-            smem = (size_t)need;
-            break;
+    for (uint32_t passes = (batch + bt_max - 1) / bt_max; smem == 0; ++passes) {
+        if (passes > batch) return SQNN_E_UNSUPPORTED;           // rows too long
+        g.bt = (batch + passes - 1) / passes;
+        g.N = (8 * g.bt * PIECES + 15) / 16 * 16;
+        g.slots = g.N <= 64 ? 2u : 1u;
+        const size_t x_bytes = (size_t)(g.kq / 64) * g.N * 128 + 1024;
+        for (uint64_t RC = R;; RC = (RC + 1) / 2) {
+            const uint64_t tiles = (RC * n + tile_bits - 1) / tile_bits + 1;
+            const uint64_t region_words = (tiles * TW + slack + 3) & ~3ull;
+            g.alpha_words = (uint32_t)((RC * A.n_q + 3) & ~3ull);
+            g.part_words = (uint32_t)((TC_GROUPS * RC * g.bt + 3) & ~3ull);
+            const uint64_t need = tab + (uint64_t)(A.n_q + 1) * region_words * 4 + 4ull * (g.alpha_words + g.part_words) + x_bytes;
+            if (need <= limit) {
+                g.region_words = (uint32_t)region_words;
+                g.rows_per_chunk = (uint32_t)RC;
+                smem = (size_t)need;
+                break;
+            }
+            if (RC <= 8) break;
         }
-        if (RC <= 8) return SQNN_E_UNSUPPORTED;                  // rows too long for chunks that fill a tile half
     }
     g.x_vec = (((uintptr_t)d_x & 15) == 0 && (ldx * (int64_t)sizeof(XT)) % 16 == 0) ? 1u : 0u;
     return n % 128 == 0 ? launch_kernel(k_gemv_tc<N_OUT, N_IN, XT, true>, (uint32_t)grid, TC_THREADS, smem, st, g)
