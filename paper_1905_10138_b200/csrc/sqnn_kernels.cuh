@@ -8,6 +8,8 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 namespace sqnn {
 
 // ------------------------------------------------------------------------------------------
@@ -194,159 +196,211 @@ SQNN_DEV void stage_mask(uint32_t *mask_s, const uint32_t *__restrict__ mask32, 
     }
 }
 
-// K2: decoded, masked, rescaled weights as bf16.  Lane j of an iteration writes the 8 weights
-// of byte j of a 32-byte group of the tile's bit run, so a warp stores 512 contiguous bytes.
-// The tile's mask words arrive by cp.async while the tile is decoded; a lane keeps the scales
-// of the row it is in.  NQ = number of planes when it is 1, 2 or 3, 0 = any.
-// With one plane a weight is +-bf16(alpha) or 0, so four weights at a time come from a table indexed
-// by (mask nibble, bit nibble): a keep-mask and a sign-flip per weight, applied to the row's scale
-// with one logic operation per pair of weights (exact for any alpha; a pruned weight is +0).  The
-// table is kept in 8 copies, lane l reads copy l % 8, so that lookups of different entries do not
-// share banks.
-constexpr uint32_t BF16_LUT_COPIES = 8;
-constexpr uint32_t BF16_LUT_WORDS = 256 * BF16_LUT_COPIES * 4;
+// K2: decoded, masked, rescaled weights as bf16.  A lane takes 32 weights (one word of every plane and of the mask)
+// at a time and writes them as 64 bytes of a 2 KB buffer of its warp, which leaves by a bulk copy while the
+// next one is filled.
+//
+// With up to three planes a weight is +-V[a], where the sign is plane 0's bit and a says which of the other
+// planes disagree with it: at most four bf16 values per row, eight bytes, from which one byte permutation picks
+// two weights.  Selectors, signs and keep masks come out of words in which even and odd columns have been
+// separated, by a shift and an AND each (4.5 instructions per weight with three planes; sums of the scales per
+// weight took about 20, and 64 us for 2^26 weights of three planes).  Negating all terms of a sum negates it
+// exactly, except when it is zero or not finite; rows with such a value take the plain loop, as do words that
+// straddle two rows in the chunk of 8 where they do, and layers of four and more planes.
 constexpr uint32_t BF16_THREADS = 768;                   // one block per SM, as many warps as shared memory holds
+constexpr uint32_t BF16_STAGE_WORDS = 2 * 512;           // two buffers of 2 KB per warp
+
+// The bf16 values of a row: V[0] | V[1] << 16, V[2] | V[3] << 16; plain: the sign trick does not hold.
+struct RowValues {
+    uint64_t row;
+    uint32_t v0, v1;
+    bool plain;
+};
+template <int NQ>
+SQNN_DEV RowValues row_values(const float *__restrict__ alpha, uint64_t r)
+{
+    static_assert(NQ >= 1 && NQ <= 3, "up to four values");
+    RowValues t{r, 0u, 0u, false};
+    float a[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) a[i] = __ldg(alpha + r * NQ + i);
+    uint32_t h[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        float s = a[0];
+        if constexpr (NQ >= 2) s = __fadd_rn(s, (e & 1) ? -a[1] : a[1]);
+        if constexpr (NQ >= 3) s = __fadd_rn(s, (e & 2) ? -a[2] : a[2]);
+        h[e] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(s));
+        if (s == 0.0f || (__float_as_uint(s) & 0x7f800000u) == 0x7f800000u) t.plain = true;
+    }
+    t.v0 = h[0] | (h[1] << 16);
+    t.v1 = h[2] | (h[3] << 16);
+    return t;
+}
+
+// 16 columns as eight words of two bf16.  zm: even columns' (mask, minus) bit pairs in the low half, odd ones'
+// in the high half; qe: bytes even 0-7, odd 0-7, even 8-15, odd 8-15 of (e1, e2) pairs, e_i = plane i differs
+// from plane 0.
+template <int NQ>
+SQNN_DEV void weights16(uint32_t zm, uint32_t qe, const RowValues &t, uint32_t (&out)[8])
+{
+#pragma unroll
+    for (uint32_t j = 0; j < 4; ++j) {
+        uint32_t lo, hi;
+        if constexpr (NQ >= 2) {
+            const uint32_t sel = ((qe >> (2 * j)) & 0x03030303u) * 0x22u + 0x10101010u;
+            lo = __byte_perm(t.v0, t.v1, sel);
+            hi = __byte_perm(t.v0, t.v1, sel >> 16);
+        } else {
+            lo = hi = __byte_perm(t.v0, 0u, 0x1010);
+        }
+#pragma unroll
+        for (uint32_t k = 0; k < 2; ++k) {
+            const uint32_t f = j + 4 * k;                        // columns 2 f, 2 f + 1
+            const uint32_t keep = ((zm >> (2 * f)) & 0x00010001u) * 0xffffu;
+            out[f] = ((k ? hi : lo) ^ ((zm << (14 - 2 * f)) & 0x80008000u)) & keep;
+        }
+    }
+}
+
 template <int N_OUT, int N_IN, int NQ>
 __global__ void __launch_bounds__(BF16_THREADS, 1)
 k_decode_bf16(DecodeArgs A, const uint32_t *__restrict__ mask32, const float *__restrict__ alpha,
               uint64_t n, __nv_bfloat16 *__restrict__ out)
 {
     extern __shared__ __align__(16) uint32_t smem[];
+    wait_prior_grid();
+    launch_dependents();
     tables_request(A, smem);
-    uint4 *lut = reinterpret_cast<uint4 *>(smem + A.tab_words);          // [256][copies]: keep masks (x, y), sign flips (z, w)
-    if constexpr (NQ == 1) {
-        for (uint32_t e = threadIdx.x; e < 256; e += blockDim.x) {
-            uint32_t keep[4], flip[4];
-#pragma unroll
-            for (uint32_t k = 0; k < 4; ++k) {
-                const uint32_t m = (e >> (4 + k)) & 1u, b = (e >> k) & 1u;
-                keep[k] = m ? 0xffffu : 0u;
-                flip[k] = (m && !b) ? 0x8000u : 0u;
-            }
-            const uint4 v = make_uint4(keep[0] | (keep[1] << 16), keep[2] | (keep[3] << 16),
-                                       flip[0] | (flip[1] << 16), flip[2] | (flip[3] << 16));
-#pragma unroll
-            for (uint32_t c = 0; c < BF16_LUT_COPIES; ++c) lut[e * BF16_LUT_COPIES + c] = v;
-        }
-    }
     cp_async_wait_all();
     __syncthreads();
     const uint32_t W = words_per_lane<N_OUT>(A);
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const uint32_t n_q = A.n_q;
-    const uint32_t per_warp = (n_q + 1) * 32 * W;
-    uint32_t *region = smem + A.tab_words + (NQ == 1 ? BF16_LUT_WORDS : 0u) + warp * per_warp;
-    uint32_t *mask_s = region + n_q * 32 * W;
-    const uint8_t *mask_s8 = reinterpret_cast<const uint8_t *>(mask_s);
-    const uint32_t tile_bytes = 128 * W;                 // bytes of bits per tile and plane
+    const uint32_t n_q = NQ ? NQ : A.n_q;
+    uint32_t *region = smem + A.tab_words + warp * (n_q * 32 * W + BF16_STAGE_WORDS);
+    uint32_t *stage = region + n_q * 32 * W;
     const uint64_t mask_words = A.words64 * 2;
-    const bool mask_vec = (reinterpret_cast<uintptr_t>(mask32) & 15) == 0;
-    constexpr int NR = NQ > 0 ? NQ : 1;
+    // A lane's four chunks of 8 weights are produced in an order that starts at `turn`, so that the 16-byte stores
+    // of eight neighbouring lanes fall into different banks.
+    const uint32_t turn = (lane >> 1) & 3u;
+    const bool long_rows = n > 1024;
+    uint32_t buf = 0;
+    RowValues t{~0ull, 0u, 0u, true};
     for (uint64_t tile = (uint64_t)blockIdx.x * nwarps + warp; tile < A.ktiles; tile += (uint64_t)gridDim.x * nwarps) {
-        const uint64_t p_tile = tile * (uint64_t)tile_bytes * 8;
-        if (p_tile >= A.mn) continue;
-        stage_mask(mask_s, mask32, tile * 32 * W, mask_words, 32 * W, lane, 32, mask_vec);
+        const uint64_t p_tile = tile * (uint64_t)W * 1024;
+        if (p_tile >= A.mn) break;
+        uint64_t r = (p_tile + 32ull * lane) / n;                // row and column of the lane's first weight
+        uint64_t c = (p_tile + 32ull * lane) - r * n;
+        const uint64_t w_tile = tile * 32 * W;
+        uint32_t m_next = w_tile + lane < mask_words ? __ldg(mask32 + w_tile + lane) : 0u;
         for (uint32_t i = 0; i < n_q; ++i)
             decode_warp_tile<N_OUT, N_IN>(A, i, tile, region + i * 32 * W, smem, lane);
-        cp_async_wait_all();
-        __syncwarp();
-        // byte t of the tile's bit run holds the weights p_tile + 8 t ..; bytes below nfull lie wholly inside
-        // the plane, bytes below nbytes hold at least one of its weights
-        const uint64_t left = A.mn - p_tile;
-        const uint32_t nbytes = left >= 8ull * tile_bytes ? tile_bytes : (uint32_t)((left + 7) / 8);
-        const uint32_t nfull = left >= 8ull * tile_bytes ? tile_bytes : (uint32_t)(left / 8);
-        __nv_bfloat16 *out_t = out + p_tile;
-        const uint8_t *bits_s8 = reinterpret_cast<const uint8_t *>(region);
-        const uint32_t lut_lane = lane & (BF16_LUT_COPIES - 1);
-        uint64_t r = (p_tile + 8ull * lane) / n;         // row and column of the lane's first weight
-        uint64_t c = (p_tile + 8ull * lane) - r * n;
-        float al[NR];
-        uint32_t ab2 = 0;                                // bf16(alpha) of the row, twice (one plane)
-        uint64_t r_al = ~0ull;
-        for (uint32_t t = lane; t < nbytes; t += 32, c += 256) {
-            while (c >= n) { c -= n; ++r; }
-            const uint32_t mk = mask_s8[t];
-            const uint64_t p = p_tile + 8ull * t;        // (the slow path's)
-            if (NQ == 1 && c + 8 <= n && t < nfull) {
-                if (r != r_al) {
-                    al[0] = __ldg(alpha + r);
-                    r_al = r;
-                    const uint32_t ab = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(al[0]));
-                    ab2 = ab | (ab << 16);
+        for (uint32_t it = 0; it < W; ++it) {
+            const uint64_t p_it = p_tile + 1024ull * it;         // first weight of the warp's 1024
+            if (p_it >= A.mn) break;
+            const uint32_t wi = 32 * it + lane, m = m_next;
+            if (it + 1 < W) m_next = w_tile + wi + 32 < mask_words ? __ldg(mask32 + w_tile + wi + 32) : 0u;
+            uint32_t *to = stage + buf * 512 + lane * 16;
+            if (lane == 0) bulk_wait_read<1>();                  // the copy out of this buffer is over
+            __syncwarp();
+            bool fast = false;
+            if constexpr (NQ != 0) {
+                if (c + 32 <= n) {
+                    if (r != t.row) t = row_values<NQ>(alpha, r);
+                    fast = !t.plain;
                 }
-                const uint32_t bt = bits_s8[t];
-                const uint4 e0 = lut[((((mk & 15u) << 4) | (bt & 15u))) * BF16_LUT_COPIES + lut_lane];
-                const uint4 e1 = lut[((mk & 0xf0u) | (bt >> 4)) * BF16_LUT_COPIES + lut_lane];
-                *reinterpret_cast<uint4 *>(out_t + 8 * t) = make_uint4((ab2 & e0.x) ^ e0.z, (ab2 & e0.y) ^ e0.w,
-                                                                       (ab2 & e1.x) ^ e1.z, (ab2 & e1.y) ^ e1.w);
-            } else if (NQ > 0 && c + 8 <= n && t < nfull) {
-                if (r != r_al) {
-#pragma unroll
-                    for (int i = 0; i < NR; ++i) al[i] = __ldg(alpha + r * n_q + i);
-                    r_al = r;
-                }
-                uint32_t bits[NR];
-#pragma unroll
-                for (int i = 0; i < NR; ++i) bits[i] = reinterpret_cast<const uint8_t *>(region + i * 32 * W)[t];
-                uint32_t w[4];
-#pragma unroll
-                for (uint32_t h = 0; h < 4; ++h) {
-                    float two[2];
-#pragma unroll
-                    for (uint32_t e = 0; e < 2; ++e) {
-                        const uint32_t k = 2 * h + e;
-                        float s = 0.0f;
-#pragma unroll
-                        for (int i = 0; i < NR; ++i) {
-                            const float term = ((bits[i] >> k) & 1u) ? al[i] : -al[i];
-                            s = i == 0 ? term : __fadd_rn(s, term);
-                        }
-                        two[e] = ((mk >> k) & 1u) ? s : 0.0f;
+                if (fast) {
+                    const uint32_t b0 = region[wi], sgn = ~b0;
+                    // rotated so that chunk `turn` comes first
+                    const uint32_t mr = __funnelshift_r(m, m, 8 * turn), sr = __funnelshift_r(sgn, sgn, 8 * turn);
+                    const uint32_t me = (mr & 0x55555555u) | ((sr << 1) & 0xaaaaaaaau), mo = ((mr >> 1) & 0x55555555u) | (sr & 0xaaaaaaaau);
+                    uint32_t qe = 0, qo = 0;
+                    if constexpr (NQ >= 2) {
+                        uint32_t e1 = b0 ^ region[32 * W + wi], e2 = 0;
+                        if constexpr (NQ >= 3) e2 = b0 ^ region[64 * W + wi];
+                        e1 = __funnelshift_r(e1, e1, 8 * turn);
+                        e2 = __funnelshift_r(e2, e2, 8 * turn);
+                        qe = (e1 & 0x55555555u) | ((e2 << 1) & 0xaaaaaaaau);
+                        qo = ((e1 >> 1) & 0x55555555u) | (e2 & 0xaaaaaaaau);
                     }
-                    const __nv_bfloat162 pk = __floats2bfloat162_rn(two[0], two[1]);
-                    w[h] = *reinterpret_cast<const uint32_t *>(&pk);
+#pragma unroll
+                    for (uint32_t h = 0; h < 2; ++h) {           // 16 weights: chunks 2 h and 2 h + 1 of the rotated word
+                        uint32_t o[8];
+                        weights16<NQ>(__byte_perm(me, mo, h ? 0x7632 : 0x5410), __byte_perm(qe, qo, h ? 0x7362 : 0x5140), t, o);
+                        *reinterpret_cast<uint4 *>(to + 4 * ((2 * h + turn) & 3u)) = make_uint4(o[0], o[1], o[2], o[3]);
+                        *reinterpret_cast<uint4 *>(to + 4 * ((2 * h + 1 + turn) & 3u)) = make_uint4(o[4], o[5], o[6], o[7]);
+                    }
                 }
-                *reinterpret_cast<uint4 *>(out_t + 8 * t) = make_uint4(w[0], w[1], w[2], w[3]);
-            } else {
+            }
+            if (!fast) {
                 uint64_t rr = r, cc = c;
-                for (uint32_t k = 0; k < 8 && p + k < A.mn; ++k) {
-                    if (cc >= n) { cc -= n; ++rr; }
-                    float s = 0.0f;
-                    if ((mk >> k) & 1u) {
-                        for (uint32_t i = 0; i < n_q; ++i) {
-                            const float a = __ldg(alpha + rr * n_q + i);
-                            const uint32_t bi = reinterpret_cast<const uint8_t *>(region + i * 32 * W)[t];
-                            s = __fadd_rn(s, ((bi >> k) & 1u) ? a : -a);
+#pragma unroll 1
+                for (uint32_t ch = 0; ch < 4; ++ch) {            // chunks of 8 weights
+                    while (cc >= n) { cc -= n; ++rr; }
+                    const uint32_t mk = (m >> (8 * ch)) & 0xffu;
+                    if constexpr (NQ != 0) {
+                        if (cc + 8 <= n && p_it + 32 * lane + 8 * ch < A.mn) {       // one row
+                            if (rr != t.row) t = row_values<NQ>(alpha, rr);
+                            if (!t.plain) {
+                                const uint32_t b0 = region[wi] >> (8 * ch), sr = ~b0;
+                                uint32_t e1 = 0, e2 = 0;
+                                if constexpr (NQ >= 2) e1 = b0 ^ (region[32 * W + wi] >> (8 * ch));
+                                if constexpr (NQ >= 3) e2 = b0 ^ (region[64 * W + wi] >> (8 * ch));
+                                const uint32_t me = (mk & 0x55u) | ((sr << 1) & 0xaau), mo = ((mk >> 1) & 0x55u) | (sr & 0xaau);
+                                const uint32_t qe = (e1 & 0x55u) | ((e2 << 1) & 0xaau), qo = ((e1 >> 1) & 0x55u) | (e2 & 0xaau);
+                                uint32_t o[8];
+                                weights16<NQ>(me | (mo << 16), qe | (qo << 8), t, o);
+                                *reinterpret_cast<uint4 *>(to + 4 * ch) = make_uint4(o[0], o[1], o[2], o[3]);
+                                cc += 8;
+                                continue;
+                            }
                         }
                     }
-                    out[p + k] = __float2bfloat16_rn(s);
-                    ++cc;
+#pragma unroll 1
+                    for (uint32_t k = 0; k < 8; ++k) {
+                        while (cc >= n) { cc -= n; ++rr; }
+                        float sum = 0.0f;
+                        if (((mk >> k) & 1u) && p_it + 32 * lane + 8 * ch + k < A.mn)
+                            for (uint32_t i = 0; i < n_q; ++i) {
+                                const float a = __ldg(alpha + rr * n_q + i);
+                                sum = __fadd_rn(sum, ((region[i * 32 * W + wi] >> (8 * ch + k)) & 1u) ? a : -a);
+                            }
+                        reinterpret_cast<__nv_bfloat16 *>(to)[8 * ch + k] = __float2bfloat16_rn(sum);
+                        ++cc;
+                    }
                 }
+            }
+            if (p_it + 1024 <= A.mn) {
+                fence_async_smem();
+                __syncwarp();
+                if (lane == 0) bulk_store(out + p_it, stage + buf * 512, 2048);
+            } else {                                             // the last weights, one by one
+                __syncwarp();
+                const __nv_bfloat16 *from = reinterpret_cast<const __nv_bfloat16 *>(stage + buf * 512);
+                for (uint32_t k = lane; p_it + k < A.mn; k += 32) out[p_it + k] = from[k];
+                __syncwarp();
+            }
+            buf ^= 1u;
+            c += 1024;
+            if (c >= n) {
+                if (long_rows) { c -= n; ++r; }
+                else { const uint32_t q = (uint32_t)c / (uint32_t)n; c -= (uint64_t)q * n; r += q; }
             }
         }
         __syncwarp();
     }
+    if (lane == 0) bulk_wait_read<0>();                          // shared memory must outlive the copies
 }
 
 // ------------------------------------------------------------------------------------------
 // launchers
 // ------------------------------------------------------------------------------------------
-// Picks warps per block so the dynamic shared memory fits; returns 0 if not even one warp fits.
-inline uint32_t pick_warps(const DecodeArgs &A, uint32_t regions, size_t *smem_bytes, uint32_t max_warps, size_t limit)
+// A layer with fewer tiles than all SMs have warps: as many blocks as SMs with as few warps as that takes.
+inline uint32_t spread_warps(uint64_t tiles, uint32_t most)
 {
-    const size_t tab = (size_t)A.tab_words * 4;
-    const size_t per_warp = (size_t)regions * 32 * A.W * 4;
-    if (tab + per_warp > limit) return 0;
-    uint32_t warps = (uint32_t)((limit - tab) / per_warp);
-    if (warps > max_warps) warps = max_warps;
-    *smem_bytes = tab + warps * per_warp;
-    return warps;
-}
-
-template <typename K>
-inline int prepare(K kernel, size_t smem)
-{
-    return ensure_dynamic_smem(reinterpret_cast<const void *>(kernel), smem);
+    const uint64_t share = (tiles + sm_count() - 1) / sm_count();
+    const uint32_t want = share > 4 ? (share < most ? (uint32_t)share : most) : 4u;
+    return want < most ? want : most;
 }
 
 inline uint32_t grid_for(uint64_t warp_tiles, uint32_t warps, uint32_t blocks_per_sm)
@@ -374,10 +428,7 @@ inline int launch_decode(const DecodeArgs &A, sqnn_out_mode mode, const uint64_t
         if (tab + per_warp > limit) return SQNN_E_UNSUPPORTED;
         uint32_t warps = (uint32_t)((limit - tab) / per_warp);
         if (warps > DECODE_BITS_THREADS / 32) warps = DECODE_BITS_THREADS / 32;
-        // a layer with fewer tiles than all SMs have warps: as many blocks as SMs with as few warps as that takes
-        const uint64_t share = (live * A.n_q + sm_count() - 1) / sm_count();
-        const uint32_t want = share > 4 ? (share < 32 ? (uint32_t)share : 32u) : 4u;
-        if (warps > want) warps = want;
+        warps = spread_warps(live * A.n_q, warps);
         smem = tab + warps * per_warp;
         const uint32_t grid = grid_for(live * A.n_q, warps, 1);
 #define SQNN_BITS_LAUNCH2(SINKV, ONEV, REPV)                                                             \
@@ -398,17 +449,16 @@ inline int launch_decode(const DecodeArgs &A, sqnn_out_mode mode, const uint64_t
 #undef SQNN_BITS_LAUNCH2
 #undef SQNN_BITS_LAUNCH
     } else {
-        const size_t lut_bytes = A.n_q == 1 ? (size_t)BF16_LUT_WORDS * 4 : 0;
-        const uint32_t warps = pick_warps(A, A.n_q + 1, &smem, BF16_THREADS / 32, 224 * 1024 - lut_bytes);
-        if (!warps) return SQNN_E_UNSUPPORTED;
-        smem += lut_bytes;
+        const size_t limit = 224 * 1024, tab = (size_t)A.tab_words * 4, per_warp = (size_t)(A.n_q * 32 * A.W + BF16_STAGE_WORDS) * 4;
+        if (tab + per_warp > limit) return SQNN_E_UNSUPPORTED;
         const uint64_t live = (A.words64 * 2 + 32ull * A.W - 1) / (32ull * A.W);
+        const uint32_t warps = spread_warps(live, (uint32_t)std::min<size_t>((limit - tab) / per_warp, BF16_THREADS / 32));
+        smem = tab + warps * per_warp;
         const uint32_t grid = grid_for(live, warps, 1);
 #define SQNN_BF16_LAUNCH(NQV)                                                                            \
     do {                                                                                                 \
-        auto k = k_decode_bf16<N_OUT, N_IN, NQV>;                                                        \
-        if (prepare(k, smem)) return SQNN_E_CUDA;                                                        \
-        k<<<grid, warps * 32, smem, st>>>(A, (const uint32_t *)d_mask, d_alpha, n, (__nv_bfloat16 *)d_out); \
+        return launch_kernel(k_decode_bf16<N_OUT, N_IN, NQV>, grid, warps * 32, smem, st, A, (const uint32_t *)d_mask, \
+                             d_alpha, n, (__nv_bfloat16 *)d_out);                                        \
     } while (0)
         if (A.n_q == 1) SQNN_BF16_LAUNCH(1);
         else if (A.n_q == 2) SQNN_BF16_LAUNCH(2);
