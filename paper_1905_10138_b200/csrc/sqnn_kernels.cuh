@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 namespace sqnn {
 
@@ -200,49 +201,60 @@ SQNN_DEV void stage_mask(uint32_t *mask_s, const uint32_t *__restrict__ mask32, 
 // at a time and writes them as 64 bytes of a 2 KB buffer of its warp, which leaves by a bulk copy while the
 // next one is filled.
 //
-// With up to three planes a weight is +-V[a], where the sign is plane 0's bit and a says which of the other
+// With up to three planes a weight is 0 or +-V[a], where the sign is plane 0's bit and a says which of the other
 // planes disagree with it: at most four bf16 values per row, eight bytes, from which one byte permutation picks
-// two weights.  Selectors, signs and keep masks come out of words in which even and odd columns have been
-// separated, by a shift and an AND each (4.5 instructions per weight with three planes; sums of the scales per
-// weight took about 20, and 64 us for 2^26 weights of three planes).  Negating all terms of a sum negates it
-// exactly, except when it is zero or not finite; rows with such a value take the plain loop, as do words that
-// straddle two rows in the chunk of 8 where they do, and layers of four and more planes.
+// two weights.  Mask and sign bits, moved to the top of a half word, are the bf16 numbers 0, 2 and -2, so a
+// multiply-add with V / 2 does the rest.  Selectors and those numbers come out of words in which even and odd
+// columns have been separated, by a shift and an AND each: 3 instructions per weight with three planes.  (Sums of
+// the scales per weight took about 20, and 64 us for 2^26 weights of three planes.)  Negating all terms of a sum
+// negates it exactly, except when it is zero or not finite, and halving is exact except for the tiniest
+// numbers; rows with such a value take the plain loop, as do chunks of 8 weights that straddle rows, and
+// layers of four and more planes.
 constexpr uint32_t BF16_THREADS = 768;                   // one block per SM, as many warps as shared memory holds
 constexpr uint32_t BF16_STAGE_WORDS = 2 * 512;           // two buffers of 2 KB per warp
 
-// The bf16 values of a row: V[0] | V[1] << 16, V[2] | V[3] << 16; plain: the sign trick does not hold.
+// Half the bf16 values of a row: V[0] | V[1] << 16, V[2] | V[3] << 16; plain: see above.
+template <typename IT>
 struct RowValues {
-    uint64_t row;
+    IT row;
     uint32_t v0, v1;
     bool plain;
 };
-template <int NQ>
-SQNN_DEV RowValues row_values(const float *__restrict__ alpha, uint64_t r)
+template <int NQ, typename IT>
+SQNN_DEV RowValues<IT> row_values(const float *__restrict__ alpha, IT r)
 {
     static_assert(NQ >= 1 && NQ <= 3, "up to four values");
-    RowValues t{r, 0u, 0u, false};
+    RowValues<IT> t{r, 0u, 0u, false};
     float a[3] = {0.0f, 0.0f, 0.0f};
 #pragma unroll
-    for (int i = 0; i < NQ; ++i) a[i] = __ldg(alpha + r * NQ + i);
+    for (int i = 0; i < NQ; ++i) a[i] = __ldg(alpha + (uint64_t)r * NQ + i);
     uint32_t h[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
         float s = a[0];
         if constexpr (NQ >= 2) s = __fadd_rn(s, (e & 1) ? -a[1] : a[1]);
         if constexpr (NQ >= 3) s = __fadd_rn(s, (e & 2) ? -a[2] : a[2]);
-        h[e] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(s));
-        if (s == 0.0f || (__float_as_uint(s) & 0x7f800000u) == 0x7f800000u) t.plain = true;
+        if (!(fabsf(s) > 1e-36f && fabsf(s) < 1e38f)) t.plain = true;
+        h[e] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(s)) - 0x0080u;       // exponent less one
     }
-    t.v0 = h[0] | (h[1] << 16);
-    t.v1 = h[2] | (h[3] << 16);
+    t.v0 = __byte_perm(h[0], h[1], 0x5410);
+    t.v1 = __byte_perm(h[2], h[3], 0x5410);
     return t;
+}
+
+// a * b + 0 on two bf16 numbers (the + 0 turns -0 into 0)
+SQNN_DEV uint32_t bf16x2_mul0(uint32_t a, uint32_t b)
+{
+    uint32_t r;
+    asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(0u));
+    return r;
 }
 
 // 16 columns as eight words of two bf16.  zm: even columns' (mask, minus) bit pairs in the low half, odd ones'
 // in the high half; qe: bytes even 0-7, odd 0-7, even 8-15, odd 8-15 of (e1, e2) pairs, e_i = plane i differs
 // from plane 0.
-template <int NQ>
-SQNN_DEV void weights16(uint32_t zm, uint32_t qe, const RowValues &t, uint32_t (&out)[8])
+template <int NQ, typename IT>
+SQNN_DEV void weights16(uint32_t zm, uint32_t qe, const RowValues<IT> &t, uint32_t (&out)[8])
 {
 #pragma unroll
     for (uint32_t j = 0; j < 4; ++j) {
@@ -252,72 +264,91 @@ SQNN_DEV void weights16(uint32_t zm, uint32_t qe, const RowValues &t, uint32_t (
             lo = __byte_perm(t.v0, t.v1, sel);
             hi = __byte_perm(t.v0, t.v1, sel >> 16);
         } else {
-            lo = hi = __byte_perm(t.v0, 0u, 0x1010);
+            lo = hi = t.v0;                                      // V[0] = V[1]
         }
-#pragma unroll
-        for (uint32_t k = 0; k < 2; ++k) {
-            const uint32_t f = j + 4 * k;                        // columns 2 f, 2 f + 1
-            const uint32_t keep = ((zm >> (2 * f)) & 0x00010001u) * 0xffffu;
-            out[f] = ((k ? hi : lo) ^ ((zm << (14 - 2 * f)) & 0x80008000u)) & keep;
-        }
+        out[j] = bf16x2_mul0(lo, (zm << (14 - 2 * j)) & 0xc000c000u);                  // columns 2 j, 2 j + 1
+        out[j + 4] = bf16x2_mul0(hi, (zm << (6 - 2 * j)) & 0xc000c000u);               // columns 8 + 2 j, 9 + 2 j
     }
 }
 
 template <int N_OUT, int N_IN, int NQ>
 __global__ void __launch_bounds__(BF16_THREADS, 1)
 k_decode_bf16(DecodeArgs A, const uint32_t *__restrict__ mask32, const float *__restrict__ alpha,
-              uint64_t n, __nv_bfloat16 *__restrict__ out)
+              uint64_t n64, __nv_bfloat16 *__restrict__ out)
 {
+    using IT = typename std::conditional<NQ != 0, uint32_t, uint64_t>::type;       // rows and columns
     extern __shared__ __align__(16) uint32_t smem[];
     wait_prior_grid();
     launch_dependents();
     tables_request(A, smem);
     cp_async_wait_all();
     __syncthreads();
+    const IT n = (IT)n64;
     const uint32_t W = words_per_lane<N_OUT>(A);
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const uint32_t n_q = NQ ? NQ : A.n_q;
     uint32_t *region = smem + A.tab_words + warp * (n_q * 32 * W + BF16_STAGE_WORDS);
     uint32_t *stage = region + n_q * 32 * W;
-    const uint64_t mask_words = A.words64 * 2;
     // A lane's four chunks of 8 weights are produced in an order that starts at `turn`, so that the 16-byte stores
     // of eight neighbouring lanes fall into different banks.
     const uint32_t turn = (lane >> 1) & 3u;
-    const bool long_rows = n > 1024;
     uint32_t buf = 0;
-    RowValues t{~0ull, 0u, 0u, true};
+    RowValues<IT> t{(IT)~0ull, 0u, 0u, true};
     for (uint64_t tile = (uint64_t)blockIdx.x * nwarps + warp; tile < A.ktiles; tile += (uint64_t)gridDim.x * nwarps) {
         const uint64_t p_tile = tile * (uint64_t)W * 1024;
         if (p_tile >= A.mn) break;
-        uint64_t r = (p_tile + 32ull * lane) / n;                // row and column of the lane's first weight
-        uint64_t c = (p_tile + 32ull * lane) - r * n;
-        const uint64_t w_tile = tile * 32 * W;
-        uint32_t m_next = w_tile + lane < mask_words ? __ldg(mask32 + w_tile + lane) : 0u;
-        for (uint32_t i = 0; i < n_q; ++i)
-            decode_warp_tile<N_OUT, N_IN>(A, i, tile, region + i * 32 * W, smem, lane);
-        for (uint32_t it = 0; it < W; ++it) {
-            const uint64_t p_it = p_tile + 1024ull * it;         // first weight of the warp's 1024
-            if (p_it >= A.mn) break;
-            const uint32_t wi = 32 * it + lane, m = m_next;
-            if (it + 1 < W) m_next = w_tile + wi + 32 < mask_words ? __ldg(mask32 + w_tile + wi + 32) : 0u;
+        const uint32_t here = A.mn - p_tile < (uint64_t)W * 1024 ? (uint32_t)(A.mn - p_tile) : W * 1024;   // weights of this tile
+        const uint64_t p_lane = p_tile + 32ull * lane, r64 = p_lane / n64;
+        IT r = (IT)r64, c = (IT)(p_lane - r64 * n64);            // row and column of the lane's first weight
+        const uint32_t *mp = mask32 + tile * 32 * W + lane;      // this lane's mask words: those below `here`
+        uint32_t m_next = 32 * lane < here ? __ldg(mp) : 0u;
+        if constexpr (N_OUT != 0 && NQ != 0) {
+            // all planes' seeds and patch runs are requested together, then all patch entries
+            using S = Shape<N_OUT, N_IN>;
+            TileSeeds<N_OUT, N_IN> seeds[NQ];
+            TileRun run[NQ];
+            uint32_t pw[NQ][PATCH_AHEAD];
+#pragma unroll
+            for (int i = 0; i < NQ; ++i) {
+                run[i] = fetch_run(A.pl[i], tile);
+                fetch_seeds<N_OUT, N_IN>(A.pl[i], tile, lane, seeds[i]);
+            }
+#pragma unroll
+            for (int i = 0; i < NQ; ++i) fetch_patches(A, A.pl[i], run[i], lane, pw[i]);
+#pragma unroll
+            for (int i = 0; i < NQ; ++i) tile_expand<N_OUT, N_IN>(seeds[i], region + i * 32 * W, smem, lane);
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < NQ; ++i) tile_patch(A, A.pl[i], run[i], pw[i], region + i * 32 * W, 0u, S::TILE_BITS, lane);
+            __syncwarp();
+        } else {
+            for (uint32_t i = 0; i < n_q; ++i)
+                decode_warp_tile<N_OUT, N_IN>(A, i, tile, region + i * 32 * W, smem, lane);
+        }
+        __nv_bfloat16 *to_g = out + p_tile;
+        const uint32_t *bits = region + lane;
+        for (uint32_t at = 0; at < here; at += 1024, bits += 32, to_g += 1024) {
+            const uint32_t m = m_next;
+            mp += 32;
+            if (at + 1024 + 32 * lane < here) m_next = __ldg(mp); else m_next = 0u;
             uint32_t *to = stage + buf * 512 + lane * 16;
             if (lane == 0) bulk_wait_read<1>();                  // the copy out of this buffer is over
             __syncwarp();
             bool fast = false;
             if constexpr (NQ != 0) {
-                if (c + 32 <= n) {
-                    if (r != t.row) t = row_values<NQ>(alpha, r);
+                if (n - c >= 32 && at + 32 * lane < here) {
+                    if (r != t.row) t = row_values<NQ, IT>(alpha, r);
                     fast = !t.plain;
                 }
                 if (fast) {
-                    const uint32_t b0 = region[wi], sgn = ~b0;
+                    const uint32_t b0 = bits[0], sgn = ~b0;
                     // rotated so that chunk `turn` comes first
                     const uint32_t mr = __funnelshift_r(m, m, 8 * turn), sr = __funnelshift_r(sgn, sgn, 8 * turn);
                     const uint32_t me = (mr & 0x55555555u) | ((sr << 1) & 0xaaaaaaaau), mo = ((mr >> 1) & 0x55555555u) | (sr & 0xaaaaaaaau);
                     uint32_t qe = 0, qo = 0;
                     if constexpr (NQ >= 2) {
-                        uint32_t e1 = b0 ^ region[32 * W + wi], e2 = 0;
-                        if constexpr (NQ >= 3) e2 = b0 ^ region[64 * W + wi];
+                        uint32_t e1 = b0 ^ bits[32 * W], e2 = 0;
+                        if constexpr (NQ >= 3) e2 = b0 ^ bits[64 * W];
                         e1 = __funnelshift_r(e1, e1, 8 * turn);
                         e2 = __funnelshift_r(e2, e2, 8 * turn);
                         qe = (e1 & 0x55555555u) | ((e2 << 1) & 0xaaaaaaaau);
@@ -326,30 +357,30 @@ k_decode_bf16(DecodeArgs A, const uint32_t *__restrict__ mask32, const float *__
 #pragma unroll
                     for (uint32_t h = 0; h < 2; ++h) {           // 16 weights: chunks 2 h and 2 h + 1 of the rotated word
                         uint32_t o[8];
-                        weights16<NQ>(__byte_perm(me, mo, h ? 0x7632 : 0x5410), __byte_perm(qe, qo, h ? 0x7362 : 0x5140), t, o);
+                        weights16<NQ, IT>(__byte_perm(me, mo, h ? 0x7632 : 0x5410), __byte_perm(qe, qo, h ? 0x7362 : 0x5140), t, o);
                         *reinterpret_cast<uint4 *>(to + 4 * ((2 * h + turn) & 3u)) = make_uint4(o[0], o[1], o[2], o[3]);
                         *reinterpret_cast<uint4 *>(to + 4 * ((2 * h + 1 + turn) & 3u)) = make_uint4(o[4], o[5], o[6], o[7]);
                     }
                 }
             }
             if (!fast) {
-                uint64_t rr = r, cc = c;
+                IT rr = r, cc = c;
 #pragma unroll 1
-                for (uint32_t ch = 0; ch < 4; ++ch) {            // chunks of 8 weights
+                for (uint32_t ch = 0; ch < 4 && at + 32 * lane + 8 * ch < here; ++ch) {      // chunks of 8 weights
                     while (cc >= n) { cc -= n; ++rr; }
                     const uint32_t mk = (m >> (8 * ch)) & 0xffu;
                     if constexpr (NQ != 0) {
-                        if (cc + 8 <= n && p_it + 32 * lane + 8 * ch < A.mn) {       // one row
-                            if (rr != t.row) t = row_values<NQ>(alpha, rr);
+                        if (n - cc >= 8) {                       // one row
+                            if (rr != t.row) t = row_values<NQ, IT>(alpha, rr);
                             if (!t.plain) {
-                                const uint32_t b0 = region[wi] >> (8 * ch), sr = ~b0;
+                                const uint32_t b0 = bits[0] >> (8 * ch), sr = ~b0;
                                 uint32_t e1 = 0, e2 = 0;
-                                if constexpr (NQ >= 2) e1 = b0 ^ (region[32 * W + wi] >> (8 * ch));
-                                if constexpr (NQ >= 3) e2 = b0 ^ (region[64 * W + wi] >> (8 * ch));
+                                if constexpr (NQ >= 2) e1 = b0 ^ (bits[32 * W] >> (8 * ch));
+                                if constexpr (NQ >= 3) e2 = b0 ^ (bits[64 * W] >> (8 * ch));
                                 const uint32_t me = (mk & 0x55u) | ((sr << 1) & 0xaau), mo = ((mk >> 1) & 0x55u) | (sr & 0xaau);
                                 const uint32_t qe = (e1 & 0x55u) | ((e2 << 1) & 0xaau), qo = ((e1 >> 1) & 0x55u) | (e2 & 0xaau);
                                 uint32_t o[8];
-                                weights16<NQ>(me | (mo << 16), qe | (qo << 8), t, o);
+                                weights16<NQ, IT>(me | (mo << 16), qe | (qo << 8), t, o);
                                 *reinterpret_cast<uint4 *>(to + 4 * ch) = make_uint4(o[0], o[1], o[2], o[3]);
                                 cc += 8;
                                 continue;
@@ -357,34 +388,34 @@ k_decode_bf16(DecodeArgs A, const uint32_t *__restrict__ mask32, const float *__
                         }
                     }
 #pragma unroll 1
-                    for (uint32_t k = 0; k < 8; ++k) {
+                    for (uint32_t k = 0; k < 8 && at + 32 * lane + 8 * ch + k < here; ++k) {
                         while (cc >= n) { cc -= n; ++rr; }
                         float sum = 0.0f;
-                        if (((mk >> k) & 1u) && p_it + 32 * lane + 8 * ch + k < A.mn)
+                        if ((mk >> k) & 1u)
                             for (uint32_t i = 0; i < n_q; ++i) {
-                                const float a = __ldg(alpha + rr * n_q + i);
-                                sum = __fadd_rn(sum, ((region[i * 32 * W + wi] >> (8 * ch + k)) & 1u) ? a : -a);
+                                const float a = __ldg(alpha + (uint64_t)rr * n_q + i);
+                                sum = __fadd_rn(sum, ((bits[i * 32 * W] >> (8 * ch + k)) & 1u) ? a : -a);
                             }
                         reinterpret_cast<__nv_bfloat16 *>(to)[8 * ch + k] = __float2bfloat16_rn(sum);
                         ++cc;
                     }
                 }
             }
-            if (p_it + 1024 <= A.mn) {
+            if (at + 1024 <= here) {
                 fence_async_smem();
                 __syncwarp();
-                if (lane == 0) bulk_store(out + p_it, stage + buf * 512, 2048);
+                if (lane == 0) bulk_store(to_g, stage + buf * 512, 2048);
             } else {                                             // the last weights, one by one
                 __syncwarp();
                 const __nv_bfloat16 *from = reinterpret_cast<const __nv_bfloat16 *>(stage + buf * 512);
-                for (uint32_t k = lane; p_it + k < A.mn; k += 32) out[p_it + k] = from[k];
+                for (uint32_t k = lane; at + k < here; k += 32) to_g[k] = from[k];
                 __syncwarp();
             }
             buf ^= 1u;
             c += 1024;
             if (c >= n) {
-                if (long_rows) { c -= n; ++r; }
-                else { const uint32_t q = (uint32_t)c / (uint32_t)n; c -= (uint64_t)q * n; r += q; }
+                if (n > 1024) { c -= n; ++r; }
+                else { const uint32_t q = (uint32_t)c / (uint32_t)n; c -= (IT)(q * (uint32_t)n); r += q; }
             }
         }
         __syncwarp();
@@ -460,7 +491,8 @@ inline int launch_decode(const DecodeArgs &A, sqnn_out_mode mode, const uint64_t
         return launch_kernel(k_decode_bf16<N_OUT, N_IN, NQV>, grid, warps * 32, smem, st, A, (const uint32_t *)d_mask, \
                              d_alpha, n, (__nv_bfloat16 *)d_out);                                        \
     } while (0)
-        if (A.n_q == 1) SQNN_BF16_LAUNCH(1);
+        if (n >= (1ull << 31) || A.mn / n >= (1ull << 31)) SQNN_BF16_LAUNCH(0);       // 64-bit rows and columns
+        else if (A.n_q == 1) SQNN_BF16_LAUNCH(1);
         else if (A.n_q == 2) SQNN_BF16_LAUNCH(2);
         else if (A.n_q == 3) SQNN_BF16_LAUNCH(3);
         else SQNN_BF16_LAUNCH(0);
