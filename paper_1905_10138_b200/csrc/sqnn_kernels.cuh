@@ -210,7 +210,8 @@ SQNN_DEV void stage_mask(uint32_t *mask_s, const uint32_t *__restrict__ mask32, 
 // negates it exactly, except when it is zero or not finite, and halving is exact except for the tiniest
 // numbers; rows with such a value take the plain loop, as do chunks of 8 weights that straddle rows, and
 // layers of four and more planes.
-constexpr uint32_t BF16_THREADS = 768;                   // one block per SM, as many warps as shared memory holds
+// One block per SM, as many warps as shared memory holds, fewer where a lane's entries need the registers.
+SQNN_HD constexpr uint32_t bf16_threads(uint32_t n_out) { return n_out > 128 ? 512 : 768; }
 constexpr uint32_t BF16_STAGE_WORDS = 2 * 512;           // two buffers of 2 KB per warp
 
 // Half the bf16 values of a row: V[0] | V[1] << 16, V[2] | V[3] << 16; plain: see above.
@@ -272,7 +273,7 @@ SQNN_DEV void weights16(uint32_t zm, uint32_t qe, const RowValues<IT> &t, uint32
 }
 
 template <int N_OUT, int N_IN, int NQ>
-__global__ void __launch_bounds__(BF16_THREADS, 1)
+__global__ void __launch_bounds__(bf16_threads(N_OUT), 1)
 k_decode_bf16(DecodeArgs A, const uint32_t *__restrict__ mask32, const float *__restrict__ alpha,
               uint64_t n64, __nv_bfloat16 *__restrict__ out)
 {
@@ -281,11 +282,31 @@ k_decode_bf16(DecodeArgs A, const uint32_t *__restrict__ mask32, const float *__
     wait_prior_grid();
     launch_dependents();
     tables_request(A, smem);
-    cp_async_wait_all();
-    __syncthreads();
     const IT n = (IT)n64;
     const uint32_t W = words_per_lane<N_OUT>(A);
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const uint32_t ktiles = (uint32_t)((A.mn + (uint64_t)W * 1024 - 1) / ((uint64_t)W * 1024)), stride = gridDim.x * nwarps;
+    // All planes' seeds and patch runs of a tile are requested together, the first tile's ahead of the tables and
+    // every other tile's before the weights of the one before it are made; then all its patch entries.
+    constexpr bool AHEAD = N_OUT != 0 && NQ != 0;
+    constexpr int NF = AHEAD ? NQ : 1;
+    TileSeeds<AHEAD ? N_OUT : 40, AHEAD ? N_IN : 12> seeds[NF];
+    TileRun run[NF];
+    auto request = [&](uint32_t tile) {
+        if constexpr (AHEAD) {
+            if (tile < ktiles) {
+#pragma unroll
+                for (int i = 0; i < NQ; ++i) {
+                    run[i] = fetch_run(A.pl[i], tile);
+                    fetch_seeds<N_OUT, N_IN>(A.pl[i], tile, lane, seeds[i]);
+                }
+            }
+        }
+    };
+    const uint32_t first = blockIdx.x * nwarps + warp;
+    request(first);
+    cp_async_wait_all();
+    __syncthreads();
     const uint32_t n_q = NQ ? NQ : A.n_q;
     uint32_t *region = smem + A.tab_words + warp * (n_q * 32 * W + BF16_STAGE_WORDS);
     uint32_t *stage = region + n_q * 32 * W;
@@ -294,25 +315,16 @@ k_decode_bf16(DecodeArgs A, const uint32_t *__restrict__ mask32, const float *__
     const uint32_t turn = (lane >> 1) & 3u;
     uint32_t buf = 0;
     RowValues<IT> t{(IT)~0ull, 0u, 0u, true};
-    for (uint64_t tile = (uint64_t)blockIdx.x * nwarps + warp; tile < A.ktiles; tile += (uint64_t)gridDim.x * nwarps) {
+    for (uint32_t tile = first; tile < ktiles; tile += stride) {
         const uint64_t p_tile = tile * (uint64_t)W * 1024;
-        if (p_tile >= A.mn) break;
         const uint32_t here = A.mn - p_tile < (uint64_t)W * 1024 ? (uint32_t)(A.mn - p_tile) : W * 1024;   // weights of this tile
         const uint64_t p_lane = p_tile + 32ull * lane, r64 = p_lane / n64;
         IT r = (IT)r64, c = (IT)(p_lane - r64 * n64);            // row and column of the lane's first weight
-        const uint32_t *mp = mask32 + tile * 32 * W + lane;      // this lane's mask words: those below `here`
+        const uint32_t *mp = mask32 + (uint64_t)tile * 32 * W + lane;      // this lane's mask words: those below `here`
         uint32_t m_next = 32 * lane < here ? __ldg(mp) : 0u;
-        if constexpr (N_OUT != 0 && NQ != 0) {
-            // all planes' seeds and patch runs are requested together, then all patch entries
+        if constexpr (AHEAD) {
             using S = Shape<N_OUT, N_IN>;
-            TileSeeds<N_OUT, N_IN> seeds[NQ];
-            TileRun run[NQ];
             uint32_t pw[NQ][PATCH_AHEAD];
-#pragma unroll
-            for (int i = 0; i < NQ; ++i) {
-                run[i] = fetch_run(A.pl[i], tile);
-                fetch_seeds<N_OUT, N_IN>(A.pl[i], tile, lane, seeds[i]);
-            }
 #pragma unroll
             for (int i = 0; i < NQ; ++i) fetch_patches(A, A.pl[i], run[i], lane, pw[i]);
 #pragma unroll
@@ -321,6 +333,7 @@ k_decode_bf16(DecodeArgs A, const uint32_t *__restrict__ mask32, const float *__
 #pragma unroll
             for (int i = 0; i < NQ; ++i) tile_patch(A, A.pl[i], run[i], pw[i], region + i * 32 * W, 0u, S::TILE_BITS, lane);
             __syncwarp();
+            request(tile + stride);
         } else {
             for (uint32_t i = 0; i < n_q; ++i)
                 decode_warp_tile<N_OUT, N_IN>(A, i, tile, region + i * 32 * W, smem, lane);
@@ -394,7 +407,8 @@ k_decode_bf16(DecodeArgs A, const uint32_t *__restrict__ mask32, const float *__
                         if ((mk >> k) & 1u)
                             for (uint32_t i = 0; i < n_q; ++i) {
                                 const float a = __ldg(alpha + (uint64_t)rr * n_q + i);
-                                sum = __fadd_rn(sum, ((bits[i * 32 * W] >> (8 * ch + k)) & 1u) ? a : -a);
+                                const float term = ((bits[i * 32 * W] >> (8 * ch + k)) & 1u) ? a : -a;
+                                sum = i == 0 ? term : __fadd_rn(sum, term);
                             }
                         reinterpret_cast<__nv_bfloat16 *>(to)[8 * ch + k] = __float2bfloat16_rn(sum);
                         ++cc;
@@ -483,7 +497,8 @@ inline int launch_decode(const DecodeArgs &A, sqnn_out_mode mode, const uint64_t
         const size_t limit = 224 * 1024, tab = (size_t)A.tab_words * 4, per_warp = (size_t)(A.n_q * 32 * A.W + BF16_STAGE_WORDS) * 4;
         if (tab + per_warp > limit) return SQNN_E_UNSUPPORTED;
         const uint64_t live = (A.words64 * 2 + 32ull * A.W - 1) / (32ull * A.W);
-        const uint32_t warps = spread_warps(live, (uint32_t)std::min<size_t>((limit - tab) / per_warp, BF16_THREADS / 32));
+        if (live >= (1ull << 31)) return SQNN_E_UNSUPPORTED;
+        const uint32_t warps = spread_warps(live, (uint32_t)std::min<size_t>((limit - tab) / per_warp, bf16_threads(N_OUT) / 32));
         smem = tab + warps * per_warp;
         const uint32_t grid = grid_for(live, warps, 1);
 #define SQNN_BF16_LAUNCH(NQV)                                                                            \
