@@ -13,9 +13,9 @@
 //
 // and e can be taken in the order of its size: once the best count is B, sizes above B cannot matter.  Almost
 // all slices are done after sizes 0 (consistent: no wrong bit), 1 and 2: about 80 candidates for r = 12
-// instead of 4096.  One thread per slice does that much; the few slices that need larger sets are finished by
-// the whole warp, which walks all 2^r sets in Gray-code order, and slices with more dependent rows than V has
-// bits for by trying all seeds.
+// instead of 4096.  One thread per slice does that much; slices that need larger sets are finished by the whole
+// warp: sets of three (which decide nearly all of them), then all 2^r sets in Gray-code order; slices with more
+// dependent rows than V has bits for by trying all seeds.
 //
 // Bound: integer instructions.  600 000 slices of 60 x 12 (20 % care bits): see the measured figure at the
 // launch below.
@@ -105,6 +105,21 @@ SQNN_DEV uint32_t try_all_sets(const unsigned long long *v, unsigned long long v
             if (i != 0) x ^= v[((uint32_t)__ffs((int)i) - 1u) * SEARCH_THREADS];
             const uint32_t wrong = size0 + (uint32_t)__popc(i ^ (i >> 1)) + (uint32_t)__popcll(x >> 20);
             best = min(best, (wrong << 20) | ((uint32_t)x & 0xfffffu));
+        }
+    }
+    return warp_min(best);
+}
+
+// The whole warp tries all sets of three wrong pivots: the lanes split the pairs, each walks the third.
+SQNN_DEV uint32_t try_triples(const unsigned long long *v, unsigned long long v0, uint32_t r, uint32_t lane)
+{
+    uint32_t best = 0xffffffffu;
+    for (uint32_t q = lane; q < r * (r - 1) / 2; q += 32) {
+        const uint32_t i = (uint32_t)((1.0f + sqrtf(1.0f + 8.0f * (float)q)) * 0.5f), h = q - i * (i - 1) / 2;     // h < i
+        const unsigned long long y = v0 ^ v[i * SEARCH_THREADS] ^ v[h * SEARCH_THREADS];
+        for (uint32_t g = 0; g < h; ++g) {
+            const unsigned long long x = y ^ v[g * SEARCH_THREADS];
+            best = min(best, ((3u + (uint32_t)__popcll(x >> 20)) << 20) | ((uint32_t)x & 0xfffffu));
         }
     }
     return warp_min(best);
@@ -217,20 +232,10 @@ k_search_seeds(const __grid_constant__ SearchArgs S)
                         best = min(best, ((2u + (uint32_t)__popcll(x >> 20)) << 20) | ((uint32_t)x & 0xfffffu));
                     }
                 }
-            // three by this thread alone where the whole warp would have far more than that to walk
-            if (r > 12 && (best >> 20) >= 3)
-                for (uint32_t i = 2; i < r; ++i)
-                    for (uint32_t h = 1; h < i; ++h) {
-                        const unsigned long long y = v0 ^ v[i * SEARCH_THREADS] ^ v[h * SEARCH_THREADS];
-                        for (uint32_t g = 0; g < h; ++g) {
-                            const unsigned long long x = y ^ v[g * SEARCH_THREADS];
-                            best = min(best, ((3u + (uint32_t)__popcll(x >> 20)) << 20) | ((uint32_t)x & 0xfffffu));
-                        }
-                    }
         }
         __syncwarp();
         // what is left for the whole warp: larger sets could still win or tie, or V has no room
-        uint32_t more = __ballot_sync(0xffffffffu, wide || (live && syn != 0 && (best >> 20) > (r > 12 ? 3u : 2u)));
+        uint32_t more = __ballot_sync(0xffffffffu, wide || (live && syn != 0 && (best >> 20) > 2u));
         while (more) {
             const uint32_t src = (uint32_t)__ffs((int)more) - 1u;
             more &= more - 1u;
@@ -241,7 +246,10 @@ k_search_seeds(const __grid_constant__ SearchArgs S)
                 for (int k = 0; k < NW; ++k) { w_s[k] = __shfl_sync(0xffffffffu, want[k], src); c_s[k] = __shfl_sync(0xffffffffu, care[k], src); }
                 found = try_all_seeds<NW>(cols, S.n_in, w_s, c_s, lane);
             } else {
-                found = try_all_sets(&v_s[0][(threadIdx.x & ~31u) + src], __shfl_sync(0xffffffffu, v0, src), __shfl_sync(0xffffffffu, r, src), lane);
+                const unsigned long long *v_src = &v_s[0][(threadIdx.x & ~31u) + src], v0_src = __shfl_sync(0xffffffffu, v0, src);
+                const uint32_t r_src = __shfl_sync(0xffffffffu, r, src);
+                found = min(__shfl_sync(0xffffffffu, best, src), try_triples(v_src, v0_src, r_src, lane));
+                if ((found >> 20) > 3u) found = try_all_sets(v_src, v0_src, r_src, lane);
             }
             if (lane == src) best = found;
         }
