@@ -15,7 +15,7 @@
 // all slices are done after sizes 0 (consistent: no wrong bit), 1 and 2: about 80 candidates for r = 12
 // instead of 4096.  One thread per slice does that much; slices that need larger sets are finished by the whole
 // warp: sets of three (which decide nearly all of them), then all 2^r sets in Gray-code order; slices with more
-// dependent rows than V has bits for by trying all seeds.
+// dependent rows than C has bits for by trying all seeds.
 //
 // Bound: integer instructions.  600 000 slices of 60 x 12 (20 % care bits): see the measured figure at the
 // launch below.
@@ -50,7 +50,7 @@ SQNN_DEV uint32_t bits32_at(const uint64_t *__restrict__ v, uint64_t p, uint64_t
 }
 
 constexpr uint32_t SEARCH_THREADS = 128;
-constexpr uint32_t MAX_DEP = 44;                          // dependent rows a 64-bit V has room for
+constexpr uint32_t MAX_DEP = 32;                          // dependent rows a word C has room for
 
 SQNN_DEV uint32_t warp_min(uint32_t v)
 {
@@ -90,53 +90,63 @@ SQNN_DEV uint32_t try_all_seeds(const uint32_t (*cols)[NW], uint32_t n_in, const
     return warp_min(best);
 }
 
-// The whole warp tries all 2^r sets of wrong pivots of one slice (v: its V_i, one every SEARCH_THREADS).
-SQNN_DEV uint32_t try_all_sets(const unsigned long long *v, unsigned long long v0, uint32_t r, uint32_t lane)
+// A candidate's key: number of wrong care bits, then the seed.
+SQNN_DEV uint32_t set_key(uint32_t size, uint32_t c, uint32_t q) { return ((size + (uint32_t)__popc(c)) << 20) + q; }
+
+// The whole warp tries all 2^r sets of wrong pivots of one slice (v: its (C_i, Q_i), one every SEARCH_THREADS).
+SQNN_DEV uint32_t try_all_sets(const uint2 *v, uint2 v0, uint32_t r, uint32_t lane)
 {
     const uint32_t low_bits = r > 5 ? r - 5 : 0, lanes_used = r >= 5 ? 32u : (1u << r);
     uint32_t best = 0xffffffffu;
     if (lane < lanes_used) {
         const uint32_t top = lane << low_bits, size0 = (uint32_t)__popc(lane);
-        unsigned long long x = v0;
+        uint32_t c = v0.x, q = v0.y;
         for (uint32_t t = low_bits; t < r; ++t)
-            if ((top >> t) & 1u) x ^= v[t * SEARCH_THREADS];
+            if ((top >> t) & 1u) { c ^= v[t * SEARCH_THREADS].x; q ^= v[t * SEARCH_THREADS].y; }
         const uint32_t count = 1u << low_bits;
         for (uint32_t i = 0; i < count; ++i) {
-            if (i != 0) x ^= v[((uint32_t)__ffs((int)i) - 1u) * SEARCH_THREADS];
-            const uint32_t wrong = size0 + (uint32_t)__popc(i ^ (i >> 1)) + (uint32_t)__popcll(x >> 20);
-            best = min(best, (wrong << 20) | ((uint32_t)x & 0xfffffu));
+            if (i != 0) {
+                const uint2 w = v[((uint32_t)__ffs((int)i) - 1u) * SEARCH_THREADS];
+                c ^= w.x;
+                q ^= w.y;
+            }
+            best = min(best, set_key(size0 + (uint32_t)__popc(i ^ (i >> 1)), c, q));
         }
     }
     return warp_min(best);
 }
 
 // The whole warp tries all sets of three wrong pivots: the lanes split the pairs, each walks the third.
-SQNN_DEV uint32_t try_triples(const unsigned long long *v, unsigned long long v0, uint32_t r, uint32_t lane)
+SQNN_DEV uint32_t try_triples(const uint2 *v, uint2 v0, uint32_t r, uint32_t lane)
 {
     uint32_t best = 0xffffffffu;
-    for (uint32_t q = lane; q < r * (r - 1) / 2; q += 32) {
-        const uint32_t i = (uint32_t)((1.0f + sqrtf(1.0f + 8.0f * (float)q)) * 0.5f), h = q - i * (i - 1) / 2;     // h < i
-        const unsigned long long y = v0 ^ v[i * SEARCH_THREADS] ^ v[h * SEARCH_THREADS];
+    for (uint32_t p = lane; p < r * (r - 1) / 2; p += 32) {
+        const uint32_t i = (uint32_t)((1.0f + sqrtf(1.0f + 8.0f * (float)p)) * 0.5f), h = p - i * (i - 1) / 2;     // h < i
+        const uint2 a = v[i * SEARCH_THREADS], b = v[h * SEARCH_THREADS];
+        const uint32_t c = v0.x ^ a.x ^ b.x, q = v0.y ^ a.y ^ b.y;
         for (uint32_t g = 0; g < h; ++g) {
-            const unsigned long long x = y ^ v[g * SEARCH_THREADS];
-            best = min(best, ((3u + (uint32_t)__popcll(x >> 20)) << 20) | ((uint32_t)x & 0xfffffu));
+            const uint2 w = v[g * SEARCH_THREADS];
+            best = min(best, set_key(3u, c ^ w.x, q ^ w.y));
         }
     }
     return warp_min(best);
 }
 
-// NI >= n_in: rows and bookkeeping of the elimination sit in registers, indexed by pivot column at compile time.
+// NI >= n_in.  Rows and bookkeeping of the elimination sit in registers; every loop over columns or pivots has a
+// fixed length, and a column without a pivot row or a pivot that does not exist is a zero that changes nothing
+// (a set with such a pivot only counts one error more than the set without it), so that the lanes of a warp,
+// which have different numbers of care bits and pivots, stay together.
 template <int NI, int NW>
 __global__ void __launch_bounds__(SEARCH_THREADS)
 k_search_seeds(const __grid_constant__ SearchArgs S)
 {
     __shared__ uint32_t rows_s[SQNN_MAX_N_OUT];
     __shared__ uint32_t cols[SQNN_MAX_N_IN][NW];                          // column t of M as an n_out-bit word
-    __shared__ unsigned long long v_s[NI][SEARCH_THREADS];
+    __shared__ uint2 v_s[NI][SEARCH_THREADS];
     wait_prior_grid();
     launch_dependents();
     const uint32_t lane = threadIdx.x & 31;
-    for (uint32_t j = threadIdx.x; j < S.n_out; j += SEARCH_THREADS) rows_s[j] = S.rows[j] & (uint32_t)((1ull << S.n_in) - 1ull);
+    for (uint32_t j = threadIdx.x; j < SQNN_MAX_N_OUT; j += SEARCH_THREADS) rows_s[j] = S.rows[j] & (uint32_t)((1ull << S.n_in) - 1ull);
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < S.n_in * NW; i += SEARCH_THREADS) {
         const uint32_t t = i / NW, k = i % NW;
@@ -145,7 +155,6 @@ k_search_seeds(const __grid_constant__ SearchArgs S)
         cols[t][k] = w;
     }
     __syncthreads();
-    unsigned long long *v = &v_s[0][threadIdx.x];
     const uint64_t total = S.slices * S.n_q;
     const uint64_t step = (uint64_t)gridDim.x * SEARCH_THREADS;
     for (uint64_t job0 = (uint64_t)blockIdx.x * SEARCH_THREADS + (threadIdx.x & ~31u); job0 < total; job0 += step) {
@@ -166,39 +175,39 @@ k_search_seeds(const __grid_constant__ SearchArgs S)
             }
         }
         // elimination: row[c] = the pivot row whose lowest set column is c, sub[c] = the original pivots it is the
-        // sum of (numbered as they come), bits = the original pivots' wanted bits
-        uint32_t row[NI], sub[NI], have = 0, bits = 0, r = 0, dep = 0;
-        unsigned long long syn = 0;
+        // sum of (numbered as they come), bits = the original pivots' wanted bits, dc[i] = C_i
+        uint32_t row[NI], sub[NI], dc[NI], bits = 0, r = 0, dep = 0, syn = 0;
 #pragma unroll
-        for (int c = 0; c < NI; ++c) { row[c] = sub[c] = 0; v[c * SEARCH_THREADS] = 0; }
+        for (int c = 0; c < NI; ++c) row[c] = sub[c] = dc[c] = 0;
 #pragma unroll
-        for (int k = 0; k < NW; ++k) {
-            uint32_t left = care[k];
+        for (int k = 0; k < NW; k += 2) {
+            unsigned long long left = care[k], wanted = want[k];
+            if (k + 1 < NW) {
+                left |= (unsigned long long)care[k + 1 < NW ? k + 1 : k] << 32;
+                wanted |= (unsigned long long)want[k + 1 < NW ? k + 1 : k] << 32;
+            }
             while (left) {
-                const uint32_t j = (uint32_t)__ffs((int)left) - 1u;
-                left &= left - 1u;
+                const uint32_t j = (uint32_t)__ffsll((long long)left) - 1u;
+                left &= left - 1ull;
                 uint32_t a = rows_s[32 * k + j], of = 0;
-                const uint32_t b = (want[k] >> j) & 1u;
+                const uint32_t b = (uint32_t)(wanted >> j) & 1u;
 #pragma unroll
-                for (int c = 0; c < NI; ++c) {
-                    const bool set = (a >> c) & 1u, pivot = (have >> c) & 1u;
-                    if (set && pivot) { a ^= row[c]; of ^= sub[c]; }
-                    if (set && !pivot) {                                  // a new pivot
-                        row[c] = a;
-                        sub[c] = of | (1u << r);
-                        have |= 1u << c;
-                        bits |= b << r;
-                        ++r;
-                        a = 0;
-                        of = 0x80000000u;
-                    }
-                }
-                if (!(of & 0x80000000u)) {                                // the sum of the pivots in `of`
-                    if (dep < MAX_DEP) {
-                        const unsigned long long bit = 1ull << (20 + dep);
-                        if ((b ^ (uint32_t)__popc(bits & of)) & 1u) syn |= bit;
-                        for (uint32_t o = of; o; o &= o - 1u) v[((uint32_t)__ffs((int)o) - 1u) * SEARCH_THREADS] |= bit;
-                    }
+                for (int c = 0; c < NI; ++c)
+                    if ((a >> c) & 1u) { a ^= row[c]; of ^= sub[c]; }
+                if (a) {                                                  // a new pivot
+                    const uint32_t low = a & (0u - a);
+                    of |= 1u << r;
+#pragma unroll
+                    for (int c = 0; c < NI; ++c)
+                        if (low == (1u << c)) { row[c] = a; sub[c] = of; }
+                    bits |= b << r;
+                    ++r;
+                } else {                                                  // the sum of the pivots in `of`
+                    const uint32_t bit = dep < MAX_DEP ? 1u << dep : 0u;
+                    if ((b ^ (uint32_t)__popc(bits & of)) & 1u) syn |= bit;
+#pragma unroll
+                    for (int i = 0; i < NI; ++i)
+                        if ((of >> i) & 1u) dc[i] |= bit;
                     ++dep;
                 }
             }
@@ -208,33 +217,37 @@ k_search_seeds(const __grid_constant__ SearchArgs S)
         for (int c = NI - 2; c >= 0; --c) {
 #pragma unroll
             for (int d = c + 1; d < NI; ++d)
-                if ((row[c] >> d) & (have >> d) & 1u) { row[c] ^= row[d]; sub[c] ^= sub[d]; }
+                if ((row[c] >> d) & 1u) { row[c] ^= row[d]; sub[c] ^= sub[d]; }
         }
         uint32_t seed = 0;
 #pragma unroll
         for (int c = 0; c < NI; ++c) seed |= ((uint32_t)__popc(bits & sub[c]) & 1u) << c;
-        const unsigned long long v0 = syn | seed;
-        uint32_t best = ((uint32_t)__popcll(syn) << 20) | seed;
+        uint32_t best = set_key(0u, syn, seed);
         const bool wide = live && dep > MAX_DEP;
         if (syn != 0 && !wide) {
+            uint32_t dq[NI];                                              // Q_i
 #pragma unroll
-            for (int c = 0; c < NI; ++c)
-                for (uint32_t o = sub[c]; o; o &= o - 1u) v[((uint32_t)__ffs((int)o) - 1u) * SEARCH_THREADS] |= 1ull << c;
-            for (uint32_t i = 0; i < r; ++i) {                            // one wrong pivot
-                const unsigned long long x = v0 ^ v[i * SEARCH_THREADS];
-                best = min(best, ((1u + (uint32_t)__popcll(x >> 20)) << 20) | ((uint32_t)x & 0xfffffu));
+            for (int i = 0; i < NI; ++i) {
+                dq[i] = 0;
+#pragma unroll
+                for (int c = 0; c < NI; ++c) dq[i] |= ((sub[c] >> i) & 1u) << c;
+                best = min(best, set_key(1u, syn ^ dc[i], seed ^ dq[i])); // one wrong pivot
             }
-            if ((best >> 20) >= 2)
-                for (uint32_t i = 1; i < r; ++i) {                        // two
-                    const unsigned long long y = v0 ^ v[i * SEARCH_THREADS];
-                    for (uint32_t h = 0; h < i; ++h) {
-                        const unsigned long long x = y ^ v[h * SEARCH_THREADS];
-                        best = min(best, ((2u + (uint32_t)__popcll(x >> 20)) << 20) | ((uint32_t)x & 0xfffffu));
-                    }
+            if ((best >> 20) >= 2) {
+#pragma unroll
+                for (int i = 1; i < NI; ++i) {                            // two
+                    const uint32_t c = syn ^ dc[i], q = seed ^ dq[i];
+#pragma unroll
+                    for (int h = 0; h < i; ++h) best = min(best, set_key(2u, c ^ dc[h], q ^ dq[h]));
                 }
+            }
+            if ((best >> 20) > 2u) {
+#pragma unroll
+                for (int i = 0; i < NI; ++i) v_s[i][threadIdx.x] = make_uint2(dc[i], dq[i]);
+            }
         }
         __syncwarp();
-        // what is left for the whole warp: larger sets could still win or tie, or V has no room
+        // what is left for the whole warp: larger sets could still win or tie, or C has no room
         uint32_t more = __ballot_sync(0xffffffffu, wide || (live && syn != 0 && (best >> 20) > 2u));
         while (more) {
             const uint32_t src = (uint32_t)__ffs((int)more) - 1u;
@@ -246,10 +259,11 @@ k_search_seeds(const __grid_constant__ SearchArgs S)
                 for (int k = 0; k < NW; ++k) { w_s[k] = __shfl_sync(0xffffffffu, want[k], src); c_s[k] = __shfl_sync(0xffffffffu, care[k], src); }
                 found = try_all_seeds<NW>(cols, S.n_in, w_s, c_s, lane);
             } else {
-                const unsigned long long *v_src = &v_s[0][(threadIdx.x & ~31u) + src], v0_src = __shfl_sync(0xffffffffu, v0, src);
+                const uint2 *v = &v_s[0][(threadIdx.x & ~31u) + src];
+                const uint2 v0 = make_uint2(__shfl_sync(0xffffffffu, syn, src), __shfl_sync(0xffffffffu, seed, src));
                 const uint32_t r_src = __shfl_sync(0xffffffffu, r, src);
-                found = min(__shfl_sync(0xffffffffu, best, src), try_triples(v_src, v0_src, r_src, lane));
-                if ((found >> 20) > 3u) found = try_all_sets(v_src, v0_src, r_src, lane);
+                found = min(__shfl_sync(0xffffffffu, best, src), try_triples(v, v0, r_src, lane));
+                if ((found >> 20) > 3u) found = try_all_sets(v, v0, r_src, lane);
             }
             if (lane == src) best = found;
         }
