@@ -37,10 +37,8 @@ UNIT = "weights/s"
 WORKLOAD = "alexnet-fc6 4096x9216, n_q=1, M 100x10, S=0.91, bf16 activations, batch 1"
 # DRAM bytes (read + write) of one launch, from one ncu capture of each kernel as it stands now on exactly
 # these workloads (summaries under profiles/).  An entry is None while its kernel has changed since the
-# counters were taken.  k_decode_gemv: 5.654 MB read, nothing written.  k_decode_bits at 2^30 weights,
-# 100x10, S = 0.90: 29.796 MB read + 74.684 MB written while the kernel ran; the other 59.5 MB of its
-# 134.2 MB of output were still in L2 when it ended and reach DRAM afterwards.
-NCU_DRAM_BYTES_PER_LAUNCH = {"k_decode_gemv": 5.654e6, "k_decode_bits": 104.48e6}
+# counters were taken.
+NCU_DRAM_BYTES_PER_LAUNCH = {"k_gemv_tc": None, "k_decode_bits": None}
 LANES_PER_SM = 128
 SMS = 148
 
@@ -365,8 +363,8 @@ def run_ours(args):
     alg_ops = layer.mn * layer.n_q + int(layer.mask.sum()) * layer.n_q
     alu_peak = SMS * LANES_PER_SM * peaks["sm_max_mhz"] * 1e6 / 1e12
     roofline = {"bound": "alu", "achieved": alg_ops / kern_s / 1e12, "peak": alu_peak, "unit": "Tlane-op/s",
-                "frac": alg_ops / kern_s / 1e12 / alu_peak, "traffic": NCU_DRAM_BYTES_PER_LAUNCH["k_decode_gemv"],
-                "kernel": "k_decode_gemv", "peak_source": f"148 SMs x 128 lanes x {peaks['sm_max_mhz']:.0f} MHz (max SM clock)",
+                "frac": alg_ops / kern_s / 1e12 / alu_peak, "traffic": NCU_DRAM_BYTES_PER_LAUNCH["k_gemv_tc"],
+                "kernel": "k_gemv_tc", "peak_source": f"148 SMs x 128 lanes x {peaks['sm_max_mhz']:.0f} MHz (max SM clock)",
                 "per_step_event_intervals_ms_median": float(np.median(times)),
                 "hbm_achieved_gbs": alg_bytes / kern_s / 1e9,
                 "hbm_frac_of_measured": alg_bytes / kern_s / 1e9 / peaks["hbm_gbs"],

@@ -30,7 +30,9 @@
  *    stay valid until the work queued on the stream has run.
  *  - Device entry points only queue work on the given CUDA stream (a cudaStream_t passed as
  *    void*, NULL = the legacy default stream) and do not synchronise.  They allocate no
- *    device memory and create no streams.
+ *    device memory and create no streams.  Their kernels are launched with programmatic stream
+ *    serialization: one may be set up while the kernel queued before it finishes, and waits for that
+ *    kernel before it touches anything that kernel may write.
  *  - Host buffers the library returns (blob, unpacked arrays) are released with sqnn_free.
  *  - d_status (device, one uint32, may be NULL) receives a sticky non-zero code when a
  *    kernel had to skip a malformed patch entry (1: position outside its tile, 2: a tile's
@@ -276,12 +278,14 @@ int sqnn_decode(const sqnn_desc *desc, const void *d_blob, const uint64_t *d_mas
  * SQNN_X_BF16), row stride ldx elements.  d_y: device fp32, batch rows of m, row stride ldy;
  * fully overwritten.
  *  - batch <= 15: one kernel; every block decodes the slices that cover its own rows into shared
- *    memory and accumulates in fp32 on the plain ALUs (weights exact).  Each Y[b][r] is summed in
- *    a fixed order, so results are bit-identical from run to run.  No workspace is used.  A row
- *    must fit shared memory as bits: n * (n_q + 1) <= 1 400 000, else UNSUPPORTED.
+ *    memory, expands them to bf16 signs and multiplies on the tensor cores with fp32 accumulation
+ *    (weights and F32 activations exact); rows too long for that are walked on the plain ALUs.
+ *    Each Y[b][r] is summed in a fixed order, so results are bit-identical from run to run.  No
+ *    workspace is used.  A row must fit shared memory as bits: n * (n_q + 1) <= 1 400 000, else
+ *    UNSUPPORTED.
  *  - batch >= 16: two kernels.  The decode kernel writes the planes as packed bits (1 bit per
- *    weight and plane) into d_workspace; the tcgen05 kernel reads boxes of them, expands them to
- *    bf16 tiles in shared memory and multiplies with fp32 accumulation in tensor memory.
+ *    weight and plane) into d_workspace; the tcgen05 kernel reads them, expands them to bf16 signs
+ *    in tensor memory and multiplies with fp32 accumulation there (weights exact).
  *    Activations must be BF16 with a 16-byte aligned base and a row pitch that is a multiple of
  *    16 bytes.  d_workspace: device scratch of at least sqnn_workspace_bytes(desc, batch) bytes,
  *    256-byte aligned, contents undefined before and after; required.  Column ranges handled by

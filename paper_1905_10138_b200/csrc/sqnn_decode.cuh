@@ -126,12 +126,6 @@ SQNN_DEV uint32_t settle(uint32_t v)
     return r;
 }
 
-// Flips one bit of a shared-memory word (address given as a 32-bit shared address).
-SQNN_DEV void smem_flip(uint32_t region_sa, uint32_t bit)
-{
-    asm volatile("red.shared.xor.b32 [%0], %1;\n" :: "r"(region_sa + ((bit >> 5) << 2)), "r"(1u << (bit & 31u)) : "memory");
-}
-
 // Starts the copy of the lookup tables from the blob into shared memory (all threads of the
 // block; one commit group).  Wait for the group and pass a block barrier before the first lookup.
 SQNN_DEV void tables_request(const DecodeArgs &A, uint32_t *tab_s)
