@@ -356,8 +356,8 @@ def run_ours(args):
     e2e = {"value": whole_job_rate(world, units, e2e_ms / args.steps), "unit": UNIT,
            "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h}
 
-    # roofline of the dominant kernel (fused decode-GEMV).  It is bound by plain ALU work: one
-    # table-driven expansion per weight bit plus one multiply-add per unpruned weight.
+    # roofline of the dominant kernel (fused decode-GEMV), against plain ALU work: one table-driven
+    # expansion per weight bit plus one multiply-add per unpruned weight.
     alg_bytes = stream_bytes(stats, layer, True) + layer.alpha.nbytes + x1.size * 2 + layer.m * 4
     kern_s = ms_per_step_local * 1e-3
     alg_ops = layer.mn * layer.n_q + int(layer.mask.sum()) * layer.n_q
@@ -417,7 +417,7 @@ def product_rows(torch, sqnn, layer, desc, d_blob, d_mask, d_alpha, status, flus
                "dense_bf16_hbm_floor_us": dense_floor_us,
                "fused_us_cold_l2": 1e3 * time_interval(torch, fused, reps, flush),
                "fused_us_warm_l2": 1e3 * time_interval(torch, fused, reps),
-               "path": "fp32 ALU (one kernel)" if batch <= 15 else "decode to packed bits + tcgen05 (two kernels)"}
+               "path": "tcgen05 (one kernel)" if batch <= 15 else "decode to packed bits + tcgen05 (two kernels)"}
         # the same four figures with the timed calls replayed from a CUDA graph (both sides alike)
         for key, f, fl in (("dense_bf16_us_cold_l2", dense, flush), ("dense_bf16_us_warm_l2", dense, None),
                            ("fused_us_cold_l2", fused, flush), ("fused_us_warm_l2", fused, None)):
