@@ -81,6 +81,20 @@ bool enough(Py_ssize_t nargs, Py_ssize_t want)
     return false;
 }
 
+// Other Python threads run while a C function is under way: a launch waits when the stream's queue is full, and in
+// checked mode the call waits for its stream.  Everything a call needs has been read out of its Python
+// arguments before; the caller's references keep them alive until it returns.
+class Unlocked {
+  public:
+    Unlocked() : state_(PyEval_SaveThread()) {}
+    ~Unlocked() { PyEval_RestoreThread(state_); }
+    Unlocked(const Unlocked &) = delete;
+    Unlocked &operator=(const Unlocked &) = delete;
+
+  private:
+    PyThreadState *state_;
+};
+
 // C++ exceptions of torch (a tensor without storage, for instance) must not cross into C.
 template <typename F>
 PyObject *guarded(F &&f)
@@ -107,8 +121,17 @@ PyObject *decode(PyObject *, PyObject *const *a, Py_ssize_t nargs)
             return nullptr;
         const long mode = PyLong_AsLong(a[4]);
         if (mode == -1 && PyErr_Occurred()) return nullptr;
-        return PyLong_FromLong(f_decode(d, ptr<void>(blob), ptr<uint64_t>(mask), ptr<float>(alpha), (sqnn_out_mode)mode,
-                                        ptr<void>(out), bytes_of(out), ptr<uint32_t>(status), st));
+        void *const p_blob = ptr<void>(blob), *const p_out = ptr<void>(out);
+        const uint64_t *const p_mask = ptr<uint64_t>(mask);
+        const float *const p_alpha = ptr<float>(alpha);
+        uint32_t *const p_status = ptr<uint32_t>(status);
+        const size_t out_bytes = bytes_of(out);
+        int rc;
+        {
+            Unlocked u;
+            rc = f_decode(d, p_blob, p_mask, p_alpha, (sqnn_out_mode)mode, p_out, out_bytes, p_status, st);
+        }
+        return PyLong_FromLong(rc);
     });
 }
 
@@ -118,6 +141,20 @@ bool product_shapes(const at::Tensor *x, const at::Tensor *y)
     PyErr_SetString(PyExc_ValueError, "X and Y must be 2-D with unit inner stride");
     return false;
 }
+
+// What both products take out of their tensors.
+struct Operands {
+    void *blob, *x;
+    uint64_t *mask;
+    float *alpha, *y;
+    uint32_t *status;
+    uint32_t batch;
+    int64_t ldx, ldy;
+    Operands(const at::Tensor *blob_, const at::Tensor *mask_, const at::Tensor *alpha_, const at::Tensor *x_, const at::Tensor *y_,
+             const at::Tensor *status_)
+        : blob(ptr<void>(blob_)), x(ptr<void>(x_)), mask(ptr<uint64_t>(mask_)), alpha(ptr<float>(alpha_)), y(ptr<float>(y_)),
+          status(ptr<uint32_t>(status_)), batch((uint32_t)x_->size(0)), ldx(x_->stride(0)), ldy(y_->stride(0)) {}
+};
 
 // matmul(desc, blob, mask, alpha, x, y, workspace, status, stream) -> status code
 PyObject *matmul(PyObject *, PyObject *const *a, Py_ssize_t nargs)
@@ -138,9 +175,15 @@ PyObject *matmul(PyObject *, PyObject *const *a, Py_ssize_t nargs)
         else { PyErr_SetString(PyExc_ValueError, "X must be float32 or bfloat16"); return nullptr; }
         if (y->scalar_type() != at::kFloat) { PyErr_SetString(PyExc_ValueError, "Y must be float32"); return nullptr; }
         if (!stream_arg(a[8], &st)) return nullptr;
-        return PyLong_FromLong(f_matmul(d, ptr<void>(blob), ptr<uint64_t>(mask), ptr<float>(alpha), ptr<void>(x), xdt,
-                                        (uint32_t)x->size(0), x->stride(0), ptr<float>(y), y->stride(0), ptr<void>(ws),
-                                        bytes_of(ws), ptr<uint32_t>(status), st));
+        const Operands o(blob, mask, alpha, x, y, status);
+        void *const p_ws = ptr<void>(ws);
+        const size_t ws_bytes = bytes_of(ws);
+        int rc;
+        {
+            Unlocked u;
+            rc = f_matmul(d, o.blob, o.mask, o.alpha, o.x, xdt, o.batch, o.ldx, o.y, o.ldy, p_ws, ws_bytes, o.status, st);
+        }
+        return PyLong_FromLong(rc);
     });
 }
 
@@ -161,9 +204,13 @@ PyObject *matmul_static(PyObject *, PyObject *const *a, Py_ssize_t nargs)
             return nullptr;
         }
         if (!stream_arg(a[7], &st)) return nullptr;
-        return PyLong_FromLong(f_matmul_static(d, ptr<void>(blob), ptr<uint64_t>(mask), ptr<float>(alpha), ptr<void>(x),
-                                               SQNN_X_BF16, (uint32_t)x->size(0), x->stride(0), ptr<float>(y),
-                                               y->stride(0), ptr<uint32_t>(status), st));
+        const Operands o(blob, mask, alpha, x, y, status);
+        int rc;
+        {
+            Unlocked u;
+            rc = f_matmul_static(d, o.blob, o.mask, o.alpha, o.x, SQNN_X_BF16, o.batch, o.ldx, o.y, o.ldy, o.status, st);
+        }
+        return PyLong_FromLong(rc);
     });
 }
 
