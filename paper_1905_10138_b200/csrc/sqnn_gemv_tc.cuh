@@ -184,14 +184,20 @@ k_gemv_tc(const TcArgs g)
     const uint64_t row0 = (uint64_t)blockIdx.x * g.rows_per_block;
     const uint64_t row_end = row0 + g.rows_per_block < g.m ? row0 + g.rows_per_block : g.m;
 
-    if (warp == nwarps - 1) tmem_alloc(&tmem_slot, 512);
+    // The block takes all tensor memory of its SM.  A block of the next grid does so too, and may become resident here
+    // as soon as this grid has let it in; if it got the columns first, it would hold them while it waits for this
+    // grid, which could then never end.  So the next grid is let in (a block counts as soon as one of its threads
+    // has) by the warp that allocates, after its allocation: then every block of this grid has its columns, and
+    // a later one's allocation waits until they are given back.
+    const bool holder = warp == nwarps - 1;
+    if (holder) tmem_alloc(&tmem_slot, 512);
     if (threadIdx.x == 0) {
         for (uint32_t i = 0; i < 3 * TC_GROUPS; ++i) mbar_init(bars_sa + 8 * i, 1);
         abort_word = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     wait_prior_grid();
-    launch_dependents();
+    if (holder) launch_dependents();
     uint32_t slot_seq = 0, parts_done = 0;                       // per group: A slots filled, accumulators read
     bool first = true;
 
@@ -385,7 +391,7 @@ k_gemv_tc(const TcArgs g)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == nwarps - 1) tmem_dealloc(tmem_slot, 512);
+    if (holder) tmem_dealloc(tmem_slot, 512);
 }
 
 // ------------------------------------------------------------------------------------------

@@ -203,7 +203,7 @@ k_decode_mma(const __grid_constant__ CUtensorMap xmap, const MmaArgs M)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_slot;
-    launch_dependents();
+    launch_dependents();                                     // after the allocation: see k_gemv_tc
 
     if (warp < 4 * groups) {
         // ------------------------------ expander groups ------------------------------

@@ -204,3 +204,51 @@ def test_a_bounded_wait_that_runs_out_reports_a_timeout_and_the_kernel_returns()
     torch.cuda.synchronize()
     assert dev.status_value() == 0
     assert H.rel_err(d_y.cpu().numpy(), ref) <= 2e-4
+
+
+def test_products_queued_back_to_back_and_from_two_threads():
+    """Consecutive kernels overlap (a grid is let in while the one before it runs) and both tensor-core kernels take
+    an SM's whole tensor memory.  Small and large batches and decodes are queued in turn without a pause, from
+    two threads with a stream each, so that grids of both streams meet on the SMs as well; every result is the one
+    that the same call gives alone."""
+    import threading
+    import torch
+    from paper_1905_10138_b200 import sqnn
+    jobs = []
+    for layer, batches in ((wl.make_layer(1), (1, 16)), (wl.make_layer(3, m=203, n=3000), (1, 8, 32)), (wl.make_layer(2, m=300, n=2048), (2, 64))):
+        layer.x_dtype = "bf16"
+        dev = H.DeviceLayer(layer, H.blob_from_library(layer)[0])
+        for batch in batches:
+            x = layer.activations(batch)
+            jobs.append((dev, torch.from_numpy(x).cuda().to(torch.bfloat16), dev.matmul(x, torch.bfloat16), batch))
+    failures = []
+
+    def worker(rounds):
+        try:
+            stream = torch.cuda.Stream()
+            ws = [torch.empty(max(sqnn.sqnn_workspace_bytes(d.desc, b), 256), dtype=torch.uint8, device="cuda") for d, _, _, b in jobs]
+            bits = [torch.empty(d.layer.n_q * d.words64, dtype=torch.int64, device="cuda") for d, _, _, _ in jobs]
+            ys = [[torch.empty((b, d.layer.m), device="cuda") for d, _, _, b in jobs] for _ in range(rounds)]
+            stream.wait_stream(torch.cuda.default_stream())
+            for r in range(rounds):
+                for i, (d, x, _, _) in enumerate(jobs):
+                    sqnn.sqnn_decode_matmul(d.desc, d.blob, d.mask, d.alpha, x, ys[r][i], ws[i], d.status, stream)
+                    if (r + i) % 3 == 0:
+                        sqnn.sqnn_decode(d.desc, d.blob, None, None, sqnn.OUT_BITS, bits[i], d.status, stream)
+            stream.synchronize()
+            for r in range(rounds):
+                for i, (_, _, want, batch) in enumerate(jobs):
+                    got = ys[r][i].cpu().numpy()
+                    # up to 15 vectors: a fixed order of summation; above: fp32 reductions in any order
+                    if not (np.array_equal(got, want) if batch <= 15 else H.rel_err(got, want) <= 2e-4):
+                        failures.append((r, i))
+        except Exception as e:                                   # noqa: BLE001 -- reported by the main thread
+            failures.append(repr(e))
+
+    threads = [threading.Thread(target=worker, args=(40,)) for _ in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failures, failures[:5]
+    assert all(d.status_value() == 0 for d, _, _, _ in jobs)
