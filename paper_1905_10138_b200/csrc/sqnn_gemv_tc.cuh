@@ -19,6 +19,14 @@
 // from different banks, whatever the row length.  Sums over the 8 ranges (shuffles) and the four groups (shared
 // memory) have a fixed order: results are bit-identical from run to run.
 //
+// Every wait on an mbarrier is bounded.  An expander warp whose wait gives up sets SQNN_E_TIMEOUT in the status word,
+// makes the arrivals its MMA warp still counts on and leaves its loop; the MMA warp reaches the end of its list, and
+// the block returns without storing this pass of Y, after a bounded wait for the MMAs it issued.  The barriers
+// between the two only count: an arrival for a slot's next use while another warp had not yet arrived for the one
+// before would complete the wrong one, and the MMA warp would wait for good; so the late arrivals follow the number
+// of slots the MMA warp has taken.  (mbarriers with bounded waits between the two would need no such care, but FC6
+// batch 1 takes 9.8 us with them against 9.5, 3001 x 4099 with four fp32 vectors 16.9 against 16.3.)
+//
 // Bound: integer instructions of the expansion (1.4 per weight and plane, against 42 per unpruned weight of the
 // walk over care bits in sqnn_gemv.cuh, 3.8 per weight at 9 % density) and the latency of the block's phases
 // (launch, staging, decode, product, reduction).
@@ -32,7 +40,7 @@ constexpr uint32_t TC_GROUPS = 4;                         // expander groups
 constexpr uint32_t TC_THREADS = TC_GROUPS * 128 + TC_GROUPS * 32;
 constexpr uint32_t TC_TILE_ROWS = 16, TC_RANGES = 8;
 constexpr uint32_t TC_MAX_Q = 12;                         // activation columns (vectors x pieces) per pass: N <= 96
-constexpr uint64_t TC_WAIT_LIMIT = 2000000000ull;         // about a second
+constexpr uint64_t TC_WAIT_LIMIT = 2000000000ull;         // cycles a bounded wait may take: about a second
 
 struct TcArgs {
     DecodeArgs A;
@@ -53,10 +61,23 @@ struct TcArgs {
     uint32_t slots;               // A slots (64 columns) per group: 1 or 2
     uint32_t alpha_words, part_words;
     uint32_t x_vec;               // rows of X start on 16-byte boundaries
+    uint32_t skip_mma;            // test only: the MMA warps issue nothing
+    uint64_t wait_limit;          // cycles a bounded wait may take
 };
 
 SQNN_DEV void named_arrive(uint32_t id) { asm volatile("bar.arrive %0, 160;\n" :: "r"(id) : "memory"); }
 SQNN_DEV void named_sync(uint32_t id) { asm volatile("bar.sync %0, 160;\n" :: "r"(id) : "memory"); }
+// The arrivals of a warp that has given up, for slots [from, to) of its group: each once the MMA warp has taken the
+// use before it of the same barrier (it waits for nothing but these arrivals; bounded all the same).
+static __device__ __noinline__ void arrive_for_the_rest(const volatile uint32_t *taken, uint32_t barrier, uint32_t slot_mask, uint32_t from, uint32_t to, uint64_t limit)
+{
+    const long long t0 = clock64();
+    for (; from != to; ++from) {
+        while ((int32_t)(*taken - (from - slot_mask)) < 0 && (uint64_t)(clock64() - t0) <= limit) {}
+        __syncwarp();
+        named_arrive(barrier + (from & slot_mask));
+    }
+}
 
 // 128 columns of one row from bit `o` of a packed vector in shared memory (address sa, 16-byte aligned).
 template <bool ALIGNED>
@@ -163,7 +184,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 k_gemv_tc(const TcArgs g)
 {
     extern __shared__ __align__(16) uint32_t smem[];
-    __shared__ uint64_t bars[3 * TC_GROUPS];              // per group: two A slots free, accumulator complete
+    __shared__ uint64_t bars[4 * TC_GROUPS];              // per group: two A slots free, accumulator complete; all MMAs over (after a timeout)
+    __shared__ volatile uint32_t taken_s[TC_GROUPS];      // A slots the group's MMA warp has taken
     __shared__ uint32_t tmem_slot, abort_word;
     constexpr uint32_t PIECES = sizeof(XT) == 4 ? 3 : 1;
     const DecodeArgs &A = g.A;
@@ -192,7 +214,8 @@ k_gemv_tc(const TcArgs g)
     const bool holder = warp == nwarps - 1;
     if (holder) tmem_alloc(&tmem_slot, 512);
     if (threadIdx.x == 0) {
-        for (uint32_t i = 0; i < 3 * TC_GROUPS; ++i) mbar_init(bars_sa + 8 * i, 1);
+        for (uint32_t i = 0; i < 4 * TC_GROUPS; ++i) mbar_init(bars_sa + 8 * i, 1);
+        for (uint32_t i = 0; i < TC_GROUPS; ++i) taken_s[i] = 0;
         abort_word = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
@@ -289,6 +312,7 @@ k_gemv_tc(const TcArgs g)
             if (warp < 4 * TC_GROUPS) {
                 const uint32_t quad = warp & 3, kq = lane & 7, lane_sel = (quad * 32) << 16;
                 const uint32_t mask_sa = smem_addr(mask_s), bits_sa = smem_addr(bits_s);
+                const uint32_t seq_end = slot_seq + 2 * (u_end - u_begin);
                 float acc[TC_MAX_Q];
 #pragma unroll
                 for (uint32_t q = 0; q < TC_MAX_Q; ++q) acc[q] = 0.0f;
@@ -309,7 +333,10 @@ k_gemv_tc(const TcArgs g)
                             expand32(mw[2 * h + 1], bw[2 * h + 1], v + 16);
                             const uint32_t slot = slot_seq & slot_mask, use = slot_seq >> slot_shift;
                             if (use > 0) {
-                                mbar_wait_warp(free_a + 8 * slot, (use - 1) & 1u, abort_flag, A.status, TC_WAIT_LIMIT);
+                                if (!mbar_wait_warp(free_a + 8 * slot, (use - 1) & 1u, abort_flag, A.status, g.wait_limit)) {
+                                    arrive_for_the_rest(taken_s + grp, 1 + 2 * grp, slot_mask, slot_seq, seq_end, g.wait_limit);
+                                    goto pass_over;
+                                }
                                 tc_fence_after();
                             }
                             tmem_st16(a_tmem + lane_sel + slot * 32, v);
@@ -322,7 +349,10 @@ k_gemv_tc(const TcArgs g)
                     u += len;
                     // the part's accumulator: this lane's range, scaled
                     const float al = 0.5f * alpha_s[rl * n_q + pl];
-                    mbar_wait_warp(done, parts_done & 1u, abort_flag, A.status, TC_WAIT_LIMIT);
+                    if (!mbar_wait_warp(done, parts_done & 1u, abort_flag, A.status, g.wait_limit)) {
+                        arrive_for_the_rest(taken_s + grp, 1 + 2 * grp, slot_mask, slot_seq, seq_end, g.wait_limit);
+                        goto pass_over;
+                    }
                     ++parts_done;
                     tc_fence_after();
 #pragma unroll
@@ -362,12 +392,20 @@ k_gemv_tc(const TcArgs g)
                 const uint32_t idesc = instr_desc_bf16(g.N);
                 const uint64_t x_desc0 = smem_desc_sw128(x_sa);
                 const uint32_t box_step = g.N * 128 >> 4;
-                for (uint32_t u = u_begin; u < u_end;) {
+                if (g.skip_mma) {
+                    for (uint32_t k = 0; k < 2 * (u_end - u_begin); ++k) {
+                        named_sync(1 + 2 * grp + (slot_seq & slot_mask));
+                        ++slot_seq;
+                        if (lane == 0) taken_s[grp] = slot_seq;
+                    }
+                }
+                for (uint32_t u = g.skip_mma ? u_end : u_begin; u < u_end;) {
                     const uint32_t it = u / g.units, t0 = u - it * g.units;
                     const uint32_t len = min(g.units - t0, u_end - u);
                     for (uint32_t k = 0; k < 2 * len; ++k, ++slot_seq) {
                         const uint32_t slot = slot_seq & slot_mask;
                         named_sync(1 + 2 * grp + slot);
+                        if (lane == 0) taken_s[grp] = slot_seq + 1;
                         tc_fence_after();
                         mma_slot<4>(d_tmem, a_tmem + slot * 32, x_desc0 + (2 * t0 + k) * box_step, idesc, k, free_a + 8 * slot, 0);
                     }
@@ -375,7 +413,9 @@ k_gemv_tc(const TcArgs g)
                     u += len;
                 }
             }
+        pass_over:
             __syncthreads();
+            const uint32_t gave_up = *abort_flag;                // (no role sets it between this barrier and the next)
             for (uint32_t q = warp; q < g.bt && bc + q < g.batch; q += nwarps)
                 for (uint32_t rl = lane; rl < nrows; rl += 32) {
                     float sum = 0.0f;
@@ -384,9 +424,16 @@ k_gemv_tc(const TcArgs g)
                     if ((__float_as_uint(sum) & 0x7f800000u) == 0x7f800000u)
                         sum = tc_walk<XT>(g, reinterpret_cast<const XT *>(g.x) + (int64_t)(bc + q) * g.ldx, mask_s, bits_s,
                                           alpha_s + rl * n_q, (uint32_t)((ra + rl) * n - gw0 * 32));
-                    g.y[(int64_t)(bc + q) * g.ldy + (int64_t)(ra + rl)] = sum;
+                    if (!gave_up) g.y[(int64_t)(bc + q) * g.ldy + (int64_t)(ra + rl)] = sum;
                 }
+            if (gave_up) goto leave;
         }
+    }
+leave:
+    if (*abort_flag && warp >= 4 * TC_GROUPS) {                  // tensor and shared memory must outlive the MMAs
+        const uint32_t over = bars_sa + 8 * (3 * TC_GROUPS + warp - 4 * TC_GROUPS);
+        mma_commit(over);
+        mbar_drain(over, 0, g.wait_limit);
     }
     tc_fence_before();
     __syncthreads();
@@ -447,6 +494,9 @@ inline int launch_gemv_tc(const DecodeArgs &A, const uint64_t *d_mask, const flo
             if (RC <= 8) break;
         }
     }
+    const DebugKnobs dbg = debug_knobs();
+    g.skip_mma = (dbg.flags & 2u) ? 1u : 0u;
+    g.wait_limit = dbg.wait_cycles ? dbg.wait_cycles : TC_WAIT_LIMIT;
     g.x_vec = (((uintptr_t)d_x & 15) == 0 && (ldx * (int64_t)sizeof(XT)) % 16 == 0) ? 1u : 0u;
     return n % 128 == 0 ? launch_kernel(k_gemv_tc<N_OUT, N_IN, XT, true>, (uint32_t)grid, TC_THREADS, smem, st, g)
                         : launch_kernel(k_gemv_tc<N_OUT, N_IN, XT, false>, (uint32_t)grid, TC_THREADS, smem, st, g);

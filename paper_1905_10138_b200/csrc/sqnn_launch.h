@@ -32,6 +32,13 @@ inline int launch_kernel(void (*kernel)(P...), uint32_t grid, uint32_t threads, 
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...) == cudaSuccess ? SQNN_OK : SQNN_E_CUDA;
 }
+// What sqnn_set_debug_flags was given last (zeros in normal use).
+struct DebugKnobs {
+    uint32_t flags;
+    uint64_t wait_cycles;
+};
+DebugKnobs debug_knobs();
+
 size_t mma_workspace_bytes(const sqnn_desc *desc, uint32_t batch);
 int mma_dispatch(const sqnn_desc *desc, const DecodeArgs &A, const uint64_t *d_mask, const float *d_alpha,
                  const void *d_x, int64_t ldx, uint32_t batch, float *d_y, int64_t ldy, void *d_workspace,

@@ -390,6 +390,8 @@ EncodeTiledFn encode_tiled_fn()
 
 }  // namespace
 
+DebugKnobs debug_knobs() { return DebugKnobs{g_debug_flags.load(), g_debug_wait_cycles.load()}; }
+
 // Workspace of the two-stage form: the decoded planes as packed bits (1 bit per weight and plane).
 size_t mma_workspace_bytes(const sqnn_desc *desc, uint32_t)
 {
@@ -418,9 +420,9 @@ int mma_dispatch(const sqnn_desc *desc, const DecodeArgs &A0, const uint64_t *d_
     M.n_q = desc->n_q;
     M.batch = batch;
     M.status = A0.status;
-    const uint32_t dbg = g_debug_flags.load();
-    M.skip_loads = (dbg & 1u) ? 1u : 0u;
-    M.wait_limit = g_debug_wait_cycles.load() ? g_debug_wait_cycles.load() : WAIT_LIMIT_CYCLES;
+    const DebugKnobs dbg = debug_knobs();
+    M.skip_loads = (dbg.flags & 1u) ? 1u : 0u;
+    M.wait_limit = dbg.wait_cycles ? dbg.wait_cycles : WAIT_LIMIT_CYCLES;
 
     // Units of a tile: all planes of 128 rows share the activation tile, up to four; more planes are taken in equal
     // groups.  (One plane with 256 rows per tile uses an activation tile twice but cuts the columns into twice as
@@ -472,9 +474,9 @@ int mma_dispatch(const sqnn_desc *desc, const DecodeArgs &A0, const uint64_t *d_
 
 }  // namespace sqnn
 
-// For the library's own tests: bit 0 of `flags` makes the tensor-core kernel's loader issue no loads, so that
-// the bounded waits of its consumers run out; wait_limit_cycles (0 = default, about 2 s) is the number of
-// clock cycles such a wait may take.  Affects calls made after it; not meant for applications.
+// For the library's own tests: bit 0 of `flags` makes the large-batch kernel's loader issue no loads, bit 1 the
+// small-batch kernel's MMA warps no MMAs, so that the bounded waits of the roles behind them run out;
+// wait_limit_cycles (0 = the kernel's default, one or two seconds) is the number of clock cycles such a wait may take.  Affects calls made after it; not meant for applications.
 extern "C" void sqnn_set_debug_flags(uint32_t flags, uint64_t wait_limit_cycles)
 {
     sqnn::g_debug_flags.store(flags);

@@ -206,6 +206,36 @@ def test_a_bounded_wait_that_runs_out_reports_a_timeout_and_the_kernel_returns()
     assert H.rel_err(d_y.cpu().numpy(), ref) <= 2e-4
 
 
+@pytest.mark.parametrize("dtype,batch", [("bf16", 1), ("bf16", 15), ("f32", 9)])      # one, two and three passes
+def test_a_bounded_wait_of_the_small_batch_kernel_that_runs_out_reports_a_timeout(dtype, batch):
+    """With the library's test knob the MMA warps issue nothing: slots are never freed and accumulators never complete,
+    the expanders' waits run out after about a millisecond, the kernel reports 6 (-SQNN_E_TIMEOUT), stores no
+    result and returns; the same call made normally right afterwards is correct."""
+    import torch
+    from paper_1905_10138_b200 import sqnn
+    layer = wl.make_layer(3, m=700, n=3000)                             # several slots and parts per group
+    layer.x_dtype = dtype
+    x = layer.activations(batch)
+    ref = reference(layer, x)
+    dev = H.DeviceLayer(layer, H.blob_from_library(layer)[0])
+    d_x = torch.from_numpy(x).cuda().to(torch.float32 if dtype == "f32" else torch.bfloat16)
+    d_y = torch.full((batch, layer.m), float("nan"), dtype=torch.float32, device="cuda")
+    call = lambda: sqnn.sqnn_decode_matmul(dev.desc, dev.blob, dev.mask, dev.alpha, d_x, d_y, None, dev.status)
+    try:
+        sqnn.sqnn_set_debug_flags(2, 2_000_000)
+        call()
+        torch.cuda.synchronize()
+        assert dev.status_value() == -sqnn.E_TIMEOUT
+        assert torch.isnan(d_y).all()
+    finally:
+        sqnn.sqnn_set_debug_flags(0, 0)
+    dev.status.zero_()
+    call()
+    torch.cuda.synchronize()
+    assert dev.status_value() == 0
+    assert H.rel_err(d_y.cpu().numpy(), ref) <= TOL_F32
+
+
 def test_products_queued_back_to_back_and_from_two_threads():
     """Consecutive kernels overlap (a grid is let in while the one before it runs) and both tensor-core kernels take
     an SM's whole tensor memory.  Small and large batches and decodes are queued in turn without a pause, from
