@@ -15,8 +15,9 @@
 // xs[c][BT].  Rows that do not fit shared memory at once are taken in chunks.
 // With one activation vector and 16-byte aligned operands the tables, the activations and the mask
 // range of a block's first chunk are fetched by three bulk copies (cp.async.bulk, completion on an
-// mbarrier, bounded wait) that thread 0 issues at kernel entry; otherwise by cp.async from every
-// thread.
+// mbarrier) that thread 0 issues at kernel entry; otherwise by cp.async from every thread.  The wait
+// for those copies is bounded; a block whose wait gives up reports SQNN_E_TIMEOUT, waits once more for
+// what may be in flight and returns without storing its rows of Y.
 #pragma once
 #include "sqnn_kernels.cuh"
 
@@ -37,7 +38,10 @@ struct GemvArgs {
     uint32_t region_words;        // words of one bit vector of a chunk in shared memory (whole kernel tiles)
     uint32_t alpha_words, part_words, xs_words;
     uint32_t bulk_stage;          // tables, activations and mask may be staged by bulk copies (sizes and alignment allow it)
+    uint32_t skip_stage;          // test only: no bulk copy is issued
+    uint64_t wait_limit;          // cycles the wait for them may take
 };
+constexpr uint64_t GEMV_WAIT_LIMIT = 2000000000ull;       // about a second
 
 // One-dimensional bulk copy global -> shared by the copy engine, completion counted in bytes on an
 // mbarrier; both addresses 16-byte aligned, size a multiple of 16.
@@ -56,8 +60,8 @@ SQNN_DEV void bulk_load(void *sdst, const void *gsrc, uint32_t bytes, uint64_t *
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
                  :: "r"(smem_addr(sdst)), "l"(gsrc), "r"(bytes), "r"(smem_addr(bar)) : "memory");
 }
-// Waits for phase 0 of the barrier, for about a second at most; false if it gave up.
-SQNN_DEV bool stage_bar_wait(uint64_t *bar)
+// Waits for phase 0 of the barrier, `limit` cycles at most; false if it gave up.
+SQNN_DEV bool stage_bar_wait(uint64_t *bar, uint64_t limit)
 {
     const long long t0 = clock64();
     for (;;) {
@@ -65,7 +69,7 @@ SQNN_DEV bool stage_bar_wait(uint64_t *bar)
         asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0, %2;\n selp.u32 %0, 1, 0, p;\n}\n"
                      : "=r"(ok) : "r"(smem_addr(bar)), "r"(1000000u) : "memory");
         if (ok) return true;
-        if (clock64() - t0 > 2000000000ll) return false;
+        if ((uint64_t)(clock64() - t0) > limit) return false;
     }
 }
 
@@ -164,6 +168,7 @@ k_decode_gemv(const GemvArgs g)
     // block's first chunk -- tables, activations, mask -- to the copy engine at once, before anything else
     // runs; otherwise every thread requests its share by cp.async (three commit groups, as below).
     __shared__ uint64_t stage_bar;
+    __shared__ volatile uint32_t stage_late;                     // a thread's wait for the copies has given up
     bool bulk = false;
     if constexpr (XS && BT == 1) {
         const uint64_t tile_bits = 32ull * TW;
@@ -172,13 +177,23 @@ k_decode_gemv(const GemvArgs g)
         bulk = g.bulk_stage && row0 < row_end && k1 * TW <= g.mask_words;      // the mask range lies inside the array
         if (bulk && threadIdx.x == 0) {
             const uint32_t tab_bytes = A.tab_words * 4, x_bytes = n * (uint32_t)sizeof(XT), mask_bytes = (uint32_t)(k1 - k0) * TW * 4;
+            stage_late = 0;
             stage_bar_init(&stage_bar);
             stage_bar_expect(&stage_bar, tab_bytes + x_bytes + mask_bytes);
-            bulk_load(tab_s, A.tab, tab_bytes, &stage_bar);
-            bulk_load(xs, x, x_bytes, &stage_bar);
-            bulk_load(mask_s, g.mask32 + k0 * TW, mask_bytes, &stage_bar);
+            if (!g.skip_stage) {
+                bulk_load(tab_s, A.tab, tab_bytes, &stage_bar);
+                bulk_load(xs, x, x_bytes, &stage_bar);
+                bulk_load(mask_s, g.mask32 + k0 * TW, mask_bytes, &stage_bar);
+            }
         }
     }
+    auto bulk_ready = [&] {
+        __syncthreads();                                         // the barrier's initialisation is visible to all
+        if (!stage_bar_wait(&stage_bar, g.wait_limit)) {
+            flag(A.status, (uint32_t)(-SQNN_E_TIMEOUT));
+            stage_late = 1;
+        }
+    };
     if (!bulk) {
         tables_request(A, tab_s);                                // commit group: tables
         stage_x(0);                                              // commit group: activations
@@ -217,8 +232,7 @@ k_decode_gemv(const GemvArgs g)
             if (item < items) fetch(item);
             if (ra == row0) {
                 if (bulk) {
-                    __syncthreads();                             // the barrier's initialisation is visible to all
-                    if (!stage_bar_wait(&stage_bar)) flag(A.status, (uint32_t)(-SQNN_E_TIMEOUT));
+                    bulk_ready();
                 } else {
                     cp_async_wait_group<2>();                    // tables (the two younger groups may be pending)
                     __syncthreads();
@@ -236,8 +250,7 @@ k_decode_gemv(const GemvArgs g)
         } else {
             if (ra == row0) {
                 if (bulk) {
-                    __syncthreads();
-                    if (!stage_bar_wait(&stage_bar)) flag(A.status, (uint32_t)(-SQNN_E_TIMEOUT));
+                    bulk_ready();
                 } else {
                     cp_async_wait_group<2>();
                     __syncthreads();
@@ -250,6 +263,10 @@ k_decode_gemv(const GemvArgs g)
         }
         cp_async_wait_all();
         __syncthreads();                                         // bits, mask, scales, activations in place
+        if (bulk && stage_late) {                                // (the same for all threads: it was set before the barrier)
+            stage_bar_wait(&stage_bar, g.wait_limit);            // shared memory must outlive the copies
+            return;
+        }
 
         const uint32_t nitems = nrows * P;
         for (uint32_t bc = 0; bc < g.batch; bc += BT) {
@@ -423,6 +440,9 @@ inline int launch_gemv_bt(const DecodeArgs &A, const uint64_t *d_mask, const flo
     g.bulk_stage = (BT == 1 && xs && ((uintptr_t)d_x & 15) == 0 && (n * sizeof(XT)) % 16 == 0 &&
                     ((uintptr_t)d_mask & 15) == 0 && ((uintptr_t)A.tab & 15) == 0 && (tab + 0) % 16 == 0 &&
                     (size_t)g.region_words * 4 < (1u << 20)) ? 1u : 0u;
+    const DebugKnobs dbg = debug_knobs();
+    g.skip_stage = (dbg.flags & 4u) ? 1u : 0u;
+    g.wait_limit = dbg.wait_cycles ? dbg.wait_cycles : GEMV_WAIT_LIMIT;
 #define SQNN_GEMV_LAUNCH(XSV, NQV)                                                                       \
     do {                                                                                                 \
         return launch_kernel(k_decode_gemv<N_OUT, N_IN, BT, XT, XSV, NQV>, (uint32_t)grid, nwarps * 32, smem, st, g); \

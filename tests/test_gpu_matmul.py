@@ -236,6 +236,34 @@ def test_a_bounded_wait_of_the_small_batch_kernel_that_runs_out_reports_a_timeou
     assert H.rel_err(d_y.cpu().numpy(), ref) <= TOL_F32
 
 
+def test_the_wait_of_the_walk_for_its_staged_operands_runs_out():
+    """The same for the walk over care bits (rows too long for the tensor-core form), whose blocks wait for bulk copies of
+    their operands: blocks that gave up report it and store nothing."""
+    import torch
+    from paper_1905_10138_b200 import sqnn
+    layer = generic_layer(100, 10, 6, 48000, 0.1, 61)
+    layer.x_dtype = "bf16"
+    x = layer.activations(1)
+    ref = reference(layer, x)
+    dev = H.DeviceLayer(layer, H.blob_from_library(layer)[0])
+    d_x = torch.from_numpy(x).cuda().to(torch.bfloat16)
+    d_y = torch.full((1, layer.m), float("nan"), dtype=torch.float32, device="cuda")
+    call = lambda: sqnn.sqnn_decode_matmul(dev.desc, dev.blob, dev.mask, dev.alpha, d_x, d_y, None, dev.status)
+    try:
+        sqnn.sqnn_set_debug_flags(4, 2_000_000)
+        call()
+        torch.cuda.synchronize()
+        assert dev.status_value() == -sqnn.E_TIMEOUT
+        assert torch.isnan(d_y[0, :-1]).all()                           # (the last block's mask range ends past the array: no bulk copies)
+    finally:
+        sqnn.sqnn_set_debug_flags(0, 0)
+    dev.status.zero_()
+    call()
+    torch.cuda.synchronize()
+    assert dev.status_value() == 0
+    assert H.rel_err(d_y.cpu().numpy(), ref) <= TOL_F32
+
+
 def test_products_queued_back_to_back_and_from_two_threads():
     """Consecutive kernels overlap (a grid is let in while the one before it runs) and both tensor-core kernels take
     an SM's whole tensor memory.  Small and large batches and decodes are queued in turn without a pause, from
