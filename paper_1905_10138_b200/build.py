@@ -6,6 +6,7 @@ import os
 import subprocess
 import sys
 import sysconfig
+from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
@@ -64,23 +65,16 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if verbose:
         common += ["-Xptxas", "-v"]
     jobs = []
+    for no, ni in reversed(SHAPES):               # the longest first
+        for part in (2, 1, 0):
+            jobs.append(([f"-DSQNN_NO={no}", f"-DSQNN_NI={ni}", f"-DSQNN_PART={part}", os.path.join(CSRC, SHAPE_SOURCE)],
+                         os.path.join(objdir, f"sqnn_shape_{no}x{ni}_{part}.o")))
     for s in SOURCES:
         jobs.append(([os.path.join(CSRC, s)], os.path.join(objdir, os.path.splitext(s)[0] + ".o")))
-    for no, ni in SHAPES:
-        jobs.append(([f"-DSQNN_NO={no}", f"-DSQNN_NI={ni}", os.path.join(CSRC, SHAPE_SOURCE)],
-                     os.path.join(objdir, f"sqnn_shape_{no}x{ni}.o")))
     objs = [o for _, o in jobs]
-    width = max(1, min(len(jobs), os.cpu_count() or 4))
-    pending, running = list(jobs), []
-    while pending or running:
-        while pending and len(running) < width:
-            extra, o = pending.pop(0)
-            running.append(subprocess.Popen([_nvcc(), *common, "-c", *extra, "-o", o]))
-        if running[0].wait() != 0:
-            for r in running[1:]:
-                r.wait()
-            raise RuntimeError("nvcc failed")
-        running.pop(0)
+    with ThreadPoolExecutor(max(1, min(len(jobs), os.cpu_count() or 4))) as pool:
+        for _ in pool.map(lambda j: subprocess.run([_nvcc(), *common, "-c", *j[0], "-o", j[1]], check=True), jobs):
+            pass
     subprocess.run([_nvcc(), "-shared", "-o", LIB, *objs, "-Xcompiler", "-fopenmp", "-lgomp"], check=True)
     return LIB
 

@@ -1,13 +1,19 @@
-// Instantiates the decode and GEMV kernels for one network shape (N_OUT x N_IN given by
-// -DSQNN_NO / -DSQNN_NI; 0 x 0 is the run-time-shape fallback).
+// Instantiates the kernels of one network shape (N_OUT x N_IN given by -DSQNN_NO / -DSQNN_NI; 0 x 0 is the
+// run-time-shape fallback).  -DSQNN_PART compiles one part of them, so that the parts of a shape build side by side:
+// 0 the decode, 1 the small-batch tensor-core product, 2 the walk over care bits and the choice between the two.
 #include "sqnn_gemv_tc.cuh"
 
 #ifndef SQNN_NO
 #error "compile with -DSQNN_NO=<n_out> -DSQNN_NI=<n_in>"
 #endif
 
+#ifndef SQNN_PART
+#error "compile with -DSQNN_PART=<0, 1 or 2>"
+#endif
+
 namespace sqnn {
 
+#if SQNN_PART == 0
 template <>
 int decode_shape<SQNN_NO, SQNN_NI>(const DecodeArgs &A, sqnn_out_mode mode, const uint64_t *d_mask,
                                    const float *d_alpha, uint64_t n, void *d_out, const ClearArgs &clear,
@@ -16,18 +22,38 @@ int decode_shape<SQNN_NO, SQNN_NI>(const DecodeArgs &A, sqnn_out_mode mode, cons
     return launch_decode<SQNN_NO, SQNN_NI>(A, mode, d_mask, d_alpha, n, d_out, clear, st);
 }
 
+#else
+// the tensor-core product; SQNN_E_UNSUPPORTED: not the form to take
+template <int N_OUT, int N_IN>
+int gemv_tc_shape(const DecodeArgs &A, const uint64_t *d_mask, const float *d_alpha, const void *d_x, int x_dtype,
+                  int64_t ldx, uint32_t batch, float *d_y, int64_t ldy, uint64_t m, uint64_t n, cudaStream_t st);
+#if SQNN_PART == 1
+template <>
+int gemv_tc_shape<SQNN_NO, SQNN_NI>(const DecodeArgs &A, const uint64_t *d_mask, const float *d_alpha,
+                                    const void *d_x, int x_dtype, int64_t ldx, uint32_t batch, float *d_y,
+                                    int64_t ldy, uint64_t m, uint64_t n, cudaStream_t st)
+{
+    return x_dtype == SQNN_X_BF16
+        ? launch_gemv_tc<SQNN_NO, SQNN_NI, __nv_bfloat16>(A, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st)
+        : launch_gemv_tc<SQNN_NO, SQNN_NI, float>(A, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st);
+}
+#else
+template <>
+int gemv_tc_shape<SQNN_NO, SQNN_NI>(const DecodeArgs &, const uint64_t *, const float *, const void *, int, int64_t, uint32_t,
+                                    float *, int64_t, uint64_t, uint64_t, cudaStream_t);
+
 template <>
 int gemv_shape<SQNN_NO, SQNN_NI>(const DecodeArgs &A, const uint64_t *d_mask, const float *d_alpha,
                                  const void *d_x, int x_dtype, int64_t ldx, uint32_t batch, float *d_y,
                                  int64_t ldy, uint64_t m, uint64_t n, cudaStream_t st)
 {
-    const int rc = x_dtype == SQNN_X_BF16
-        ? launch_gemv_tc<SQNN_NO, SQNN_NI, __nv_bfloat16>(A, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st)
-        : launch_gemv_tc<SQNN_NO, SQNN_NI, float>(A, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st);
+    const int rc = gemv_tc_shape<SQNN_NO, SQNN_NI>(A, d_mask, d_alpha, d_x, x_dtype, ldx, batch, d_y, ldy, m, n, st);
     if (rc != SQNN_E_UNSUPPORTED) return rc;
     return x_dtype == SQNN_X_BF16
         ? launch_gemv<SQNN_NO, SQNN_NI, __nv_bfloat16>(A, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st)
         : launch_gemv<SQNN_NO, SQNN_NI, float>(A, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st);
 }
+#endif
+#endif
 
 }  // namespace sqnn
