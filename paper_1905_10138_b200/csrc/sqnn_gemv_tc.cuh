@@ -15,8 +15,12 @@
 //     a row and plane is applied to the accumulator, so weights are exact.  fp32 activations enter as three bf16
 //     pieces that add up to them exactly (8 + 8 + 8 bits).
 //
-// Kq is an odd multiple of 128 columns: the 8 lanes of a row then read 16-byte vectors of mask and plane bits
-// from different banks, whatever the row length.  Sums over the 8 ranges (shuffles) and the four groups (shared
+// Kq is a multiple of 128 columns (`units` of them): the 8 lanes of a row read 16-byte vectors of mask and plane bits
+// that lie 16 x units bytes apart.  With a multiple of 8 units they would all read the same four banks, and one more
+// unit is cheaper (LSTM-like layer 4096 x 8192, two planes, batch 1: 14.5 us against 15.4; 2048 x 16384: 14.5 against
+// 15.6).  An even number that is none costs two or four passes of the same banks, less than another unit of
+// expansion would: 16384 x 2048, two planes, batch 8 21.9 us with three units and 18.7 with two, 32736 x 1025
+// 35.9 and 30.0, 8192 x 4096 19.6 (five) and 17.8 (four), 2730 x 12288 32.8 (13) and 31.4 (12).  Sums over the 8 ranges (shuffles) and the four groups (shared
 // memory) have a fixed order: results are bit-identical from run to run.
 //
 // Every wait on an mbarrier is bounded.  An expander warp whose wait gives up sets SQNN_E_TIMEOUT in the status word,
@@ -462,7 +466,8 @@ inline int launch_gemv_tc(const DecodeArgs &A, const uint64_t *d_mask, const flo
     const uint64_t R = (m + sms - 1) / sms, grid = (m + R - 1) / R;
     if (R > 0xffffffffull || n > (1u << 24)) return SQNN_E_UNSUPPORTED;
     g.rows_per_block = (uint32_t)R;
-    g.units = (uint32_t)((n + 128 * TC_RANGES - 1) / (128 * TC_RANGES)) | 1u;      // odd: see above
+    g.units = (uint32_t)((n + 128 * TC_RANGES - 1) / (128 * TC_RANGES));
+    if (g.units % 8 == 0) ++g.units;                                               // see above
     g.kq = g.units * 128;
     const size_t tab = (size_t)A.tab_words * 4;
     const uint64_t TW = 32ull * A.W, tile_bits = 32 * TW;

@@ -33,6 +33,12 @@ SMALL = [
     (128, 24, 300, 640, 0.2, 8, "bf16", 15),
     (64, 16, 5000, 900, 0.25, 1, "f32", 3),
     (80, 16, 2500, 8192, 0.2, 3, "bf16", 2),
+    # ranges of 2, 3, 4, 8 and 8 + 1 units of 128 columns: banks shared by none to all lanes of a row
+    (60, 12, 40, 2048, 0.2, 2, "bf16", 8),
+    (60, 12, 40, 2049, 0.2, 2, "bf16", 8),
+    (100, 10, 200, 4096, 0.1, 1, "f32", 3),
+    (100, 10, 33, 7169, 0.1, 1, "bf16", 5),
+    (100, 10, 33, 8193, 0.1, 1, "bf16", 5),
 ]
 
 
