@@ -1,6 +1,7 @@
-// K3 for rows too long for the tensor-core form (sqnn_gemv_tc.cuh): decryption fused with
-// Y[b][r] = sum_c W[r][c] X[b][c] for small batch (<= 15), fp32 accumulation on the plain ALUs, as a template over
-// the network shape, with its launcher.
+// K3, walk over care bits: decryption fused with Y[b][r] = sum_c W[r][c] X[b][c] for small batch (<= 15), fp32
+// accumulation on the plain ALUs, as a template over the network shape, with its launcher.  It takes rows too long
+// for the tensor-core form (sqnn_gemv_tc.cuh), and small or sparse layers with one plane and bf16 activations; where
+// the line lies and why: sqnn_gemv_plan.h.
 //
 // Work split.  A block owns a run of whole rows of W.  The bits of those rows are one contiguous
 // range of every flattened plane, so the block decodes the kernel tiles that cover that range
@@ -19,6 +20,7 @@
 // for those copies is bounded; a block whose wait gives up reports SQNN_E_TIMEOUT, waits once more for
 // what may be in flight and returns without storing its rows of Y.
 #pragma once
+#include "sqnn_gemv_plan.h"
 #include "sqnn_kernels.cuh"
 
 namespace sqnn {
@@ -369,12 +371,9 @@ k_decode_gemv(const GemvArgs g)
 // launcher
 // ------------------------------------------------------------------------------------------
 template <int N_OUT, int N_IN, int BT, typename XT>
-inline int launch_gemv_bt(const DecodeArgs &A, const uint64_t *d_mask, const float *d_alpha, const void *d_x,
+inline int launch_gemv_bt(const DecodeArgs &A, const WalkPlan &plan, const uint64_t *d_mask, const float *d_alpha, const void *d_x,
                           int64_t ldx, uint32_t batch, float *d_y, int64_t ldy, uint64_t m, uint64_t n, cudaStream_t st)
 {
-    uint32_t nwarps = 32;
-    const size_t limit = 220 * 1024;
-    const uint32_t sms = (uint32_t)sm_count();
     GemvArgs g;
     g.A = A;
     g.mask32 = (const uint32_t *)d_mask;
@@ -382,73 +381,21 @@ inline int launch_gemv_bt(const DecodeArgs &A, const uint64_t *d_mask, const flo
     g.alpha = d_alpha;
     g.x = d_x; g.ldx = ldx; g.y = d_y; g.ldy = ldy;
     g.m = m; g.n = (uint32_t)n; g.batch = batch;
-    const uint64_t R = (m + sms - 1) / sms;
-    const uint64_t grid = (m + R - 1) / R;
-    if (R > 0xffffffffull) return SQNN_E_UNSUPPORTED;
-    g.rows_per_block = (uint32_t)R;
-    {
-        // a block with a few rows and a few tiles to decode gets a few warps: a thread block is cheaper to start
-        // and to synchronise the smaller it is (tiny layers are all launch and latency)
-        const uint64_t tb = 32ull * 32ull * A.W;
-        const uint64_t items = ((R * n + tb - 1) / tb + 1) * A.n_q;
-        const uint64_t want = R > items ? R : items;
-        if (want <= 4) nwarps = 4;
-        else if (want <= 8) nwarps = 8;
-        else if (want <= 16) nwarps = 16;
-    }
-    const uint64_t TW = 32ull * A.W, tile_bits = 32 * TW;
-    const size_t tab = (size_t)A.tab_words * 4;
-    const size_t xbytes = ((size_t)n * BT * sizeof(XT) + 15) & ~(size_t)15;
-    bool xs = BT == 1 && xbytes <= 128 * 1024;      // several long vectors never fit
-    // Warps sharing a row.  A warp walks its run of a row's words 32 at a time, and every item (a row, or one
-    // of `parts` runs of it) costs about one such step more for its set-up and reduction, so the walk of a chunk
-    // takes (rounds of items over the warps) x (steps per item + 1); the cheapest split wins, the smaller one on
-    // a tie.  (Measured on 41 rows of 94 words: 1 part 13.5 us, 2 parts 15.2, 3 parts 13.8, 4 parts 16.5.)
-    auto pick_parts = [&](uint64_t rows) {
-        const uint64_t row_words = (n + 31) / 32 + 1;
-        uint32_t best = 1;
-        uint64_t best_cost = ~0ull;
-        for (uint32_t p = 1; p <= 32 && p <= row_words; ++p) {
-            const uint64_t per = (row_words + p - 1) / p;
-            const uint64_t cost = ((rows * p + nwarps - 1) / nwarps) * ((per + 31) / 32 + 1);
-            if (cost < best_cost) { best = p; best_cost = cost; }
-        }
-        return best;
-    };
-    uint64_t RC = R;
-    size_t smem = 0;
-    for (;;) {
-        g.parts = pick_parts(RC);
-        const uint64_t tiles = (RC * n + tile_bits - 1) / tile_bits + 1;
-        const uint64_t region_words = tiles * TW;
-        g.alpha_words = (uint32_t)((RC * A.n_q + 3) & ~3ull);
-        g.part_words = (uint32_t)((RC * g.parts * BT + 3) & ~3ull);
-        g.xs_words = xs ? (uint32_t)(xbytes / 4) : 0u;
-        const uint64_t need = tab + (uint64_t)(A.n_q + 1) * region_words * 4 +
-                              4ull * (g.alpha_words + g.part_words + g.xs_words);
-        if (need <= limit) {
-            g.region_words = (uint32_t)region_words;
-            g.rows_per_chunk = (uint32_t)RC;
-            smem = (size_t)need;
-            break;
-        }
-        if (RC > 1) { RC = (RC + 1) / 2; continue; }
-        if (xs) { xs = false; RC = R; continue; }               // leave the activations in global memory
-        return SQNN_E_UNSUPPORTED;                               // one row of bits does not fit
-    }
+    g.rows_per_block = plan.rows_per_block; g.rows_per_chunk = plan.rows_per_chunk; g.parts = plan.parts;
+    g.region_words = plan.region_words; g.alpha_words = plan.alpha_words; g.part_words = plan.part_words; g.xs_words = plan.xs_words;
     // bulk staging of the first chunk: one activation vector in shared memory, 16-byte aligned sources and sizes
-    g.bulk_stage = (BT == 1 && xs && ((uintptr_t)d_x & 15) == 0 && (n * sizeof(XT)) % 16 == 0 &&
-                    ((uintptr_t)d_mask & 15) == 0 && ((uintptr_t)A.tab & 15) == 0 && (tab + 0) % 16 == 0 &&
+    g.bulk_stage = (BT == 1 && plan.xs && ((uintptr_t)d_x & 15) == 0 && (n * sizeof(XT)) % 16 == 0 &&
+                    ((uintptr_t)d_mask & 15) == 0 && ((uintptr_t)A.tab & 15) == 0 && A.tab_words % 4 == 0 &&
                     (size_t)g.region_words * 4 < (1u << 20)) ? 1u : 0u;
     const DebugKnobs dbg = debug_knobs();
     g.skip_stage = (dbg.flags & 4u) ? 1u : 0u;
     g.wait_limit = dbg.wait_cycles ? dbg.wait_cycles : GEMV_WAIT_LIMIT;
 #define SQNN_GEMV_LAUNCH(XSV, NQV)                                                                       \
     do {                                                                                                 \
-        return launch_kernel(k_decode_gemv<N_OUT, N_IN, BT, XT, XSV, NQV>, (uint32_t)grid, nwarps * 32, smem, st, g); \
+        return launch_kernel(k_decode_gemv<N_OUT, N_IN, BT, XT, XSV, NQV>, plan.grid, plan.warps * 32, plan.smem, st, g); \
     } while (0)
     if constexpr (BT == 1) {
-        if (xs) {
+        if (plan.xs) {
             if (A.n_q == 1) SQNN_GEMV_LAUNCH(true, 1);
             else SQNN_GEMV_LAUNCH(true, 0);
         }
@@ -459,13 +406,13 @@ inline int launch_gemv_bt(const DecodeArgs &A, const uint64_t *d_mask, const flo
 }
 
 template <int N_OUT, int N_IN, typename XT>
-inline int launch_gemv(const DecodeArgs &A, const uint64_t *d_mask, const float *d_alpha, const void *d_x,
+inline int launch_gemv(const DecodeArgs &A, const WalkPlan &plan, const uint64_t *d_mask, const float *d_alpha, const void *d_x,
                        int64_t ldx, uint32_t batch, float *d_y, int64_t ldy, uint64_t m, uint64_t n, cudaStream_t st)
 {
-    if (batch == 1) return launch_gemv_bt<N_OUT, N_IN, 1, XT>(A, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st);
-    if (batch == 2) return launch_gemv_bt<N_OUT, N_IN, 2, XT>(A, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st);
-    if (batch <= 4) return launch_gemv_bt<N_OUT, N_IN, 4, XT>(A, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st);
-    return launch_gemv_bt<N_OUT, N_IN, 8, XT>(A, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st);
+    if (plan.bt == 1) return launch_gemv_bt<N_OUT, N_IN, 1, XT>(A, plan, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st);
+    if (plan.bt == 2) return launch_gemv_bt<N_OUT, N_IN, 2, XT>(A, plan, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st);
+    if (plan.bt == 4) return launch_gemv_bt<N_OUT, N_IN, 4, XT>(A, plan, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st);
+    return launch_gemv_bt<N_OUT, N_IN, 8, XT>(A, plan, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st);
 }
 
 }  // namespace sqnn

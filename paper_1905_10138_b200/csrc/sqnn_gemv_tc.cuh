@@ -33,17 +33,14 @@
 //
 // Bound: integer instructions of the expansion (1.4 per weight and plane, against 42 per unpruned weight of the
 // walk over care bits in sqnn_gemv.cuh, 3.8 per weight at 9 % density) and the latency of the block's phases
-// (launch, staging, decode, product, reduction).
+// (launch, staging, decode, product, reduction).  Which of the two takes a call: sqnn_gemv_plan.h.
 #pragma once
 #include "sqnn_gemv.cuh"
 #include "sqnn_tc.cuh"
 
 namespace sqnn {
 
-constexpr uint32_t TC_GROUPS = 4;                         // expander groups
-constexpr uint32_t TC_THREADS = TC_GROUPS * 128 + TC_GROUPS * 32;
-constexpr uint32_t TC_TILE_ROWS = 16, TC_RANGES = 8;
-constexpr uint32_t TC_MAX_Q = 12;                         // activation columns (vectors x pieces) per pass: N <= 96
+constexpr uint32_t TC_THREADS = TC_WARPS * 32;             // per group four expander warps, and an MMA warp
 constexpr uint64_t TC_WAIT_LIMIT = 2000000000ull;         // cycles a bounded wait may take: about a second
 
 struct TcArgs {
@@ -448,14 +445,10 @@ leave:
 // ------------------------------------------------------------------------------------------
 // launcher
 // ------------------------------------------------------------------------------------------
-// Returns SQNN_E_UNSUPPORTED when this kernel is not the one to take (the caller falls back to the walk).
 template <int N_OUT, int N_IN, typename XT>
-inline int launch_gemv_tc(const DecodeArgs &A, const uint64_t *d_mask, const float *d_alpha, const void *d_x,
+inline int launch_gemv_tc(const DecodeArgs &A, const TcPlan &plan, const uint64_t *d_mask, const float *d_alpha, const void *d_x,
                           int64_t ldx, uint32_t batch, float *d_y, int64_t ldy, uint64_t m, uint64_t n, cudaStream_t st)
 {
-    constexpr uint32_t PIECES = sizeof(XT) == 4 ? 3 : 1;
-    const size_t limit = 220 * 1024;
-    const uint32_t sms = (uint32_t)sm_count();
     TcArgs g;
     g.A = A;
     g.mask32 = (const uint32_t *)d_mask;
@@ -463,48 +456,18 @@ inline int launch_gemv_tc(const DecodeArgs &A, const uint64_t *d_mask, const flo
     g.alpha = d_alpha;
     g.x = d_x; g.ldx = ldx; g.y = d_y; g.ldy = ldy;
     g.m = m; g.n = (uint32_t)n; g.batch = batch;
-    const uint64_t R = (m + sms - 1) / sms, grid = (m + R - 1) / R;
-    if (R > 0xffffffffull || n > (1u << 24)) return SQNN_E_UNSUPPORTED;
-    g.rows_per_block = (uint32_t)R;
-    g.units = (uint32_t)((n + 128 * TC_RANGES - 1) / (128 * TC_RANGES));
-    if (g.units % 8 == 0) ++g.units;                                               // see above
-    g.kq = g.units * 128;
-    const size_t tab = (size_t)A.tab_words * 4;
-    const uint64_t TW = 32ull * A.W, tile_bits = 32 * TW;
-    // bits a lane may read past the end of the last row: its range's padding and the second vector
-    const uint64_t slack = (TC_RANGES * (uint64_t)g.kq - n) / 32 + 12;
-    // Activation vectors per pass: as many as the accumulators allow, fewer where they would leave too little
-    // shared memory for a chunk of rows (every pass expands the weights again, every chunk decodes its boundary
-    // tiles again and may leave a tile of 16 rows half empty).
-    const uint32_t bt_max = TC_MAX_Q / PIECES;
-    size_t smem = 0;
-    for (uint32_t passes = (batch + bt_max - 1) / bt_max; smem == 0; ++passes) {
-        if (passes > batch) return SQNN_E_UNSUPPORTED;           // rows too long
-        g.bt = (batch + passes - 1) / passes;
-        g.N = (8 * g.bt * PIECES + 15) / 16 * 16;
-        g.slots = g.N <= 64 ? 2u : 1u;
-        const size_t x_bytes = (size_t)(g.kq / 64) * g.N * 128 + 1024;
-        for (uint64_t RC = R;; RC = (RC + 1) / 2) {
-            const uint64_t tiles = (RC * n + tile_bits - 1) / tile_bits + 1;
-            const uint64_t region_words = (tiles * TW + slack + 3) & ~3ull;
-            g.alpha_words = (uint32_t)((RC * A.n_q + 3) & ~3ull);
-            g.part_words = (uint32_t)((TC_GROUPS * RC * g.bt + 3) & ~3ull);
-            const uint64_t need = tab + (uint64_t)(A.n_q + 1) * region_words * 4 + 4ull * (g.alpha_words + g.part_words) + x_bytes;
-            if (need <= limit) {
-                g.region_words = (uint32_t)region_words;
-                g.rows_per_chunk = (uint32_t)RC;
-                smem = (size_t)need;
-                break;
-            }
-            if (RC <= 8) break;
-        }
-    }
+    g.rows_per_block = plan.rows_per_block;
+    g.rows_per_chunk = plan.rows_per_chunk;
+    g.units = plan.units;
+    g.kq = plan.units * 128;
+    g.bt = plan.bt; g.N = plan.N; g.slots = plan.slots;
+    g.region_words = plan.region_words; g.alpha_words = plan.alpha_words; g.part_words = plan.part_words;
     const DebugKnobs dbg = debug_knobs();
     g.skip_mma = (dbg.flags & 2u) ? 1u : 0u;
     g.wait_limit = dbg.wait_cycles ? dbg.wait_cycles : TC_WAIT_LIMIT;
     g.x_vec = (((uintptr_t)d_x & 15) == 0 && (ldx * (int64_t)sizeof(XT)) % 16 == 0) ? 1u : 0u;
-    return n % 128 == 0 ? launch_kernel(k_gemv_tc<N_OUT, N_IN, XT, true>, (uint32_t)grid, TC_THREADS, smem, st, g)
-                        : launch_kernel(k_gemv_tc<N_OUT, N_IN, XT, false>, (uint32_t)grid, TC_THREADS, smem, st, g);
+    return n % 128 == 0 ? launch_kernel(k_gemv_tc<N_OUT, N_IN, XT, true>, plan.grid, TC_THREADS, plan.smem, st, g)
+                        : launch_kernel(k_gemv_tc<N_OUT, N_IN, XT, false>, plan.grid, TC_THREADS, plan.smem, st, g);
 }
 
 }  // namespace sqnn

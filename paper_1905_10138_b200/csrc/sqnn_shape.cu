@@ -23,35 +23,46 @@ int decode_shape<SQNN_NO, SQNN_NI>(const DecodeArgs &A, sqnn_out_mode mode, cons
 }
 
 #else
-// the tensor-core product; SQNN_E_UNSUPPORTED: not the form to take
 template <int N_OUT, int N_IN>
-int gemv_tc_shape(const DecodeArgs &A, const uint64_t *d_mask, const float *d_alpha, const void *d_x, int x_dtype,
+int gemv_tc_shape(const DecodeArgs &A, const TcPlan &plan, const uint64_t *d_mask, const float *d_alpha, const void *d_x, int x_dtype,
                   int64_t ldx, uint32_t batch, float *d_y, int64_t ldy, uint64_t m, uint64_t n, cudaStream_t st);
 #if SQNN_PART == 1
 template <>
-int gemv_tc_shape<SQNN_NO, SQNN_NI>(const DecodeArgs &A, const uint64_t *d_mask, const float *d_alpha,
+int gemv_tc_shape<SQNN_NO, SQNN_NI>(const DecodeArgs &A, const TcPlan &plan, const uint64_t *d_mask, const float *d_alpha,
                                     const void *d_x, int x_dtype, int64_t ldx, uint32_t batch, float *d_y,
                                     int64_t ldy, uint64_t m, uint64_t n, cudaStream_t st)
 {
     return x_dtype == SQNN_X_BF16
-        ? launch_gemv_tc<SQNN_NO, SQNN_NI, __nv_bfloat16>(A, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st)
-        : launch_gemv_tc<SQNN_NO, SQNN_NI, float>(A, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st);
+        ? launch_gemv_tc<SQNN_NO, SQNN_NI, __nv_bfloat16>(A, plan, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st)
+        : launch_gemv_tc<SQNN_NO, SQNN_NI, float>(A, plan, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st);
 }
 #else
 template <>
-int gemv_tc_shape<SQNN_NO, SQNN_NI>(const DecodeArgs &, const uint64_t *, const float *, const void *, int, int64_t, uint32_t,
-                                    float *, int64_t, uint64_t, uint64_t, cudaStream_t);
+int gemv_tc_shape<SQNN_NO, SQNN_NI>(const DecodeArgs &, const TcPlan &, const uint64_t *, const float *, const void *, int, int64_t,
+                                    uint32_t, float *, int64_t, uint64_t, uint64_t, cudaStream_t);
 
 template <>
 int gemv_shape<SQNN_NO, SQNN_NI>(const DecodeArgs &A, const uint64_t *d_mask, const float *d_alpha,
                                  const void *d_x, int x_dtype, int64_t ldx, uint32_t batch, float *d_y,
                                  int64_t ldy, uint64_t m, uint64_t n, cudaStream_t st)
 {
-    const int rc = gemv_tc_shape<SQNN_NO, SQNN_NI>(A, d_mask, d_alpha, d_x, x_dtype, ldx, batch, d_y, ldy, m, n, st);
-    if (rc != SQNN_E_UNSUPPORTED) return rc;
+    uint64_t patches = 0;
+    for (uint32_t i = 0; i < A.n_q; ++i) patches += A.pl[i].n_pp;
+    const double slices = (double)A.n_q * (double)((A.mn + A.n_out - 1) / A.n_out);
+    GemvLayer L;
+    L.m = m; L.n = n; L.batch = batch; L.n_q = A.n_q;
+    L.W = A.W; L.tab_words = A.tab_words;
+    L.x_bytes = x_dtype == SQNN_X_BF16 ? 2 : 4;
+    L.sms = (uint32_t)sm_count();
+    L.density = care_density(A.n_out, A.n_in, (double)patches / slices);
+    const TcPlan tc = plan_gemv_tc(L);
+    const WalkPlan walk = plan_walk(L);
+    if (!take_walk(L, tc, walk))
+        return tc.ok ? gemv_tc_shape<SQNN_NO, SQNN_NI>(A, tc, d_mask, d_alpha, d_x, x_dtype, ldx, batch, d_y, ldy, m, n, st)
+                     : SQNN_E_UNSUPPORTED;                       // one row of bits does not fit
     return x_dtype == SQNN_X_BF16
-        ? launch_gemv<SQNN_NO, SQNN_NI, __nv_bfloat16>(A, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st)
-        : launch_gemv<SQNN_NO, SQNN_NI, float>(A, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st);
+        ? launch_gemv<SQNN_NO, SQNN_NI, __nv_bfloat16>(A, walk, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st)
+        : launch_gemv<SQNN_NO, SQNN_NI, float>(A, walk, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st);
 }
 #endif
 #endif

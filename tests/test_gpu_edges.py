@@ -51,6 +51,40 @@ def test_small_batch_product_at_tile_edges(case):
     assert H.rel_err(y, ref) <= 1e-4
 
 
+# (n_out, n_in, m, n, keep, n_q, x, batch, walk): small and sparse one-plane bf16 layers go to the walk (one, two, four and
+# eight vectors at a time, a row over several warps, chunks of rows, a second group of vectors), their neighbours do not
+FORMS = [
+    (100, 10, 300, 1024, 0.07, 1, "bf16", 1, True),
+    (100, 10, 1, 64, 0.1, 1, "bf16", 1, True),
+    (80, 8, 147, 3001, 0.1, 1, "bf16", 2, True),
+    (200, 10, 900, 700, 0.03, 1, "bf16", 4, True),
+    (200, 10, 149, 16384, 0.02, 1, "bf16", 15, False),
+    (64, 16, 40, 44001, 0.25, 1, "f32", 11, True),              # (rows too long for the other form)
+    (100, 10, 300, 1024, 0.07, 1, "f32", 1, False),
+    (100, 10, 300, 1024, 0.07, 2, "bf16", 1, False),
+    (60, 12, 2000, 3000, 0.2, 1, "bf16", 1, False),
+]
+
+
+@pytest.mark.parametrize("case", FORMS, ids=lambda c: "x".join(map(str, c)))
+def test_small_batch_product_in_the_form_that_the_rule_picks(case):
+    """Which form ran: with the library's test knob the tensor-core form issues no MMAs and reports a timeout."""
+    import torch
+    n_out, n_in, m, n, keep, n_q, x_dtype, batch, walk = case
+    layer = generic_layer(n_out, n_in, m, n, keep, 56, n_q=n_q)
+    layer.x_dtype = x_dtype
+    x = layer.activations(batch)
+    y, ref = product(layer, x, x_dtype)
+    assert H.rel_err(y, ref) <= 1e-4
+    dev = H.DeviceLayer(layer, H.blob_from_library(layer)[0])
+    try:
+        sqnn.sqnn_set_debug_flags(2, 1_000_000)
+        dev.matmul(x, torch.float32 if x_dtype == "f32" else torch.bfloat16)
+    finally:
+        sqnn.sqnn_set_debug_flags(0, 0)
+    assert dev.status_value() == (0 if walk else -sqnn.E_TIMEOUT)
+
+
 @pytest.mark.parametrize("x_dtype", ["f32", "bf16"])
 def test_pruned_weights_do_not_meet_activations_that_are_not_finite(x_dtype):
     layer = generic_layer(100, 10, 40, 700, 0.3, 52)
