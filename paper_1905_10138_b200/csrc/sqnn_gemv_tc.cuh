@@ -214,10 +214,10 @@ k_gemv_tc(const TcArgs g)
     // a later one's allocation waits until they are given back.
     const bool holder = warp == nwarps - 1;
     if (holder) tmem_alloc(&tmem_slot, 512);
-    if (threadIdx.x == 0) {
-        for (uint32_t i = 0; i < 4 * TC_GROUPS; ++i) mbar_init(bars_sa + 8 * i, 1);
-        for (uint32_t i = 0; i < TC_GROUPS; ++i) taken_s[i] = 0;
-        abort_word = 0;
+    if (warp == nwarps - 2) {
+        if (lane < 4 * TC_GROUPS) mbar_init(bars_sa + 8 * lane, 1);
+        if (lane < TC_GROUPS) taken_s[lane] = 0;
+        if (lane == 0) abort_word = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     wait_prior_grid();
@@ -334,10 +334,7 @@ k_gemv_tc(const TcArgs g)
                             expand32(mw[2 * h + 1], bw[2 * h + 1], v + 16);
                             const uint32_t slot = slot_seq & slot_mask, use = slot_seq >> slot_shift;
                             if (use > 0) {
-                                if (!mbar_wait_warp(free_a + 8 * slot, (use - 1) & 1u, abort_flag, A.status, g.wait_limit)) {
-                                    arrive_for_the_rest(taken_s + grp, 1 + 2 * grp, slot_mask, slot_seq, seq_end, g.wait_limit);
-                                    goto pass_over;
-                                }
+                                if (!mbar_wait_warp(free_a + 8 * slot, (use - 1) & 1u, abort_flag, A.status, g.wait_limit)) goto late;
                                 tc_fence_after();
                             }
                             tmem_st16(a_tmem + lane_sel + slot * 32, v);
@@ -350,10 +347,7 @@ k_gemv_tc(const TcArgs g)
                     u += len;
                     // the part's accumulator: this lane's range, scaled
                     const float al = 0.5f * alpha_s[rl * n_q + pl];
-                    if (!mbar_wait_warp(done, parts_done & 1u, abort_flag, A.status, g.wait_limit)) {
-                        arrive_for_the_rest(taken_s + grp, 1 + 2 * grp, slot_mask, slot_seq, seq_end, g.wait_limit);
-                        goto pass_over;
-                    }
+                    if (!mbar_wait_warp(done, parts_done & 1u, abort_flag, A.status, g.wait_limit)) goto late;
                     ++parts_done;
                     tc_fence_after();
 #pragma unroll
@@ -388,6 +382,9 @@ k_gemv_tc(const TcArgs g)
                         }
                     }
                 }
+                goto pass_over;
+            late:
+                arrive_for_the_rest(taken_s + grp, 1 + 2 * grp, slot_mask, slot_seq, seq_end, g.wait_limit);
             } else {
                 // the group's MMA warp: one slot at a time, in the order they are filled
                 const uint32_t idesc = instr_desc_bf16(g.N);
