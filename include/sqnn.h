@@ -279,7 +279,8 @@ int sqnn_decode(const sqnn_desc *desc, const void *d_blob, const uint64_t *d_mas
  * fully overwritten.
  *  - batch <= 15: one kernel; every block decodes the slices that cover its own rows into shared
  *    memory, expands them to bf16 signs and multiplies on the tensor cores with fp32 accumulation
- *    (weights and F32 activations exact); rows too long for that are walked on the plain ALUs.
+ *    (weights and F32 activations exact).  Rows too long for that, and small or sparse layers of one
+ *    plane with BF16 activations, are walked care bit by care bit on the plain ALUs (fp32).
  *    Each Y[b][r] is summed in a fixed order, so results are bit-identical from run to run.  No
  *    workspace is used.  A row must fit shared memory as bits: n * (n_q + 1) <= 1 400 000, else
  *    UNSUPPORTED.

@@ -54,9 +54,10 @@ struct ClearArgs {
 };
 
 // Programmatic dependent launch.  A kernel of this library may be scheduled before the kernel queued ahead of
-// it has finished; wait_prior_grid() returns once that one is complete and its results are visible, and nothing
-// in global memory is read or written before it.  launch_dependents() lets the next kernel in (it waits in
-// turn for all of this one), and is called once this kernel has nothing left to wait for.
+// it has finished; wait_prior_grid() returns once that one is complete and its results are visible.  Nothing in
+// global memory is read or written before it, with one exception: k_decode_mma reads activations and mask ahead of its
+// wait.  The decode kernel queued just before it lets it in after its own wait, so whatever was queued before the
+// two is complete by then.  launch_dependents() lets the next kernel in, which waits in turn for all of this one.
 SQNN_DEV void wait_prior_grid() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 SQNN_DEV void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 

@@ -181,7 +181,7 @@ inline WalkPlan plan_walk(const GemvLayer &L)
     // Warps sharing a row.  A warp walks its run of a row's words 32 at a time, and every item (a row, or one
     // of `parts` runs of it) costs about one such step more for its set-up and reduction, so the walk of a chunk
     // takes (rounds of items over the warps) x (steps per item + 1); the cheapest split wins, the smaller one on
-    // a tie.  (Measured on 41 rows of 94 words: 1 part 13.5 us, 2 parts 15.2, 3 parts 13.8, 4 parts 16.5.)
+    // a tie.  (Measured on 41 rows of 94 words, two planes: 1 part 13.5 us, 2 parts 15.2, 3 parts 13.8, 4 parts 16.5.)
     const uint64_t row_words = (L.n + 31) / 32 + 1;
     auto pick_parts = [&](uint64_t rows) {
         uint32_t best = 1;

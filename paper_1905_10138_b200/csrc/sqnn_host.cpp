@@ -89,8 +89,8 @@ struct Expander {
 // every column in turn (zero where there is none) and what is left is kept at its lowest column; a row that
 // reduces to 0 = 1 is the unsolvable case and is dropped (it will show up as a patch), one that reduces to 0 = 0 is
 // redundant.  Free variables are 0, so the pivot variables follow from the highest column down.  (One slice at a
-// time, with a branch for every reduction, spent most of its time on mispredicted branches: 4.6 ms against
-// the figure of the commit for 378 000 slices of 100 x 10 on 16 cores.)
+// time, with a branch for every reduction, spent most of its time on mispredicted branches: encoding 378 000 slices of
+// 100 x 10 took 4.6 ms on 16 cores, and takes 2.5 ms this way.)
 constexpr uint32_t LANES = 8;
 typedef uint32_t Vec __attribute__((vector_size(4 * LANES)));
 typedef int32_t SignedVec __attribute__((vector_size(4 * LANES)));

@@ -205,8 +205,10 @@ SQNN_DEV void stage_mask(uint32_t *mask_s, const uint32_t *__restrict__ mask32, 
 // planes disagree with it: at most four bf16 values per row, eight bytes, from which one byte permutation picks
 // two weights.  Mask and sign bits, moved to the top of a half word, are the bf16 numbers 0, 2 and -2, so a
 // multiply-add with V / 2 does the rest.  Selectors and those numbers come out of words in which even and odd
-// columns have been separated, by a shift and an AND each: 3 instructions per weight with three planes.  (Sums of
-// the scales per weight took about 20, and 64 us for 2^26 weights of three planes.)  Negating all terms of a sum
+// columns have been separated, by a shift and an AND each: 3 instructions per weight with three planes.  What surrounds
+// that -- words, separation, staging, copies, row bookkeeping -- takes nearly four more: 2^26 weights of three planes
+// take 37 us and 22.0 M warp instructions, of which 7.7 M are the decode.  (Sums of the scales per weight took about 20
+// instructions, and 64 us.)  Negating all terms of a sum
 // negates it exactly, except when it is zero or not finite, and halving is exact except for the tiniest
 // numbers; rows with such a value take the plain loop, as do chunks of 8 weights that straddle rows, and
 // layers of four and more planes.

@@ -223,7 +223,8 @@ k_decode_mma(const __grid_constant__ CUtensorMap xmap, const MmaArgs M)
             sm.open(M.mask32, M.plane_words32, c0, count);
             sb.open(M.bits32 + plane * M.plane_words32, M.plane_words32, c0, count);
             if (count) sm.fetch();
-            if (part_no == 0) wait_prior_grid();             // decoded planes and cleared Y are in place
+            // decoded planes and cleared Y are in place; mask and activations are inputs and were before (sqnn_decode.cuh)
+            if (part_no == 0) wait_prior_grid();
             if (count) sb.fetch();
             uint32_t seq = seq0;
             for (uint32_t i = 0; i < count; ++i) {

@@ -17,8 +17,9 @@
 // warp: sets of three (which decide nearly all of them), then all 2^r sets in Gray-code order; slices with more
 // dependent rows than C has bits for by trying all seeds.
 //
-// Bound: integer instructions.  600 000 slices of 60 x 12 (20 % care bits): see the measured figure at the
-// launch below.
+// Bound: integer instructions.  600 000 slices of 60 x 12 (20 % care bits, two planes of 6000 x 3000) take 127 us, 79 M
+// warp instructions with 18.5 of 32 lanes active: the loop over a slice's care bits takes as many turns as the lane with
+// the most of them needs.  (Trying all 2^12 seeds of every slice took 2540 us.)
 #include "sqnn_launch.h"
 
 #include <cuda_runtime.h>
