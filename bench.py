@@ -38,9 +38,7 @@ WORKLOAD = "alexnet-fc6 4096x9216, n_q=1, M 100x10, S=0.91, bf16 activations, ba
 # DRAM bytes (read + write) of one launch, from one ncu capture of each kernel as it stands now on exactly
 # these workloads (summaries under profiles/).  An entry is None while its kernel has changed since the
 # counters were taken.
-NCU_DRAM_BYTES_PER_LAUNCH = {"k_gemv_tc": None, "k_decode_bits": None}
-LANES_PER_SM = 128
-SMS = 148
+NCU_DRAM_BYTES_PER_LAUNCH = {"k_gemv_tc": 5690112, "k_decode_bits": 103741440}
 
 
 def measured_peaks():
@@ -199,8 +197,8 @@ def time_interval(torch, fn, reps, flush=None, rounds=3):
 
 def time_interval_graph(torch, fn, reps, flush=None, rounds=3):
     """As time_interval, but the reps x (flush + call) and the reps flushes are each captured into a CUDA
-    graph once and replayed: consecutive kernels then start without the launch grid of about 2 us that
-    separately launched kernels show on this system.  Returns None if the work cannot be captured."""
+    graph once and replayed: consecutive kernels then start without the gap of about 2 us between
+    separately launched kernels that wait for one another in full.  Returns None if the work cannot be captured."""
     try:
         side = torch.cuda.Stream()
 
@@ -330,9 +328,9 @@ def run_ours(args):
     sampler.start()
     # exactly K steps in one event interval over K x (flush + step), minus the K flushes alone, the kernels
     # launched one by one: this is the figure reported.  The same K x (flush + step) replayed from a CUDA graph
-    # is reported beside it (separately launched kernels start on a grid of about 2 us on this system; in a
-    # graph they do not, but there the flushes alone also pack tighter than flushes with a step between them,
-    # so neither difference is the kernel's bare duration).
+    # is reported beside it (separately launched kernels that wait for one another in full, as the flushes do, start
+    # about 2 us apart on this system; in a graph they do not, but there the flushes alone also pack tighter than
+    # flushes with a step between them, so neither difference is the kernel's bare duration).
     ms_stream = time_interval(torch, step, args.steps, flush, rounds=1)
     ms_graph = time_interval_graph(torch, step, args.steps, flush, rounds=1)
     ms_per_step_local = ms_stream
@@ -356,19 +354,19 @@ def run_ours(args):
     e2e = {"value": whole_job_rate(world, units, e2e_ms / args.steps), "unit": UNIT,
            "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h}
 
-    # roofline of the dominant kernel (fused decode-GEMV), against plain ALU work: one table-driven
-    # expansion per weight bit plus one multiply-add per unpruned weight.
+    # Roofline of the dominant kernel (fused decode and product): the time its bytes take at the copy bandwidth.  A
+    # block's phases follow one another and each is bound by its own latency, so the fraction is small; the tensor
+    # cores it multiplies on are nearly idle at one vector (8 ranges x 16 accumulator columns issued per weight).
     alg_bytes = stream_bytes(stats, layer, True) + layer.alpha.nbytes + x1.size * 2 + layer.m * 4
     kern_s = ms_per_step_local * 1e-3
-    alg_ops = layer.mn * layer.n_q + int(layer.mask.sum()) * layer.n_q
-    alu_peak = SMS * LANES_PER_SM * peaks["sm_max_mhz"] * 1e6 / 1e12
-    roofline = {"bound": "alu", "achieved": alg_ops / kern_s / 1e12, "peak": alu_peak, "unit": "Tlane-op/s",
-                "frac": alg_ops / kern_s / 1e12 / alu_peak, "traffic": NCU_DRAM_BYTES_PER_LAUNCH["k_gemv_tc"],
-                "kernel": "k_gemv_tc", "peak_source": f"148 SMs x 128 lanes x {peaks['sm_max_mhz']:.0f} MHz (max SM clock)",
-                "per_step_event_intervals_ms_median": float(np.median(times)),
-                "hbm_achieved_gbs": alg_bytes / kern_s / 1e9,
-                "hbm_frac_of_measured": alg_bytes / kern_s / 1e9 / peaks["hbm_gbs"],
-                "algorithmic_bytes": alg_bytes, "peaks": peaks["source"]}
+    mma_flops = 2.0 * layer.mn * layer.n_q * 16
+    roofline = {"bound": "hbm", "achieved": alg_bytes / kern_s / 1e9, "peak": peaks["hbm_gbs"], "unit": "GB/s",
+                "frac": alg_bytes / kern_s / 1e9 / peaks["hbm_gbs"], "traffic": NCU_DRAM_BYTES_PER_LAUNCH["k_gemv_tc"],
+                "kernel": "k_gemv_tc", "algorithmic_bytes": alg_bytes, "peaks": peaks["source"],
+                "limited_by": "latency of the phases of a block (start, staging, decode, expansion, reduction)",
+                "tensor_issued_tflops": mma_flops / kern_s / 1e12,
+                "tensor_issued_frac_of_burst": mma_flops / kern_s / 1e12 / peaks["bf16_tflops"],
+                "per_step_event_intervals_ms_median": float(np.median(times))}
 
     out = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
            "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True,
@@ -417,7 +415,7 @@ def product_rows(torch, sqnn, layer, desc, d_blob, d_mask, d_alpha, status, flus
                "dense_bf16_hbm_floor_us": dense_floor_us,
                "fused_us_cold_l2": 1e3 * time_interval(torch, fused, reps, flush),
                "fused_us_warm_l2": 1e3 * time_interval(torch, fused, reps),
-               "path": "tcgen05 (one kernel)" if batch <= 15 else "decode to packed bits + tcgen05 (two kernels)"}
+               "path": "one kernel" if batch <= 15 else "decode to packed bits + tcgen05 (two kernels)"}
         # the same four figures with the timed calls replayed from a CUDA graph (both sides alike)
         for key, f, fl in (("dense_bf16_us_cold_l2", dense, flush), ("dense_bf16_us_warm_l2", dense, None),
                            ("fused_us_cold_l2", fused, flush), ("fused_us_warm_l2", fused, None)):
@@ -590,7 +588,7 @@ def run_reference(args):
     from oracle import oracle as orc
     from paper_1905_10138_b200 import workloads as wl
     layer = wl.make_layer(2)
-    rows = 2048
+    rows = layer.m
     _, sub_mask, arrays = oracle_sample(layer, rows)
     x64 = layer.activations(1).astype(np.float64)
     for _ in range(args.warmup):
@@ -600,11 +598,11 @@ def run_reference(args):
         oracle_step(layer, rows, sub_mask, arrays, x64)
     dt = (time.perf_counter() - t0) / args.steps
     value = rows * layer.n * layer.n_q / dt
-    sample = f"first {rows} of {layer.m} rows per step (bounded sample), decode + fp64 product, batch 1"
+    sample = f"all {rows} rows per step, decode + fp64 product, batch 1"
     out = {"impl": "reference", "metric": METRIC, "value": value, "unit": UNIT,
            "n_gpus": int(os.environ.get("WORLD_SIZE", "1")), "steps": args.steps, "warmup": args.warmup,
            "ms_per_step": dt * 1e3, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-           "dtype": "f64", "data": "synthetic", "config": {"workload": WORKLOAD, "sample": sample},
+           "dtype": "f64", "data": "synthetic", "config": {"workload": WORKLOAD, "parallelism": "host cores", "timing": sample},
            "cpu_baseline": {"value": value, "unit": UNIT, "cores": orc.num_threads(), "kind": "oracle",
                             "sample": sample},
            "e2e": {"value": value, "unit": UNIT, "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
