@@ -5,8 +5,9 @@
     python -m paper_1905_10138_b200.profile_case bf16    --cfg 3
     python -m paper_1905_10138_b200.profile_case matmul  --cfg 2 --batch 1
     python -m paper_1905_10138_b200.profile_case search  --cfg 2          (exhaustive seed search)
+    python -m paper_1905_10138_b200.profile_case case    --name bits_odd  (a listed case of perf/cases.py)
 
---cfg 1..4 picks a layer of the benchmark configurations (optionally --rows / --cols smaller),
+Run it from the root of the repository.  --cfg 1..4 picks a layer of the benchmark configurations (optionally --rows / --cols smaller),
 --sweep I_S I_M a point of the decode-only sweep (prune rate index, network index).
 Prints the CUDA-event time of every iteration.
 """
@@ -17,11 +18,24 @@ import argparse
 import numpy as np
 
 
+def run_case(name: str, iters: int) -> None:
+    """Inputs of a listed performance case (seed 7), then `iters` passes through the public entry points."""
+    import torch
+    from perf import cases
+    case = next(c for c in cases.listed() if c["name"] == name)
+    state = cases.prepare(case, 7)
+    for _ in range(iters):
+        cases.run(state)
+    torch.cuda.synchronize()
+    print(f"{name}: {iters} passes, status {int(state['status'].item()) if 'status' in state else 0}")
+
+
 def main():
     import torch
     from . import sqnn, workloads as wl
     ap = argparse.ArgumentParser()
-    ap.add_argument("what", choices=["decode", "sink", "bf16", "matmul", "search"])
+    ap.add_argument("what", choices=["decode", "sink", "bf16", "matmul", "search", "case"])
+    ap.add_argument("--name", help="with `case`: the case's name")
     ap.add_argument("--cfg", type=int, default=0)
     ap.add_argument("--sweep", type=int, nargs=2, default=None)
     ap.add_argument("--repeat", type=int, default=0,
@@ -32,6 +46,9 @@ def main():
     ap.add_argument("--iters", type=int, default=3)
     ap.add_argument("--flush", action="store_true", help="write 256 MB between iterations (evict L2)")
     a = ap.parse_args()
+    if a.what == "case":
+        run_case(a.name, a.iters)
+        return
     if a.sweep is not None:
         layer = wl.make_sweep_layer(a.sweep[0], a.sweep[1], m=a.rows or 32768, n=a.cols or 32768)
     else:
