@@ -30,7 +30,8 @@
 // take units and column ranges in turn, so that consecutive slots come from different groups.
 //
 // Every wait on an mbarrier is bounded; a wait that gives up sets SQNN_E_TIMEOUT in the status word and
-// makes all roles leave their loops, so the kernel always frees its tensor memory and returns.
+// makes all roles leave their loops; after a bounded wait for the copies and MMAs in flight the kernel frees its tensor
+// memory and returns.
 #include "sqnn_launch.h"
 #include "sqnn_tc.cuh"
 
@@ -173,12 +174,13 @@ __global__ void __launch_bounds__(threads_of(UNITS), 1)
 k_decode_mma(const __grid_constant__ CUtensorMap xmap, const MmaArgs M)
 {
     extern __shared__ __align__(16) uint8_t smem_raw[];
-    __shared__ uint64_t bars[2 * MAX_UNITS * MAX_SLOTS + 2 * MAX_XSTAGES + 2];
+    __shared__ uint64_t bars[2 * MAX_UNITS * MAX_SLOTS + 2 * MAX_XSTAGES + 2 + MAX_UNITS];
     __shared__ uint32_t tmem_slot, abort_word;
     volatile uint32_t *abort_flag = &abort_word;
     // barriers by shared address: barrier i of a kind is 8 i bytes further on
     const uint32_t full_a = smem_addr(bars), empty_a = full_a + 8 * MAX_UNITS * MAX_SLOTS, full_x = empty_a + 8 * MAX_UNITS * MAX_SLOTS;
     const uint32_t empty_x = full_x + 8 * MAX_XSTAGES, accum = empty_x + 8 * MAX_XSTAGES, acc_free = accum + 8;
+    const uint32_t mma_over = acc_free + 8;                      // per unit, after a timeout: its MMAs are over
     const uint32_t x_sa = (smem_addr(smem_raw) + 1023u) & ~1023u;
     const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     constexpr uint32_t units = UNITS, PHASES = phases_of(UNITS), groups = units * PHASES;
@@ -195,6 +197,7 @@ k_decode_mma(const __grid_constant__ CUtensorMap xmap, const MmaArgs M)
         if (lane == 31) {
             mbar_init(accum, units);
             mbar_init(acc_free, 4 * groups);
+            for (uint32_t u = 0; u < units; ++u) mbar_init(mma_over + 8 * u, 1);
             abort_word = 0;
         }
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -369,6 +372,17 @@ leave:
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (*abort_flag) {                                           // (the same for all: nobody waits any more)
+        // tensor and shared memory must outlive the MMAs that were issued
+        if (warp > 4 * groups) {
+            const uint32_t over = mma_over + 8 * (warp - (4 * groups + 1));
+            mma_commit(over);
+            mbar_drain(over, 0, M.wait_limit);
+        }
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+    }
     if (warp == 4 * groups + 1) tmem_dealloc(tmem_base, 512);
 }
 
