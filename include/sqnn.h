@@ -344,7 +344,7 @@ int sqnn_store_probe(void *d_out, size_t bytes, uint32_t chunk_bytes, void *cuda
 
 /* For the library's own tests (the paper has no counterpart; not meant for applications).  Bit 0 of
  * `flags` makes the loader role of the tensor-core kernel for large batches issue no loads, bit 1 the MMA
- * role of the one for small batches no MMAs, bit 2 the walk over care bits no bulk copies, so that the
+ * role of the one for small batches report no completion, bit 2 the walk over care bits no bulk copies, so that the
  * bounded waits of what comes after them run out: the kernel then reports 6 (= -SQNN_E_TIMEOUT)
  * through d_status, frees what it holds and returns; Y is left incomplete.  wait_limit_cycles is the number of SM clock cycles such a wait may
  * take (0 = the default, one to two seconds).  Applies to calls made

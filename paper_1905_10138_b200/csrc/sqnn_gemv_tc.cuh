@@ -20,8 +20,8 @@
 // unit is cheaper (LSTM-like layer 4096 x 8192, two planes, batch 1: 14.5 us against 15.4; 2048 x 16384: 14.5 against
 // 15.6).  An even number that is none costs two or four passes of the same banks, less than another unit of
 // expansion would: 16384 x 2048, two planes, batch 8 21.9 us with three units and 18.7 with two, 32736 x 1025
-// 35.9 and 30.0, 8192 x 4096 19.6 (five) and 17.8 (four), 2730 x 12288 32.8 (13) and 31.4 (12).  Sums over the 8 ranges (shuffles) and the four groups (shared
-// memory) have a fixed order: results are bit-identical from run to run.
+// 35.9 and 30.0, 8192 x 4096 19.6 (five) and 17.8 (four), 2730 x 12288 32.8 (13) and 31.4 (12).  Sums over the 8
+// ranges (shuffles) and the four groups (shared memory) have a fixed order: results are bit-identical from run to run.
 //
 // Every wait on an mbarrier is bounded.  An expander warp whose wait gives up sets SQNN_E_TIMEOUT in the status word,
 // makes the arrivals its MMA warp still counts on and leaves its loop; the MMA warp reaches the end of its list, and
@@ -29,7 +29,7 @@
 // between the two only count: an arrival for a slot's next use while another warp had not yet arrived for the one
 // before would complete the wrong one, and the MMA warp would wait for good; so the late arrivals follow the number
 // of slots the MMA warp has taken.  (mbarriers with bounded waits between the two would need no such care, but FC6
-// batch 1 takes 9.8 us with them against 9.5, 3001 x 4099 with four fp32 vectors 16.9 against 16.3.)
+// batch 1 takes 9.8 us with them against 9.5, 3001 x 4099 with four fp32 vectors 16.9 against 16.2.)
 //
 // Bound: integer instructions of the expansion (1.4 per weight and plane, against 42 per unpruned weight of the
 // walk over care bits in sqnn_gemv.cuh, 3.8 per weight at 9 % density) and the latency of the block's phases
@@ -62,7 +62,7 @@ struct TcArgs {
     uint32_t slots;               // A slots (64 columns) per group: 1 or 2
     uint32_t alpha_words, part_words;
     uint32_t x_vec;               // rows of X start on 16-byte boundaries
-    uint32_t skip_mma;            // test only: the MMA warps issue nothing
+    uint32_t unheard;             // test only: completions are reported to barriers this far past the real ones (else 0)
     uint64_t wait_limit;          // cycles a bounded wait may take
 };
 
@@ -185,7 +185,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 k_gemv_tc(const TcArgs g)
 {
     extern __shared__ __align__(16) uint32_t smem[];
-    __shared__ uint64_t bars[4 * TC_GROUPS];              // per group: two A slots free, accumulator complete; all MMAs over (after a timeout)
+    // per group: two A slots free, accumulator complete; then per group: all MMAs over (after a timeout); then for tests
+    // the first three again, where nobody waits
+    __shared__ uint64_t bars[7 * TC_GROUPS];
     __shared__ volatile uint32_t taken_s[TC_GROUPS];      // A slots the group's MMA warp has taken
     __shared__ uint32_t tmem_slot, abort_word;
     constexpr uint32_t PIECES = sizeof(XT) == 4 ? 3 : 1;
@@ -215,7 +217,7 @@ k_gemv_tc(const TcArgs g)
     const bool holder = warp == nwarps - 1;
     if (holder) tmem_alloc(&tmem_slot, 512);
     if (warp == nwarps - 2) {
-        if (lane < 4 * TC_GROUPS) mbar_init(bars_sa + 8 * lane, 1);
+        if (lane < 7 * TC_GROUPS) mbar_init(bars_sa + 8 * lane, 1);
         if (lane < TC_GROUPS) taken_s[lane] = 0;
         if (lane == 0) abort_word = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -223,6 +225,7 @@ k_gemv_tc(const TcArgs g)
     wait_prior_grid();
     if (holder) launch_dependents();
     uint32_t slot_seq = 0, parts_done = 0;                       // per group: A slots filled, accumulators read
+    uint32_t gave_up = 0;                                        // a wait of this warp
     bool first = true;
 
     for (uint64_t ra = row0; ra < row_end; ra += g.rows_per_chunk) {
@@ -384,20 +387,14 @@ k_gemv_tc(const TcArgs g)
                 }
                 goto pass_over;
             late:
+                gave_up = 1;
                 arrive_for_the_rest(taken_s + grp, 1 + 2 * grp, slot_mask, slot_seq, seq_end, g.wait_limit);
             } else {
                 // the group's MMA warp: one slot at a time, in the order they are filled
                 const uint32_t idesc = instr_desc_bf16(g.N);
                 const uint64_t x_desc0 = smem_desc_sw128(x_sa);
                 const uint32_t box_step = g.N * 128 >> 4;
-                if (g.skip_mma) {
-                    for (uint32_t k = 0; k < 2 * (u_end - u_begin); ++k) {
-                        named_sync(1 + 2 * grp + (slot_seq & slot_mask));
-                        ++slot_seq;
-                        if (lane == 0) taken_s[grp] = slot_seq;
-                    }
-                }
-                for (uint32_t u = g.skip_mma ? u_end : u_begin; u < u_end;) {
+                for (uint32_t u = u_begin; u < u_end;) {
                     const uint32_t it = u / g.units, t0 = u - it * g.units;
                     const uint32_t len = min(g.units - t0, u_end - u);
                     for (uint32_t k = 0; k < 2 * len; ++k, ++slot_seq) {
@@ -405,15 +402,14 @@ k_gemv_tc(const TcArgs g)
                         named_sync(1 + 2 * grp + slot);
                         if (lane == 0) taken_s[grp] = slot_seq + 1;
                         tc_fence_after();
-                        mma_slot<4>(d_tmem, a_tmem + slot * 32, x_desc0 + (2 * t0 + k) * box_step, idesc, k, free_a + 8 * slot, 0);
+                        mma_slot<4>(d_tmem, a_tmem + slot * 32, x_desc0 + (2 * t0 + k) * box_step, idesc, k, free_a + g.unheard + 8 * slot, 0);
                     }
-                    mma_commit(done);
+                    mma_commit(done + g.unheard);
                     u += len;
                 }
             }
         pass_over:
-            __syncthreads();
-            const uint32_t gave_up = *abort_flag;                // (no role sets it between this barrier and the next)
+            if (__syncthreads_or(gave_up)) goto quit;
             for (uint32_t q = warp; q < g.bt && bc + q < g.batch; q += nwarps)
                 for (uint32_t rl = lane; rl < nrows; rl += 32) {
                     float sum = 0.0f;
@@ -422,17 +418,18 @@ k_gemv_tc(const TcArgs g)
                     if ((__float_as_uint(sum) & 0x7f800000u) == 0x7f800000u)
                         sum = tc_walk<XT>(g, reinterpret_cast<const XT *>(g.x) + (int64_t)(bc + q) * g.ldx, mask_s, bits_s,
                                           alpha_s + rl * n_q, (uint32_t)((ra + rl) * n - gw0 * 32));
-                    if (!gave_up) g.y[(int64_t)(bc + q) * g.ldy + (int64_t)(ra + rl)] = sum;
+                    g.y[(int64_t)(bc + q) * g.ldy + (int64_t)(ra + rl)] = sum;
                 }
-            if (gave_up) goto leave;
         }
     }
-leave:
-    if (*abort_flag && warp >= 4 * TC_GROUPS) {                  // tensor and shared memory must outlive the MMAs
+    goto leave;
+quit:
+    if (warp >= 4 * TC_GROUPS) {                                 // tensor and shared memory must outlive the MMAs
         const uint32_t over = bars_sa + 8 * (3 * TC_GROUPS + warp - 4 * TC_GROUPS);
         mma_commit(over);
         mbar_drain(over, 0, g.wait_limit);
     }
+leave:
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -460,7 +457,7 @@ inline int launch_gemv_tc(const DecodeArgs &A, const TcPlan &plan, const uint64_
     g.bt = plan.bt; g.N = plan.N; g.slots = plan.slots;
     g.region_words = plan.region_words; g.alpha_words = plan.alpha_words; g.part_words = plan.part_words;
     const DebugKnobs dbg = debug_knobs();
-    g.skip_mma = (dbg.flags & 2u) ? 1u : 0u;
+    g.unheard = (dbg.flags & 2u) ? 8 * 4 * TC_GROUPS : 0u;
     g.wait_limit = dbg.wait_cycles ? dbg.wait_cycles : TC_WAIT_LIMIT;
     g.x_vec = (((uintptr_t)d_x & 15) == 0 && (ldx * (int64_t)sizeof(XT)) % 16 == 0) ? 1u : 0u;
     return n % 128 == 0 ? launch_kernel(k_gemv_tc<N_OUT, N_IN, XT, true>, plan.grid, TC_THREADS, plan.smem, st, g)

@@ -491,7 +491,7 @@ int mma_dispatch(const sqnn_desc *desc, const DecodeArgs &A0, const uint64_t *d_
 }  // namespace sqnn
 
 // For the library's own tests: bit 0 of `flags` makes the large-batch kernel's loader issue no loads, bit 1 the
-// small-batch kernel's MMA warps no MMAs, bit 2 the walk no bulk copies, so that the bounded waits of the roles behind them run out;
+// small-batch kernel's MMA warps report no completion, bit 2 the walk no bulk copies, so that the bounded waits of the roles behind them run out;
 // wait_limit_cycles (0 = the kernel's default, one or two seconds) is the number of clock cycles such a wait may take.  Affects calls made after it; not meant for applications.
 extern "C" void sqnn_set_debug_flags(uint32_t flags, uint64_t wait_limit_cycles)
 {

@@ -342,7 +342,7 @@ def sqnn_store_probe(d_out, chunk_bytes: int = 3200, stream=None):
 
 def sqnn_set_debug_flags(flags: int, wait_limit_cycles: int = 0) -> None:
     """Test knob: bit 0 = the large-batch kernel's loader issues no loads, bit 1 = the small-batch kernel's MMA
-    warps issue nothing, bit 2 = the walk over care bits issues no bulk copies; wait_limit_cycles bounds their waits."""
+    warps report no completion, bit 2 = the walk over care bits issues no bulk copies; wait_limit_cycles bounds their waits."""
     lib().sqnn_set_debug_flags(int(flags), int(wait_limit_cycles))
 
 

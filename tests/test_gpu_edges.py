@@ -68,7 +68,7 @@ FORMS = [
 
 @pytest.mark.parametrize("case", FORMS, ids=lambda c: "x".join(map(str, c)))
 def test_small_batch_product_in_the_form_that_the_rule_picks(case):
-    """Which form ran: with the library's test knob the tensor-core form issues no MMAs and reports a timeout."""
+    """Which form ran: with the library's test knob the tensor-core form hears of no completion and reports a timeout."""
     import torch
     n_out, n_in, m, n, keep, n_q, x_dtype, batch, walk = case
     layer = generic_layer(n_out, n_in, m, n, keep, 56, n_q=n_q)

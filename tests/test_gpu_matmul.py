@@ -207,7 +207,7 @@ def test_a_bounded_wait_that_runs_out_reports_a_timeout_and_the_kernel_returns()
 
 @pytest.mark.parametrize("dtype,batch", [("bf16", 1), ("bf16", 15), ("f32", 9)])      # one, two and three passes
 def test_a_bounded_wait_of_the_small_batch_kernel_that_runs_out_reports_a_timeout(dtype, batch):
-    """With the library's test knob the MMA warps issue nothing: slots are never freed and accumulators never complete,
+    """With the library's test knob the MMA warps report no completion: slots are never freed, accumulators never complete,
     the expanders' waits run out after about a millisecond, the kernel reports 6 (-SQNN_E_TIMEOUT), stores no
     result and returns; the same call made normally right afterwards is correct."""
     import torch
