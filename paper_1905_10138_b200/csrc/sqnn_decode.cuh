@@ -51,6 +51,7 @@ struct ClearArgs {
     uint64_t m;
     int64_t ldy;
     uint32_t batch;
+    uint64_t per_block;    // elements a block clears, counted without the gaps between rows (set by the launcher)
 };
 
 // Programmatic dependent launch.  A kernel of this library may be scheduled before the kernel queued ahead of

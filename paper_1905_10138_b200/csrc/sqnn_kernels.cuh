@@ -59,32 +59,35 @@ inline uint32_t decode_bits_table_words(const DecodeArgs &A, bool rep)
 }
 // ONE_PLANE: the layer has a single plane (its stream pointers are then kernel constants instead of
 // being looked up by a plane index in every step).
+//
+// A small layer (the first half of a product with a batch, a tile or two per warp) is all latency.  What depends on
+// the arguments alone is worked out before the wait for the grid ahead or comes from the launcher; the first fetches go out
+// before tables and clearing; and a warp without a next tile does not take delivery of its patch entries
+// before it expands.
+struct BitsArgs {
+    uint32_t live;         // tiles that hold at least one real word, per plane
+    uint32_t full_tiles;   // tiles before this one lie wholly inside the plane and end on a whole word
+};
 template <int N_OUT, int N_IN, bool SINK, bool ONE_PLANE, bool REP>
 __global__ void __launch_bounds__(DECODE_BITS_THREADS, 1)
-k_decode_bits(DecodeArgs A, uint64_t *__restrict__ out, const ClearArgs clear)
+k_decode_bits(DecodeArgs A, uint64_t *__restrict__ out, const ClearArgs clear, const BitsArgs B)
 {
     extern __shared__ __align__(16) uint32_t smem[];
-    wait_prior_grid();
-    launch_dependents();
-    uint32_t tab_words_s;
-    if constexpr (N_OUT != 0 && REP) {
-        tab_words_s = table_words_replicated(N_OUT, N_IN);       // filled below, after the first fetches are out
-    } else {
-        tables_request(A, smem);
-        tab_words_s = A.tab_words;
-    }
     const uint32_t W = words_per_lane<N_OUT>(A);
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    // the tables: replicated ones are filled below, after the first fetches are out
+    const uint32_t tab_words_s = N_OUT != 0 && REP ? table_words_replicated(N_OUT, N_IN) : A.tab_words;
     uint32_t *region = smem + tab_words_s + warp * 32 * W;
     const uint64_t tail_bits = A.mn & 63;
-    // tiles that hold at least one real word, per plane (the launcher keeps the count below 2^31)
-    const uint32_t live = (uint32_t)((A.words64 + 16 * W - 1) / (16 * W));
-    // tiles before this one lie wholly inside the plane and end on a whole word
-    const uint32_t full_tiles = (uint32_t)(A.words64 / (16 * W)) -
-                                ((tail_bits != 0 && A.words64 % (16 * W) == 0) ? 1u : 0u);
+    const uint32_t live = B.live, full_tiles = B.full_tiles;
     const uint32_t stride = gridDim.x * nwarps;
-    const TilePos p_first = advance(TilePos{0u, 0u}, blockIdx.x * nwarps + warp, live, A.n_q);
+    TilePos p_first = advance(TilePos{0u, 0u}, blockIdx.x * nwarps + warp, live, A.n_q);
+    const uint64_t clear_lo = blockIdx.x * clear.per_block;
     uint64_t sink = 0;
+    p_first.plane = settle(p_first.plane);
+    p_first.tile = settle(p_first.tile);
+    wait_prior_grid();
+    launch_dependents();
 
     auto write_out = [&](TilePos p) {
         uint64_t *pbase = out + (uint64_t)p.plane * A.words64;
@@ -105,19 +108,21 @@ k_decode_bits(DecodeArgs A, uint64_t *__restrict__ out, const ClearArgs clear)
         }
     };
 
-    if (clear.batch) {
-        // every block clears a run of Y's elements (counted without the gaps between rows)
-        const uint64_t total = clear.m * clear.batch, per = (total + gridDim.x - 1) / gridDim.x;
-        const uint64_t lo = blockIdx.x * per, hi = lo + per < total ? lo + per : total;
+    // every block clears a run of Y's elements
+    auto clear_y = [&] {
+        const uint64_t total = clear.m * clear.batch;
+        if (clear_lo >= total) return;
+        const uint32_t count = (uint32_t)min(clear.per_block, total - clear_lo);
         if (clear.ldy == (int64_t)clear.m) {
-            for (uint64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) clear.y[i] = 0.0f;
+            float *y = clear.y + clear_lo;
+            for (uint32_t i = threadIdx.x; i < count; i += blockDim.x) y[i] = 0.0f;
         } else {
-            for (uint64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+            for (uint64_t i = clear_lo + threadIdx.x; i < clear_lo + count; i += blockDim.x) {
                 const uint64_t b = i / clear.m;
                 clear.y[(int64_t)b * clear.ldy + (int64_t)(i - b * clear.m)] = 0.0f;
             }
         }
-    }
+    };
     auto plane_of = [&](const TilePos &p) -> const PlanePtrs & { return ONE_PLANE ? A.pl[0] : A.pl[p.plane]; };
     if constexpr (N_OUT != 0) {
         using S = Shape<N_OUT, N_IN>;
@@ -131,20 +136,24 @@ k_decode_bits(DecodeArgs A, uint64_t *__restrict__ out, const ClearArgs clear)
         if (pa.plane < A.n_q) { fetch_seeds<N_OUT, N_IN>(plane_of(pa), pa.tile, lane, sa); ra = fetch_run(plane_of(pa), pa.tile); }
         if (pb.plane < A.n_q) { fetch_seeds<N_OUT, N_IN>(plane_of(pb), pb.tile, lane, sb); rb = fetch_run(plane_of(pb), pb.tile); }
         if constexpr (REP) tables_replicate<entry_words_padded(N_OUT)>(A, smem);
+        else tables_request(A, smem);
+        if (clear.batch) clear_y();
         if (pa.plane < A.n_q) fetch_patches(A, plane_of(pa), ra, lane, wa);
         if constexpr (!REP) cp_async_wait_all();
         __syncthreads();                                 // the tables are in place
         auto step = [&](TilePos &p0, TileSeeds<N_OUT, N_IN> &s0, TileRun &r0, uint32_t (&w0)[PATCH_AHEAD],
                         TilePos &p1, TileRun &r1, uint32_t (&w1)[PATCH_AHEAD],
                         TilePos &p2, TileSeeds<N_OUT, N_IN> &s2, TileRun &r2) {
-            // everything this step consumes was requested at least a step ago: take delivery of it now,
-            // before the loads of this step are issued
+            if (p1.plane < A.n_q) {
+                // everything this step consumes was requested at least a step ago: take delivery of it now,
+                // before the loads of this step are issued
 #pragma unroll
-            for (uint32_t k = 0; k < S::NRAW; ++k) s0.raw[k] = settle(s0.raw[k]);
+                for (uint32_t k = 0; k < S::NRAW; ++k) s0.raw[k] = settle(s0.raw[k]);
 #pragma unroll
-            for (uint32_t k = 0; k < PATCH_AHEAD; ++k) w0[k] = settle(w0[k]);
-            r0.base = settle(r0.base); r0.end = settle(r0.end);
-            r1.base = settle(r1.base); r1.end = settle(r1.end);
+                for (uint32_t k = 0; k < PATCH_AHEAD; ++k) w0[k] = settle(w0[k]);
+                r0.base = settle(r0.base); r0.end = settle(r0.end);
+                r1.base = settle(r1.base); r1.end = settle(r1.end);
+            }
             p2 = advance(p1, stride, live, A.n_q);
             if (p1.plane < A.n_q) fetch_patches(A, plane_of(p1), r1, lane, w1);
             if (p2.plane < A.n_q) { fetch_seeds<N_OUT, N_IN>(plane_of(p2), p2.tile, lane, s2); r2 = fetch_run(plane_of(p2), p2.tile); }
@@ -163,6 +172,8 @@ k_decode_bits(DecodeArgs A, uint64_t *__restrict__ out, const ClearArgs clear)
             }
         }
     } else {
+        tables_request(A, smem);
+        if (clear.batch) clear_y();
         cp_async_wait_all();
         __syncthreads();
         for (TilePos p = p_first; p.plane < A.n_q; p = advance(p, stride, live, A.n_q)) {
@@ -478,10 +489,14 @@ inline int launch_decode(const DecodeArgs &A, sqnn_out_mode mode, const uint64_t
         warps = spread_warps(live * A.n_q, warps);
         smem = tab + warps * per_warp;
         const uint32_t grid = grid_for(live * A.n_q, warps, 1);
+        const uint64_t whole = A.words64 / (16ull * A.W);
+        const BitsArgs B{(uint32_t)live, (uint32_t)(whole - (A.mn % 64 != 0 && whole * 16 * A.W == A.words64 ? 1 : 0))};
+        ClearArgs c = clear;
+        c.per_block = (clear.m * clear.batch + grid - 1) / grid;
 #define SQNN_BITS_LAUNCH2(SINKV, ONEV, REPV)                                                             \
     do {                                                                                                 \
         auto k = k_decode_bits<N_OUT, N_IN, SINKV, ONEV, REPV>;                                          \
-        return launch_kernel(k, grid, warps * 32, smem, st, A, (uint64_t *)d_out, clear);                \
+        return launch_kernel(k, grid, warps * 32, smem, st, A, (uint64_t *)d_out, c, B);                 \
     } while (0)
 #define SQNN_BITS_LAUNCH(SINKV, ONEV)                                                                    \
     do {                                                                                                 \

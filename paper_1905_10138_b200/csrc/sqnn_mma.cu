@@ -477,7 +477,7 @@ int mma_dispatch(const sqnn_desc *desc, const DecodeArgs &A0, const uint64_t *d_
         return SQNN_E_CUDA;
 
     // stage 1: the decode kernel writes the planes as packed bits into the workspace and clears Y
-    const int rc = decode_bits_dispatch(A0, d_workspace, ClearArgs{d_y, desc->m, ldy, batch}, st);
+    const int rc = decode_bits_dispatch(A0, d_workspace, ClearArgs{d_y, desc->m, ldy, batch, 0}, st);
     if (rc != SQNN_OK) return rc;
 #define SQNN_MMA_PICK(U, COLS) (aligned ? k_decode_mma<U, true, COLS> : k_decode_mma<U, false, COLS>)
     auto k = units == 1   ? SQNN_MMA_PICK(1, 64)
