@@ -1,25 +1,26 @@
 // Exhaustive seed search on the device (Section 5.2): for every slice of every plane the seed with the fewest
 // wrong care bits among all 2^n_in is found (the smallest seed among equals).
 //
-// The seeds are not tried one by one.  Let r_j be the rows of M at the slice's care positions and b_j the
-// wanted bits.  Elimination in ascending position makes some rows pivots (r of them, r = the rank); every
-// other row is the sum of pivot rows in a known subset.  A seed is then a choice of the set e of pivots it
-// gets wrong: which dependent rows are wrong follows (their syndrome s plus the columns C_i of the pivots in
-// e), and so does the smallest seed with exactly these errors: the one with all free variables 0 when every
-// pivot column is the lowest possible one, which is linear in the pivots' bits (columns Q_i).  So with
-// V_i = C_i << 20 | Q_i the search is
+// The seeds are not tried one by one.  Column c of M, restricted to the slice's care positions, is a bit vector v_c; a
+// seed is a choice of columns and its error vector is (wanted bits) ^ xor of the chosen v_c.  Column operations bring
+// the v_c into reduced form: in ascending order, a column that is not zero by then takes its lowest bit as its pivot, which is
+// removed from all other columns and from the wanted bits, and t_c keeps the seed that belongs to v_c.  What is
+// left of the wanted bits, E, is the error vector of the seed that gets every pivot bit right, and a set e of wrong pivots has
 //
-//     min over e of  (|e| + |C part|) << 20 | Q part,   V(e) = V_0 ^ xor of V_i, i in e,
+//     key(e) = popcount(E ^ xor of v_c, c in e) << 20 | seed(E) ^ xor of t_c, c in e,      at least |e| errors.
 //
-// and e can be taken in the order of its size: once the best count is B, sizes above B cannot matter.  Almost
-// all slices are done after sizes 0 (consistent: no wrong bit), 1 and 2: about 80 candidates for r = 12
-// instead of 4096.  One thread per slice does that much; slices that need larger sets are finished by the whole
-// warp: sets of three (which decide nearly all of them), then all 2^r sets in Gray-code order; slices with more
-// dependent rows than C has bits for by trying all seeds.
+// The search is the minimum of the keys, taken in the order of |e|: once the best count is B, sizes above B cannot
+// matter.  (Ties go to the smallest seed.  Pivot columns are the lowest possible ones, so the seed with all other bits 0, which
+// the keys hold, is the smallest of those with the same errors.)  Sizes 0 and 1 are done by a thread per slice and decide
+// 92 % of them; of the rest the warp finishes one slice after the other, the lanes sharing the pairs, then, for one
+// slice in a hundred, the triples, then all 2^n_in sets in Gray-code order.
 //
-// Bound: integer instructions.  600 000 slices of 60 x 12 (20 % care bits, two planes of 6000 x 3000) take 127 us, 79 M
-// warp instructions with 18.5 of 32 lanes active: the loop over a slice's care bits takes as many turns as the lane with
-// the most of them needs.  (Trying all 2^12 seeds of every slice took 2540 us.)
+// The care positions of a slice are squeezed together first: up to 32 of them make one word per column, up to 64 two, whatever
+// n_out is.  A step takes each lane's next care position; its row of M, with the bits of four columns in the four
+// bytes of a word, is added to the columns' bytes shifted by the step's number, so that eight steps fill a byte of every column with
+// three additions each, for 12 columns.  Slices with more care bits than that try all seeds.
+//
+// Bound: integer instructions.
 #include "sqnn_launch.h"
 
 #include <cuda_runtime.h>
@@ -51,7 +52,7 @@ SQNN_DEV uint32_t bits32_at(const uint64_t *__restrict__ v, uint64_t p, uint64_t
 }
 
 constexpr uint32_t SEARCH_THREADS = 128;
-constexpr uint32_t MAX_DEP = 32;                          // dependent rows a word C has room for
+constexpr uint32_t MAX_CARE = 64;                         // care bits the vectors have room for
 
 SQNN_DEV uint32_t warp_min(uint32_t v)
 {
@@ -91,68 +92,235 @@ SQNN_DEV uint32_t try_all_seeds(const uint32_t (*cols)[NW], uint32_t n_in, const
     return warp_min(best);
 }
 
-// A candidate's key: number of wrong care bits, then the seed.
-SQNN_DEV uint32_t set_key(uint32_t size, uint32_t c, uint32_t q) { return ((size + (uint32_t)__popc(c)) << 20) + q; }
+// The reduced columns of one slice per thread, for the slices the whole warp finishes: v_c and t_c.
+template <int NI, int KW>
+struct Columns {
+    uint32_t v[KW][NI][SEARCH_THREADS], t[NI][SEARCH_THREADS];
+};
+// A candidate: an error vector and its seed.
+template <int KW>
+struct Candidate {
+    uint32_t e[KW], seed;
+    SQNN_DEV uint32_t key() const
+    {
+        uint32_t wrong = 0;
+#pragma unroll
+        for (int k = 0; k < KW; ++k) wrong += (uint32_t)__popc(e[k]);
+        return (wrong << 20) + seed;
+    }
+    template <int NI, int CW>
+    SQNN_DEV void add(const Columns<NI, CW> &col, uint32_t c, uint32_t slot)
+    {
+#pragma unroll
+        for (int k = 0; k < KW; ++k) e[k] ^= col.v[k][c][slot];
+        seed ^= col.t[c][slot];
+    }
+};
 
-// The whole warp tries all 2^r sets of wrong pivots of one slice (v: its (C_i, Q_i), one every SEARCH_THREADS).
-SQNN_DEV uint32_t try_all_sets(const uint2 *v, uint2 v0, uint32_t r, uint32_t lane)
+// The whole warp tries all 2^n_in sets of columns of one slice: the lanes split them by the top bits.
+template <int KW, int NI, int CW>
+SQNN_DEV uint32_t try_all_sets(const Columns<NI, CW> &col, uint32_t slot, Candidate<KW> x, uint32_t n_in, uint32_t lane)
 {
-    const uint32_t low_bits = r > 5 ? r - 5 : 0, lanes_used = r >= 5 ? 32u : (1u << r);
+    const uint32_t low_bits = n_in > 5 ? n_in - 5 : 0, lanes_used = n_in >= 5 ? 32u : (1u << n_in);
     uint32_t best = 0xffffffffu;
     if (lane < lanes_used) {
-        const uint32_t top = lane << low_bits, size0 = (uint32_t)__popc(lane);
-        uint32_t c = v0.x, q = v0.y;
-        for (uint32_t t = low_bits; t < r; ++t)
-            if ((top >> t) & 1u) { c ^= v[t * SEARCH_THREADS].x; q ^= v[t * SEARCH_THREADS].y; }
+        for (uint32_t c = low_bits; c < n_in; ++c)
+            if ((lane >> (c - low_bits)) & 1u) x.add(col, c, slot);
         const uint32_t count = 1u << low_bits;
         for (uint32_t i = 0; i < count; ++i) {
-            if (i != 0) {
-                const uint2 w = v[((uint32_t)__ffs((int)i) - 1u) * SEARCH_THREADS];
-                c ^= w.x;
-                q ^= w.y;
-            }
-            best = min(best, set_key(size0 + (uint32_t)__popc(i ^ (i >> 1)), c, q));
+            if (i != 0) x.add(col, (uint32_t)__ffs((int)i) - 1u, slot);
+            best = min(best, x.key());
         }
     }
     return warp_min(best);
 }
 
-// The whole warp tries all sets of three wrong pivots: the lanes split the pairs, each walks the third.
-SQNN_DEV uint32_t try_triples(const uint2 *v, uint2 v0, uint32_t r, uint32_t lane)
+// The pair with number p of the list (1,0), (2,0), (2,1), (3,0), ..: the larger one, and the smaller one from it.  (At the
+// first pair of a larger one, 1 + 8 p is a square; p + 1/8 leaves room for the approximation's error, p < 190.)
+SQNN_DEV uint32_t pair_high(uint32_t p)
 {
-    uint32_t best = 0xffffffffu;
-    for (uint32_t p = lane; p < r * (r - 1) / 2; p += 32) {
-        const uint32_t i = (uint32_t)((1.0f + sqrtf(1.0f + 8.0f * (float)p)) * 0.5f), h = p - i * (i - 1) / 2;     // h < i
-        const uint2 a = v[i * SEARCH_THREADS], b = v[h * SEARCH_THREADS];
-        const uint32_t c = v0.x ^ a.x ^ b.x, q = v0.y ^ a.y ^ b.y;
-        for (uint32_t g = 0; g < h; ++g) {
-            const uint2 w = v[g * SEARCH_THREADS];
-            best = min(best, set_key(3u, c ^ w.x, q ^ w.y));
-        }
+    float root;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(root) : "f"(2.0f + 8.0f * (float)p));
+    return (uint32_t)((1.0f + root) * 0.5f);
+}
+SQNN_DEV uint32_t pair_low(uint32_t p, uint32_t high) { return p - high * (high - 1) / 2; }
+
+// The whole warp finishes one slice whose best set of at most one column has two errors or more: pairs, where three errors or
+// more are left triples (the lanes split the pairs, each walks the third column), then all sets.
+template <int KW, int NI, int CW>
+SQNN_DEV uint32_t try_larger_sets(const Columns<NI, CW> &col, uint32_t slot, const Candidate<KW> &x0, uint32_t best, uint32_t n_in, uint32_t lane)
+{
+    const uint32_t pairs = n_in * (n_in - 1) / 2;
+    for (uint32_t p = lane; p < pairs; p += 32) {
+        const uint32_t i = pair_high(p);
+        Candidate<KW> x = x0;
+        x.add(col, i, slot);
+        x.add(col, pair_low(p, i), slot);
+        best = min(best, x.key());
     }
-    return warp_min(best);
+    best = warp_min(best);
+    if ((best >> 20) > 2u) {
+        for (uint32_t p = lane; p < pairs; p += 32) {
+            const uint32_t i = pair_high(p), h = pair_low(p, i);
+            Candidate<KW> x = x0;
+            x.add(col, i, slot);
+            x.add(col, h, slot);
+            for (uint32_t g = 0; g < h; ++g) {
+                Candidate<KW> y = x;
+                y.add(col, g, slot);
+                best = min(best, y.key());
+            }
+        }
+        best = warp_min(best);
+        if ((best >> 20) > 3u) best = min(best, try_all_sets<KW>(col, slot, x0, n_in, lane));
+    }
+    return best;
 }
 
-// NI >= n_in.  Rows and bookkeeping of the elimination sit in registers; every loop over columns or pivots has a
-// fixed length, and a column without a pivot row or a pivot that does not exist is a zero that changes nothing
-// (a set with such a pivot only counts one error more than the set without it), so that the lanes of a warp,
-// which have different numbers of care bits and pivots, stay together.
+// A lane's care positions in ascending order.  Up to two words sit in registers, more in the lane's slots of shared memory.
+template <int NW>
+struct CareBits {
+    uint32_t care, want, base, care1, want1;
+    const uint32_t *rest;                                                 // care and want of word k: 2 k, 2 k + 1
+    // Position of the next care bit, 32 * NW if there is none, and its wanted bit.
+    SQNN_DEV uint32_t next(uint32_t &bit)
+    {
+        if constexpr (NW <= 2) {
+            if (care == 0) { care = care1; want = want1; care1 = 0; base = 32 * (NW - 1); }
+        } else {
+            while (care == 0 && base < 32 * (NW - 1)) {
+                base += 32;
+                care = rest[(base / 16) * SEARCH_THREADS];
+                want = rest[(base / 16 + 1) * SEARCH_THREADS];
+            }
+        }
+        const uint32_t j = (uint32_t)__clz((int)__brev(care));            // 32 for no bit
+        bit = __funnelshift_rc(want, 0u, j) & 1u;                        // 0 for no bit
+        care &= care - 1u;
+        return base + j;
+    }
+};
+
+// The search over one slice per lane; care bits of a slice fit KW words.  rows_s: byte b of word [w][j] is bit 4 w + b
+// of row j of M.  Lanes without a slice have no care bits.
+template <int KW, int NI, int NW, int CW>
+SQNN_DEV uint32_t search_slices(const uint32_t (&rows_s)[(NI + 3) / 4][32 * NW + 1], Columns<NI, CW> &col, CareBits<NW> bits, uint32_t most,
+                                uint32_t n_in, uint32_t lane)
+{
+    constexpr int NB = (NI + 3) / 4;
+    uint32_t v[KW][NI], t[NI], e[KW], seed = 0;
+#pragma unroll
+    for (int k = 0; k < KW; ++k) {
+        e[k] = 0;
+#pragma unroll
+        for (int c = 0; c < NI; ++c) v[k][c] = 0;
+#pragma unroll 1
+        for (uint32_t byte = 0; byte < 4 && 32 * k + 8 * byte < most; ++byte) {
+            uint32_t acc[NB], wanted = 0;
+#pragma unroll
+            for (int w = 0; w < NB; ++w) acc[w] = 0;
+#pragma unroll
+            for (uint32_t half = 0; half < 2; ++half) {
+                if (half == 1 && 32 * k + 8 * byte + 4 >= most) break;
+#pragma unroll
+                for (uint32_t i = 4 * half; i < 4 * half + 4; ++i) {
+                    uint32_t bit;
+                    const uint32_t j = bits.next(bit);
+#pragma unroll
+                    for (int w = 0; w < NB; ++w) acc[w] += rows_s[w][j] << i;
+                    wanted += bit << i;
+                }
+            }
+            e[k] |= wanted << (8 * byte);
+            // byte c % 4 of acc[c / 4] becomes this byte of column c
+            const uint32_t keep = 0x3210u & ~(0xfu << (4 * byte));
+#pragma unroll
+            for (int c = 0; c < NI; ++c) v[k][c] = __byte_perm(v[k][c], acc[c / 4], keep | ((4u + c % 4) << (4 * byte)));
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < NI; ++c) t[c] = (uint32_t)c < n_in ? 1u << c : 0u;
+#pragma unroll
+    for (int c = 0; c < NI; ++c) {
+        uint32_t p[KW];                                                   // the lowest bit of column c
+        p[0] = v[0][c] & (0u - v[0][c]);
+        if constexpr (KW == 2) p[1] = v[0][c] ? 0u : v[1][c] & (0u - v[1][c]);
+        auto has = [&](uint32_t a0, uint32_t a1) {
+            if constexpr (KW == 2) return ((a0 & p[0]) | (a1 & p[KW - 1])) != 0;
+            else return (a0 & p[0]) != 0;
+        };
+        if (has(e[0], e[KW - 1])) {
+#pragma unroll
+            for (int k = 0; k < KW; ++k) e[k] ^= v[k][c];
+            seed ^= t[c];
+        }
+#pragma unroll
+        for (int d = 0; d < NI; ++d)
+            if (d != c && has(v[0][d], v[KW - 1][d])) {
+#pragma unroll
+                for (int k = 0; k < KW; ++k) v[k][d] ^= v[k][c];
+                t[d] ^= t[c];
+            }
+    }
+    Candidate<KW> x;
+    uint32_t any = 0;
+#pragma unroll
+    for (int k = 0; k < KW; ++k) { x.e[k] = e[k]; any |= e[k]; }
+    x.seed = seed;
+    uint32_t best = x.key();
+    if (any) {                                                            // sets of one
+#pragma unroll
+        for (int c = 0; c < NI; ++c) {
+            Candidate<KW> y;
+#pragma unroll
+            for (int k = 0; k < KW; ++k) y.e[k] = e[k] ^ v[k][c];
+            y.seed = seed ^ t[c];
+            best = min(best, y.key());
+        }
+    }
+    const bool open = (best >> 20) >= 2u;
+    if (open) {
+#pragma unroll
+        for (int c = 0; c < NI; ++c) {
+#pragma unroll
+            for (int k = 0; k < KW; ++k) col.v[k][c][threadIdx.x] = v[k][c];
+            col.t[c][threadIdx.x] = t[c];
+        }
+    }
+    __syncwarp();
+    for (uint32_t more = __ballot_sync(0xffffffffu, open); more; more &= more - 1u) {
+        const uint32_t src = (uint32_t)__ffs((int)more) - 1u;
+        Candidate<KW> from;
+#pragma unroll
+        for (int k = 0; k < KW; ++k) from.e[k] = __shfl_sync(0xffffffffu, e[k], src);
+        from.seed = __shfl_sync(0xffffffffu, seed, src);
+        const uint32_t found = try_larger_sets<KW>(col, (threadIdx.x & ~31u) + src, from, __shfl_sync(0xffffffffu, best, src), n_in, lane);
+        if (lane == src) best = found;
+    }
+    return best;
+}
+
+// NI >= n_in, 32 NW >= n_out.  The loops over columns have a fixed length; a column past n_in is a zero that changes nothing.
 template <int NI, int NW>
 __global__ void __launch_bounds__(SEARCH_THREADS)
 k_search_seeds(const __grid_constant__ SearchArgs S)
 {
-    __shared__ uint32_t rows_s[SQNN_MAX_N_OUT];
+    __shared__ uint32_t rows_s[(NI + 3) / 4][32 * NW + 1];                // rows past n_out are zero
     __shared__ uint32_t cols[SQNN_MAX_N_IN][NW];                          // column t of M as an n_out-bit word
-    __shared__ uint2 v_s[NI][SEARCH_THREADS];
+    __shared__ uint32_t rest_s[NW > 2 ? 2 * NW : 1][SEARCH_THREADS];
+    __shared__ Columns<NI, 2> col_s;
     wait_prior_grid();
     launch_dependents();
     const uint32_t lane = threadIdx.x & 31;
-    for (uint32_t j = threadIdx.x; j < SQNN_MAX_N_OUT; j += SEARCH_THREADS) rows_s[j] = S.rows[j] & (uint32_t)((1ull << S.n_in) - 1ull);
-    __syncthreads();
+    for (uint32_t j = threadIdx.x; j < 32 * NW + 1; j += SEARCH_THREADS) {
+        const uint32_t row = j < S.n_out ? S.rows[j] & (uint32_t)((1ull << S.n_in) - 1ull) : 0u;
+#pragma unroll
+        for (uint32_t w = 0; w < (NI + 3) / 4; ++w) rows_s[w][j] = (((row >> (4 * w)) & 0xfu) * 0x00204081u) & 0x01010101u;
+    }
     for (uint32_t i = threadIdx.x; i < S.n_in * NW; i += SEARCH_THREADS) {
         const uint32_t t = i / NW, k = i % NW;
         uint32_t w = 0;
-        for (uint32_t j = 32 * k; j < S.n_out && j < 32 * k + 32; ++j) w |= ((rows_s[j] >> t) & 1u) << (j - 32 * k);
+        for (uint32_t j = 32 * k; j < S.n_out && j < 32 * k + 32; ++j) w |= ((S.rows[j] >> t) & 1u) << (j - 32 * k);
         cols[t][k] = w;
     }
     __syncthreads();
@@ -161,7 +329,7 @@ k_search_seeds(const __grid_constant__ SearchArgs S)
     for (uint64_t job0 = (uint64_t)blockIdx.x * SEARCH_THREADS + (threadIdx.x & ~31u); job0 < total; job0 += step) {
         const uint64_t job = job0 + lane;
         const bool live = job < total;
-        uint32_t want[NW], care[NW];
+        uint32_t want[NW], care[NW], count = 0;
 #pragma unroll
         for (int k = 0; k < NW; ++k) want[k] = care[k] = 0;
         if (live) {
@@ -175,97 +343,28 @@ k_search_seeds(const __grid_constant__ SearchArgs S)
                 want[k] = bits32_at(S.planes + (uint64_t)plane * S.words64, p0 + 32 * k, limit);
             }
         }
-        // elimination: row[c] = the pivot row whose lowest set column is c, sub[c] = the original pivots it is the
-        // sum of (numbered as they come), bits = the original pivots' wanted bits, dc[i] = C_i
-        uint32_t row[NI], sub[NI], dc[NI], bits = 0, r = 0, dep = 0, syn = 0;
 #pragma unroll
-        for (int c = 0; c < NI; ++c) row[c] = sub[c] = dc[c] = 0;
+        for (int k = 0; k < NW; ++k) count += (uint32_t)__popc(care[k]);
+        const bool wide = count > MAX_CARE;
+        CareBits<NW> bits{wide ? 0u : care[0], want[0], 0u, 0u, 0u, nullptr};
+        if constexpr (NW == 2) { bits.care1 = wide ? 0u : care[1]; bits.want1 = want[1]; }
+        if constexpr (NW > 2) {
 #pragma unroll
-        for (int k = 0; k < NW; k += 2) {
-            unsigned long long left = care[k], wanted = want[k];
-            if (k + 1 < NW) {
-                left |= (unsigned long long)care[k + 1 < NW ? k + 1 : k] << 32;
-                wanted |= (unsigned long long)want[k + 1 < NW ? k + 1 : k] << 32;
+            for (int k = 0; k < NW; ++k) {
+                rest_s[2 * k][threadIdx.x] = wide ? 0u : care[k];
+                rest_s[2 * k + 1][threadIdx.x] = want[k];
             }
-            while (left) {
-                const uint32_t j = (uint32_t)__ffsll((long long)left) - 1u;
-                left &= left - 1ull;
-                uint32_t a = rows_s[32 * k + j], of = 0;
-                const uint32_t b = (uint32_t)(wanted >> j) & 1u;
-#pragma unroll
-                for (int c = 0; c < NI; ++c)
-                    if ((a >> c) & 1u) { a ^= row[c]; of ^= sub[c]; }
-                if (a) {                                                  // a new pivot
-                    const uint32_t low = a & (0u - a);
-                    of |= 1u << r;
-#pragma unroll
-                    for (int c = 0; c < NI; ++c)
-                        if (low == (1u << c)) { row[c] = a; sub[c] = of; }
-                    bits |= b << r;
-                    ++r;
-                } else {                                                  // the sum of the pivots in `of`
-                    const uint32_t bit = dep < MAX_DEP ? 1u << dep : 0u;
-                    if ((b ^ (uint32_t)__popc(bits & of)) & 1u) syn |= bit;
-#pragma unroll
-                    for (int i = 0; i < NI; ++i)
-                        if ((of >> i) & 1u) dc[i] |= bit;
-                    ++dep;
-                }
-            }
+            bits.rest = &rest_s[0][threadIdx.x];
         }
-        // reduced form: no pivot row contains another pivot's column
-#pragma unroll
-        for (int c = NI - 2; c >= 0; --c) {
-#pragma unroll
-            for (int d = c + 1; d < NI; ++d)
-                if ((row[c] >> d) & 1u) { row[c] ^= row[d]; sub[c] ^= sub[d]; }
-        }
-        uint32_t seed = 0;
-#pragma unroll
-        for (int c = 0; c < NI; ++c) seed |= ((uint32_t)__popc(bits & sub[c]) & 1u) << c;
-        uint32_t best = set_key(0u, syn, seed);
-        const bool wide = live && dep > MAX_DEP;
-        if (syn != 0 && !wide) {
-            uint32_t dq[NI];                                              // Q_i
-#pragma unroll
-            for (int i = 0; i < NI; ++i) {
-                dq[i] = 0;
-#pragma unroll
-                for (int c = 0; c < NI; ++c) dq[i] |= ((sub[c] >> i) & 1u) << c;
-                best = min(best, set_key(1u, syn ^ dc[i], seed ^ dq[i])); // one wrong pivot
-            }
-            if ((best >> 20) >= 2) {
-#pragma unroll
-                for (int i = 1; i < NI; ++i) {                            // two
-                    const uint32_t c = syn ^ dc[i], q = seed ^ dq[i];
-#pragma unroll
-                    for (int h = 0; h < i; ++h) best = min(best, set_key(2u, c ^ dc[h], q ^ dq[h]));
-                }
-            }
-            if ((best >> 20) > 2u) {
-#pragma unroll
-                for (int i = 0; i < NI; ++i) v_s[i][threadIdx.x] = make_uint2(dc[i], dq[i]);
-            }
-        }
-        __syncwarp();
-        // what is left for the whole warp: larger sets could still win or tie, or C has no room
-        uint32_t more = __ballot_sync(0xffffffffu, wide || (live && syn != 0 && (best >> 20) > 2u));
-        while (more) {
+        const uint32_t most = __reduce_max_sync(0xffffffffu, wide ? 0u : count);
+        uint32_t best = most <= 32 ? search_slices<1, NI, NW>(rows_s, col_s, bits, most, S.n_in, lane)
+                                   : search_slices<2, NI, NW>(rows_s, col_s, bits, most, S.n_in, lane);
+        for (uint32_t more = __ballot_sync(0xffffffffu, wide); more; more &= more - 1u) {
             const uint32_t src = (uint32_t)__ffs((int)more) - 1u;
-            more &= more - 1u;
-            uint32_t found;
-            if (__shfl_sync(0xffffffffu, wide ? 1u : 0u, src)) {
-                uint32_t w_s[NW], c_s[NW];
+            uint32_t w_s[NW], c_s[NW];
 #pragma unroll
-                for (int k = 0; k < NW; ++k) { w_s[k] = __shfl_sync(0xffffffffu, want[k], src); c_s[k] = __shfl_sync(0xffffffffu, care[k], src); }
-                found = try_all_seeds<NW>(cols, S.n_in, w_s, c_s, lane);
-            } else {
-                const uint2 *v = &v_s[0][(threadIdx.x & ~31u) + src];
-                const uint2 v0 = make_uint2(__shfl_sync(0xffffffffu, syn, src), __shfl_sync(0xffffffffu, seed, src));
-                const uint32_t r_src = __shfl_sync(0xffffffffu, r, src);
-                found = min(__shfl_sync(0xffffffffu, best, src), try_triples(v, v0, r_src, lane));
-                if ((found >> 20) > 3u) found = try_all_sets(v, v0, r_src, lane);
-            }
+            for (int k = 0; k < NW; ++k) { w_s[k] = __shfl_sync(0xffffffffu, want[k], src); c_s[k] = __shfl_sync(0xffffffffu, care[k], src); }
+            const uint32_t found = try_all_seeds<NW>(cols, S.n_in, w_s, c_s, lane);
             if (lane == src) best = found;
         }
         if (live) {

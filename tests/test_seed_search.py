@@ -47,7 +47,29 @@ SEARCH = [
     ("8x3", lambda: generic_layer(8, 3, 9, 77, 0.6, 32)),
     ("200x10", lambda: generic_layer(200, 10, 11, 1000, 0.1, 33)),
     ("40x14", lambda: generic_layer(40, 14, 5, 333, 0.4, 34)),
+    # one and two words of care bits side by side, more care bits than two words hold, few and many words per slice,
+    # more seed bits than positions, the smallest network, a single slice
+    ("64x11-mixed", lambda: generic_layer(64, 11, 23, 100, 0.5, 35)),
+    ("128x9-two-words", lambda: generic_layer(128, 9, 19, 201, 0.35, 36)),
+    ("200x7-wide", lambda: generic_layer(200, 7, 13, 401, 0.32, 37)),
+    ("256x12", lambda: generic_layer(256, 12, 16, 640, 0.08, 38)),
+    ("50x17", lambda: generic_layer(50, 17, 4, 251, 0.6, 39)),
+    ("7x12", lambda: generic_layer(7, 12, 9, 50, 0.6, 40)),
+    ("3x1", lambda: generic_layer(3, 1, 5, 77, 0.2, 41)),
+    ("96x10-one-slice", lambda: generic_layer(96, 10, 1, 50, 0.5, 42)),
+    ("64x10-rank-3", lambda: low_rank_layer(64, 10, 3, 43)),
 ]
+
+
+def low_rank_layer(n_out, n_in, rank, seed):
+    """A network whose columns are sums of `rank` of them, with empty columns: many seeds with the same errors."""
+    layer = generic_layer(n_out, n_in, 21, 100, 0.7, seed)
+    rng = np.random.default_rng(seed)
+    basis = layer.M[:, :rank]
+    mix = rng.integers(0, 2, (rank, n_in))
+    mix[:, [0, n_in // 2]] = 0
+    layer.M[:] = (basis @ mix % 2).astype(layer.M.dtype)
+    return layer
 
 
 @pytest.mark.gpu
