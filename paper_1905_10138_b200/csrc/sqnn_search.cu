@@ -12,8 +12,8 @@
 // The search is the minimum of the keys, taken in the order of |e|: once the best count is B, sizes above B cannot
 // matter.  (Ties go to the smallest seed.  Pivot columns are the lowest possible ones, so the seed with all other bits 0, which
 // the keys hold, is the smallest of those with the same errors.)  Sizes 0 and 1 are done by a thread per slice and decide
-// 92 % of them; of the rest the warp finishes one slice after the other, the lanes sharing the pairs, then, for one
-// slice in a hundred, the triples, then all 2^n_in sets in Gray-code order.
+// 92 % of them; of the rest the warp finishes one slice after the other, the lanes sharing the pairs and, for one slice in a
+// hundred, sets of three to five columns; what remains tries all 2^n_in sets in Gray-code order.
 //
 // The care positions of a slice are squeezed together first: up to 32 of them make one word per column, up to 64 two, whatever
 // n_out is.  A step takes each lane's next care position; its row of M, with the bits of four columns in the four
@@ -135,46 +135,73 @@ SQNN_DEV uint32_t try_all_sets(const Columns<NI, CW> &col, uint32_t slot, Candid
     return warp_min(best);
 }
 
-// The pair with number p of the list (1,0), (2,0), (2,1), (3,0), ..: the larger one, and the smaller one from it.  (At the
-// first pair of a larger one, 1 + 8 p is a square; p + 1/8 leaves room for the approximation's error, p < 190.)
-SQNN_DEV uint32_t pair_high(uint32_t p)
+// The pairs of columns, numbered (1,0), (2,0), (2,1), (3,0), ..: those below column c are the first c (c - 1) / 2.  Lane l keeps
+// the sums of pairs l, l + 32, ..  (At the first pair of a larger column, 1 + 8 p is a square; the 1 more leaves room for the
+// approximation's error, p < 190.)
+template <int NI>
+constexpr int PAIRS_PER_LANE = (NI * (NI - 1) / 2 + 31) / 32;
+template <int KW, int NI, int CW>
+SQNN_DEV Candidate<KW> pair_sum(const Columns<NI, CW> &col, uint32_t slot, Candidate<KW> x, uint32_t p)
 {
     float root;
     asm("sqrt.approx.f32 %0, %1;" : "=f"(root) : "f"(2.0f + 8.0f * (float)p));
-    return (uint32_t)((1.0f + root) * 0.5f);
+    const uint32_t high = (uint32_t)((1.0f + root) * 0.5f);
+    x.add(col, high, slot);
+    x.add(col, p - high * (high - 1) / 2, slot);
+    return x;
 }
-SQNN_DEV uint32_t pair_low(uint32_t p, uint32_t high) { return p - high * (high - 1) / 2; }
 
-// The whole warp finishes one slice whose best set of at most one column has two errors or more: pairs, where three errors or
-// more are left triples (the lanes split the pairs, each walks the third column), then all sets.
-template <int KW, int NI, int CW>
-SQNN_DEV uint32_t try_larger_sets(const Columns<NI, CW> &col, uint32_t slot, const Candidate<KW> &x0, uint32_t best, uint32_t n_in, uint32_t lane)
+// The best of all sets of MORE columns below `top` and a pair below those, added to x (`pair`: this lane's pair sums).  The warp
+// walks the columns together, the lanes share the pairs.
+template <int MORE, int KW, int NI, int CW>
+SQNN_DEV uint32_t walk_sets(const Columns<NI, CW> &col, uint32_t slot, const Candidate<KW> (&pair)[PAIRS_PER_LANE<NI>], const Candidate<KW> &x,
+                            uint32_t top, uint32_t lane, uint32_t best)
 {
-    const uint32_t pairs = n_in * (n_in - 1) / 2;
-    for (uint32_t p = lane; p < pairs; p += 32) {
-        const uint32_t i = pair_high(p);
-        Candidate<KW> x = x0;
-        x.add(col, i, slot);
-        x.add(col, pair_low(p, i), slot);
-        best = min(best, x.key());
-    }
-    best = warp_min(best);
-    if ((best >> 20) > 2u) {
-        for (uint32_t p = lane; p < pairs; p += 32) {
-            const uint32_t i = pair_high(p), h = pair_low(p, i);
-            Candidate<KW> x = x0;
-            x.add(col, i, slot);
-            x.add(col, h, slot);
-            for (uint32_t g = 0; g < h; ++g) {
-                Candidate<KW> y = x;
-                y.add(col, g, slot);
-                best = min(best, y.key());
-            }
+    if constexpr (MORE == 0) {
+        const uint32_t count = top * (top - 1) / 2;
+#pragma unroll
+        for (uint32_t k = 0; k < (uint32_t)PAIRS_PER_LANE<NI>; ++k) {
+            if (32 * k >= count) break;
+            Candidate<KW> y = x;
+#pragma unroll
+            for (int j = 0; j < KW; ++j) y.e[j] ^= pair[k].e[j];
+            y.seed ^= pair[k].seed;
+            if (32 * k + lane < count) best = min(best, y.key());
         }
-        best = warp_min(best);
-        if ((best >> 20) > 3u) best = min(best, try_all_sets<KW>(col, slot, x0, n_in, lane));
+    } else {
+#pragma unroll 1
+        for (uint32_t c = MORE + 1; c < top; ++c) {
+            Candidate<KW> y = x;
+            y.add(col, c, slot);
+            best = walk_sets<MORE - 1>(col, slot, pair, y, c, lane, best);
+        }
     }
     return best;
+}
+
+// The whole warp finishes one slice whose best set of at most one column has two errors or more: pairs, then larger sets as
+// long as the best count exceeds the sets' size, up to five columns; then all sets.  (Slices far from being consistent, with
+// many care bits for their seed bits, go there at once: the next sizes would not decide them.)
+template <int KW, int NI, int CW>
+SQNN_DEV uint32_t try_larger_sets(const Columns<NI, CW> &col, uint32_t slot, const Candidate<KW> &x, uint32_t best, uint32_t n_in, uint32_t lane)
+{
+    Candidate<KW> pair[PAIRS_PER_LANE<NI>];
+#pragma unroll
+    for (uint32_t k = 0; k < (uint32_t)PAIRS_PER_LANE<NI>; ++k) {
+        pair[k] = Candidate<KW>{};
+        if (32 * k + lane < n_in * (n_in - 1) / 2) pair[k] = pair_sum<KW>(col, slot, pair[k], 32 * k + lane);
+    }
+    best = warp_min(walk_sets<0>(col, slot, pair, x, n_in, lane, best));
+    if ((best >> 20) <= 2u) return best;
+    best = warp_min(walk_sets<1>(col, slot, pair, x, n_in, lane, best));
+    if ((best >> 20) <= 3u) return best;
+    if ((best >> 20) <= 6u) {
+        best = warp_min(walk_sets<2>(col, slot, pair, x, n_in, lane, best));
+        if ((best >> 20) <= 4u) return best;
+        best = warp_min(walk_sets<3>(col, slot, pair, x, n_in, lane, best));
+        if ((best >> 20) <= 5u) return best;
+    }
+    return min(best, try_all_sets<KW>(col, slot, x, n_in, lane));
 }
 
 // A lane's care positions in ascending order.  Up to two words sit in registers, more in the lane's slots of shared memory.
@@ -317,11 +344,12 @@ k_search_seeds(const __grid_constant__ SearchArgs S)
 #pragma unroll
         for (uint32_t w = 0; w < (NI + 3) / 4; ++w) rows_s[w][j] = (((row >> (4 * w)) & 0xfu) * 0x00204081u) & 0x01010101u;
     }
-    for (uint32_t i = threadIdx.x; i < S.n_in * NW; i += SEARCH_THREADS) {
-        const uint32_t t = i / NW, k = i % NW;
-        uint32_t w = 0;
-        for (uint32_t j = 32 * k; j < S.n_out && j < 32 * k + 32; ++j) w |= ((S.rows[j] >> t) & 1u) << (j - 32 * k);
-        cols[t][k] = w;
+    for (uint32_t k = threadIdx.x >> 5; k < NW; k += SEARCH_THREADS / 32) {
+        const uint32_t row = 32 * k + lane < S.n_out ? S.rows[32 * k + lane] : 0u;
+        for (uint32_t t = 0; t < S.n_in; ++t) {
+            const uint32_t word = __ballot_sync(0xffffffffu, (row >> t) & 1u);
+            if (lane == 0) cols[t][k] = word;
+        }
     }
     __syncthreads();
     const uint64_t total = S.slices * S.n_q;
