@@ -20,7 +20,9 @@
 // bytes of a word, is added to the columns' bytes shifted by the step's number, so that eight steps fill a byte of every column with
 // three additions each, for 12 columns.  Slices with more care bits than that try all seeds.
 //
-// Bound: integer instructions.
+// Bound: integer instructions.  600 000 slices of 60 x 12 (20 % care bits, two planes of 6000 x 3000) take 53 us: 31.7 M warp
+// instructions with 30.6 of 32 lanes active, 19.7 M of them on the integer pipe, which starts one every other cycle and is
+// busy 70 % of the time.  (Elimination of rows in a loop over the care bits: 126 us, 79 M instructions with 18.5 lanes active.)
 #include "sqnn_launch.h"
 
 #include <cuda_runtime.h>
@@ -38,17 +40,26 @@ struct SearchArgs {
     uint16_t *np;
 };
 
-// 32 bits of a packed vector starting at position p; positions >= limit (<= vector length) read 0
-SQNN_DEV uint32_t bits32_at(const uint64_t *__restrict__ v, uint64_t p, uint64_t limit)
+// NW words of a packed vector (`words` 32-bit words long) from bit p on; words past its end read 0.
+template <int NW>
+SQNN_DEV void load_bits(const uint64_t *__restrict__ vec, uint64_t words, uint64_t p, uint32_t (&out)[NW])
 {
-    if (p >= limit) return 0u;
-    const uint64_t w = p >> 6;
-    const uint32_t sh = (uint32_t)(p & 63);
-    uint64_t x = __ldg(v + w) >> sh;
-    if (sh > 32 && limit > ((w + 1) << 6)) x |= __ldg(v + w + 1) << (64 - sh);   // next word holds wanted positions
-    uint32_t r = (uint32_t)x;
-    if (p + 32 > limit) r &= (1u << (uint32_t)(limit - p)) - 1u;
-    return r;
+    const uint64_t w = p >> 5;
+    const uint32_t *from = reinterpret_cast<const uint32_t *>(vec) + w;
+    const uint32_t left = words - w < NW + 1 ? (uint32_t)(words - w) : NW + 1;
+    uint32_t raw[NW + 1];
+#pragma unroll
+    for (uint32_t k = 0; k < NW + 1; ++k) raw[k] = k < left ? __ldg(from + k) : 0u;
+#pragma unroll
+    for (int k = 0; k < NW; ++k) out[k] = __funnelshift_r(raw[k], raw[k + 1], (uint32_t)p & 31u);
+}
+
+// Row j of M, another j in every lane: by a generic load, since the lanes of a constant load take turns.
+SQNN_DEV uint32_t row_of(const SearchArgs &S, uint32_t j)
+{
+    uint32_t row;
+    asm("ld.u32 %0, [%1];" : "=r"(row) : "l"(S.rows + j));
+    return row;
 }
 
 constexpr uint32_t SEARCH_THREADS = 128;
@@ -92,14 +103,11 @@ SQNN_DEV uint32_t try_all_seeds(const uint32_t (*cols)[NW], uint32_t n_in, const
     return warp_min(best);
 }
 
-// The reduced columns of one slice per thread, for the slices the whole warp finishes: v_c and t_c.
-template <int NI, int KW>
-struct Columns {
-    uint32_t v[KW][NI][SEARCH_THREADS], t[NI][SEARCH_THREADS];
-};
-// A candidate: an error vector and its seed.
-template <int KW>
-struct Candidate {
+// How v_c and t_c are held: KW = 1 or 2 words of care bits and a word of t_c; KW = 0 for both in one word, t_c in its low NI bits,
+// where the care bits fit above them (for the LSTM gates 20 are enough for seven warps of eight: a third of the
+// elimination's instructions less).
+template <int KW, int NI>
+struct Candidate {                                                        // an error vector and its seed
     uint32_t e[KW], seed;
     SQNN_DEV uint32_t key() const
     {
@@ -108,72 +116,144 @@ struct Candidate {
         for (int k = 0; k < KW; ++k) wrong += (uint32_t)__popc(e[k]);
         return (wrong << 20) + seed;
     }
-    template <int NI, int CW>
-    SQNN_DEV void add(const Columns<NI, CW> &col, uint32_t c, uint32_t slot)
+    SQNN_DEV bool none() const
+    {
+        uint32_t any = 0;
+#pragma unroll
+        for (int k = 0; k < KW; ++k) any |= e[k];
+        return any == 0;
+    }
+    SQNN_DEV void add(const Candidate &o)
     {
 #pragma unroll
-        for (int k = 0; k < KW; ++k) e[k] ^= col.v[k][c][slot];
-        seed ^= col.t[c][slot];
+        for (int k = 0; k < KW; ++k) e[k] ^= o.e[k];
+        seed ^= o.seed;
+    }
+    SQNN_DEV Candidate lowest() const                                     // its lowest care bit, if any
+    {
+        Candidate p{};
+        p.e[0] = e[0] & (0u - e[0]);
+        if constexpr (KW == 2) p.e[KW - 1] = e[0] ? 0u : e[KW - 1] & (0u - e[KW - 1]);
+        return p;
+    }
+    SQNN_DEV bool has(const Candidate &p) const
+    {
+        uint32_t any = 0;
+#pragma unroll
+        for (int k = 0; k < KW; ++k) any |= e[k] & p.e[k];
+        return any != 0;
+    }
+    SQNN_DEV Candidate from(uint32_t src) const
+    {
+        Candidate x;
+#pragma unroll
+        for (int k = 0; k < KW; ++k) x.e[k] = __shfl_sync(0xffffffffu, e[k], src);
+        x.seed = __shfl_sync(0xffffffffu, seed, src);
+        return x;
+    }
+};
+template <int NI>
+struct Candidate<0, NI> {
+    static constexpr uint32_t CARE = ~((1u << NI) - 1u);
+    uint32_t w;
+    SQNN_DEV uint32_t key() const { return ((uint32_t)__popc(w & CARE) << 20) + (w & ~CARE); }
+    SQNN_DEV bool none() const { return (w & CARE) == 0; }
+    SQNN_DEV void add(const Candidate &o) { w ^= o.w; }
+    SQNN_DEV Candidate lowest() const { return Candidate{(w & CARE) & (0u - (w & CARE))}; }
+    SQNN_DEV bool has(const Candidate &p) const { return (w & p.w) != 0; }
+    SQNN_DEV Candidate from(uint32_t src) const { return Candidate{__shfl_sync(0xffffffffu, w, src)}; }
+};
+
+// The reduced columns of one slice per thread, for the slices the whole warp finishes.
+template <int NI>
+struct Columns {
+    uint32_t word[3][NI][SEARCH_THREADS];
+    template <int KW>
+    SQNN_DEV void put(uint32_t c, uint32_t slot, const Candidate<KW, NI> &x)
+    {
+        if constexpr (KW == 0) {
+            word[0][c][slot] = x.w;
+        } else {
+#pragma unroll
+            for (int k = 0; k < KW; ++k) word[k][c][slot] = x.e[k];
+            word[2][c][slot] = x.seed;
+        }
+    }
+    template <int KW>
+    SQNN_DEV Candidate<KW, NI> get(uint32_t c, uint32_t slot) const
+    {
+        Candidate<KW, NI> x;
+        if constexpr (KW == 0) {
+            x.w = word[0][c][slot];
+        } else {
+#pragma unroll
+            for (int k = 0; k < KW; ++k) x.e[k] = word[k][c][slot];
+            x.seed = word[2][c][slot];
+        }
+        return x;
     }
 };
 
 // The whole warp tries all 2^n_in sets of columns of one slice: the lanes split them by the top bits.
-template <int KW, int NI, int CW>
-SQNN_DEV uint32_t try_all_sets(const Columns<NI, CW> &col, uint32_t slot, Candidate<KW> x, uint32_t n_in, uint32_t lane)
+template <int KW, int NI>
+SQNN_DEV uint32_t try_all_sets(const Columns<NI> &col, uint32_t slot, Candidate<KW, NI> x, uint32_t n_in, uint32_t lane)
 {
     const uint32_t low_bits = n_in > 5 ? n_in - 5 : 0, lanes_used = n_in >= 5 ? 32u : (1u << n_in);
     uint32_t best = 0xffffffffu;
     if (lane < lanes_used) {
         for (uint32_t c = low_bits; c < n_in; ++c)
-            if ((lane >> (c - low_bits)) & 1u) x.add(col, c, slot);
+            if ((lane >> (c - low_bits)) & 1u) x.add(col.template get<KW>(c, slot));
         const uint32_t count = 1u << low_bits;
         for (uint32_t i = 0; i < count; ++i) {
-            if (i != 0) x.add(col, (uint32_t)__ffs((int)i) - 1u, slot);
+            if (i != 0) x.add(col.template get<KW>((uint32_t)__ffs((int)i) - 1u, slot));
             best = min(best, x.key());
         }
     }
     return warp_min(best);
 }
 
-// The pairs of columns, numbered (1,0), (2,0), (2,1), (3,0), ..: those below column c are the first c (c - 1) / 2.  Lane l keeps
-// the sums of pairs l, l + 32, ..  (At the first pair of a larger column, 1 + 8 p is a square; the 1 more leaves room for the
-// approximation's error, p < 190.)
+// The pairs of columns, numbered (1,0), (2,0), (2,1), (3,0), ..: those below column c are the first c (c - 1) / 2.  Lane l looks
+// after pairs l, l + 32, ..; `lanes_pairs` holds the larger column of each with the smaller one in its upper half.
 template <int NI>
 constexpr int PAIRS_PER_LANE = (NI * (NI - 1) / 2 + 31) / 32;
-template <int KW, int NI, int CW>
-SQNN_DEV Candidate<KW> pair_sum(const Columns<NI, CW> &col, uint32_t slot, Candidate<KW> x, uint32_t p)
+template <int NI>
+SQNN_DEV void number_pairs(uint32_t lane, uint32_t (&lanes_pairs)[PAIRS_PER_LANE<NI>])
 {
-    float root;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(root) : "f"(2.0f + 8.0f * (float)p));
-    const uint32_t high = (uint32_t)((1.0f + root) * 0.5f);
-    x.add(col, high, slot);
-    x.add(col, p - high * (high - 1) / 2, slot);
-    return x;
+    uint32_t high = 1, before = 0;                                        // pairs before those of `high`
+#pragma unroll
+    for (uint32_t k = 0; k < (uint32_t)PAIRS_PER_LANE<NI>; ++k) {
+        while (before + high <= 32 * k + lane) before += high++;
+        lanes_pairs[k] = high < NI ? high | (32 * k + lane - before) << 16 : 1u;
+    }
 }
 
-// The best of all sets of MORE columns below `top` and a pair below those, added to x (`pair`: this lane's pair sums).  The warp
-// walks the columns together, the lanes share the pairs.
-template <int MORE, int KW, int NI, int CW>
-SQNN_DEV uint32_t walk_sets(const Columns<NI, CW> &col, uint32_t slot, const Candidate<KW> (&pair)[PAIRS_PER_LANE<NI>], const Candidate<KW> &x,
-                            uint32_t top, uint32_t lane, uint32_t best)
+// The best of all sets of MORE columns below `top` and a pair below those, added to x (`pair`: this lane's pair sums, v: all columns,
+// the same in every lane).  The warp walks the columns together, the lanes share the pairs.  The innermost columns are walked
+// in straight-line code: a slice that gets here holds up its warp, and a loop over them is all latency.
+template <int MORE, int KW, int NI>
+SQNN_DEV uint32_t walk_sets(const Columns<NI> &col, uint32_t slot, const Candidate<KW, NI> (&v)[NI], const Candidate<KW, NI> (&pair)[PAIRS_PER_LANE<NI>],
+                            const Candidate<KW, NI> &x, uint32_t top, uint32_t lane, uint32_t best)
 {
-    if constexpr (MORE == 0) {
-        const uint32_t count = top * (top - 1) / 2;
+    if constexpr (MORE == 1) {
 #pragma unroll
-        for (uint32_t k = 0; k < (uint32_t)PAIRS_PER_LANE<NI>; ++k) {
-            if (32 * k >= count) break;
-            Candidate<KW> y = x;
+        for (uint32_t c = 2; c < NI; ++c) {
+            if (c >= top) break;
+            Candidate<KW, NI> y = x;
+            y.add(v[c]);
+            const uint32_t count = c * (c - 1) / 2;
 #pragma unroll
-            for (int j = 0; j < KW; ++j) y.e[j] ^= pair[k].e[j];
-            y.seed ^= pair[k].seed;
-            if (32 * k + lane < count) best = min(best, y.key());
+            for (uint32_t k = 0; 32 * k < count; ++k) {
+                Candidate<KW, NI> z = y;
+                z.add(pair[k]);
+                if (32 * k + 32 <= count || 32 * k + lane < count) best = min(best, z.key());
+            }
         }
     } else {
 #pragma unroll 1
         for (uint32_t c = MORE + 1; c < top; ++c) {
-            Candidate<KW> y = x;
-            y.add(col, c, slot);
-            best = walk_sets<MORE - 1>(col, slot, pair, y, c, lane, best);
+            Candidate<KW, NI> y = x;
+            y.add(col.template get<KW>(c, slot));
+            best = walk_sets<MORE - 1>(col, slot, v, pair, y, c, lane, best);
         }
     }
     return best;
@@ -182,23 +262,33 @@ SQNN_DEV uint32_t walk_sets(const Columns<NI, CW> &col, uint32_t slot, const Can
 // The whole warp finishes one slice whose best set of at most one column has two errors or more: pairs, then larger sets as
 // long as the best count exceeds the sets' size, up to five columns; then all sets.  (Slices far from being consistent, with
 // many care bits for their seed bits, go there at once: the next sizes would not decide them.)
-template <int KW, int NI, int CW>
-SQNN_DEV uint32_t try_larger_sets(const Columns<NI, CW> &col, uint32_t slot, const Candidate<KW> &x, uint32_t best, uint32_t n_in, uint32_t lane)
+template <int KW, int NI>
+SQNN_DEV uint32_t try_larger_sets(const Columns<NI> &col, uint32_t slot, const uint32_t (&lanes_pairs)[PAIRS_PER_LANE<NI>], const Candidate<KW, NI> &x,
+                                  uint32_t best, uint32_t n_in, uint32_t lane)
 {
-    Candidate<KW> pair[PAIRS_PER_LANE<NI>];
+    Candidate<KW, NI> pair[PAIRS_PER_LANE<NI>];
 #pragma unroll
     for (uint32_t k = 0; k < (uint32_t)PAIRS_PER_LANE<NI>; ++k) {
-        pair[k] = Candidate<KW>{};
-        if (32 * k + lane < n_in * (n_in - 1) / 2) pair[k] = pair_sum<KW>(col, slot, pair[k], 32 * k + lane);
+        pair[k] = col.template get<KW>(lanes_pairs[k] & 0xffffu, slot);
+        pair[k].add(col.template get<KW>(lanes_pairs[k] >> 16, slot));
     }
-    best = warp_min(walk_sets<0>(col, slot, pair, x, n_in, lane, best));
+#pragma unroll
+    for (uint32_t k = 0; k < (uint32_t)PAIRS_PER_LANE<NI>; ++k) {
+        Candidate<KW, NI> y = x;
+        y.add(pair[k]);
+        if (32 * k + lane < n_in * (n_in - 1) / 2) best = min(best, y.key());
+    }
+    best = warp_min(best);
     if ((best >> 20) <= 2u) return best;
-    best = warp_min(walk_sets<1>(col, slot, pair, x, n_in, lane, best));
+    Candidate<KW, NI> v[NI];
+#pragma unroll
+    for (int c = 0; c < NI; ++c) v[c] = col.template get<KW>(c, slot);
+    best = warp_min(walk_sets<1>(col, slot, v, pair, x, n_in, lane, best));
     if ((best >> 20) <= 3u) return best;
     if ((best >> 20) <= 6u) {
-        best = warp_min(walk_sets<2>(col, slot, pair, x, n_in, lane, best));
+        best = warp_min(walk_sets<2>(col, slot, v, pair, x, n_in, lane, best));
         if ((best >> 20) <= 4u) return best;
-        best = warp_min(walk_sets<3>(col, slot, pair, x, n_in, lane, best));
+        best = warp_min(walk_sets<3>(col, slot, v, pair, x, n_in, lane, best));
         if ((best >> 20) <= 5u) return best;
     }
     return min(best, try_all_sets<KW>(col, slot, x, n_in, lane));
@@ -230,17 +320,19 @@ struct CareBits {
 
 // The search over one slice per lane; care bits of a slice fit KW words.  rows_s: byte b of word [w][j] is bit 4 w + b
 // of row j of M.  Lanes without a slice have no care bits.
-template <int KW, int NI, int NW, int CW>
-SQNN_DEV uint32_t search_slices(const uint32_t (&rows_s)[(NI + 3) / 4][32 * NW + 1], Columns<NI, CW> &col, CareBits<NW> bits, uint32_t most,
-                                uint32_t n_in, uint32_t lane)
+template <int KW, int NI, int NW>
+SQNN_DEV uint32_t search_slices(const uint32_t (&rows_s)[(NI + 3) / 4][32 * NW + 1], Columns<NI> &col, const uint32_t (&lanes_pairs)[PAIRS_PER_LANE<NI>],
+                                CareBits<NW> bits, uint32_t most, uint32_t n_in, uint32_t lane)
 {
-    constexpr int NB = (NI + 3) / 4;
-    uint32_t v[KW][NI], t[NI], e[KW], seed = 0;
+    constexpr int NB = (NI + 3) / 4, VW = KW == 0 ? 1 : KW;
+    Candidate<KW, NI> v[NI], x{};
 #pragma unroll
-    for (int k = 0; k < KW; ++k) {
-        e[k] = 0;
+    for (int c = 0; c < NI; ++c) v[c] = Candidate<KW, NI>{};
 #pragma unroll
-        for (int c = 0; c < NI; ++c) v[k][c] = 0;
+    for (int k = 0; k < VW; ++k) {
+        uint32_t squeezed[NI], wants = 0;
+#pragma unroll
+        for (int c = 0; c < NI; ++c) squeezed[c] = 0;
 #pragma unroll 1
         for (uint32_t byte = 0; byte < 4 && 32 * k + 8 * byte < most; ++byte) {
             uint32_t acc[NB], wanted = 0;
@@ -258,70 +350,55 @@ SQNN_DEV uint32_t search_slices(const uint32_t (&rows_s)[(NI + 3) / 4][32 * NW +
                     wanted += bit << i;
                 }
             }
-            e[k] |= wanted << (8 * byte);
+            wants |= wanted << (8 * byte);
             // byte c % 4 of acc[c / 4] becomes this byte of column c
             const uint32_t keep = 0x3210u & ~(0xfu << (4 * byte));
 #pragma unroll
-            for (int c = 0; c < NI; ++c) v[k][c] = __byte_perm(v[k][c], acc[c / 4], keep | ((4u + c % 4) << (4 * byte)));
+            for (int c = 0; c < NI; ++c) squeezed[c] = __byte_perm(squeezed[c], acc[c / 4], keep | ((4u + c % 4) << (4 * byte)));
+        }
+        if constexpr (KW == 0) {
+            x.w = wants << NI;
+#pragma unroll
+            for (int c = 0; c < NI; ++c) v[c].w = squeezed[c] << NI;
+        } else {
+            x.e[k] = wants;
+#pragma unroll
+            for (int c = 0; c < NI; ++c) v[c].e[k] = squeezed[c];
         }
     }
-#pragma unroll
-    for (int c = 0; c < NI; ++c) t[c] = (uint32_t)c < n_in ? 1u << c : 0u;
 #pragma unroll
     for (int c = 0; c < NI; ++c) {
-        uint32_t p[KW];                                                   // the lowest bit of column c
-        p[0] = v[0][c] & (0u - v[0][c]);
-        if constexpr (KW == 2) p[1] = v[0][c] ? 0u : v[1][c] & (0u - v[1][c]);
-        auto has = [&](uint32_t a0, uint32_t a1) {
-            if constexpr (KW == 2) return ((a0 & p[0]) | (a1 & p[KW - 1])) != 0;
-            else return (a0 & p[0]) != 0;
-        };
-        if (has(e[0], e[KW - 1])) {
+        const uint32_t t = (uint32_t)c < n_in ? 1u << c : 0u;
+        if constexpr (KW == 0) v[c].w += t;
+        else v[c].seed = t;
+    }
 #pragma unroll
-            for (int k = 0; k < KW; ++k) e[k] ^= v[k][c];
-            seed ^= t[c];
-        }
+    for (int c = 0; c < NI; ++c) {
+        const Candidate<KW, NI> p = v[c].lowest();
+        if (x.has(p)) x.add(v[c]);
 #pragma unroll
         for (int d = 0; d < NI; ++d)
-            if (d != c && has(v[0][d], v[KW - 1][d])) {
-#pragma unroll
-                for (int k = 0; k < KW; ++k) v[k][d] ^= v[k][c];
-                t[d] ^= t[c];
-            }
+            if (d != c && v[d].has(p)) v[d].add(v[c]);
     }
-    Candidate<KW> x;
-    uint32_t any = 0;
-#pragma unroll
-    for (int k = 0; k < KW; ++k) { x.e[k] = e[k]; any |= e[k]; }
-    x.seed = seed;
     uint32_t best = x.key();
-    if (any) {                                                            // sets of one
+    if (!x.none()) {                                                      // sets of one
 #pragma unroll
         for (int c = 0; c < NI; ++c) {
-            Candidate<KW> y;
-#pragma unroll
-            for (int k = 0; k < KW; ++k) y.e[k] = e[k] ^ v[k][c];
-            y.seed = seed ^ t[c];
+            Candidate<KW, NI> y = x;
+            y.add(v[c]);
             best = min(best, y.key());
         }
     }
     const bool open = (best >> 20) >= 2u;
     if (open) {
 #pragma unroll
-        for (int c = 0; c < NI; ++c) {
-#pragma unroll
-            for (int k = 0; k < KW; ++k) col.v[k][c][threadIdx.x] = v[k][c];
-            col.t[c][threadIdx.x] = t[c];
-        }
+        for (int c = 0; c < NI; ++c) col.put(c, threadIdx.x, v[c]);
     }
     __syncwarp();
     for (uint32_t more = __ballot_sync(0xffffffffu, open); more; more &= more - 1u) {
         const uint32_t src = (uint32_t)__ffs((int)more) - 1u;
-        Candidate<KW> from;
-#pragma unroll
-        for (int k = 0; k < KW; ++k) from.e[k] = __shfl_sync(0xffffffffu, e[k], src);
-        from.seed = __shfl_sync(0xffffffffu, seed, src);
-        const uint32_t found = try_larger_sets<KW>(col, (threadIdx.x & ~31u) + src, from, __shfl_sync(0xffffffffu, best, src), n_in, lane);
+        const uint32_t found = try_larger_sets<KW>(col, (threadIdx.x & ~31u) + src, lanes_pairs, x.from(src), __shfl_sync(0xffffffffu, best, src),
+                                                   n_in, lane);
         if (lane == src) best = found;
     }
     return best;
@@ -335,23 +412,25 @@ k_search_seeds(const __grid_constant__ SearchArgs S)
     __shared__ uint32_t rows_s[(NI + 3) / 4][32 * NW + 1];                // rows past n_out are zero
     __shared__ uint32_t cols[SQNN_MAX_N_IN][NW];                          // column t of M as an n_out-bit word
     __shared__ uint32_t rest_s[NW > 2 ? 2 * NW : 1][SEARCH_THREADS];
-    __shared__ Columns<NI, 2> col_s;
-    wait_prior_grid();
-    launch_dependents();
+    __shared__ Columns<NI> col_s;
     const uint32_t lane = threadIdx.x & 31;
+    uint32_t lanes_pairs[PAIRS_PER_LANE<NI>];
+    number_pairs<NI>(lane, lanes_pairs);
     for (uint32_t j = threadIdx.x; j < 32 * NW + 1; j += SEARCH_THREADS) {
-        const uint32_t row = j < S.n_out ? S.rows[j] & (uint32_t)((1ull << S.n_in) - 1ull) : 0u;
+        const uint32_t row = j < S.n_out ? row_of(S, j) & (uint32_t)((1ull << S.n_in) - 1ull) : 0u;
 #pragma unroll
         for (uint32_t w = 0; w < (NI + 3) / 4; ++w) rows_s[w][j] = (((row >> (4 * w)) & 0xfu) * 0x00204081u) & 0x01010101u;
     }
     for (uint32_t k = threadIdx.x >> 5; k < NW; k += SEARCH_THREADS / 32) {
-        const uint32_t row = 32 * k + lane < S.n_out ? S.rows[32 * k + lane] : 0u;
+        const uint32_t row = 32 * k + lane < S.n_out ? row_of(S, 32 * k + lane) : 0u;
         for (uint32_t t = 0; t < S.n_in; ++t) {
             const uint32_t word = __ballot_sync(0xffffffffu, (row >> t) & 1u);
             if (lane == 0) cols[t][k] = word;
         }
     }
     __syncthreads();
+    wait_prior_grid();
+    launch_dependents();
     const uint64_t total = S.slices * S.n_q;
     const uint64_t step = (uint64_t)gridDim.x * SEARCH_THREADS;
     for (uint64_t job0 = (uint64_t)blockIdx.x * SEARCH_THREADS + (threadIdx.x & ~31u); job0 < total; job0 += step) {
@@ -361,15 +440,16 @@ k_search_seeds(const __grid_constant__ SearchArgs S)
 #pragma unroll
         for (int k = 0; k < NW; ++k) want[k] = care[k] = 0;
         if (live) {
-            const uint32_t plane = (uint32_t)(job / S.slices);
-            const uint64_t p0 = (job - (uint64_t)plane * S.slices) * S.n_out;
-            const uint64_t limit = p0 + S.n_out < S.mn ? p0 + S.n_out : S.mn;   // slice end (ragged tail)
+            uint64_t slice = job;
+            const uint64_t *plane = S.planes;
+            while (slice >= S.slices) { slice -= S.slices; plane += S.words64; }
+            const uint64_t p0 = slice * S.n_out;
+            load_bits<NW>(S.mask, 2 * S.words64, p0, care);
+            load_bits<NW>(plane, 2 * S.words64, p0, want);
+            const uint32_t bits = S.mn - p0 < S.n_out ? (uint32_t)(S.mn - p0) : S.n_out;        // the last slice may be shorter
 #pragma unroll
-            for (int k = 0; k < NW; ++k) {
-                if (32u * k >= S.n_out) break;
-                care[k] = bits32_at(S.mask, p0 + 32 * k, limit);
-                want[k] = bits32_at(S.planes + (uint64_t)plane * S.words64, p0 + 32 * k, limit);
-            }
+            for (uint32_t k = 0; k < NW; ++k)
+                if (bits < 32 * k + 32) care[k] &= bits > 32 * k ? (1u << (bits - 32 * k)) - 1u : 0u;
         }
 #pragma unroll
         for (int k = 0; k < NW; ++k) count += (uint32_t)__popc(care[k]);
@@ -385,8 +465,9 @@ k_search_seeds(const __grid_constant__ SearchArgs S)
             bits.rest = &rest_s[0][threadIdx.x];
         }
         const uint32_t most = __reduce_max_sync(0xffffffffu, wide ? 0u : count);
-        uint32_t best = most <= 32 ? search_slices<1, NI, NW>(rows_s, col_s, bits, most, S.n_in, lane)
-                                   : search_slices<2, NI, NW>(rows_s, col_s, bits, most, S.n_in, lane);
+        uint32_t best = most + NI <= 32 ? search_slices<0, NI, NW>(rows_s, col_s, lanes_pairs, bits, most, S.n_in, lane)
+                        : most <= 32    ? search_slices<1, NI, NW>(rows_s, col_s, lanes_pairs, bits, most, S.n_in, lane)
+                                        : search_slices<2, NI, NW>(rows_s, col_s, lanes_pairs, bits, most, S.n_in, lane);
         for (uint32_t more = __ballot_sync(0xffffffffu, wide); more; more &= more - 1u) {
             const uint32_t src = (uint32_t)__ffs((int)more) - 1u;
             uint32_t w_s[NW], c_s[NW];
@@ -434,7 +515,7 @@ static int search_seeds_queue(const sqnn_xornet *net, uint64_t m, uint64_t n, ui
     S.planes = d_planes; S.mask = d_mask; S.wc = d_wc; S.np = d_np;
     const uint64_t jobs = S.slices * n_q;
     uint64_t blocks = (jobs + SEARCH_THREADS - 1) / SEARCH_THREADS;
-    const uint64_t cap = (uint64_t)sm_count() * 64;
+    const uint64_t cap = (uint64_t)sm_count() * 16;         // about twice what is resident: few tables, an even end
     if (blocks > cap) blocks = cap;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     return net->n_in <= 8    ? launch_search<8>(S, (uint32_t)blocks, st)
