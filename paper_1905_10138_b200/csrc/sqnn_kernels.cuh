@@ -177,6 +177,8 @@ k_decode_bits(DecodeArgs A, uint64_t *__restrict__ out, const ClearArgs clear, c
         cp_async_wait_all();
         __syncthreads();
         for (TilePos p = p_first; p.plane < A.n_q; p = advance(p, stride, live, A.n_q)) {
+            if (!SINK && lane == 0) bulk_wait_read<0>();         // the copy out of the region is over
+            __syncwarp();
             decode_ktile_generic(A, p.plane, p.tile, region, smem, lane);
             write_out(p);
         }

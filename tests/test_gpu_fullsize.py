@@ -117,3 +117,16 @@ def test_decode_loop_with_many_tiles_per_warp_run_time_shape():
     blob, _ = H.blob_from_library(layer)
     dev = H.DeviceLayer(layer, blob)
     check_whole_decode(layer, dev, blob, n_samples=20)
+
+
+def test_decode_loop_with_long_tiles_run_time_shape():
+    """The same with tiles of 6400 bytes (200 x 20): the copy of one tile takes long enough that the warp's next
+    tile meets it, and must wait for it."""
+    layer = generic_layer(200, 20, 14000, 16384, 0.1, 52)      # 229 M weights, more than one tile of 51 200 bits for every warp
+    blob, _ = H.blob_from_library(layer)
+    dev = H.DeviceLayer(layer, blob)
+    words = dev.decode_bits()
+    wc, np_, dp = sqnn.sqnn_unpack_host(blob, 0)
+    bits = orc.decode_plane(layer.M, layer.mn, wc.astype(np.uint64), np_, dp)
+    assert np.array_equal(words[0], wl.pack_bits(bits))
+    assert dev.status_value() == 0
