@@ -42,10 +42,10 @@ int fill_decode_args(const sqnn_desc *d, const void *d_blob, uint32_t *d_status,
     A->mn = d->m * d->n;
     A->words64 = (A->mn + 63) / 64;
     A->n_out = d->n_out; A->n_in = d->n_in; A->n_q = d->n_q;
-    A->KT = format_tiles_per_kernel_tile(d->n_out);
-    A->G = 8 * A->KT;
-    A->W = A->G * d->n_out / 32;
-    A->ktiles = d->slices_padded / (32ull * A->G);
+    A->slices = (A->mn + d->n_out - 1) / d->n_out;
+    A->inv_n_out = d->n_out > 1 ? ~0ull / d->n_out + 1 + (0xffffffffffffffffull % d->n_out == d->n_out - 1 ? 1 : 0) : 0;
+    A->KT = format_tiles_per_kernel_tile(d->n_out);           // launchers may cut the tiles of run-time shapes smaller
+    A->W = 8 * A->KT * d->n_out / 32;
     A->nw = entry_words(d->n_out);
     A->nwp = entry_words_padded(d->n_out);
     A->nchunks = table_chunks(d->n_in, A->nwp);

@@ -1,11 +1,11 @@
 // Device-side decryption of one warp tile: seeds -> XOR-gate network (table lookup) ->
 // patch flips, producing a run of consecutive output words in shared memory.
 //
-// Work split.  A lane owns G consecutive slices, G = 8 * KT with KT the number of format tiles
-// (256 slices) per kernel tile, chosen so that G * n_out is a multiple of 32 bits; its
-// W = G * n_out / 32 output words are private to it while it expands.  A kernel tile is therefore
-// 32 * G consecutive slices = 32 * W consecutive 32-bit words of the flattened plane.  In the
-// seed stream a lane's 8 slices of one format tile are n_in consecutive bytes.
+// Work split.  A kernel tile is 32 * W consecutive 32-bit words of the flattened plane, decoded by a warp.
+// As a rule it is KT format tiles (256 slices), KT chosen so that 8 * KT * n_out is a multiple of 32 bits: a lane owns 8 * KT
+// consecutive slices, whose W output words are private to it while it expands; in the seed stream a lane's 8 slices of
+// one format tile are n_in consecutive bytes.  (Shapes with compile-time kernels have KT = 1.)  In small layers of other
+// shapes it is a part of a format tile, so that all warps have something to decode: see decode_range.
 //
 // The network (Section 3.1, w~ = M . w^c) is evaluated with the lookup tables stored in the
 // blob (geometry in sqnn_layout.h), copied to shared memory once per block.
@@ -34,9 +34,11 @@ struct PlanePtrs {
 struct DecodeArgs {
     uint64_t mn;           // weights per plane
     uint64_t words64;      // ceil(mn / 64)
-    uint64_t ktiles;       // kernel tiles per plane (padded stream)
+    uint64_t slices;       // slices per plane that hold weights
+    uint64_t inv_n_out;    // floor(2^64 / n_out) + 1: the upper half of its product with a bit position (< 2^40) is the slice (n_out > 1)
     uint32_t n_out, n_in, n_q;
-    uint32_t KT, G, W;     // format tiles per kernel tile, slices and words per lane
+    uint32_t KT;           // format tiles per kernel tile; 0: a kernel tile is a part of one (run-time shapes, small layers)
+    uint32_t W;            // words of a kernel tile per lane
     uint32_t nw, nwp;      // words per table entry: used, padded (1, 2, 4, 8)
     uint32_t nchunks, cb;  // table chunks, bits per chunk
     uint32_t tab_words;    // words of all tables (multiple of 4)
@@ -274,29 +276,44 @@ SQNN_DEV void fetch_patches(const DecodeArgs &A, const PlanePtrs &P, TileRun &ru
     }
 }
 
-// One patch entry: flips bit bit0 + pos of the region if the entry belongs to the run (t < total,
-// t = its index minus the run's base, as unsigned) and pos lies inside the tile.  Branch-free: the
-// reduction is predicated.  Returns pos if the entry belongs to the run, else 0 (for the range check).
-SQNN_DEV uint32_t flip_entry(uint32_t region_sa, uint32_t bit0, uint32_t tile_bits, uint32_t pos, uint32_t t, uint32_t total)
+// One patch entry: flips the bit at pos of the format tile if the entry belongs to the run (t < total, t = its index minus
+// the run's base, as unsigned) and pos lies inside the tile.  Branch-free: the reduction is predicated.  The region
+// holds the tile or, PART, `bits` bits from bit -offset of it on (the others are passed over).  Returns pos if the entry
+// belongs to the run, else 0 (for the range check).
+template <bool PART>
+SQNN_DEV uint32_t flip_entry(uint32_t region_sa, uint32_t offset, uint32_t bits, uint32_t tile_bits, uint32_t pos, uint32_t t, uint32_t total)
 {
     uint32_t seen;
-    asm volatile("{\n .reg .pred p, q;\n .reg .b32 a, v, s, b;\n"
-                 " setp.lt.u32 q, %3, %4;\n"                    // the entry belongs to the run
-                 " setp.lt.and.u32 p, %2, %5, q;\n"             // ... and its position lies inside the tile
-                 " selp.u32 %0, %2, 0, q;\n"
-                 " add.u32 b, %2, %6;\n"
-                 " shr.u32 a, b, 5;\n shl.b32 a, a, 2;\n add.u32 a, a, %1;\n"
-                 " and.b32 s, b, 31;\n shl.b32 v, 1, s;\n"
-                 " @p red.shared.xor.b32 [a], v;\n}"
-                 : "=r"(seen) : "r"(region_sa), "r"(pos), "r"(t), "r"(total), "r"(tile_bits), "r"(bit0) : "memory");
+    if constexpr (PART) {
+        asm volatile("{\n .reg .pred p, q;\n .reg .b32 a, v, s, b;\n"
+                     " setp.lt.u32 q, %3, %4;\n"
+                     " setp.lt.and.u32 p, %2, %5, q;\n"
+                     " selp.u32 %0, %2, 0, q;\n"
+                     " add.u32 b, %2, %6;\n"
+                     " setp.lt.and.u32 p, b, %7, p;\n"
+                     " shr.u32 a, b, 5;\n shl.b32 a, a, 2;\n add.u32 a, a, %1;\n"
+                     " and.b32 s, b, 31;\n shl.b32 v, 1, s;\n"
+                     " @p red.shared.xor.b32 [a], v;\n}"
+                     : "=r"(seen) : "r"(region_sa), "r"(pos), "r"(t), "r"(total), "r"(tile_bits), "r"(offset), "r"(bits) : "memory");
+    } else {
+        asm volatile("{\n .reg .pred p, q;\n .reg .b32 a, v, s;\n"
+                     " setp.lt.u32 q, %3, %4;\n"                    // the entry belongs to the run
+                     " setp.lt.and.u32 p, %2, %5, q;\n"             // ... and its position lies inside the tile
+                     " selp.u32 %0, %2, 0, q;\n"
+                     " shr.u32 a, %2, 5;\n shl.b32 a, a, 2;\n add.u32 a, a, %1;\n"
+                     " and.b32 s, %2, 31;\n shl.b32 v, 1, s;\n"
+                     " @p red.shared.xor.b32 [a], v;\n}"
+                     : "=r"(seen) : "r"(region_sa), "r"(pos), "r"(t), "r"(total), "r"(tile_bits) : "memory");
+    }
     return seen;
 }
 
-// Flips the patched positions of one format tile (Section 3.2) whose first bit is bit `bit0` of
-// the region.  Every lane's words of the tile must be in place (warp barrier before), and the
+// Flips the patched positions of one format tile (Section 3.2) in the region (PART, offset, bits: see flip_entry).
+// Every lane's words of the tile must be in place (warp barrier before), and the
 // region is complete after the warp barrier that follows.  `pw`: words fetched by fetch_patches.
+template <bool PART = false>
 SQNN_DEV void tile_patch(const DecodeArgs &A, const PlanePtrs &P, const TileRun &run, const uint32_t (&pw)[PATCH_AHEAD],
-                         uint32_t *region, uint32_t bit0, uint32_t tile_bits, uint32_t lane)
+                         uint32_t *region, uint32_t tile_bits, uint32_t lane, uint32_t offset = 0, uint32_t bits = 0)
 {
     if (run.end == run.base) return;                             // the same in every lane
     const uint32_t region_sa = smem_addr(region);
@@ -308,8 +325,8 @@ SQNN_DEV void tile_patch(const DecodeArgs &A, const PlanePtrs &P, const TileRun 
     uint32_t top = 0;                                            // largest position seen
 #pragma unroll
     for (uint32_t k = 0; k < PATCH_AHEAD; ++k) {
-        top = max(top, flip_entry(region_sa, bit0, tile_bits, pw[k] & 0xffffu, t0 + 64 * k, total));
-        top = max(top, flip_entry(region_sa, bit0, tile_bits, pw[k] >> 16, t0 + 64 * k + 1, total));
+        top = max(top, flip_entry<PART>(region_sa, offset, bits, tile_bits, pw[k] & 0xffffu, t0 + 64 * k, total));
+        top = max(top, flip_entry<PART>(region_sa, offset, bits, tile_bits, pw[k] >> 16, t0 + 64 * k + 1, total));
     }
     // longer runs: eight words (sixteen entries) per lane and round; the words of the next round are
     // requested before this round's are used
@@ -332,8 +349,8 @@ SQNN_DEV void tile_patch(const DecodeArgs &A, const PlanePtrs &P, const TileRun 
             const uint32_t t = 2 * (a0 + lane) - run.base;
 #pragma unroll
             for (uint32_t k = 0; k < RB; ++k) {
-                top = max(top, flip_entry(region_sa, bit0, tile_bits, cur[k] & 0xffffu, t + 64 * k, total));
-                top = max(top, flip_entry(region_sa, bit0, tile_bits, cur[k] >> 16, t + 64 * k + 1, total));
+                top = max(top, flip_entry<PART>(region_sa, offset, bits, tile_bits, cur[k] & 0xffffu, t + 64 * k, total));
+                top = max(top, flip_entry<PART>(region_sa, offset, bits, tile_bits, cur[k] >> 16, t + 64 * k + 1, total));
             }
 #pragma unroll
             for (uint32_t k = 0; k < RB; ++k) cur[k] = nxt[k];
@@ -413,23 +430,18 @@ SQNN_DEV void tile_expand(const TileSeeds<N_OUT, N_IN> &in, uint32_t *region, co
     }
 }
 
-// Table entry e of NWP words (run-time shapes).
-template <int NWP>
-SQNN_DEV void xor_entry(const uint32_t *tab, uint32_t e, uint32_t (&x)[NWP])
-{
-    uint32_t y[NWP];
-    load_entry<NWP, false>(tab, e, 0, y);
-#pragma unroll
-    for (int k = 0; k < NWP; ++k) x[k] ^= y[k];
-}
+// Entry e of the tables in shared memory is the XOR of one entry per chunk of the seed (run-time shapes).
 template <int NWP>
 SQNN_DEV void lookup(const DecodeArgs &A, const uint32_t *tab, uint32_t seed, uint32_t (&x)[NWP])
 {
     const uint32_t cb = A.cb, cmask = (1u << cb) - 1u;
     load_entry<NWP, false>(tab, seed & cmask, 0, x);
     for (uint32_t ch = 1; ch < A.nchunks; ++ch) {
+        uint32_t y[NWP];
         seed >>= cb;
-        xor_entry<NWP>(tab, (ch << cb) | (seed & cmask), x);
+        load_entry<NWP, false>(tab, (ch << cb) | (seed & cmask), 0, y);
+#pragma unroll
+        for (int k = 0; k < NWP; ++k) x[k] ^= y[k];
     }
 }
 
@@ -513,8 +525,8 @@ SQNN_DEV void expand_shifted(const DecodeArgs &A, const PlanePtrs &P, uint64_t k
     }
 }
 
-// Run-time shape: one kernel tile.  Ends with the warp synchronised.
-SQNN_DEV void decode_ktile_generic(const DecodeArgs &A, uint32_t plane, uint64_t ktile, uint32_t *region, const uint32_t *tab, uint32_t lane)
+// Run-time shape, whole format tiles.  Ends with the warp synchronised.
+SQNN_DEV void decode_whole_tiles(const DecodeArgs &A, uint32_t plane, uint64_t ktile, uint32_t *region, const uint32_t *tab, uint32_t lane)
 {
     const PlanePtrs &P = A.pl[plane];
     const uint32_t tile_bits = SQNN_TILE_SLICES * A.n_out;
@@ -542,13 +554,143 @@ SQNN_DEV void decode_ktile_generic(const DecodeArgs &A, uint32_t plane, uint64_t
     fetch_patches(A, P, run, lane, pw);
     __syncwarp();
     for (uint32_t f = 0; f < A.KT; ++f) {                        // one format tile after the other
-        tile_patch(A, P, run, pw, region, f * tile_bits, tile_bits, lane);
+        tile_patch(A, P, run, pw, region + f * (tile_bits / 32), tile_bits, lane);
         if (f + 1 < A.KT) {
             run = fetch_run(P, ktile * A.KT + f + 1);
             fetch_patches(A, P, run, lane, pw);
         }
     }
     __syncwarp();
+}
+
+// A kernel tile that is a part of a format tile: `words` words; the slices that overlap it, the first one starting at bit pos0 <= 0 of
+// it and at bit `bit` of the words at wc, are taken by the lanes in turn.
+struct RangeTile {
+    const uint32_t *wc;
+    uint32_t bit, slices, words;         // slices: those left in the plane
+    int32_t pos0;
+};
+constexpr uint32_t SEEDS_AHEAD = 4;      // turns whose seeds are requested together
+struct RangeSeeds {
+    uint32_t lo[SEEDS_AHEAD], hi[SEEDS_AHEAD];
+};
+SQNN_DEV void request_seeds(const DecodeArgs &A, const RangeTile &T, uint32_t turn, uint32_t lane, RangeSeeds &s)
+{
+#pragma unroll
+    for (uint32_t k = 0; k < SEEDS_AHEAD; ++k) {
+        const uint32_t i = 32 * (turn + k) + lane;
+        const uint32_t *w = T.wc + ((T.bit + i * A.n_in) >> 5);
+        s.lo[k] = s.hi[k] = 0u;
+        if (T.pos0 + (int32_t)(i * A.n_out) < (int32_t)(32 * T.words) && i < T.slices) { s.lo[k] = ldg_ahead(w); s.hi[k] = ldg_ahead(w + 1); }   // sections end with slack
+    }
+}
+
+// Expands the tile's slices.  Slices of 33 bits and more share a word with one neighbour at most: its part is handed up
+// the lanes, and from one turn to the next, to the slice the word ends in, which stores it.  Shorter ones are
+// added to zeros by reductions.
+template <int NWP>
+SQNN_DEV void expand_range(const DecodeArgs &A, const RangeTile &T, RangeSeeds &s, uint32_t *region, const uint32_t *tab, uint32_t lane)
+{
+    const uint32_t n_out = A.n_out, n_in = A.n_in, smask = n_in >= 32 ? 0xffffffffu : (1u << n_in) - 1u, words = T.words;
+    const uint32_t region_sa = smem_addr(region);
+    if constexpr (NWP == 1) {
+        for (uint32_t w = 4 * lane; w < words; w += 128) *reinterpret_cast<uint4 *>(region + w) = make_uint4(0u, 0u, 0u, 0u);
+        __syncwarp();
+    }
+    uint32_t carry = 0;                                          // part of the first slice's first word from the turn before
+    int32_t first = T.pos0;                                      // where lane 0's slice starts
+    for (uint32_t turn = 0;; turn += SEEDS_AHEAD) {
+        RangeSeeds ahead;
+        request_seeds(A, T, turn + SEEDS_AHEAD, lane, ahead);
+#pragma unroll
+        for (uint32_t j = 0; j < SEEDS_AHEAD; ++j, first += (int32_t)(32 * n_out)) {
+            const uint32_t i = 32 * (turn + j) + lane;
+            if (first >= (int32_t)(32 * words) || 32 * (turn + j) >= T.slices) return;
+            const int32_t pos = first + (int32_t)(lane * n_out);
+            const bool live = i < T.slices && pos < (int32_t)(32 * words);
+            uint32_t x[NWP];
+            lookup<NWP>(A, tab, __funnelshift_r(s.lo[j], s.hi[j], (T.bit + i * n_in) & 31u) & smask, x);
+            const uint32_t sh = (uint32_t)pos & 31u, full = (sh + n_out) >> 5;                   // words that end in it
+            const int32_t w = pos >> 5;
+            uint32_t prev = 0;
+            if constexpr (NWP == 1) {
+#pragma unroll
+                for (int k = 0; k <= 1; ++k) {
+                    const uint32_t word = k == 0 ? x[0] << sh : __funnelshift_l(x[0], 0u, sh);
+                    if (live && (uint32_t)(w + k) < words && word)
+                        asm volatile("red.shared.xor.b32 [%0], %1;" :: "r"(region_sa + 4 * (uint32_t)(w + k)), "r"(word) : "memory");
+                }
+            } else {
+                uint32_t out[NWP + 1], tail = 0;
+#pragma unroll
+                for (int k = 0; k <= NWP; ++k) {
+                    const uint32_t cur = k < NWP ? x[k < NWP ? k : 0] : 0u;
+                    out[k] = __funnelshift_l(prev, cur, sh);
+                    prev = cur;
+                    if (k > 0 && (uint32_t)k == full) tail = out[k];                             // (0 where no word is shared)
+                }
+                const uint32_t up = __shfl_up_sync(0xffffffffu, tail, 1);
+                out[0] |= lane ? up : carry;
+                carry = __shfl_sync(0xffffffffu, tail, 31);
+                const uint32_t store = i + 1 == T.slices ? full + 1 : full;                      // the plane's last word may not end
+#pragma unroll
+                for (int k = 0; k <= NWP; ++k)
+                    if (live && (uint32_t)k < store && (uint32_t)(w + k) < words)
+                        asm volatile("st.shared.u32 [%0], %1;" :: "r"(region_sa + 4 * (uint32_t)(w + k)), "r"(out[k]) : "memory");
+            }
+        }
+        s = ahead;
+    }
+}
+
+// Run-time shape, part of a format tile (or parts of two).  A whole format tile per warp leaves most warps of a small layer idle
+// while one walks its lanes' chains of 8, 16 or 32 slices.
+// Before / with parts, us: planes of 223 x 673 with 33 x 20 11.4 / 4.3; bf16 of 1024 x 2560, three planes, 64 x 16 15.7 / 9.9; products
+// of 4864 x 1152 with 128 x 24, batch 129 21.7 / 14.8, of 960 x 1984, two planes, 33 x 20, batch 1 15.5 / 9.8, of 512 x 192 with
+// 200 x 20, batch 35 14.9 / 8.1.  Which layers: cut_tiles.  Ends with the warp synchronised.
+SQNN_DEV void decode_range(const DecodeArgs &A, uint32_t plane, uint64_t ktile, uint32_t *region, const uint32_t *tab, uint32_t lane)
+{
+    const PlanePtrs &P = A.pl[plane];
+    const uint32_t n_out = A.n_out, words = 32 * A.W, tile_bits = SQNN_TILE_SLICES * n_out;
+    const uint64_t bit0 = ktile * (32ull * words), s0 = n_out > 1 ? __umul64hi(bit0, A.inv_n_out) : bit0;
+    uint64_t ftile = s0 / SQNN_TILE_SLICES;
+    uint32_t offset = (uint32_t)(ftile * tile_bits - bit0);      // of the format tile inside the kernel tile, as a signed number
+    auto goes_on = [&] { return (int32_t)(offset + tile_bits) < (int32_t)(32 * words) && (ftile + 1) * SQNN_TILE_SLICES < A.slices; };
+    // the patch runs of the first two format tiles it overlaps, and the first seeds
+    TileRun run = fetch_run(P, ftile), run2{0u, 0u};
+    if (goes_on()) run2 = fetch_run(P, ftile + 1);
+    const uint64_t sbit = s0 * A.n_in, left = A.slices - s0;
+    const RangeTile T{P.wc + (sbit >> 5), (uint32_t)sbit & 31u, left < 0x7fffffffu ? (uint32_t)left : 0x7fffffffu, words, -(int32_t)(uint32_t)(bit0 - s0 * n_out)};
+    RangeSeeds seeds;
+    request_seeds(A, T, 0, lane, seeds);
+    uint32_t pw[PATCH_AHEAD], pw2[PATCH_AHEAD];
+    fetch_patches(A, P, run, lane, pw);
+    fetch_patches(A, P, run2, lane, pw2);
+    switch (A.nwp) {
+        case 1: expand_range<1>(A, T, seeds, region, tab, lane); break;
+        case 2: expand_range<2>(A, T, seeds, region, tab, lane); break;
+        case 4: expand_range<4>(A, T, seeds, region, tab, lane); break;
+        default: expand_range<8>(A, T, seeds, region, tab, lane); break;
+    }
+    __syncwarp();
+    for (;;) {                                                   // one format tile after the other
+        tile_patch<true>(A, P, run, pw, region, tile_bits, lane, offset, 32 * words);
+        if (!goes_on()) break;
+        offset += tile_bits;
+        ++ftile;
+        run = run2;
+#pragma unroll
+        for (uint32_t k = 0; k < PATCH_AHEAD; ++k) pw[k] = pw2[k];
+        if (goes_on()) { run2 = fetch_run(P, ftile + 1); fetch_patches(A, P, run2, lane, pw2); }
+    }
+    __syncwarp();
+}
+
+// Run-time shape: one kernel tile.
+SQNN_DEV void decode_ktile_generic(const DecodeArgs &A, uint32_t plane, uint64_t ktile, uint32_t *region, const uint32_t *tab, uint32_t lane)
+{
+    if (A.KT) decode_whole_tiles(A, plane, ktile, region, tab, lane);
+    else decode_range(A, plane, ktile, region, tab, lane);
 }
 
 // Fetch + expand + patch of one kernel tile without overlap (for the kernels that do more work per
@@ -567,7 +709,7 @@ SQNN_DEV void decode_warp_tile(const DecodeArgs &A, uint32_t plane, uint64_t til
         fetch_patches(A, P, run, lane, pw);
         tile_expand<N_OUT, N_IN>(in, region, tab, lane);
         __syncwarp();
-        tile_patch(A, P, run, pw, region, 0u, S::TILE_BITS, lane);
+        tile_patch(A, P, run, pw, region, S::TILE_BITS, lane);
         __syncwarp();
     } else {
         decode_ktile_generic(A, plane, tile, region, tab, lane);

@@ -277,7 +277,7 @@ k_gemv_tc(const TcArgs g)
                 uint32_t *region = bits_s + pl * g.region_words + t * TW;
                 tile_expand<N_OUT, N_IN>(s, region, tab_s, lane);
                 __syncwarp();
-                tile_patch(A, A.pl[pl], run, pw, region, 0u, S::TILE_BITS, lane);
+                tile_patch(A, A.pl[pl], run, pw, region, S::TILE_BITS, lane);
                 item += nwarps;
                 if (item < items) { fetch(item); fetch_patches(A, A.pl[item % n_q], run, lane, pw); }
             }

@@ -49,7 +49,8 @@ SQNN_DEV TilePos advance(TilePos p, uint32_t by, uint32_t live, uint32_t n_q)
 // flight.  REP: the lookup tables sit in shared memory in replicated form (every lane of a load
 // wavefront reads its own copy in its own banks); filling them takes a few microseconds, which pays
 // once a warp has several tiles to decode.  One block per SM.
-// SINK = true: XOR of all those words instead of storing them.
+// SINK = true: XOR of all those words instead of storing them.  Run-time shapes: REP says that kernel tiles are parts of
+// format tiles (KT = 0); two kernels, since the code of both in one costs large layers 1 %.
 constexpr uint32_t DECODE_BITS_THREADS = 768;
 template <int N_OUT, int N_IN>
 inline uint32_t decode_bits_table_words(const DecodeArgs &A, bool rep)
@@ -159,7 +160,7 @@ k_decode_bits(DecodeArgs A, uint64_t *__restrict__ out, const ClearArgs clear, c
             if (p2.plane < A.n_q) { fetch_seeds<N_OUT, N_IN>(plane_of(p2), p2.tile, lane, s2); r2 = fetch_run(plane_of(p2), p2.tile); }
             tile_expand<N_OUT, N_IN, !SINK, REP>(s0, region, smem, lane);
             __syncwarp();
-            tile_patch(A, plane_of(p0), r0, w0, region, 0u, S::TILE_BITS, lane);
+            tile_patch(A, plane_of(p0), r0, w0, region, S::TILE_BITS, lane);
             __syncwarp();
             write_out(p0);
             return p1.plane < A.n_q;
@@ -179,7 +180,8 @@ k_decode_bits(DecodeArgs A, uint64_t *__restrict__ out, const ClearArgs clear, c
         for (TilePos p = p_first; p.plane < A.n_q; p = advance(p, stride, live, A.n_q)) {
             if (!SINK && lane == 0) bulk_wait_read<0>();         // the copy out of the region is over
             __syncwarp();
-            decode_ktile_generic(A, p.plane, p.tile, region, smem, lane);
+            if constexpr (REP) decode_range(A, p.plane, p.tile, region, smem, lane);
+            else decode_whole_tiles(A, p.plane, p.tile, region, smem, lane);
             write_out(p);
         }
     }
@@ -346,7 +348,7 @@ k_decode_bf16(DecodeArgs A, const uint32_t *__restrict__ mask32, const float *__
             for (int i = 0; i < NQ; ++i) tile_expand<N_OUT, N_IN>(seeds[i], region + i * 32 * W, smem, lane);
             __syncwarp();
 #pragma unroll
-            for (int i = 0; i < NQ; ++i) tile_patch(A, A.pl[i], run[i], pw[i], region + i * 32 * W, 0u, S::TILE_BITS, lane);
+            for (int i = 0; i < NQ; ++i) tile_patch(A, A.pl[i], run[i], pw[i], region + i * 32 * W, S::TILE_BITS, lane);
             __syncwarp();
             request(tile + stride);
         } else {
@@ -472,17 +474,24 @@ inline uint32_t grid_for(uint64_t warp_tiles, uint32_t warps, uint32_t blocks_pe
 }
 
 template <int N_OUT, int N_IN>
-inline int launch_decode(const DecodeArgs &A, sqnn_out_mode mode, const uint64_t *d_mask,
+inline int launch_decode(const DecodeArgs &A0, sqnn_out_mode mode, const uint64_t *d_mask,
                          const float *d_alpha, uint64_t n, void *d_out, const ClearArgs &clear,
                          cudaStream_t st)
 {
     size_t smem = 0;
+    DecodeArgs A = A0;
+    if constexpr (N_OUT == 0) {
+        const uint64_t planes = mode == SQNN_OUT_BF16 ? 1 : A.n_q;       // a warp takes a tile of one plane or of all
+        cut_tiles(A.n_out, &A.KT, &A.W, [&](uint32_t words) {
+            return (A.words64 + 16ull * words - 1) / (16ull * words) * planes <= DECODE_BITS_THREADS / 32 * (uint64_t)sm_count();
+        });
+    }
     if (mode == SQNN_OUT_BITS || mode == SQNN_OUT_SINK) {
         // one block per SM: the tables and one region per warp.  The replicated tables are worth their
         // fill only when a warp gets several tiles.
         const uint64_t live = (A.words64 + 16ull * A.W - 1) / (16ull * A.W);
         if (live * A.n_q >= (1ull << 31)) return SQNN_E_UNSUPPORTED;
-        const bool rep = N_OUT != 0 && live * A.n_q >= 3ull * (DECODE_BITS_THREADS / 32) * (uint64_t)sm_count();
+        const bool rep = N_OUT == 0 ? A.KT == 0 : live * A.n_q >= 3ull * (DECODE_BITS_THREADS / 32) * (uint64_t)sm_count();
         const size_t tab = (size_t)decode_bits_table_words<N_OUT, N_IN>(A, rep) * 4, per_warp = (size_t)32 * A.W * 4;
         const size_t limit = 224 * 1024;
         if (tab + per_warp > limit) return SQNN_E_UNSUPPORTED;

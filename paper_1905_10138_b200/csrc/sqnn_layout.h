@@ -57,6 +57,33 @@ SQNN_HD constexpr uint32_t format_tiles_per_kernel_tile(uint32_t n_out)
     return (n_out % 4 == 0) ? 1u : (n_out % 2 == 0) ? 2u : 4u;
 }
 
+// Run-time shapes: words per lane of a kernel tile that is a part of a format tile, `turns` turns of 32 slices.  Where n_out is no
+// multiple of 32 the tile may start inside a slice and overlap one slice more than its length tells, which should not
+// cost another turn.
+SQNN_HD constexpr uint32_t range_words(uint32_t n_out, uint32_t turns)
+{
+    return n_out % 32 == 0 ? turns * n_out / 32 : (turns * 32 - 1) * n_out / 1024 ? (turns * 32 - 1) * n_out / 1024 : 1u;
+}
+// Cuts the kernel tiles (W words per lane, KT format tiles each) of a run-time shape smaller if there are idle warps:
+// the smallest parts, in turns, with which `fits(words per lane)` still finds a warp for every tile.  Large parts are not
+// worth it: their slices wait for one another from turn to turn, where a whole tile's are expanded side by side.  The
+// line is a third of the whole (part / whole, us: 3648 x 3072, 33 x 20, three planes, 10 turns of 32: 8.6 / 10.6; 5055 x 8957,
+// 50 x 20, 10 of 16: 9.5 / 8.4; 5003 x 7001, 200 x 20, two planes, 4 of 8: 10.1 / 8.7), and a single turn where a slice is whole
+// words, which takes no shifting in a whole tile (64 x 16, three planes, product of 1152 x 1664, 2 of 8: 9.9 / 9.5).
+template <typename F>
+inline void cut_tiles(uint32_t n_out, uint32_t *KT, uint32_t *W, F fits)
+{
+    const uint32_t most = n_out % 32 == 0 ? 1 : 8 * *KT / 3;
+    for (uint32_t turns = 1; turns <= most; ++turns) {
+        const uint32_t words = range_words(n_out, turns);
+        if (words < *W && fits(words)) {
+            *KT = 0;
+            *W = words;
+            return;
+        }
+    }
+}
+
 // Words of the replicated tables in shared memory.
 SQNN_HD constexpr uint32_t table_words_replicated(uint32_t n_out, uint32_t n_in)
 {

@@ -42,18 +42,24 @@ int gemv_tc_shape<SQNN_NO, SQNN_NI>(const DecodeArgs &, const TcPlan &, const ui
                                     uint32_t, float *, int64_t, uint64_t, uint64_t, cudaStream_t);
 
 template <>
-int gemv_shape<SQNN_NO, SQNN_NI>(const DecodeArgs &A, const uint64_t *d_mask, const float *d_alpha,
+int gemv_shape<SQNN_NO, SQNN_NI>(const DecodeArgs &A0, const uint64_t *d_mask, const float *d_alpha,
                                  const void *d_x, int x_dtype, int64_t ldx, uint32_t batch, float *d_y,
                                  int64_t ldy, uint64_t m, uint64_t n, cudaStream_t st)
 {
+    DecodeArgs A = A0;
     uint64_t patches = 0;
     for (uint32_t i = 0; i < A.n_q; ++i) patches += A.pl[i].n_pp;
     const double slices = (double)A.n_q * (double)((A.mn + A.n_out - 1) / A.n_out);
     GemvLayer L;
     L.m = m; L.n = n; L.batch = batch; L.n_q = A.n_q;
-    L.W = A.W; L.tab_words = A.tab_words;
+    L.tab_words = A.tab_words;
     L.x_bytes = x_dtype == SQNN_X_BF16 ? 2 : 4;
     L.sms = (uint32_t)sm_count();
+    if (SQNN_NO == 0) cut_tiles(A.n_out, &A.KT, &A.W, [&](uint32_t words) {
+        L.W = words;
+        return covering_tiles(L, (m + L.sms - 1) / L.sms) * L.n_q <= TC_WARPS;
+    });
+    L.W = A.W;
     L.density = care_density(A.n_out, A.n_in, (double)patches / slices);
     const TcPlan tc = plan_gemv_tc(L);
     const WalkPlan walk = plan_walk(L);

@@ -139,3 +139,37 @@ def test_output_buffer_size_and_alignment_are_checked():
     with pytest.raises(sqnn.SqnnError):
         sqnn.sqnn_decode(dev.desc, dev.blob, None, None, sqnn.OUT_BF16,
                          torch.zeros(16 * 80, dtype=torch.bfloat16, device="cuda"))   # mask / alpha missing
+
+
+# Run-time shapes around the sizes where slices start to share words with one neighbour only, are whole words, or take
+# another table width; layers so small that kernel tiles are parts of format tiles (a tile starts inside a slice, a slice
+# ends past the last tile, patch runs of two format tiles with more entries than are fetched ahead), and
+# layers so large that they are whole ones.
+PARTS = [(31, 6, 9, 1203, 0.5, 2), (32, 9, 7, 1999, 0.6, 1), (33, 7, 40, 1504, 0.7, 3), (50, 20, 23, 997, 0.9, 2), (63, 9, 5, 4001, 0.5, 1),
+         (64, 11, 64, 512, 0.9, 1), (65, 10, 31, 1776, 0.4, 2), (127, 12, 3, 9001, 0.3, 1), (129, 8, 17, 2000, 0.6, 1), (255, 13, 12, 3001, 0.5, 2),
+         (33, 7, 2600, 16001, 0.25, 1), (50, 8, 2600, 16001, 0.2, 1), (96, 14, 2600, 16001, 0.15, 1)]
+
+
+@pytest.mark.parametrize("n_out,n_in,m,n,keep,n_q", PARTS, ids=[f"{a}x{b}-{c}x{d}" for a, b, c, d, _, _ in PARTS])
+def test_kernel_tiles_of_run_time_shapes(n_out, n_in, m, n, keep, n_q):
+    import torch
+    layer = generic_layer(n_out, n_in, m, n, keep, 60 + n_out, n_q=n_q)
+    blob, _ = H.blob_from_library(layer)
+    dev = H.DeviceLayer(layer, blob)
+    ref = np.empty((n_q, m, n), dtype=np.uint8)
+    got = dev.decode_bits()
+    for i in range(n_q):
+        wc, np_, dp = sqnn.sqnn_unpack_host(blob, i)
+        bits = orc.decode_plane(layer.M, layer.mn, wc.astype(np.uint64), np_, dp)
+        assert np.array_equal(got[i], wl.pack_bits(bits)), i
+        ref[i] = bits.reshape(m, n)
+    if layer.mn < 1 << 22:
+        _, want = orc.reconstruct(ref, layer.mask, layer.alpha, want_f32=False)
+        assert np.array_equal(dev.decode_bf16(), want)
+    for batch, dtype in ((1, torch.bfloat16), (3, torch.float32), (17, torch.bfloat16)):
+        if batch > 15 and n % 8:                                 # a batch needs rows on 16-byte boundaries
+            continue
+        x = torch.randn((batch, n), generator=torch.Generator().manual_seed(batch)).to(dtype).float().numpy()
+        # weights and activations enter exactly: what is left are fp32 sums, whose tolerance is the reading taken for all products
+        assert H.rel_err(dev.matmul(x, dtype), orc.matmul(ref, layer.mask, layer.alpha, x.astype(np.float64))) <= 1e-4
+    assert dev.status_value() == 0
