@@ -30,6 +30,11 @@ SQNN_FOR_SHAPES(SQNN_DECLARE)
 SQNN_DECLARE(0, 0)
 #undef SQNN_DECLARE
 
+// Up to how many format tiles per SM (bf16 output, us, compile-time shape / run-time shape in parts): 1.2 tiles (2287 x 3943, 200 x 10)
+// 34.9 / 10.5, 2.8 (5516 x 1166, 60 x 12, three planes) 29.5 / 15.9, 3.7 (4544 x 2496, 80 x 8) 14.4 / 10.1, 4.1 (1408 x 4416, 40 x 16)
+// 7.0 / 7.3, 6.9 (2048 x 5120, 40 x 16) 7.3 / 11.7.
+constexpr uint64_t SMALL_TILES_PER_SM = 4;
+
 int fill_decode_args(const sqnn_desc *d, const void *d_blob, uint32_t *d_status, DecodeArgs *A)
 {
     if (!d || !d_blob) return SQNN_E_INVALID_ARG;
@@ -182,6 +187,11 @@ static int decode_queue(const sqnn_desc *desc, const void *d_blob, const uint64_
     if (out_bytes < need) return SQNN_E_INVALID_ARG;
     if (mode == SQNN_OUT_BF16 && (!d_mask || !d_alpha)) return SQNN_E_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)cuda_stream;
+    // bf16 weights of a small layer: whole format tiles (a warp expands all planes of one and writes its 256 n_out
+    // weights) leave most warps idle, the parts that the run-time-shape kernels cut do not.
+    const uint64_t whole = (A.mn + SQNN_TILE_SLICES * (uint64_t)A.n_out - 1) / (SQNN_TILE_SLICES * (uint64_t)A.n_out);
+    if (mode == SQNN_OUT_BF16 && whole <= SMALL_TILES_PER_SM * (uint64_t)sm_count())
+        return decode_shape<0, 0>(A, mode, d_mask, d_alpha, desc->n, d_out, ClearArgs{}, st);
 #define SQNN_DECODE_CASE(NO, NI) \
     if (A.n_out == NO && A.n_in == NI) return decode_shape<NO, NI>(A, mode, d_mask, d_alpha, desc->n, d_out, ClearArgs{}, st);
     SQNN_FOR_SHAPES(SQNN_DECODE_CASE)

@@ -694,7 +694,7 @@ SQNN_DEV void decode_ktile_generic(const DecodeArgs &A, uint32_t plane, uint64_t
 }
 
 // Fetch + expand + patch of one kernel tile without overlap (for the kernels that do more work per
-// tile).  `tab`: the tables in shared memory.  Ends with the warp synchronised.
+// tile).  Run-time shapes: N_IN = 1 for parts of format tiles, else whole ones.  `tab`: the tables in shared memory.  Ends with the warp synchronised.
 template <int N_OUT, int N_IN>
 SQNN_DEV void decode_warp_tile(const DecodeArgs &A, uint32_t plane, uint64_t tile,
                                uint32_t *region, const uint32_t *tab, uint32_t lane)
@@ -711,8 +711,10 @@ SQNN_DEV void decode_warp_tile(const DecodeArgs &A, uint32_t plane, uint64_t til
         __syncwarp();
         tile_patch(A, P, run, pw, region, S::TILE_BITS, lane);
         __syncwarp();
+    } else if constexpr (N_IN == 1) {
+        decode_range(A, plane, tile, region, tab, lane);
     } else {
-        decode_ktile_generic(A, plane, tile, region, tab, lane);
+        decode_whole_tiles(A, plane, tile, region, tab, lane);
     }
 }
 

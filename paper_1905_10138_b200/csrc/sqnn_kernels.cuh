@@ -225,8 +225,9 @@ SQNN_DEV void stage_mask(uint32_t *mask_s, const uint32_t *__restrict__ mask32, 
 // take 37 us and 22.0 M warp instructions, of which 7.7 M are the decode.  (Sums of the scales per weight took about 20
 // instructions, and 64 us.)  Negating all terms of a sum
 // negates it exactly, except when it is zero or not finite, and halving is exact except for the tiniest
-// numbers; rows with such a value take the plain loop, as do chunks of 8 weights that straddle rows, and
-// layers of four and more planes.
+// numbers; rows with such a value take the plain loop, as do rows of less than 32 weights and layers of four and
+// more planes.  A lane whose 32 weights straddle two rows makes them for both and keeps the second row's from its first column on
+// (with the straddling chunk weight by weight 5516 x 1166, three planes, 60 x 12 takes 15.9 us, 13.1 so).
 // One block per SM, as many warps as shared memory holds, fewer where a lane's entries need the registers.
 SQNN_HD constexpr uint32_t bf16_threads(uint32_t n_out) { return n_out > 128 ? 512 : 768; }
 constexpr uint32_t BF16_STAGE_WORDS = 2 * 512;           // two buffers of 2 KB per warp
@@ -289,7 +290,9 @@ SQNN_DEV void weights16(uint32_t zm, uint32_t qe, const RowValues<IT> &t, uint32
     }
 }
 
-template <int N_OUT, int N_IN, int NQ>
+// Run-time shapes: N_IN = 1 says that kernel tiles are parts of format tiles (KT = 0).
+// ENDS: rows may end inside a lane's 32 weights (n no multiple of 32; a kernel of its own, since it costs the others 5 to 15 %).
+template <int N_OUT, int N_IN, int NQ, bool ENDS>
 __global__ void __launch_bounds__(bf16_threads(N_OUT), 1)
 k_decode_bf16(DecodeArgs A, const uint32_t *__restrict__ mask32, const float *__restrict__ alpha,
               uint64_t n64, __nv_bfloat16 *__restrict__ out)
@@ -366,9 +369,16 @@ k_decode_bf16(DecodeArgs A, const uint32_t *__restrict__ mask32, const float *__
             __syncwarp();
             bool fast = false;
             if constexpr (NQ != 0) {
-                if (n - c >= 32 && at + 32 * lane < here) {
+                // the next row begins inside the lane's 32 weights
+                const bool next = ENDS && n - c < 32 && at + 32 * lane + (uint32_t)(n - c) < here;
+                RowValues<IT> t2 = t;
+                if ((!ENDS || n >= 32) && at + 32 * lane < here) {
                     if (r != t.row) t = row_values<NQ, IT>(alpha, r);
                     fast = !t.plain;
+                    if (next) {
+                        t2 = row_values<NQ, IT>(alpha, r + 1);
+                        fast = fast && !t2.plain;
+                    }
                 }
                 if (fast) {
                     const uint32_t b0 = bits[0], sgn = ~b0;
@@ -390,6 +400,21 @@ k_decode_bf16(DecodeArgs A, const uint32_t *__restrict__ mask32, const float *__
                         weights16<NQ, IT>(__byte_perm(me, mo, h ? 0x7632 : 0x5410), __byte_perm(qe, qo, h ? 0x7362 : 0x5140), t, o);
                         *reinterpret_cast<uint4 *>(to + 4 * ((2 * h + turn) & 3u)) = make_uint4(o[0], o[1], o[2], o[3]);
                         *reinterpret_cast<uint4 *>(to + 4 * ((2 * h + 1 + turn) & 3u)) = make_uint4(o[4], o[5], o[6], o[7]);
+                    }
+                    if (next) {                                  // once more with the next row's values, from its first column on
+                        const uint32_t k = (uint32_t)(n - c);
+#pragma unroll
+                        for (uint32_t h = 0; h < 2; ++h) {
+                            uint32_t o[8];
+                            weights16<NQ, IT>(__byte_perm(me, mo, h ? 0x7632 : 0x5410), __byte_perm(qe, qo, h ? 0x7362 : 0x5140), t2, o);
+#pragma unroll
+                            for (uint32_t j = 0; j < 8; ++j) {
+                                const uint32_t word = 4 * ((2 * h + j / 4 + turn) & 3u) + j % 4;
+                                if (2 * word >= k) to[word] = o[j];
+                                else if (2 * word + 1 == k) to[word] = __byte_perm(to[word], o[j], 0x7610);
+                            }
+                        }
+                        t = t2;
                     }
                 }
             }
@@ -529,10 +554,16 @@ inline int launch_decode(const DecodeArgs &A0, sqnn_out_mode mode, const uint64_
         const uint32_t warps = spread_warps(live, (uint32_t)std::min<size_t>((limit - tab) / per_warp, bf16_threads(N_OUT) / 32));
         smem = tab + warps * per_warp;
         const uint32_t grid = grid_for(live, warps, 1);
+        const bool ends = n % 32 != 0;
+#define SQNN_BF16_LAUNCH2(NQV, PARTSV)                                                                   \
+    do {                                                                                                 \
+        return launch_kernel(ends ? k_decode_bf16<N_OUT, N_OUT ? N_IN : PARTSV, NQV, NQV != 0>           \
+                                  : k_decode_bf16<N_OUT, N_OUT ? N_IN : PARTSV, NQV, false>,             \
+                             grid, warps * 32, smem, st, A, (const uint32_t *)d_mask, d_alpha, n, (__nv_bfloat16 *)d_out); \
+    } while (0)
 #define SQNN_BF16_LAUNCH(NQV)                                                                            \
     do {                                                                                                 \
-        return launch_kernel(k_decode_bf16<N_OUT, N_IN, NQV>, grid, warps * 32, smem, st, A, (const uint32_t *)d_mask, \
-                             d_alpha, n, (__nv_bfloat16 *)d_out);                                        \
+        if (N_OUT == 0 && A.KT == 0) SQNN_BF16_LAUNCH2(NQV, 1); else SQNN_BF16_LAUNCH2(NQV, 0);          \
     } while (0)
         if (n >= (1ull << 31) || A.mn / n >= (1ull << 31)) SQNN_BF16_LAUNCH(0);       // 64-bit rows and columns
         else if (A.n_q == 1) SQNN_BF16_LAUNCH(1);
@@ -540,6 +571,7 @@ inline int launch_decode(const DecodeArgs &A0, sqnn_out_mode mode, const uint64_
         else if (A.n_q == 3) SQNN_BF16_LAUNCH(3);
         else SQNN_BF16_LAUNCH(0);
 #undef SQNN_BF16_LAUNCH
+#undef SQNN_BF16_LAUNCH2
     }
     return cudaGetLastError() == cudaSuccess ? SQNN_OK : SQNN_E_CUDA;
 }

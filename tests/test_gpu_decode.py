@@ -173,3 +173,28 @@ def test_kernel_tiles_of_run_time_shapes(n_out, n_in, m, n, keep, n_q):
         # weights and activations enter exactly: what is left are fp32 sums, whose tolerance is the reading taken for all products
         assert H.rel_err(dev.matmul(x, dtype), orc.matmul(ref, layer.mask, layer.alpha, x.astype(np.float64))) <= 1e-4
     assert dev.status_value() == 0
+
+
+# Rows that end at every place of a lane's 32 weights, next to rows whose values take the plain way (zero, infinite, NaN scales); in
+# parts of format tiles (small layers) and, the last three, whole ones.
+ENDS = [(40, 12, 70, 31, 3), (40, 12, 70, 33, 3), (60, 12, 65, 63, 2), (100, 10, 300, 47, 1), (80, 8, 40, 1025, 2), (33, 7, 90, 95, 3),
+        (40, 12, 6100, 1037, 3), (80, 16, 15000, 1001, 1), (60, 12, 130, 75011, 2)]
+
+
+@pytest.mark.parametrize("n_out,n_in,m,n,n_q", ENDS, ids=[f"{a}x{b}-{c}x{d}-q{q}" for a, b, c, d, q in ENDS])
+def test_bf16_rows_that_end_inside_a_word(n_out, n_in, m, n, n_q):
+    layer = generic_layer(n_out, n_in, m, n, 0.3, 70 + n % 7, n_q=n_q)
+    layer.alpha[m // 3, 0] = np.inf
+    layer.alpha[m // 2, :] = 0.0
+    layer.alpha[m // 2 + 2, n_q - 1] = np.nan
+    blob, _ = H.blob_from_library(layer)
+    dev = H.DeviceLayer(layer, blob)
+    ref = np.empty((n_q, m, n), dtype=np.uint8)
+    for i in range(n_q):
+        wc, np_, dp = sqnn.sqnn_unpack_host(blob, i)
+        ref[i] = orc.decode_plane(layer.M, layer.mn, wc.astype(np.uint64), np_, dp).reshape(m, n)
+    _, want = orc.reconstruct(ref, layer.mask, layer.alpha, want_f32=False)
+    got = dev.decode_bf16()
+    nan = (want & 0x7fff) > 0x7f80
+    assert np.array_equal((got & 0x7fff) > 0x7f80, nan) and np.array_equal(got[~nan], want[~nan])
+    assert dev.status_value() == 0
