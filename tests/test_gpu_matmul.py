@@ -309,3 +309,27 @@ def test_products_queued_back_to_back_and_from_two_threads():
         t.join()
     assert not failures, failures[:5]
     assert all(d.status_value() == 0 for d, _, _, _ in jobs)
+
+
+@pytest.mark.parametrize("m,batch,ahead,gap", [(37, 391, 0, 0), (4, 16, 0, 0), (333, 500, 1, 0), (64, 301, 0, 3), (130, 130, 2, 1)])
+def test_y_of_a_large_batch_is_cleared_whatever_its_alignment(m, batch, ahead, gap):
+    """Few tiles and a large Y: blocks without a tile clear their share of it (16 bytes at a time where Y allows)."""
+    import torch
+    layer = wl.make_layer(1, m=m, n=256)
+    blob, _ = H.blob_from_library(layer)
+    dev = H.DeviceLayer(layer, blob)
+    x = layer.activations(batch).astype(np.float32)
+    x = torch.from_numpy(x).to(torch.bfloat16)
+    buf = torch.full((ahead + batch * (m + gap) + 4,), float("nan"), dtype=torch.float32, device="cuda")
+    y = buf[ahead:ahead + batch * (m + gap)].view(batch, m + gap)[:, :m]
+    ws = torch.empty(max(sqnn.sqnn_workspace_bytes(dev.desc, batch), 256), dtype=torch.uint8, device="cuda")
+    sqnn.sqnn_decode_matmul(dev.desc, dev.blob, dev.mask, dev.alpha, x.cuda(), y, ws, dev.status)
+    torch.cuda.synchronize()
+    wc, np_, dp = sqnn.sqnn_unpack_host(blob, 0)
+    bits = orc.decode_plane(layer.M, layer.mn, wc.astype(np.uint64), np_, dp).reshape(1, m, 256)
+    assert H.rel_err(y.cpu().numpy(), orc.matmul(bits, layer.mask, layer.alpha, x.double().numpy())) <= 2e-4
+    # nothing else was touched
+    assert torch.isnan(buf[:ahead]).all() and torch.isnan(buf[ahead + batch * (m + gap):]).all()
+    if gap:
+        assert torch.isnan(buf[ahead:ahead + batch * (m + gap)].view(batch, m + gap)[:, m:]).all()
+    assert dev.status_value() == 0
