@@ -3,6 +3,7 @@ import numpy as np
 import pytest
 
 from oracle import oracle as orc
+from paper_1905_10138_b200 import sqnn
 from paper_1905_10138_b200 import workloads as wl
 from tests import helpers as H
 from tests.test_gpu_decode import generic_layer
