@@ -76,7 +76,9 @@ int fill_decode_args(const sqnn_desc *d, const void *d_blob, uint32_t *d_status,
 
 int ensure_dynamic_smem(const void *kernel, size_t smem)
 {
-    if (smem <= 48 * 1024) return SQNN_OK;
+    // A kernel may have 48 KB without asking, its static variables included (704 bytes at most, next to dynamic memory).
+    constexpr size_t STATIC_ROOM = 1024;
+    if (smem <= 48 * 1024 - STATIC_ROOM) return SQNN_OK;
     static std::mutex mu;
     static std::map<std::pair<const void *, int>, size_t> granted;
     int dev = 0;

@@ -121,6 +121,25 @@ def test_tensor_core_product_at_tile_edges(case):
     assert H.rel_err(y, ref) <= 2e-4
 
 
+# The product's dynamic shared memory ends less than its static variables below 48 KB (49136, 49152, 48976 and 49008 bytes), where a
+# launch needs a larger limit although the dynamic part alone does not.
+JUST_BELOW_48_KB = [
+    (100, 10, 18, 930, 0.1, 2, "f32", 2),
+    (100, 10, 34, 1018, 0.1, 2, "bf16", 6),
+    (96, 14, 47, 1031, 0.15, 2, "f32", 3),
+    (64, 16, 56, 1049, 0.25, 3, "bf16", 10),
+]
+
+
+@pytest.mark.parametrize("case", JUST_BELOW_48_KB, ids=lambda c: "x".join(map(str, c)))
+def test_small_batch_product_with_just_below_48_kb_of_shared_memory(case):
+    n_out, n_in, m, n, keep, n_q, x_dtype, batch = case
+    layer = generic_layer(n_out, n_in, m, n, keep, 57, n_q=n_q)
+    layer.x_dtype = x_dtype
+    y, ref = product(layer, layer.activations(batch), x_dtype)
+    assert H.rel_err(y, ref) <= 1e-4
+
+
 # n below, at and above the 8, 32 and 1024 columns at which a lane's words cross rows; whole-word and shifted
 # run-time network shapes; scales whose sums vanish, are infinite or tiny
 BF16 = [(40, 12, 50, 7, 2), (100, 10, 40, 33, 1), (60, 12, 9, 1024, 3), (60, 12, 9, 1025, 3), (200, 10, 30, 2001, 2),
