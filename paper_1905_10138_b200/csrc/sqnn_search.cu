@@ -13,7 +13,9 @@
 // matter.  (Ties go to the smallest seed.  Pivot columns are the lowest possible ones, so the seed with all other bits 0, which
 // the keys hold, is the smallest of those with the same errors.)  Sizes 0 and 1 are done by a thread per slice and decide
 // 92 % of them; of the rest the warp finishes one slice after the other, the lanes sharing the pairs and, for one slice in a
-// hundred, sets of three to five columns; what remains tries all 2^n_in sets in Gray-code order.
+// hundred, sets of three to five columns; what remains tries all 2^rank sets in Gray-code order.
+// Columns that the elimination leaves zero are only sorted out for what the pairs have not decided: a test of all columns in every slice's
+// own thread costs the LSTM gates 4 %.
 //
 // The care positions of a slice are squeezed together first: up to 32 of them make one word per column, up to 64 two, whatever
 // n_out is.  A step takes each lane's next care position; its row of M, with the bits of four columns in the four
@@ -167,7 +169,7 @@ struct Candidate<0, NI> {
 // The reduced columns of one slice per thread, for the slices the whole warp finishes.
 template <int NI>
 struct Columns {
-    uint32_t word[3][NI][SEARCH_THREADS];
+    uint32_t word[3][NI][SEARCH_THREADS + 1];                            // + 1: the columns of a slice in different banks
     template <int KW>
     SQNN_DEV void put(uint32_t c, uint32_t slot, const Candidate<KW, NI> &x)
     {
@@ -194,14 +196,32 @@ struct Columns {
     }
 };
 
-// The whole warp tries all 2^n_in sets of columns of one slice: the lanes split them by the top bits.
+// Columns that are zero after the elimination (sums of others, or empty at the care positions) add nothing to a set: one slice's go behind its
+// other columns, whose number, the rank, is returned.  A network of rank 10 with 20 columns has 2^10 sets to try for a
+// slice, not 2^20 (300 x 300, 64 x 20, us: 7745 with the zero columns among the others).
 template <int KW, int NI>
-SQNN_DEV uint32_t try_all_sets(const Columns<NI> &col, uint32_t slot, Candidate<KW, NI> x, uint32_t n_in, uint32_t lane)
+SQNN_DEV uint32_t gather_columns(Columns<NI> &col, uint32_t slot, uint32_t lane)
 {
-    const uint32_t low_bits = n_in > 5 ? n_in - 5 : 0, lanes_used = n_in >= 5 ? 32u : (1u << n_in);
+    Candidate<KW, NI> own{};
+    if (lane < NI) own = col.template get<KW>(lane, slot);
+    const uint32_t some = __ballot_sync(0xffffffffu, !own.none()), rank = (uint32_t)__popc(some);
+    if (some & (some + 1u)) {
+        const uint32_t before = (uint32_t)__popc(some & ((1u << lane) - 1u));
+        __syncwarp();
+        if (lane < NI) col.put((some >> lane) & 1u ? before : rank + lane - before, slot, own);
+        __syncwarp();
+    }
+    return rank;
+}
+
+// The whole warp tries all 2^rank sets of columns of one slice: the lanes split them by the top bits.
+template <int KW, int NI>
+SQNN_DEV uint32_t try_all_sets(const Columns<NI> &col, uint32_t slot, Candidate<KW, NI> x, uint32_t rank, uint32_t lane)
+{
+    const uint32_t low_bits = rank > 5 ? rank - 5 : 0, lanes_used = rank >= 5 ? 32u : (1u << rank);
     uint32_t best = 0xffffffffu;
     if (lane < lanes_used) {
-        for (uint32_t c = low_bits; c < n_in; ++c)
+        for (uint32_t c = low_bits; c < rank; ++c)
             if ((lane >> (c - low_bits)) & 1u) x.add(col.template get<KW>(c, slot));
         const uint32_t count = 1u << low_bits;
         for (uint32_t i = 0; i < count; ++i) {
@@ -263,15 +283,18 @@ SQNN_DEV uint32_t walk_sets(const Columns<NI> &col, uint32_t slot, const Candida
 // long as the best count exceeds the sets' size, up to five columns; then all sets.  (Slices far from being consistent, with
 // many care bits for their seed bits, go there at once: the next sizes would not decide them.)
 template <int KW, int NI>
-SQNN_DEV uint32_t try_larger_sets(const Columns<NI> &col, uint32_t slot, const uint32_t (&lanes_pairs)[PAIRS_PER_LANE<NI>], const Candidate<KW, NI> &x,
+SQNN_DEV uint32_t try_larger_sets(Columns<NI> &col, uint32_t slot, const uint32_t (&lanes_pairs)[PAIRS_PER_LANE<NI>], const Candidate<KW, NI> &x,
                                   uint32_t best, uint32_t n_in, uint32_t lane)
 {
     Candidate<KW, NI> pair[PAIRS_PER_LANE<NI>];
+    auto load_pairs = [&] {
 #pragma unroll
-    for (uint32_t k = 0; k < (uint32_t)PAIRS_PER_LANE<NI>; ++k) {
-        pair[k] = col.template get<KW>(lanes_pairs[k] & 0xffffu, slot);
-        pair[k].add(col.template get<KW>(lanes_pairs[k] >> 16, slot));
-    }
+        for (uint32_t k = 0; k < (uint32_t)PAIRS_PER_LANE<NI>; ++k) {
+            pair[k] = col.template get<KW>(lanes_pairs[k] & 0xffffu, slot);
+            pair[k].add(col.template get<KW>(lanes_pairs[k] >> 16, slot));
+        }
+    };
+    load_pairs();
 #pragma unroll
     for (uint32_t k = 0; k < (uint32_t)PAIRS_PER_LANE<NI>; ++k) {
         Candidate<KW, NI> y = x;
@@ -280,18 +303,20 @@ SQNN_DEV uint32_t try_larger_sets(const Columns<NI> &col, uint32_t slot, const u
     }
     best = warp_min(best);
     if ((best >> 20) <= 2u) return best;
+    const uint32_t rank = gather_columns<KW>(col, slot, lane);
+    if (rank < n_in) load_pairs();
     Candidate<KW, NI> v[NI];
 #pragma unroll
     for (int c = 0; c < NI; ++c) v[c] = col.template get<KW>(c, slot);
-    best = warp_min(walk_sets<1>(col, slot, v, pair, x, n_in, lane, best));
+    best = warp_min(walk_sets<1>(col, slot, v, pair, x, rank, lane, best));
     if ((best >> 20) <= 3u) return best;
     if ((best >> 20) <= 6u) {
-        best = warp_min(walk_sets<2>(col, slot, v, pair, x, n_in, lane, best));
+        best = warp_min(walk_sets<2>(col, slot, v, pair, x, rank, lane, best));
         if ((best >> 20) <= 4u) return best;
-        best = warp_min(walk_sets<3>(col, slot, v, pair, x, n_in, lane, best));
+        best = warp_min(walk_sets<3>(col, slot, v, pair, x, rank, lane, best));
         if ((best >> 20) <= 5u) return best;
     }
-    return min(best, try_all_sets<KW>(col, slot, x, n_in, lane));
+    return min(best, try_all_sets<KW>(col, slot, x, rank, lane));
 }
 
 // A lane's care positions in ascending order.  Up to two words sit in registers, more in the lane's slots of shared memory.
@@ -405,8 +430,10 @@ SQNN_DEV uint32_t search_slices(const uint32_t (&rows_s)[(NI + 3) / 4][32 * NW +
 }
 
 // NI >= n_in, 32 NW >= n_out.  The loops over columns have a fixed length; a column past n_in is a zero that changes nothing.
+// Blocks per SM: what the elimination's 64, 80, 96 or 128 registers allow.  Left to itself the compiler takes 15 more for some and a block
+// less is resident (LSTM gates, with five blocks instead of six, 55.6 -> 58.5 us), and 168 to 220 for 20 columns of eight words.
 template <int NI, int NW>
-__global__ void __launch_bounds__(SEARCH_THREADS)
+__global__ void __launch_bounds__(SEARCH_THREADS, NI <= 8 ? 8 : NI <= 12 ? (NW <= 2 ? 6 : 5) : NI <= 16 && NW <= 2 ? 5 : 4)
 k_search_seeds(const __grid_constant__ SearchArgs S)
 {
     __shared__ uint32_t rows_s[(NI + 3) / 4][32 * NW + 1];                // rows past n_out are zero

@@ -58,6 +58,8 @@ SEARCH = [
     ("3x1", lambda: generic_layer(3, 1, 5, 77, 0.2, 41)),
     ("96x10-one-slice", lambda: generic_layer(96, 10, 1, 50, 0.5, 42)),
     ("64x10-rank-3", lambda: low_rank_layer(64, 10, 3, 43)),
+    ("64x20-rank-10", lambda: low_rank_layer(64, 20, 10, 44)),
+    ("100x16-rank-12", lambda: low_rank_layer(100, 16, 12, 45)),
 ]
 
 
@@ -70,6 +72,35 @@ def low_rank_layer(n_out, n_in, rank, seed):
     mix[:, [0, n_in // 2]] = 0
     layer.M[:] = (basis @ mix % 2).astype(layer.M.dtype)
     return layer
+
+
+@pytest.mark.gpu
+def test_gpu_seed_search_tries_sets_of_independent_columns_only():
+    """20 columns of rank 10 have 2^10 different sums.  A search that goes through 2^20 sets of columns takes some 300 times as long as the
+    search for a network of full rank, whose slices are decided by small sets; this one about twice as long."""
+    import torch
+
+    def milliseconds(layer):
+        planes_words, mask_words = packed(layer)
+        l = (layer.mn + layer.n_out - 1) // layer.n_out
+        d_planes, d_mask = (torch.from_numpy(a.view(np.int64)).cuda() for a in (planes_words, mask_words))
+        d_wc = torch.zeros(l, dtype=torch.int32, device="cuda")
+        d_np = torch.zeros(l, dtype=torch.int16, device="cuda")
+        times = []
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(10):
+                sqnn.sqnn_search_seeds(wl.network_rows(layer.M), layer.n_in, layer.m, layer.n, 1, d_planes, d_mask, d_wc, d_np)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b) / 10)
+        return min(times)
+
+    full = generic_layer(64, 20, 300, 300, 0.3, 46)
+    low = generic_layer(64, 20, 300, 300, 0.3, 46)
+    low.M[:, 10:] = low.M[:, :10] @ np.random.default_rng(47).integers(0, 2, (10, 10)) % 2
+    assert milliseconds(low) < 30 * milliseconds(full)
 
 
 @pytest.mark.gpu
