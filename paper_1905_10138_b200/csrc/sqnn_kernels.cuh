@@ -69,6 +69,14 @@ struct BitsArgs {
     uint32_t live;         // tiles that hold at least one real word, per plane
     uint32_t full_tiles;   // tiles before this one lie wholly inside the plane and end on a whole word
 };
+// Networks with two lookups a slice in tables of four words and more (80 x 16, 200 x 10) need more registers than a thread has.  On large layers they
+// spill in worse places with the counts that the launcher hands over and a branch around the deliveries (2^30 weights, us, with / without:
+// 200 x 10, S = 0.95 39.4 / 36.3, 0.90 56.4 / 52.6, 0.80 83.9 / 80.2; 80 x 16, S = 0.90 34.0 / 32.1, 0.95 30.1 / 30.5), so there they keep
+// the plain form; the others gain 1 % from it (100 x 10, S = 0.95 28.4 / 28.7).
+SQNN_HD constexpr bool short_of_registers(uint32_t n_out, uint32_t n_in)
+{
+    return entry_words_padded(n_out) >= 4 && table_chunks(n_in, entry_words_padded(n_out)) > 1;
+}
 template <int N_OUT, int N_IN, bool SINK, bool ONE_PLANE, bool REP>
 __global__ void __launch_bounds__(DECODE_BITS_THREADS, 1)
 k_decode_bits(DecodeArgs A, uint64_t *__restrict__ out, const ClearArgs clear, const BitsArgs B)
@@ -80,15 +88,24 @@ k_decode_bits(DecodeArgs A, uint64_t *__restrict__ out, const ClearArgs clear, c
     const uint32_t tab_words_s = N_OUT != 0 && REP ? table_words_replicated(N_OUT, N_IN) : A.tab_words;
     uint32_t *region = smem + tab_words_s + warp * 32 * W;
     const uint64_t tail_bits = A.mn & 63;
-    const uint32_t live = B.live, full_tiles = B.full_tiles;
+    constexpr bool IN_KERNEL = N_OUT != 0 && REP && short_of_registers(N_OUT, N_IN);
+    uint32_t live = B.live, full_tiles = B.full_tiles;
+    if constexpr (IN_KERNEL) {
+        wait_prior_grid();
+        launch_dependents();
+        live = (uint32_t)((A.words64 + 16 * W - 1) / (16 * W));
+        full_tiles = (uint32_t)(A.words64 / (16 * W)) - ((tail_bits != 0 && A.words64 % (16 * W) == 0) ? 1u : 0u);
+    }
     const uint32_t stride = gridDim.x * nwarps;
     TilePos p_first = advance(TilePos{0u, 0u}, blockIdx.x * nwarps + warp, live, A.n_q);
     const uint64_t clear_lo = blockIdx.x * clear.per_block;
     uint64_t sink = 0;
-    p_first.plane = settle(p_first.plane);
-    p_first.tile = settle(p_first.tile);
-    wait_prior_grid();
-    launch_dependents();
+    if constexpr (!IN_KERNEL) {
+        p_first.plane = settle(p_first.plane);
+        p_first.tile = settle(p_first.tile);
+        wait_prior_grid();
+        launch_dependents();
+    }
 
     auto write_out = [&](TilePos p) {
         uint64_t *pbase = out + (uint64_t)p.plane * A.words64;
@@ -150,7 +167,7 @@ k_decode_bits(DecodeArgs A, uint64_t *__restrict__ out, const ClearArgs clear, c
         auto step = [&](TilePos &p0, TileSeeds<N_OUT, N_IN> &s0, TileRun &r0, uint32_t (&w0)[PATCH_AHEAD],
                         TilePos &p1, TileRun &r1, uint32_t (&w1)[PATCH_AHEAD],
                         TilePos &p2, TileSeeds<N_OUT, N_IN> &s2, TileRun &r2) {
-            if (p1.plane < A.n_q) {
+            if (IN_KERNEL || p1.plane < A.n_q) {
                 // everything this step consumes was requested at least a step ago: take delivery of it now,
                 // before the loads of this step are issued
 #pragma unroll
