@@ -260,7 +260,7 @@ k_decode_gemv(const GemvArgs g)
             }
             for (; item < items; item += nwarps) {
                 const uint32_t t = item / n_q, pl = item - t * n_q;
-                decode_ktile_generic(A, pl, kt0 + t, bits_s + pl * g.region_words + t * TW, tab_s, lane);
+                decode_warp_tile<N_OUT, N_IN>(A, pl, kt0 + t, bits_s + pl * g.region_words + t * TW, tab_s, lane);
             }
         }
         cp_async_wait_all();
@@ -392,7 +392,9 @@ inline int launch_gemv_bt(const DecodeArgs &A, const WalkPlan &plan, const uint6
     g.wait_limit = dbg.wait_cycles ? dbg.wait_cycles : GEMV_WAIT_LIMIT;
 #define SQNN_GEMV_LAUNCH(XSV, NQV)                                                                       \
     do {                                                                                                 \
-        return launch_kernel(k_decode_gemv<N_OUT, N_IN, BT, XT, XSV, NQV>, plan.grid, plan.warps * 32, plan.smem, st, g); \
+        auto k = k_decode_gemv<N_OUT, N_IN, BT, XT, XSV, NQV>;                                           \
+        if constexpr (N_OUT == 0) if (A.KT == 0) k = k_decode_gemv<0, 1, BT, XT, XSV, NQV>;              \
+        return launch_kernel(k, plan.grid, plan.warps * 32, plan.smem, st, g);                           \
     } while (0)
     if constexpr (BT == 1) {
         if (plan.xs) {
