@@ -5,7 +5,7 @@
 // As a rule it is KT format tiles (256 slices), KT chosen so that 8 * KT * n_out is a multiple of 32 bits: a lane owns 8 * KT
 // consecutive slices, whose W output words are private to it while it expands; in the seed stream a lane's 8 slices of
 // one format tile are n_in consecutive bytes.  (Shapes with compile-time kernels have KT = 1.)  In small layers of other
-// shapes it is a part of a format tile, so that all warps have something to decode: see decode_range.
+// shapes it is a run of a few turns of 32 slices, wherever it starts, so that more warps have something to decode: see decode_range.
 //
 // The network (Section 3.1, w~ = M . w^c) is evaluated with the lookup tables stored in the
 // blob (geometry in sqnn_layout.h), copied to shared memory once per block.
@@ -643,11 +643,12 @@ SQNN_DEV void expand_range(const DecodeArgs &A, const RangeTile &T, RangeSeeds &
     }
 }
 
-// Run-time shape, part of a format tile (or parts of two).  A whole format tile per warp leaves most warps of a small layer idle
+// Run-time shape, part of a format tile, as the parts are called: up to 10 turns of 32 slices that start anywhere, so that one may overlap three
+// format tiles (of 8 turns) and take from three patch runs.  A whole format tile per warp leaves most warps of a small layer idle
 // while one walks its lanes' chains of 8, 16 or 32 slices.
 // Before / with parts, us: planes of 223 x 673 with 33 x 20 11.4 / 4.3; bf16 of 1024 x 2560, three planes, 64 x 16 15.7 / 9.9; products
 // of 4864 x 1152 with 128 x 24, batch 129 21.7 / 14.8, of 960 x 1984, two planes, 33 x 20, batch 1 15.5 / 9.8, of 512 x 192 with
-// 200 x 20, batch 35 14.9 / 8.1.  Which layers: cut_tiles.  Ends with the warp synchronised.
+// 200 x 20, batch 35 14.9 / 8.1.  Which layers: most_parts_per_sm, cut_gemv_tiles.  Ends with the warp synchronised.
 SQNN_DEV void decode_range(const DecodeArgs &A, uint32_t plane, uint64_t ktile, uint32_t *region, const uint32_t *tab, uint32_t lane)
 {
     const PlanePtrs &P = A.pl[plane];

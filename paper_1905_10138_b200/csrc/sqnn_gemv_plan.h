@@ -12,9 +12,9 @@
 // small and the sparse layer with few vectors, where the expanding form's longer chain of phases and its units of
 // 16 rows x 1024 columns cost more than the care bits do.  Expanding / walk, one vector:
 //   2048 x 1024, 7 % kept 5.7 / 4.4 us     1024 x 3072, 7 % kept 6.1 / 4.8     4096 x 9216, 9 % kept 9.8 / 11.5
-// Over 1048 random calls of that kind (2^16 to 2^26 weights, 2 to 50 % kept, 1 to 15 vectors) the rule takes 172 to the
+// Over 1048 random calls of that kind (2^16 to 2^26 weights, 2 to 50 % kept, 1 to 15 vectors), all in whole format tiles, the rule takes 172 to the
 // walk; none loses more than 5 %, and all 1048 together gain 3 % (geometric mean), where always choosing right
-// would gain 4 %.
+// would gain 4 %.  Layers of run-time shapes that have room for parts: cut_gemv_tiles.
 // The walk is also faster on sparse or wide layers with fp32 activations or several planes (2048 x 1024, 3.5 % kept, 8
 // fp32 vectors: 10.2 / 7.5 us; 4096 x 12288, 10 % kept, 4 fp32 vectors, where the expanding form runs out of shared
 // memory: 67 / 36).  It does not get those calls: its sums lie further from the 64-bit product.  Relative errors over
@@ -27,6 +27,8 @@
 #include <math.h>
 #include <stddef.h>
 #include <stdint.h>
+
+#include "sqnn_layout.h"
 
 namespace sqnn {
 
@@ -44,6 +46,7 @@ struct GemvLayer {
     uint32_t x_bytes;             // of an activation: 2 (bf16) or 4 (fp32)
     uint32_t sms;
     double density;               // share of unpruned weights, estimated (care_density); read for one plane and bf16 only
+    double tile_us = 0.0;         // estimated time a warp takes to decode a tile; 0: by W, the constants of whole tiles
 };
 
 // The mask's density is on the device.  What the blob says of it: a slice with k care bits of rank r needs about
@@ -74,7 +77,7 @@ struct TcPlan {
 };
 
 // Estimates for bf16 activations and one plane, with constants fitted to the calls above (standard deviation of the
-// logarithm: 16 %).  Fixed costs, decode (per word of a lane's tile and warp), and per pass of a chunk its staging, set-up and
+// logarithm: 16 %).  Fixed costs, decode (per word of a lane's tile and warp, or GemvLayer::tile_us), and per pass of a chunk its staging, set-up and
 // expansion: e us per 128 columns of 16 rows x 8 ranges and group, more with N (above 64 there is one A slot per
 // group, and expansion and MMA take turns).
 inline double tc_estimate_us(const GemvLayer &L, const TcPlan &p, uint32_t passes)
@@ -89,7 +92,7 @@ inline double tc_estimate_us(const GemvLayer &L, const TcPlan &p, uint32_t passe
         chunks += times;
         left -= times * rows;
     }
-    us += chunks * 0.056 * L.W * (double)((covering_tiles(L, p.rows_per_chunk) * L.n_q + TC_WARPS - 1) / TC_WARPS);
+    us += chunks * (L.tile_us > 0 ? L.tile_us : 0.056 * L.W) * (double)((covering_tiles(L, p.rows_per_chunk) * L.n_q + TC_WARPS - 1) / TC_WARPS);
     return us + (passes > 1 ? passes * chunks : 1) * 0.016 * p.bt * p.units;
 }
 
@@ -161,7 +164,7 @@ inline double walk_estimate_us(const GemvLayer &L, const WalkPlan &p)
         chunks += times;
         left -= times * rows;
     }
-    return us + chunks * 0.07 * L.W * (double)((covering_tiles(L, p.rows_per_chunk) * L.n_q + p.warps - 1) / p.warps);
+    return us + chunks * (L.tile_us > 0 ? L.tile_us : 0.07 * L.W) * (double)((covering_tiles(L, p.rows_per_chunk) * L.n_q + p.warps - 1) / p.warps);
 }
 
 inline WalkPlan plan_walk(const GemvLayer &L)
@@ -214,6 +217,38 @@ inline WalkPlan plan_walk(const GemvLayer &L)
         xs = false;                                       // leave the activations in global memory
         RC = R;
     }
+}
+
+// Run-time shapes: the tiles of a layer that has room for parts of format tiles (L.W: words of whole ones), for each of the two forms.  KT = 0:
+// parts.  Whole tiles of slices with a single lookup are cheap (see most_parts_per_sm): where kernel tiles are single format tiles,
+// the walk never cuts them (parts / whole, us: 960 x 576, 8 x 2 5.7 / 4.9; 8000 x 1984, 256 x 4 7.9 / 6.9; 512 x 576, 96 x 3 4.6 / 4.4) and the
+// expanding form cuts them to one turn or not at all (96 x 7, one turn 6.6 / 7.0; 112 x 3, two turns 9.0 / 8.6); of
+// two format tiles, to two turns at most (56 x 10, two of 16 7.3 / 7.8; 50 x 5, four 10.9 / 10.7).
+// Estimates: a part costs its turns; whole tiles against parts of the other form their words, at less than where both are whole.
+// 273 one-plane bf16 calls with room for parts (2^16 to 2^25 weights, 1 to 15 vectors, any network): 0.76 of the time of whole tiles for both forms,
+// 0.9 % over always choosing right; 3 of them are more than 3 % slower than with whole tiles (by 4 % at most), 15 (by 20 %) where both
+// forms cut all they can.
+struct GemvTiles {
+    uint32_t KT, W;
+};
+inline void cut_gemv_tiles(uint32_t n_out, uint32_t n_in, GemvLayer *expanding, GemvLayer *walk, GemvTiles *for_expanding, GemvTiles *for_walk)
+{
+    const GemvTiles whole{format_tiles_per_kernel_tile(n_out), expanding->W};
+    const bool cheap = table_chunks(n_in, entry_words_padded(n_out)) == 1 && whole.KT < 4;
+    auto cut = [&](GemvLayer *L, GemvTiles *T, uint32_t most, double turn_us) {
+        *T = whole;
+        const uint32_t turns = cut_tiles(n_out, most, &T->KT, &T->W, [&](uint32_t words) {
+            GemvLayer M = *L;
+            M.W = words;
+            return covering_tiles(M, (L->m + L->sms - 1) / L->sms) * L->n_q <= TC_WARPS;
+        });
+        L->W = T->W;
+        L->tile_us = turns * turn_us;
+    };
+    const uint32_t most = most_turns(n_out);
+    cut(expanding, for_expanding, cheap && whole.KT < most ? whole.KT : most, 0.8);
+    cut(walk, for_walk, cheap && whole.KT == 1 ? 0 : cheap && whole.KT < most ? whole.KT : most, 0.7);
+    if (for_expanding->KT == 0 && for_walk->KT != 0) walk->tile_us = 0.02 * whole.W;
 }
 
 inline bool take_walk(const GemvLayer &L, const TcPlan &t, const WalkPlan &w)

@@ -530,10 +530,9 @@ inline int launch_decode(const DecodeArgs &A0, sqnn_out_mode mode, const uint64_
     size_t smem = 0;
     DecodeArgs A = A0;
     if constexpr (N_OUT == 0) {
-        const uint64_t planes = mode == SQNN_OUT_BF16 ? 1 : A.n_q;       // a warp takes a tile of one plane or of all
-        cut_tiles(A.n_out, &A.KT, &A.W, [&](uint32_t words) {
-            return (A.words64 + 16ull * words - 1) / (16ull * words) * planes <= DECODE_BITS_THREADS / 32 * (uint64_t)sm_count();
-        });
+        const DecodeFor what = mode == SQNN_OUT_BF16 ? DecodeFor::BF16 : clear.batch ? DecodeFor::PRODUCT : DecodeFor::PLANES;
+        const uint32_t planes = mode == SQNN_OUT_BF16 ? 1 : A.n_q;       // a warp takes a tile of one plane or of all
+        cut_decode_tiles(what, A.n_out, A.n_in, A.words64, planes, (uint32_t)sm_count(), DECODE_BITS_THREADS / 32, &A.KT, &A.W);
     }
     if (mode == SQNN_OUT_BITS || mode == SQNN_OUT_SINK) {
         // one block per SM: the tables and one region per warp.  The replicated tables are worth their

@@ -55,15 +55,17 @@ int gemv_shape<SQNN_NO, SQNN_NI>(const DecodeArgs &A0, const uint64_t *d_mask, c
     L.tab_words = A.tab_words;
     L.x_bytes = x_dtype == SQNN_X_BF16 ? 2 : 4;
     L.sms = (uint32_t)sm_count();
-    if (SQNN_NO == 0) cut_tiles(A.n_out, &A.KT, &A.W, [&](uint32_t words) {
-        L.W = words;
-        return covering_tiles(L, (m + L.sms - 1) / L.sms) * L.n_q <= TC_WARPS;
-    });
     L.W = A.W;
     L.density = care_density(A.n_out, A.n_in, (double)patches / slices);
+    GemvLayer Lw = L;
+    GemvTiles tc_tiles{A.KT, A.W}, walk_tiles = tc_tiles;
+    if (SQNN_NO == 0) cut_gemv_tiles(A.n_out, A.n_in, &L, &Lw, &tc_tiles, &walk_tiles);
     const TcPlan tc = plan_gemv_tc(L);
-    const WalkPlan walk = plan_walk(L);
-    if (!take_walk(L, tc, walk))
+    const WalkPlan walk = plan_walk(Lw);
+    const bool expanding = !take_walk(L, tc, walk);
+    A.KT = expanding ? tc_tiles.KT : walk_tiles.KT;
+    A.W = expanding ? tc_tiles.W : walk_tiles.W;
+    if (expanding)
         return tc.ok ? gemv_tc_shape<SQNN_NO, SQNN_NI>(A, tc, d_mask, d_alpha, d_x, x_dtype, ldx, batch, d_y, ldy, m, n, st)
                      : SQNN_E_UNSUPPORTED;                       // one row of bits does not fit
     return x_dtype == SQNN_X_BF16
