@@ -30,9 +30,14 @@ SQNN_FOR_SHAPES(SQNN_DECLARE)
 SQNN_DECLARE(0, 0)
 #undef SQNN_DECLARE
 
-// Up to how many format tiles per SM (bf16 output, us, compile-time shape / run-time shape in parts): 1.2 tiles (2287 x 3943, 200 x 10)
-// 34.9 / 10.5, 2.8 (5516 x 1166, 60 x 12, three planes) 29.5 / 15.9, 3.7 (4544 x 2496, 80 x 8) 14.4 / 10.1, 4.1 (1408 x 4416, 40 x 16)
-// 7.0 / 7.3, 6.9 (2048 x 5120, 40 x 16) 7.3 / 11.7.
+// bf16 weights of a layer with few format tiles: whole tiles (a warp expands all planes of one and writes its 256 n_out weights) leave
+// most warps idle, the parts that the run-time-shape kernels cut do not.  The line lies at four tiles per SM (us, compile-time shape
+// / run-time shape in parts): one plane, 3460 x 1664, 40 x 12, 3.8 tiles 6.7 / 6.4, 4457 x 2496, 80 x 8, 3.8 10.4 / 8.3, 3613 x 7968, 200 x 10, 3.8
+// 19.3 / 14.8; 6.0 tiles 100 x 10 12.1 / 13.3; rows that end inside a lane's weights, 3.8 tiles, three planes 40 x 12 16.3 / 12.1, 200 x 10 33.3 / 23.9, 6.0
+// tiles 16.5 / 19.7 and 44.0 / 45.5; four planes (no compile-time kernel takes them all at once) at 4.0 tiles 40 x 12 64.6 / 29.0, 200 x 10 278 / 110.
+// With two or three planes and rows of whole words the compile-time kernels are ahead earlier, since they request all planes together: three planes
+// at 1.2, 1.8 and 3.6 tiles 40 x 12 8.1 / 7.7, 8.2 / 8.7, 8.0 / 10.4, at 2.4 and 3.6 60 x 12 9.6 / 9.5, 9.9 / 11.0, at 3.0 and 3.6 80 x 16 16.1 / 13.8,
+// 13.7 / 13.6; two at 1.8 and 3.6 40 x 12 7.4 / 7.2, 7.8 / 8.7, at 3.6 60 x 12 9.2 / 9.0.
 constexpr uint64_t SMALL_TILES_PER_SM = 4;
 
 int fill_decode_args(const sqnn_desc *d, const void *d_blob, uint32_t *d_status, DecodeArgs *A)
@@ -189,10 +194,9 @@ static int decode_queue(const sqnn_desc *desc, const void *d_blob, const uint64_
     if (out_bytes < need) return SQNN_E_INVALID_ARG;
     if (mode == SQNN_OUT_BF16 && (!d_mask || !d_alpha)) return SQNN_E_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    // bf16 weights of a small layer: whole format tiles (a warp expands all planes of one and writes its 256 n_out
-    // weights) leave most warps idle, the parts that the run-time-shape kernels cut do not.
-    const uint64_t whole = (A.mn + SQNN_TILE_SLICES * (uint64_t)A.n_out - 1) / (SQNN_TILE_SLICES * (uint64_t)A.n_out);
-    if (mode == SQNN_OUT_BF16 && whole <= SMALL_TILES_PER_SM * (uint64_t)sm_count())
+    const uint64_t whole = (A.mn + SQNN_TILE_SLICES * (uint64_t)A.n_out - 1) / (SQNN_TILE_SLICES * (uint64_t)A.n_out), sms = (uint64_t)sm_count();
+    const bool together = (A.n_q == 2 || A.n_q == 3) && desc->n % 32 == 0;
+    if (mode == SQNN_OUT_BF16 && whole <= SMALL_TILES_PER_SM * sms && (!together || 8 * A.n_q * whole <= A.n_out * sms))
         return decode_shape<0, 0>(A, mode, d_mask, d_alpha, desc->n, d_out, ClearArgs{}, st);
 #define SQNN_DECODE_CASE(NO, NI) \
     if (A.n_out == NO && A.n_in == NI) return decode_shape<NO, NI>(A, mode, d_mask, d_alpha, desc->n, d_out, ClearArgs{}, st);
