@@ -313,8 +313,10 @@ SQNN_DEV void weights16(uint32_t zm, uint32_t qe, const RowValues<IT> &t, uint32
 }
 
 // Run-time shapes: N_IN = 1 says that kernel tiles are parts of format tiles (KT = 0).
-// ENDS: rows may end inside a lane's 32 weights (n no multiple of 32; a kernel of its own, since it costs the others 5 to 15 %).
-template <int N_OUT, int N_IN, int NQ, bool ENDS>
+// ENDS: rows may end inside a lane's 32 weights (n no multiple of 32; kernels of their own, since it costs the others 5 to 15 %).  1: such a lane
+// makes them twice; 2: it goes through them in chunks of 8 and weight by weight, for long rows, where few lanes do and the
+// registers of the other way cost more (LONG_ROWS).
+template <int N_OUT, int N_IN, int NQ, int ENDS>
 __global__ void __launch_bounds__(bf16_threads(N_OUT), 1)
 k_decode_bf16(DecodeArgs A, const uint32_t *__restrict__ mask32, const float *__restrict__ alpha,
               uint64_t n64, __nv_bfloat16 *__restrict__ out)
@@ -392,9 +394,9 @@ k_decode_bf16(DecodeArgs A, const uint32_t *__restrict__ mask32, const float *__
             bool fast = false;
             if constexpr (NQ != 0) {
                 // the next row begins inside the lane's 32 weights
-                const bool next = ENDS && n - c < 32 && at + 32 * lane + (uint32_t)(n - c) < here;
+                const bool next = ENDS == 1 && n - c < 32 && at + 32 * lane + (uint32_t)(n - c) < here;
                 RowValues<IT> t2 = t;
-                if ((!ENDS || n >= 32) && at + 32 * lane < here) {
+                if ((ENDS == 0 || (ENDS == 1 ? n : n - c) >= 32) && at + 32 * lane < here) {
                     if (r != t.row) t = row_values<NQ, IT>(alpha, r);
                     fast = !t.plain;
                     if (next) {
@@ -504,6 +506,11 @@ k_decode_bf16(DecodeArgs A, const uint32_t *__restrict__ mask32, const float *__
 // ------------------------------------------------------------------------------------------
 // launchers
 // ------------------------------------------------------------------------------------------
+// Columns from which on the compile-time shapes up to 128 bits with two or three planes take the plain way through lanes that straddle rows (twice
+// / plain, us: 100 x 10, two, 4115 x 7228 22.2 / 19.9, 7026 x 13601 64.5 / 61.8; 40 x 12, three, 1419 x 6628 12.5 / 11.7; 40 x 16, two, 1121 x 6499
+// 11.9 / 11.1; 80 x 8, two, 21341 x 5172 61.4 / 64.6; 60 x 12, two, 6052 x 4843 18.5 / 19.8).  With one plane the registers suffice: 40 x 12,
+// 1855 x 6535 8.7 / 9.5; 100 x 10, 4465 x 4259 16.7 / 20.3.
+constexpr uint64_t LONG_ROWS = 6144;
 constexpr uint64_t CLEAR_PER_BLOCK = 4096;               // elements of Y that are worth a block
 
 // A layer with fewer tiles than all SMs have warps: as many blocks as SMs with as few warps as that takes.
@@ -582,11 +589,13 @@ inline int launch_decode(const DecodeArgs &A0, sqnn_out_mode mode, const uint64_
         smem = tab + warps * per_warp;
         const uint32_t grid = grid_for(live, warps, 1);
         const bool ends = n % 32 != 0;
+        constexpr bool LONG = N_OUT != 0 && N_OUT <= 128;
 #define SQNN_BF16_LAUNCH2(NQV, PARTSV)                                                                   \
     do {                                                                                                 \
-        return launch_kernel(ends ? k_decode_bf16<N_OUT, N_OUT ? N_IN : PARTSV, NQV, NQV != 0>           \
-                                  : k_decode_bf16<N_OUT, N_OUT ? N_IN : PARTSV, NQV, false>,             \
-                             grid, warps * 32, smem, st, A, (const uint32_t *)d_mask, d_alpha, n, (__nv_bfloat16 *)d_out); \
+        auto k = ends ? k_decode_bf16<N_OUT, N_OUT ? N_IN : PARTSV, NQV, NQV != 0>                       \
+                      : k_decode_bf16<N_OUT, N_OUT ? N_IN : PARTSV, NQV, 0>;                             \
+        if constexpr (LONG && NQV >= 2) if (ends && n >= LONG_ROWS) k = k_decode_bf16<N_OUT, N_IN, NQV, 2>; \
+        return launch_kernel(k, grid, warps * 32, smem, st, A, (const uint32_t *)d_mask, d_alpha, n, (__nv_bfloat16 *)d_out); \
     } while (0)
 #define SQNN_BF16_LAUNCH(NQV)                                                                            \
     do {                                                                                                 \
