@@ -648,7 +648,7 @@ SQNN_DEV void expand_range(const DecodeArgs &A, const RangeTile &T, RangeSeeds &
 // while one walks its lanes' chains of 8, 16 or 32 slices.
 // Before / with parts, us: planes of 223 x 673 with 33 x 20 11.4 / 4.3; bf16 of 1024 x 2560, three planes, 64 x 16 15.7 / 9.9; products
 // of 4864 x 1152 with 128 x 24, batch 129 21.7 / 14.8, of 960 x 1984, two planes, 33 x 20, batch 1 15.5 / 9.8, of 512 x 192 with
-// 200 x 20, batch 35 14.9 / 8.1.  Which layers: most_parts_per_sm, cut_gemv_tiles.  Ends with the warp synchronised.
+// 200 x 20, batch 35 14.9 / 8.1.  Which layers: most_parts_per_sm, plan_run_time_shape.  Ends with the warp synchronised.
 SQNN_DEV void decode_range(const DecodeArgs &A, uint32_t plane, uint64_t ktile, uint32_t *region, const uint32_t *tab, uint32_t lane)
 {
     const PlanePtrs &P = A.pl[plane];

@@ -14,7 +14,7 @@
 //   2048 x 1024, 7 % kept 5.7 / 4.4 us     1024 x 3072, 7 % kept 6.1 / 4.8     4096 x 9216, 9 % kept 9.8 / 11.5
 // Over 1048 random calls of that kind (2^16 to 2^26 weights, 2 to 50 % kept, 1 to 15 vectors), all in whole format tiles, the rule takes 172 to the
 // walk; none loses more than 5 %, and all 1048 together gain 3 % (geometric mean), where always choosing right
-// would gain 4 %.  Layers of run-time shapes that have room for parts: cut_gemv_tiles.
+// would gain 4 %.  Layers of run-time shapes that have room for parts: plan_run_time_shape.
 // The walk is also faster on sparse or wide layers with fp32 activations or several planes (2048 x 1024, 3.5 % kept, 8
 // fp32 vectors: 10.2 / 7.5 us; 4096 x 12288, 10 % kept, 4 fp32 vectors, where the expanding form runs out of shared
 // memory: 67 / 36).  It does not get those calls: its sums lie further from the 64-bit product.  Relative errors over
@@ -231,24 +231,45 @@ inline WalkPlan plan_walk(const GemvLayer &L)
 struct GemvTiles {
     uint32_t KT, W;
 };
-inline void cut_gemv_tiles(uint32_t n_out, uint32_t n_in, GemvLayer *expanding, GemvLayer *walk, GemvTiles *for_expanding, GemvTiles *for_walk)
+// Cuts the tiles of one form to at most `most` turns; L gets their words and, at turn_us a turn, the estimate of a part.
+inline GemvTiles cut_gemv_tiles(uint32_t n_out, uint32_t most, double turn_us, GemvLayer *L)
 {
-    const GemvTiles whole{format_tiles_per_kernel_tile(n_out), expanding->W};
-    const bool cheap = table_chunks(n_in, entry_words_padded(n_out)) == 1 && whole.KT < 4;
-    auto cut = [&](GemvLayer *L, GemvTiles *T, uint32_t most, double turn_us) {
-        *T = whole;
-        const uint32_t turns = cut_tiles(n_out, most, &T->KT, &T->W, [&](uint32_t words) {
-            GemvLayer M = *L;
-            M.W = words;
-            return covering_tiles(M, (L->m + L->sms - 1) / L->sms) * L->n_q <= TC_WARPS;
-        });
-        L->W = T->W;
-        L->tile_us = turns * turn_us;
-    };
-    const uint32_t most = most_turns(n_out);
-    cut(expanding, for_expanding, cheap && whole.KT < most ? whole.KT : most, 0.8);
-    cut(walk, for_walk, cheap && whole.KT == 1 ? 0 : cheap && whole.KT < most ? whole.KT : most, 0.7);
-    if (for_expanding->KT == 0 && for_walk->KT != 0) walk->tile_us = 0.02 * whole.W;
+    GemvTiles t{format_tiles_per_kernel_tile(n_out), L->W};
+    const uint32_t turns = cut_tiles(n_out, most, &t.KT, &t.W, [&](uint32_t words) {
+        GemvLayer M = *L;
+        M.W = words;
+        return covering_tiles(M, (L->m + L->sms - 1) / L->sms) * L->n_q <= TC_WARPS;
+    });
+    L->W = t.W;
+    L->tile_us = turns * turn_us;
+    return t;
+}
+struct GemvForms {
+    TcPlan tc;
+    WalkPlan walk;
+    GemvTiles tc_tiles, walk_tiles;
+};
+inline GemvForms plan_run_time_shape(uint32_t n_out, uint32_t n_in, const GemvLayer &whole)
+{
+    const uint32_t KT = format_tiles_per_kernel_tile(n_out), most = most_turns(n_out);
+    const bool cheap = table_chunks(n_in, entry_words_padded(n_out)) == 1 && KT < 4;
+    const uint32_t few = cheap && KT < most ? KT : most;
+    GemvForms f;
+    GemvLayer L = whole, Lw = whole;
+    f.tc_tiles = cut_gemv_tiles(n_out, most, 0.8, &L);
+    f.tc = plan_gemv_tc(L);
+    f.walk_tiles = cut_gemv_tiles(n_out, most, 0.7, &Lw);
+    f.walk = plan_walk(Lw);
+    if (!cheap) return f;
+    // ... as long as the larger tiles take nothing else away: eight planes of them may leave less room for rows, vectors or activations, or none
+    L = Lw = whole;
+    const GemvTiles t = cut_gemv_tiles(n_out, few, 0.8, &L), w = cut_gemv_tiles(n_out, KT == 1 ? 0 : few, 0.7, &Lw);
+    if (t.KT == 0 && w.KT != 0) Lw.tile_us = 0.02 * Lw.W;
+    const TcPlan tc = plan_gemv_tc(L);
+    const WalkPlan walk = plan_walk(Lw);
+    if (tc.ok && tc.rows_per_chunk == f.tc.rows_per_chunk && tc.bt == f.tc.bt) { f.tc = tc; f.tc_tiles = t; }
+    if (walk.ok && walk.rows_per_chunk == f.walk.rows_per_chunk && walk.xs == f.walk.xs) { f.walk = walk; f.walk_tiles = w; }
+    return f;
 }
 
 inline bool take_walk(const GemvLayer &L, const TcPlan &t, const WalkPlan &w)

@@ -57,20 +57,17 @@ int gemv_shape<SQNN_NO, SQNN_NI>(const DecodeArgs &A0, const uint64_t *d_mask, c
     L.sms = (uint32_t)sm_count();
     L.W = A.W;
     L.density = care_density(A.n_out, A.n_in, (double)patches / slices);
-    GemvLayer Lw = L;
-    GemvTiles tc_tiles{A.KT, A.W}, walk_tiles = tc_tiles;
-    if (SQNN_NO == 0) cut_gemv_tiles(A.n_out, A.n_in, &L, &Lw, &tc_tiles, &walk_tiles);
-    const TcPlan tc = plan_gemv_tc(L);
-    const WalkPlan walk = plan_walk(Lw);
-    const bool expanding = !take_walk(L, tc, walk);
-    A.KT = expanding ? tc_tiles.KT : walk_tiles.KT;
-    A.W = expanding ? tc_tiles.W : walk_tiles.W;
+    const GemvTiles own{A.KT, A.W};
+    const GemvForms f = SQNN_NO == 0 ? plan_run_time_shape(A.n_out, A.n_in, L) : GemvForms{plan_gemv_tc(L), plan_walk(L), own, own};
+    const bool expanding = !take_walk(L, f.tc, f.walk);
+    A.KT = expanding ? f.tc_tiles.KT : f.walk_tiles.KT;
+    A.W = expanding ? f.tc_tiles.W : f.walk_tiles.W;
     if (expanding)
-        return tc.ok ? gemv_tc_shape<SQNN_NO, SQNN_NI>(A, tc, d_mask, d_alpha, d_x, x_dtype, ldx, batch, d_y, ldy, m, n, st)
-                     : SQNN_E_UNSUPPORTED;                       // one row of bits does not fit
+        return f.tc.ok ? gemv_tc_shape<SQNN_NO, SQNN_NI>(A, f.tc, d_mask, d_alpha, d_x, x_dtype, ldx, batch, d_y, ldy, m, n, st)
+                       : SQNN_E_UNSUPPORTED;                       // one row of bits does not fit
     return x_dtype == SQNN_X_BF16
-        ? launch_gemv<SQNN_NO, SQNN_NI, __nv_bfloat16>(A, walk, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st)
-        : launch_gemv<SQNN_NO, SQNN_NI, float>(A, walk, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st);
+        ? launch_gemv<SQNN_NO, SQNN_NI, __nv_bfloat16>(A, f.walk, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st)
+        : launch_gemv<SQNN_NO, SQNN_NI, float>(A, f.walk, d_mask, d_alpha, d_x, ldx, batch, d_y, ldy, m, n, st);
 }
 #endif
 #endif

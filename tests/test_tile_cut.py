@@ -51,12 +51,17 @@ int main()
             const unsigned turns = cut_decode_tiles(what, n_out, n_in, (m * n + 63) / 64, what == DecodeFor::BF16 ? 1 : n_q, sms, decode_warps, &KT, &W);
             std::printf("%u %u %u ", turns, KT, W);
         }
-        GemvLayer e, w;
-        e.m = m; e.n = n; e.n_q = n_q; e.sms = sms; e.W = whole_words;
-        w = e;
-        GemvTiles te, tw;
-        cut_gemv_tiles(n_out, n_in, &e, &w, &te, &tw);
-        std::printf("%u %u %u %u %u %u ", te.KT ? 0 : (unsigned)(e.tile_us / 0.8 + 0.5), te.KT, e.W, tw.KT ? 0 : (unsigned)(w.tile_us / 0.7 + 0.5), tw.KT, w.W);
+        GemvLayer L;
+        L.m = m; L.n = n; L.n_q = n_q; L.sms = sms; L.W = whole_words;
+        L.batch = 1; L.x_bytes = 2; L.tab_words = table_words(n_out, n_in); L.density = 0.1;
+        const GemvForms f = plan_run_time_shape(n_out, n_in, L);
+        for (const GemvTiles &t : {f.tc_tiles, f.walk_tiles}) {
+            unsigned turns = 0;
+            for (unsigned k = 1; t.KT == 0 && turns == 0; ++k) if (range_words(n_out, k) == t.W) turns = k;
+            std::printf("%u %u %u ", turns, t.KT, t.W);
+        }
+        // whether a row fits: the two forms with whole tiles, and as cut
+        std::printf("%u %u %u %u ", plan_gemv_tc(L).ok, f.tc.ok, plan_walk(L).ok, f.walk.ok);
         for (unsigned turns = 1; turns <= 10; ++turns) std::printf("%u ", range_words(n_out, turns));
         std::printf("\n");
     }
@@ -75,15 +80,15 @@ def cuts(tmp_path_factory):
     def run(layers):
         text = "\n".join(f"{n_out} {n_in} {m} {n} {n_q} {SMS} {DECODE_WARPS}" for n_out, n_in, m, n, _, n_q in layers)
         rows = [[int(x) for x in line.split()] for line in subprocess.run([exe], input=text, capture_output=True, text=True, check=True).stdout.splitlines()]
-        return [([tuple(r[3 * i:3 * i + 3]) for i in range(5)], r[15:]) for r in rows]
+        return [([tuple(r[3 * i:3 * i + 3]) for i in range(5)], r[19:], r[15:19]) for r in rows]
     return run
 
 
 def test_the_layers_below_are_cut_as_they_are_meant_to_be(cuts):
-    for (case, turns), (got, words) in zip(PARTS, cuts([c for c, _ in PARTS])):
+    for (case, turns), (got, words, _) in zip(PARTS, cuts([c for c, _ in PARTS])):
         for want, (t, kt, w) in zip(turns, got):
             assert t == want and (kt == 0) == (want > 0) and (want == 0 or w == words[want - 1]), (case, turns, got)
-    for case, (got, _) in zip(WHOLE, cuts(WHOLE)):
+    for case, (got, *_) in zip(WHOLE, cuts(WHOLE)):
         assert all(kt != 0 for _, kt, _ in got), (case, got)
 
 
@@ -99,14 +104,21 @@ TIMED = [
 
 
 def test_calls_that_whole_tiles_take_less_time_for_are_not_cut(cuts):
-    for (case, what, turns), (got, _) in zip(TIMED, cuts([c for c, _, _ in TIMED])):
+    for (case, what, turns), (got, *_) in zip(TIMED, cuts([c for c, _, _ in TIMED])):
         assert got[what][0] == turns, (case, what, turns, got)
+
+
+def test_rows_that_fit_in_parts_only_get_them_whatever_whole_tiles_would_cost(cuts):
+    """Eight planes of 254-bit slices: two whole tiles (16 KB each) of every plane and the mask do not fit an SM's shared memory."""
+    [(got, _, (tc_whole, tc, walk_whole, walk))] = cuts([(254, 8, 100, 20000, 0.05, 8)])
+    assert (tc_whole, tc, walk_whole, walk) == (0, 1, 0, 1)
+    assert got[3][1] == got[4][1] == 0
 
 
 def test_a_part_of_t_turns_overlaps_no_more_than_32_t_slices(cuts):
     """Wherever it starts.  (One word per lane is the least, so slices of less than 33 bits may need more than one turn for it.)"""
     layers = [(n_out, 1, 100, 100, 0.1, 1) for n_out in range(1, 257)]
-    for (n_out, *_), (_, words) in zip(layers, cuts(layers)):
+    for (n_out, *_), (_, words, _) in zip(layers, cuts(layers)):
         for turns in range(1, 11):
             w = words[turns - 1]
             if w == 1 and 1024 > (32 * turns - 1) * n_out:
@@ -144,6 +156,18 @@ def check(layer, bf16=True, products=((1, "bfloat16"), (3, "float32"), (16, "bfl
 def test_run_time_shapes_in_parts_of_many_turns_and_in_whole_tiles(case):
     n_out, n_in, m, n, keep, n_q = case
     check(generic_layer(n_out, n_in, m, n, keep, 80 + n_out, n_q=n_q))
+
+
+@pytest.mark.gpu
+def test_small_batch_product_of_rows_that_fit_in_parts_only():
+    import torch
+    layer = generic_layer(254, 8, 3, 20000, 0.05, 79, n_q=8)
+    ref = H.oracle_decode(layer, H.oracle_encode(layer))
+    dev = H.DeviceLayer(layer, H.blob_from_library(layer)[0])
+    for batch, dtype in ((1, torch.bfloat16), (2, torch.float32)):
+        x = torch.randn((batch, layer.n), generator=torch.Generator().manual_seed(batch)).to(dtype).float().numpy()
+        assert H.rel_err(dev.matmul(x, dtype), orc.matmul(ref, layer.mask, layer.alpha, x.astype(np.float64))) <= 1e-4
+    assert dev.status_value() == 0
 
 
 # bf16 weights of the shapes with compile-time kernels: in parts (the first), and with more than four format tiles per SM, where their own kernels
