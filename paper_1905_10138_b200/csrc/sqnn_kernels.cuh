@@ -244,7 +244,7 @@ SQNN_DEV void stage_mask(uint32_t *mask_s, const uint32_t *__restrict__ mask32, 
 // multiply-add with V / 2 does the rest.  Selectors and those numbers come out of words in which even and odd
 // columns have been separated, by a shift and an AND each: 3 instructions per weight with three planes.  What surrounds
 // that -- words, separation, staging, copies, row bookkeeping -- takes nearly four more: 2^26 weights of three planes
-// take 37 us and 22.0 M warp instructions, of which 7.7 M are the decode.  (Sums of the scales per weight took about 20
+// take 37 us and 21.8 M warp instructions, of which 7.3 M are the decode.  (Sums of the scales per weight took about 20
 // instructions, and 64 us.)  Negating all terms of a sum
 // negates it exactly, except when it is zero or not finite, and halving is exact except for the tiniest
 // numbers; rows with such a value take the plain loop, as do rows of less than 32 weights and layers of four and
